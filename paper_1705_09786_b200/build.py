@@ -6,7 +6,8 @@ _DIR = os.path.dirname(os.path.abspath(__file__))
 SRC = os.path.join(_DIR, "csrc", "ampnet.cu")
 SRC_HOST = os.path.join(_DIR, "csrc", "ir_builders.cpp")
 SRC_DIRECT = os.path.join(_DIR, "csrc", "engine_fast.cu")
-DEPS = [SRC, SRC_HOST, SRC_DIRECT, os.path.join(_DIR, "csrc", "engine.cuh"), os.path.join(_DIR, "csrc", "engine_types.h"),
+SRC_WAVE = [os.path.join(_DIR, "csrc", f) for f in ("wave_engine.cu", "wave_encode.cu")]
+DEPS = [SRC, SRC_HOST, SRC_DIRECT, *SRC_WAVE, os.path.join(_DIR, "csrc", "engine.cuh"), os.path.join(_DIR, "csrc", "engine_types.h"),
         os.path.join(os.path.dirname(_DIR), "include", "ampnet.h")]
 LIB = os.path.join(_DIR, "libampnet.so")
 
@@ -21,7 +22,7 @@ def build(force=False, verbose=False):
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
     tmp = LIB + f".tmp{os.getpid()}"
     cmd = [nvcc, "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
-           "-Xcompiler", "-fPIC", "-shared", "-o", tmp, SRC, SRC_DIRECT, SRC_HOST]
+           "-Xcompiler", "-fPIC", "-shared", "-o", tmp, SRC, SRC_DIRECT, *SRC_WAVE, SRC_HOST]
     if verbose:
         cmd.insert(1, "-Xptxas=-v")
     subprocess.check_call(cmd)

@@ -15,6 +15,7 @@
 
 #include "../../include/ampnet.h"
 #include "engine.cuh"
+#include "wave.h"
 
 using namespace amp;
 
@@ -30,6 +31,8 @@ extern "C" cudaError_t ampnet_direct_static_smem(size_t* bytes);
 extern "C" cudaError_t ampnet_direct_launch(const amp::Ctx* ctx, int n_ctas, size_t smem_bytes, cudaStream_t stream, int n_sms);
 
 namespace {
+
+constexpr size_t STAGE_BYTES = 256 << 10;
 
 struct DeviceArena {           // one allocation carved into aligned pieces
   char* base = nullptr;
@@ -49,6 +52,8 @@ struct HostDataset {
   int maxT = 1, maxM = 1, maxN = 1, maxD = 1, maxDc = 1, maxIn = 1, maxOut = 1, maxL = 1;
   long long total_pos = 0, total_edges = 0;
   DevInst dev{};
+  wave::WaveData wave;                  // message programs of the scheduled engine
+  std::pair<wave::WavePlanKey, wave::WavePlan> wave_plan[2];      // last placement: training, evaluation
   std::vector<void*> allocs;
 };
 
@@ -110,6 +115,11 @@ struct ampnet_graph {
   bool have_run = false;
   bool arenas_lent = false;           // the arenas belong to the caller of execute() (static scratch): never freed or grown
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
+  wave::WaveModel wave;                 // scheduled engine: the graph's cells and encoder tables
+  void* enc_scratch = nullptr; size_t enc_scratch_cap = 0;
+  char* stage = nullptr; size_t stage_used = 0;              // pinned: small arrays on their way to the device, where their addresses go
+  std::vector<std::pair<const void**, size_t>> staged;
+  char* host_read = nullptr; size_t host_read_cap = 0;       // pinned: what a run reads back
 };
 
 // FP32 FMA issue rate of the device, measured: every thread runs 16 independent FMA chains from registers.
@@ -190,22 +200,35 @@ int j_bucket(int in) {
   return -1;
 }
 
-template <class T>
-ampnet_status_t upload(ampnet_graph* g, HostDataset& D, const std::vector<T>& h, const T** out) {
-  void* p = dev_alloc(g, std::max<size_t>(h.size(), 1) * sizeof(T));
-  if (!p) return set_err(g, AMPNET_ENOMEM, "device allocation of %zu bytes failed", h.size() * sizeof(T));
-  D.allocs.push_back(p);
-  if (!h.empty()) CUDA_TRY(g, cudaMemcpyAsync(p, h.data(), h.size() * sizeof(T), cudaMemcpyHostToDevice, g->stream));
-  *out = reinterpret_cast<const T*>(p);
-  return AMPNET_OK;
-}
+// Arrays of a data set on their way to the device: small ones are collected in pinned memory and travel in one copy into one
+// allocation (a request of a few instances would otherwise pay for each), large ones go directly.
 template <class T>
 ampnet_status_t upload_raw(ampnet_graph* g, HostDataset& D, const T* h, size_t n, const T** out) {
-  void* p = dev_alloc(g, std::max<size_t>(n, 1) * sizeof(T));
+  const size_t bytes = std::max<size_t>(n, 1) * sizeof(T), at = (g->stage_used + 255) & ~(size_t)255;
+  if (g->stage && at + bytes <= STAGE_BYTES) {
+    if (n) std::memcpy(g->stage + at, h, n * sizeof(T));
+    g->stage_used = at + bytes;
+    g->staged.push_back({reinterpret_cast<const void**>(out), at});
+    return AMPNET_OK;
+  }
+  void* p = dev_alloc(g, bytes);
   if (!p) return set_err(g, AMPNET_ENOMEM, "device allocation of %zu bytes failed", n * sizeof(T));
   D.allocs.push_back(p);
   if (n) CUDA_TRY(g, cudaMemcpyAsync(p, h, n * sizeof(T), cudaMemcpyHostToDevice, g->stream));
   *out = reinterpret_cast<const T*>(p);
+  return AMPNET_OK;
+}
+template <class T>
+ampnet_status_t upload(ampnet_graph* g, HostDataset& D, const std::vector<T>& h, const T** out) { return upload_raw(g, D, h.data(), h.size(), out); }
+ampnet_status_t flush_uploads(ampnet_graph* g, HostDataset& D) {
+  if (g->staged.empty()) return AMPNET_OK;
+  char* p = (char*)dev_alloc(g, g->stage_used);
+  if (!p) return set_err(g, AMPNET_ENOMEM, "device allocation of %zu bytes failed", g->stage_used);
+  D.allocs.push_back(p);
+  CUDA_TRY(g, cudaMemcpyAsync(p, g->stage, g->stage_used, cudaMemcpyHostToDevice, g->stream));
+  for (auto& s : g->staged) *s.first = p + s.second;
+  g->staged.clear();
+  g->stage_used = 0;
   return AMPNET_OK;
 }
 
@@ -556,6 +579,8 @@ ampnet_status_t place(ampnet_graph* g, int n_ctas, int max_batch_rows, std::vect
   }
   return AMPNET_OK;
 }
+
+#include "wave_host.cuh"
 
 // ---- direct-delivery engine: which graphs it takes, and its placement -------------------------------------
 // It runs asynchronous epochs of graphs whose messages are single rows and whose parameter-free chains it can resolve
@@ -1025,6 +1050,106 @@ ampnet_status_t ensure_arenas(ampnet_graph* g, size_t ctl_need, size_t bulk_need
   return AMPNET_OK;
 }
 
+// Pinned memory for what a run reads back; sized when instances are loaded, so that no run allocates it.
+ampnet_status_t ensure_host_read(ampnet_graph* g, size_t bytes) {
+  if (bytes <= g->host_read_cap) return AMPNET_OK;
+  if (g->host_read) cudaFreeHost(g->host_read);
+  g->host_read = nullptr; g->host_read_cap = 0;
+  CUDA_TRY(g, cudaMallocHost((void**)&g->host_read, bytes));
+  g->host_read_cap = bytes;
+  return AMPNET_OK;
+}
+
+// Results of a run from the device's counters, and its status.
+ampnet_status_t report_run(ampnet_graph* g, const Globals& G, float ms, long long n_order, ampnet_epoch_stats_t* out, double* accuracy, ampnet_inference_stats_t* inference) {
+  if (out) {
+    std::memset(out, 0, sizeof *out);
+    out->instances = n_order; out->node_messages = (int64_t)G.node_messages; out->rounds = (int64_t)G.rounds;
+    out->seconds = ms * 1e-3; const long long n_train = n_order - (long long)G.inf_instances;
+    out->mean_loss = n_train > 0 ? G.total_loss / (double)n_train : 0.0;
+    out->max_active_observed = G.max_active; out->route_hash = G.route_hash;
+    for (auto& s : g->last_stats) {
+      out->ppt_messages += (int64_t)s.msgs; out->max_staleness = std::max(out->max_staleness, s.max_staleness);
+      out->micro_batches += (int64_t)s.batches; out->micro_batch_rows += (int64_t)s.batch_rows;
+    }
+  }
+  if (accuracy) *accuracy = G.n_pred ? (double)G.correct / (double)G.n_pred : 0.0;
+  if (inference) {
+    inference->instances = (int64_t)G.inf_instances;
+    inference->mean_loss = G.inf_instances ? G.inf_loss / (double)G.inf_instances : 0.0;
+    inference->accuracy = G.inf_pred ? (double)G.inf_correct / (double)G.inf_pred : 0.0;
+  }
+  if (G.status == ST_TIMEOUT) return set_err(g, AMPNET_ETIMEOUT, "a bounded device wait gave up (node %d, detail %d)", G.err_node, G.err_detail);
+  if (G.status == ST_OVERFLOW) return set_err(g, AMPNET_EOVERFLOW, "a queue / cache / key-space bound was exceeded (node %d, detail %d)", G.err_node, G.err_detail);
+  if (G.status != 0) return set_err(g, AMPNET_ECUDA, "device status %d", G.status);
+  return AMPNET_OK;
+}
+
+// The scheduled engine takes asynchronous runs of the graphs it has programs for, if its cells find room.
+bool wave_takes(ampnet_graph* g, HostDataset& D, int mak, int det, int eval, const ampnet_run_cfg_t* cfg, long long n_order, WavePlan& P) {
+  if (det || n_order < 1 || (cfg && cfg->max_batch_rows > 0)) return false;
+  if (const char* e = getenv("AMPNET_ENGINE")) if (strcmp(e, "scheduled")) return false;
+  if (const char* e = getenv("AMPNET_TUNE")) if (atoi(e) & (16 | 32 | 8)) return false;
+  // (the placement of the last run of this kind still holds if nothing it depends on has changed)
+  const char* env[3] = {getenv("AMPNET_DIRECT_ROWS"), getenv("AMPNET_DIRECT_COLS"), getenv("AMPNET_TENSOR_CORES")};
+  const int n_ctas = cfg && cfg->n_ctas > 0 ? std::min(cfg->n_ctas, g->n_sms) : g->n_sms;
+  wave::WavePlanKey key{D.wave.load_id, n_order, mak, cfg ? cfg->min_update_frequency : 1, eval, n_ctas, {env[0] ? atoi(env[0]) : -1, env[1] ? atoi(env[1]) : -1, env[2] ? atoi(env[2]) : -1}};
+  auto& slot = D.wave_plan[eval ? 1 : 0];
+  if (!(slot.first == key)) { slot.first = key; slot.second = wave_place(g, g->wave, D.wave, mak, key.muf, eval != 0, n_order, D.n, n_ctas); }
+  P = slot.second;
+  return P.ok;
+}
+
+ampnet_status_t wave_execute(ampnet_graph* g, HostDataset& D, const WavePlan& P, int mak, int eval, const ampnet_run_cfg_t* cfg, const long long* order, long long n_order,
+                             ampnet_epoch_stats_t* out, float* per_instance_loss, double* accuracy, const uint8_t* inference_only, ampnet_inference_stats_t* inference) {
+  wave::Run R;
+  const size_t order_bytes = order ? (size_t)n_order * sizeof(long long) : 0, mask_bytes = inference_only ? (size_t)D.n : 0;
+  wave_carve(g, D, g->wave, D.wave, P, mak, eval, cfg, n_order, true, R);
+  ampnet_status_t st = ensure_arenas(g, g->ctl.used, g->bulk.used + order_bytes + mask_bytes + BULK_EXTRA);
+  if (st != AMPNET_OK) return st;
+  const WaveScratch S = wave_carve(g, D, g->wave, D.wave, P, mak, eval, cfg, n_order, false, R);
+  if (order) { long long* d = g->bulk.take<long long>((size_t)n_order); CUDA_TRY(g, cudaMemcpyAsync(d, order, order_bytes, cudaMemcpyHostToDevice, g->stream)); R.core.order = d; }
+  if (inference_only) { unsigned char* d = g->bulk.take<unsigned char>(mask_bytes); CUDA_TRY(g, cudaMemcpyAsync(d, inference_only, mask_bytes, cudaMemcpyHostToDevice, g->stream)); R.core.inference_only = d; }
+  if ((st = ensure_host_read(g, S.read_bytes)) != AMPNET_OK) return st;
+  CUDA_TRY(g, cudaMemsetAsync(g->ctl_mem, 0, S.zero_bytes, g->stream));
+  for (auto& z : g->zero_regions) CUDA_TRY(g, cudaMemsetAsync(z.first, 0, z.second, g->stream));
+  if (getenv("AMPNET_DEBUG")) {
+    fprintf(stderr, "[ampnet] scheduled engine, %d CTAs, %zu B smem, ctl %zu B, bulk %zu B, arena %u x 16 B x %d x %d\n", P.n_ctas, P.smem, g->ctl.used, g->bulk.used, R.core.slot4, mak, R.core.copies);
+    static const char* names[] = {"LOOKUP_F", "LOOKUP_B", "LIN_F", "LIN_DX", "ACC", "HEAD", "GRU_ZR", "GRU_C", "GRU_DC", "GRU_DZR"};
+    for (auto& t : P.teams) fprintf(stderr, "[ampnet]   node %2d %-8s %3d CTAs = %d tiles x %d shards, R %d C %d BM %d%s, est %.0f cycles\n", g->ppts[t.t.ppt].node, names[t.t.kind], t.t.n, t.t.T, t.t.Sh, t.t.R, t.t.C, t.t.BM, t.t.bf16_tc ? " tc" : "", t.cycles);
+  }
+  for (auto& H : g->ppts) { H.LT = 1; }
+  for (auto& t : P.teams) { HostPPT& H = g->ppts[t.t.ppt]; if (t.t.kind == wave::LIN_F || t.t.kind == wave::HEAD || t.t.kind == wave::GRU_ZR || t.t.kind == wave::LOOKUP_F) { H.T = t.t.n; H.BM = t.t.BM; } }
+  CUDA_TRY(g, cudaEventRecord(g->ev0, g->stream));
+  const cudaError_t le = wave::launch(&R, P.n_ctas, P.smem, g->stream);
+  if (le != cudaSuccess) return set_err(g, AMPNET_ECUDA, "launch of the scheduled engine failed: %s", cudaGetErrorString(le));
+  CUDA_TRY(g, cudaEventRecord(g->ev1, g->stream));
+  CUDA_TRY(g, cudaMemcpyAsync(g->host_read, g->ctl_mem, S.read_bytes, cudaMemcpyDeviceToHost, g->stream));
+  CUDA_TRY(g, cudaStreamSynchronize(g->stream));
+  Globals G;
+  std::memcpy(&G, g->host_read, sizeof G);
+  g->last_stats.resize(g->ppts.size());
+  std::memcpy(g->last_stats.data(), g->host_read + S.stats_at, g->ppts.size() * sizeof(PPTStats));
+  g->last_node_msgs.resize(g->hnodes.size() * 2);
+  std::memcpy(g->last_node_msgs.data(), g->host_read + S.node_msgs_at, g->last_node_msgs.size() * sizeof(unsigned long long));
+  if (per_instance_loss) std::memcpy(per_instance_loss, g->host_read + S.loss_at, (size_t)D.n * sizeof(float));
+  if (getenv("AMPNET_DEBUG")) {
+    const unsigned long long* ph = reinterpret_cast<const unsigned long long*>(g->host_read + S.phases_at);
+    for (size_t k = 0; k < P.teams.size(); k++) {
+      fprintf(stderr, "[ampnet]   team %2zu kind %d node %2d cycles/round:", k, P.teams[k].t.kind, g->ppts[P.teams[k].t.ppt].node);
+      for (int q = 0; q < wave::N_PHASES; q++) fprintf(stderr, " %8.0f", (double)ph[k * wave::N_PHASES + q] / std::max<double>(1, (double)G.rounds));
+      fprintf(stderr, "\n");
+    }
+    fprintf(stderr, "[ampnet]   rounds %llu\n", (unsigned long long)G.rounds);
+  }
+  g->have_run = true;
+  g->n_keylog = 0;
+  if (!eval) for (size_t p = 0; p < g->ppts.size(); p++) g->ppts[p].opt_t += (long long)g->last_stats[p].n_updates;
+  float ms = 0;
+  CUDA_TRY(g, cudaEventElapsedTime(&ms, g->ev0, g->ev1));
+  return report_run(g, G, ms, n_order, out, accuracy, inference);
+}
+
 ampnet_status_t execute(ampnet_graph* g, int split, int mak, int det, int eval, const ampnet_run_cfg_t* cfg,
                         ampnet_epoch_stats_t* out, float* per_instance_loss, double* accuracy,
                         const uint8_t* inference_only = nullptr, ampnet_inference_stats_t* inference = nullptr) {
@@ -1043,8 +1168,10 @@ ampnet_status_t execute(ampnet_graph* g, int split, int mak, int det, int eval, 
   if (det && n_order >= (1ll << 24)) return set_err(g, AMPNET_EINVAL, "the deterministic schedule supports fewer than 2^24 instances per epoch");
   const bool dbg = getenv("AMPNET_DEBUG") != nullptr;
   CUDA_TRY(g, cudaSetDevice(g->device));
-  RunPlan R;
   g->have_run = false;                // planning re-targets the statistics pointers: the previous run's are gone from here on
+  WavePlan wp;
+  if (wave_takes(g, D, mak, det, eval, cfg, n_order, wp)) return wave_execute(g, D, wp, mak, eval, cfg, order, n_order, out, per_instance_loss, accuracy, inference_only, inference);
+  RunPlan R;
   if (dbg) fprintf(stderr, "[ampnet] planning\n");
   ampnet_status_t st = plan_run(g, split, mak, det, eval, cfg, n_order, true, R);
   if (st != AMPNET_OK) return st;
@@ -1138,27 +1265,7 @@ ampnet_status_t execute(ampnet_graph* g, int split, int mak, int det, int eval, 
     if (g->ctl_trials == 2) g->ctl_rate[0] = (double)G.node_messages / ms;
     if (g->ctl_trials == 3) { g->ctl_rate[1] = (double)G.node_messages / ms; g->ctl_choice = g->ctl_rate[1] > 1.03 * g->ctl_rate[0] ? 1 : 0; }
   }
-  if (out) {
-    std::memset(out, 0, sizeof *out);
-    out->instances = n_order; out->node_messages = (int64_t)G.node_messages; out->rounds = (int64_t)G.rounds;
-    out->seconds = ms * 1e-3; const long long n_train = n_order - (long long)G.inf_instances;
-    out->mean_loss = n_train > 0 ? G.total_loss / (double)n_train : 0.0;
-    out->max_active_observed = G.max_active; out->route_hash = G.route_hash;
-    for (auto& s : g->last_stats) {
-      out->ppt_messages += (int64_t)s.msgs; out->max_staleness = std::max(out->max_staleness, s.max_staleness);
-      out->micro_batches += (int64_t)s.batches; out->micro_batch_rows += (int64_t)s.batch_rows;
-    }
-  }
-  if (accuracy) *accuracy = G.n_pred ? (double)G.correct / (double)G.n_pred : 0.0;
-  if (inference) {
-    inference->instances = (int64_t)G.inf_instances;
-    inference->mean_loss = G.inf_instances ? G.inf_loss / (double)G.inf_instances : 0.0;
-    inference->accuracy = G.inf_pred ? (double)G.inf_correct / (double)G.inf_pred : 0.0;
-  }
-  if (G.status == ST_TIMEOUT) return set_err(g, AMPNET_ETIMEOUT, "a bounded device wait gave up (node %d, detail %d)", G.err_node, G.err_detail);
-  if (G.status == ST_OVERFLOW) return set_err(g, AMPNET_EOVERFLOW, "a queue / cache / key-space bound was exceeded (node %d, detail %d)", G.err_node, G.err_detail);
-  if (G.status != 0) return set_err(g, AMPNET_ECUDA, "device status %d", G.status);
-  return AMPNET_OK;
+  return report_run(g, G, ms, n_order, out, accuracy, inference);
 }
 
 }  // namespace
@@ -1192,6 +1299,11 @@ ampnet_status_t ampnet_graph_create(const ampnet_ir_desc_t* ir, uint64_t init_se
   }
   if (st == AMPNET_OK) st = build_topology(g);
   if (st == AMPNET_OK) st = create_params(g, init_seed);
+  if (st == AMPNET_OK) {
+    std::vector<int> pn;
+    for (auto& P : g->ppts) pn.push_back(P.node);
+    wave_model(g->hnodes, g->sources, g->has_it ? g->it_steps + 1 : 1, g->payload_bf16, g->wave, pn);
+  }
   if (st == AMPNET_OK && (cudaEventCreate(&g->ev0) != cudaSuccess || cudaEventCreate(&g->ev1) != cudaSuccess)) st = AMPNET_ECUDA;
   if (st != AMPNET_OK) {
     // keep the message readable through a static buffer: the handle is not returned
@@ -1212,6 +1324,9 @@ void ampnet_graph_destroy(ampnet_graph_t* g) {
   free_dataset(g, g->data[1]);
   dev_free(g, g->ctl_alloc);
   dev_free(g, g->bulk_mem);
+  dev_free(g, g->enc_scratch);
+  if (g->host_read) cudaFreeHost(g->host_read);
+  if (g->stage) cudaFreeHost(g->stage);
   if (g->ev0) cudaEventDestroy(g->ev0);
   if (g->ev1) cudaEventDestroy(g->ev1);
   delete g;
@@ -1301,6 +1416,8 @@ ampnet_status_t ampnet_load_instances(ampnet_graph_t* g, int32_t split, const am
   CUDA_TRY(g, cudaSetDevice(g->device));
   CUDA_TRY(g, cudaStreamSynchronize(g->stream));
   free_dataset(g, g->data[split]);
+  g->staged.clear(); g->stage_used = 0;
+  if (!g->stage) CUDA_TRY(g, cudaMallocHost((void**)&g->stage, STAGE_BYTES));
   HostDataset& D = g->data[split];
   const long long n = in->n_instances;
   D.kind = in->kind; D.n = n;
@@ -1443,6 +1560,10 @@ ampnet_status_t ampnet_load_instances(ampnet_graph_t* g, int32_t split, const am
     if ((st = upload_raw(g, D, in->labels_i, nl, &V.labels_i)) != AMPNET_OK) return st;
   }
   if (in->labels_f) if ((st = upload_raw(g, D, in->labels_f, (size_t)n, &V.labels_f)) != AMPNET_OK) return st;
+  if ((st = flush_uploads(g, D)) != AMPNET_OK) return st;
+  infer_domains(g, D);
+  if ((st = ensure_host_read(g, sizeof(Globals) + g->ppts.size() * sizeof(PPTStats) + 16384 + (size_t)n * sizeof(float))) != AMPNET_OK) return st;
+  if ((st = wave_encode(g, D, g->wave, D.wave, &g->enc_scratch, &g->enc_scratch_cap)) != AMPNET_OK) return st;
   CUDA_TRY(g, cudaStreamSynchronize(g->stream));
   D.loaded = true;
   return AMPNET_OK;
@@ -1657,7 +1778,12 @@ extern "C" ampnet_status_t ampnet_run_epoch_static(ampnet_graph_t* g, const ampn
   const long long n_order = cfg->order ? cfg->n_order : D.n;
   RunPlan plan;
   g->have_run = false;                // the dry plan re-targets the statistics pointers of the previous run
-  ampnet_status_t st = plan_run(g, 0, cfg->max_active_keys, cfg->deterministic ? 1 : 0, 0, cfg, n_order, true, plan);
+  ampnet_status_t st = AMPNET_OK;
+  WavePlan wp;
+  if (wave_takes(g, D, cfg->max_active_keys, cfg->deterministic ? 1 : 0, 0, cfg, n_order, wp)) {
+    wave::Run R;
+    wave_carve(g, D, g->wave, D.wave, wp, cfg->max_active_keys, 0, cfg, n_order, true, R);
+  } else st = plan_run(g, 0, cfg->max_active_keys, cfg->deterministic ? 1 : 0, 0, cfg, n_order, true, plan);
   if (st != AMPNET_OK) return st;
   const size_t order_bytes = cfg->order ? (size_t)std::max<long long>(n_order, 0) * sizeof(long long) : 0;
   // the very sizes execute() will ask ensure_arenas() for

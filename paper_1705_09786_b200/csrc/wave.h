@@ -1,0 +1,178 @@
+// Shared structures of the scheduled engine (asynchronous epochs and evaluation): wave_encode.cu turns loaded instances into
+// message programs, wave_engine.cu executes them, ampnet.cu plans and launches.
+//
+// Control flow depends on an instance's structure alone, never on payload values.  So the message passing of an instance can be
+// played through once, without payloads, when the instances are loaded: step t of an instance holds the messages that the
+// messages of step t - 1 caused (all parameter-free nodes fire at once).  What is left of the parameter-free nodes is, per
+// payload row, a list of terms: which rows of which producers are copied (Concat, Split) or summed (Bcast and Flatmap
+// backward, row sums) into it.  The kernel runs rounds; in every round an instance in flight executes its next step, and a
+// finished instance's key goes to the next one of the epoch's order.  Queues, join counters and routing disappear from the
+// epoch, and what a message waits for is known before it exists.
+#pragma once
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+#include <vector>
+
+#include "engine_types.h"
+
+namespace wave {
+
+constexpr int MAX_CELLS = 32;          // one polling lane per cell
+constexpr unsigned NONE = 0xffffffffu;
+
+// A cell is one piece of a parameterised node's work that a group of CTAs executes.
+enum CellKind { LOOKUP_F, LOOKUP_B, LIN_F, LIN_DX, ACC, HEAD, GRU_ZR, GRU_C, GRU_DC, GRU_DZR, N_CELL_KINDS };
+
+// Offsets into the key's arena are in units of four floats; every payload segment is padded to that.
+struct __align__(8) Term { unsigned src4; unsigned short col4, w4; };      // columns [col4, col4 + w4) += arena[src4 ..]
+
+enum { E_NT = 0xff, E_MSG_END = 1 << 8, E_OVERFLOW = 1 << 9, E_DENSE = 1 << 10, E_RAW = 1 << 11 };
+// One payload row of one message.  out4 / a4 / b4 by kind:
+//   LOOKUP_F  output row, -, table row            LOOKUP_B  -, -, table row (terms: gradient)
+//   LIN_F     output row, copy of the input or NONE, -        (terms: input)
+//   LIN_DX    input-gradient row, output row, pre-activation-gradient row        (terms: gradient)
+//   ACC       pre-activation-gradient row, where the forward version is kept, -  (terms: input; E_RAW: -, output row, -, terms:
+//             gradient, the input is the dense row)
+//   HEAD      input-gradient row, pre-activation-gradient row (a kept input behind it), label             (terms: input)
+//   GRU_*     forward block, backward block, -                (terms: input / gradient)
+//   LIN_F of an LSTM gate node: block, block, -  (terms: input, then meta >> 16 terms of the children's cells); LIN_DX: backward
+//             block, block, -
+// With more than four terms E_OVERFLOW is set and t[0].src4 is the first one's index in the overflow pool.
+struct __align__(16) Entry { unsigned out4, a4, b4, meta; Term t[4]; };
+
+struct __align__(16) InstHdr { unsigned tab; unsigned short steps, steps_eval; unsigned msgs, msgs_eval; };
+
+// ---- encoder ------------------------------------------------------------------------------------
+struct EncNode {
+  int type, fn, fn_arg, n_succ, n_pred, ppt;
+  signed char succ_node[amp::MAX_PORTS], succ_port[amp::MAX_PORTS], pred_node[amp::MAX_PORTS], pred_port[amp::MAX_PORTS];
+  int w4, U, J;                        // padded width of a Concat port / Split slice; positions and references per key of its join
+  unsigned ref_off, cnt_off;           // scratch words: references [key][J]; counters (PHI: origins, NPT_SUMROWS: row counts) [key]
+};
+struct EncPpt {
+  int kind, node, head, lstm, source_adj, src_fn, xstore;     // head: Loss node or -1; lstm: gate node or -1
+  int out4, in4, U;
+  unsigned save_off;                   // scratch words [key][3]: first output row, input rows, children's cells
+  int cell[6];                         // LOOKUP: F, B; LINEAR: F, DX, ACC; head: HEAD, ACC; GRU: ZR, C, DC, DZR, ACC c, ACC zr
+  int gates4;                          // gate node: padded width of the gates
+};
+constexpr int ENC_MAX_NODES = 40, ENC_MAX_PPTS = 16;
+struct EncModel {
+  int n_nodes, n_ppts, n_cells, n_sources, IT;
+  int sources[4];
+  EncNode nodes[ENC_MAX_NODES];
+  EncPpt ppts[ENC_MAX_PPTS];
+  unsigned char delay[MAX_CELLS], forward[MAX_CELLS];         // steps between a message and the cell's work on it; forward cell
+  // scratch of one encoding warp, in words: node tables, then the three frontiers, row records, terms
+  unsigned table_words, front_cap, row_cap, term_cap, scratch_words, stack_cap;
+  unsigned near_scratch;               // the scratch is small enough for shared memory
+  unsigned bound[MAX_CELLS], steps_cap;       // most entries of a cell, most steps, of one instance
+};
+struct EncTotals { unsigned entries[MAX_CELLS]; unsigned tab, ov, ov_used, arena4_max; unsigned steps_min, steps_eval_min; unsigned long long steps_sum, steps_eval_sum; int status; };
+
+struct Program {                       // device pointers of an encoded split
+  InstHdr* hdr;
+  const unsigned* tab[MAX_CELLS];      // per cell: number of entries before step t, instance after instance
+  const Entry* ent[MAX_CELLS];
+  const Term* ov;
+};
+
+int encode_warps_per_block();
+// Pass 1 counts (hdr, counts[cell][n], totals), pass 2 writes the entries at the prefix sums of the counts.  A handful of small
+// instances is written in one pass, each with room for the most it can need.
+cudaError_t encode_count(const EncModel* m, const amp::DevInst& inst, unsigned* scratch, int blocks, int warps, InstHdr* hdr, unsigned* counts, EncTotals* totals, cudaStream_t st);
+cudaError_t encode_emit(const EncModel* m, const amp::DevInst& inst, unsigned* scratch, int blocks, int warps, const Program& prog, unsigned* counts, Term* ov, EncTotals* totals,
+                        cudaStream_t st);
+cudaError_t encode_bounded(const EncModel* m, const amp::DevInst& inst, int blocks, int warps, const Program& prog, EncTotals* totals, cudaStream_t st);
+cudaError_t encode_scan(unsigned* counts, InstHdr* hdr, long long n, int n_cells, EncTotals* totals, cudaStream_t st);
+
+// ---- runtime ------------------------------------------------------------------------------------
+// A weight matrix in padded coordinates: output segments of out_w and input segments of in_w columns, each padded to four.
+struct Mat {
+  float *W, *b, *om, *ov;              // parameter arrays and moments of the node (unpadded)
+  long long nW, opt_t0;
+  int row0, in_real, out_w, nso, in_w, nsi, outp, inp;       // first row of the node's stacked matrices; padded sizes in floats
+  float *Wp, *WTp, *bp;                // published versions: [PUB][outp][inp], [PUB][inp][outp], [PUB][outp]
+  unsigned* ver;                       // [32]: round << 16 | publications so far, by round
+};
+constexpr int PUB = 8;                 // published versions kept (readers lag by less than DRIFT + lag rounds)
+constexpr int N_PHASES = 6;            // cycle counters of a cell's first CTA
+constexpr int DRIFT = 4;               // no CTA runs more than this many rounds ahead of another
+
+struct Team {                          // the CTAs of one cell
+  int kind, ppt, mat, cell, acc;       // acc: team that publishes the matrix (-1: none in this run)
+  int T, Sh, n;                        // tiles, message shards, CTAs
+  int R, G, BM;                        // LIN_F: columns per tile and gate groups; LIN_DX: columns per tile; ACC: tile rows; staged rows
+  int C, WO, WI, LO;                   // ACC: tile columns, warps along rows / columns, lanes along rows
+  unsigned wait_mask;                  // cells whose previous round this one reads
+  int act, bf16_tc, first, pad;        // first: lowest CTA index
+  int H4, lstm;                        // GRU / gate nodes: padded hidden width (float4), gate count
+  int keep, k4;                        // LIN_F: a summed input is stored for the accumulator; width of the rows' terms (float4)
+};
+struct PptRun {
+  int kind, node, act, muf, loss_type, source_adj;
+  amp::PPTStats* stats;
+  int* update_log; int log_cap;
+  float* A; int* touched_list;         // LOOKUP: sparse accumulator
+  float *W, *om, *ov; long long opt_t0;
+  int in_dim, out_dim, out4;
+};
+struct Core {                          // what every CTA keeps in shared memory
+  Program prog;
+  amp::Globals* g;
+  unsigned* progress;                  // [teams][16]: CTAs that have finished round r, in slot r mod 16
+  float4* arena; unsigned slot4; int copies;     // floats of a key / 4; arenas a key alternates between
+  const long long* order; long long n_order;
+  const unsigned char* inference_only;
+  float* loss_out;
+  unsigned long long* phases;          // [teams][N_PHASES]
+  const float* dense; int dense_dim;
+  int n_teams, mak, eval, bf16, lag, pace, n_ctas;      // pace: most instances admitted in one round
+  float lr; int opt; float mu, beta1, beta2, eps;
+  unsigned long long timeout_ns;
+};
+struct Run {
+  Core core;
+  Team teams[MAX_CELLS];
+  Mat mats[24]; int n_mats;
+  PptRun ppts[ENC_MAX_PPTS]; int n_ppts;
+};
+size_t smem_bytes(const Team& t, const Mat& m, int mak);
+cudaError_t launch(const Run* drun, int n_ctas, size_t smem, cudaStream_t st);
+size_t static_smem();
+int max_keys();
+
+// ---- host side: the model (per graph), an encoded split, a placement -----------------------------------------------
+struct WaveCell { int kind, ppt, mat, delay; bool forward; };
+struct WaveMat { int ppt, row0, out_w, nso, in_w, nsi, outp, inp; };
+struct WaveModel {
+  bool ok = false;
+  EncModel enc{};
+  std::vector<WaveCell> cells;
+  std::vector<WaveMat> mats;
+  std::vector<unsigned> fwd_mask, bwd_mask;      // per parameterised node: cells that produce its input / its gradient
+};
+struct WaveData {
+  bool ok = false;
+  long long load_id = 0;
+  Program prog{};
+  EncTotals tot{};
+};
+struct WavePlanKey {
+  long long load_id = -1, n_order = 0;
+  int mak = 0, muf = 0, eval = 0, n_ctas = 0, env[3] = {0, 0, 0};
+  bool operator==(const WavePlanKey& o) const {
+    return load_id == o.load_id && n_order == o.n_order && mak == o.mak && muf == o.muf && eval == o.eval && n_ctas == o.n_ctas && env[0] == o.env[0] && env[1] == o.env[1] && env[2] == o.env[2];
+  }
+};
+struct WaveTeam { Team t; double cycles = 0; };
+struct WavePlan {
+  bool ok = false;
+  std::vector<WaveTeam> teams;
+  int n_ctas = 0;
+  size_t smem = 0;
+  int copies = 2, pace = 1;
+};
+
+}  // namespace wave

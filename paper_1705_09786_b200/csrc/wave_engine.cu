@@ -1,0 +1,1564 @@
+// Scheduled engine: asynchronous epochs and evaluation as a persistent kernel that executes message programs (wave.h).
+//
+// Every CTA belongs to one cell.  Four helper warps run ahead and assemble the rows of the next rounds (which instances are in
+// flight, which program entries their steps hold): they depend on the programs alone, never on another CTA.  Sixteen compute
+// warps take those chunks of rows: wait until the cells whose rows they read have finished the previous round (one counter per
+// cell and round, one polling lane per cell), gather the rows, multiply with the weights that stay in shared memory, store
+// the results and count themselves.  There are no queues, no join counters and no atomics on payloads; one hop is
+// stores -> one release add -> the consumers' poll.
+//
+// Weights: an accumulator cell (ACC) owns the master copy of a rectangle of the matrix, adds up the gradients of the rounds'
+// rows in order, updates exactly at the gradient that reaches min_update_frequency (Sec. 3) and publishes the new version;
+// forward and input-gradient cells reload it `lag` rounds later (1 with a single key in flight, where an instance must see the
+// updates of the one before; 2 otherwise: the reload then never waits).
+#include <cuda_bf16.h>
+
+#include "tc_tile.cuh"
+#include "wave.h"
+
+namespace wave {
+using namespace amp;
+
+constexpr int CT = 512, CW = CT / 32;         // compute threads
+constexpr int HT = 128;                       // helper threads
+constexpr int NT = CT + HT;
+constexpr int SLOT_WORDS = 6;
+constexpr int ACC_RED = CW * 8 * 32 * 4;       // floats of an accumulator's merge buffer
+constexpr int NEAR = 128;                     // touched pieces of embedding rows a warp lists in shared memory
+
+enum { H_FIRST = 1, H_LAST = 2, H_UPDATE = 4, H_END = 8, H_COPIES = 16 };      // H_COPIES: every row is one or two copies
+struct __align__(16) RowD { unsigned out4, a4, b4, meta; Term t[4]; int inst; unsigned base4; unsigned pad[2]; };
+struct Head { int round, count, flags, n_upd, upd_t, n_updates, total, pad; };
+
+struct Shared {
+  Core core; Team team; Mat mat; PptRun ppt;
+  Head hd[2];
+  unsigned long long full[2], empty[2], tc_mbar;
+  unsigned tmem;
+  int stop, ok, ok2;
+  unsigned long long ver;                      // what the ACC team had published `lag` rounds ago: updates << 32 | publications << 16 | round
+  int warp_sum[4], sel;
+  unsigned long long batches, batch_rows, msgs, tc_batches;
+  unsigned max_pending;
+  unsigned stale_hist[64]; int max_stale;
+  int team_n[MAX_CELLS];
+  unsigned long long phase[N_PHASES]; long long mark;
+};
+__shared__ Shared S;
+// Pointers into shared memory that reach a function as arguments would be dereferenced as generic addresses.
+#define IN_SMEM(p) __builtin_assume(__isShared(p))
+
+// Cycles of the cell's first CTA: waiting for the helpers, waiting for other cells, gathers, products, the rest.
+__device__ __forceinline__ void phase(const int k) { if (threadIdx.x == 0) { const long long n = clock64(); S.phase[k] += (unsigned long long)(n - S.mark); S.mark = n; } }
+
+// ---- small helpers ---------------------------------------------------------------------------------------------
+__device__ __forceinline__ unsigned smem_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ unsigned ld_acq(const unsigned* p) { unsigned v; asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory"); return v; }
+__device__ __forceinline__ unsigned long long ld_acq64(const unsigned long long* p) { unsigned long long v; asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory"); return v; }
+// (a fence and a relaxed add: the fence also orders the adds of later rounds that have nothing of their own to publish)
+__device__ __forceinline__ void red_release(unsigned* p) { asm volatile("fence.acq_rel.gpu;\nred.relaxed.gpu.global.add.u32 [%0], 1;" :: "l"(p) : "memory"); }
+__device__ __forceinline__ void red_relaxed(unsigned* p) { asm volatile("red.relaxed.gpu.global.add.u32 [%0], 1;" :: "l"(p) : "memory"); }
+__device__ __forceinline__ unsigned long long gtime() { unsigned long long t; asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t)); return t; }
+__device__ __forceinline__ void bar_compute() { asm volatile("bar.sync 1, 512;" ::: "memory"); }
+__device__ __forceinline__ void bar_helper() { asm volatile("bar.sync 2, 128;" ::: "memory"); }
+__device__ __forceinline__ bool bar_helper_or(bool v) {
+  unsigned r;
+  asm volatile("{\n.reg .pred p, q;\nsetp.ne.u32 p, %1, 0;\nbarrier.cta.red.or.pred.aligned q, 2, 128, p;\nselp.u32 %0, 1, 0, q;\n}" : "=r"(r) : "r"((unsigned)v) : "memory");
+  return r != 0;
+}
+__device__ __forceinline__ void mbar_init(unsigned long long* b, int n) { asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" :: "r"(smem_u32(b)), "r"(n) : "memory"); }
+__device__ __forceinline__ void mbar_arrive(unsigned long long* b) { asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(smem_u32(b)) : "memory"); }
+__device__ __forceinline__ bool mbar_try(unsigned long long* b, unsigned parity) {
+  unsigned ok;
+  asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}" : "=r"(ok) : "r"(smem_u32(b)), "r"(parity) : "memory");
+  return ok != 0;
+}
+__device__ __noinline__ void fail(Globals* g, int code, int node, int detail) {
+  if (atomicCAS(&g->status, 0, code) == 0) { g->err_node = node; g->err_detail = detail; }
+  __threadfence();
+  asm volatile("st.release.gpu.global.u32 [%0], 1;" :: "l"(&g->abort_flag) : "memory");
+}
+__device__ __forceinline__ bool over(const unsigned long long t0, int where) {
+  if (ld_acq(&S.core.g->abort_flag)) return true;
+  if (gtime() - t0 <= S.core.timeout_ns) return false;
+  fail(S.core.g, ST_TIMEOUT, S.ppt.node, where);
+  return true;
+}
+// Waits for a phase of a shared-memory barrier; false when the run is being aborted.
+__device__ __forceinline__ bool mbar_wait(unsigned long long* b, unsigned parity, const unsigned long long t0, int where) {
+  for (unsigned it = 1;; it++) {
+    if (mbar_try(b, parity)) return true;
+    if ((it & 255u) == 0 && (*(volatile int*)&S.stop || over(t0, where))) { *(volatile int*)&S.stop = 1; return false; }
+  }
+}
+__device__ __forceinline__ void cp16(float* dst, const void* src) { asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(smem_u32(dst)), "l"(src) : "memory"); }
+__device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+__device__ __forceinline__ float4 ldcg4(const float4* p) { return __ldcg(p); }
+__device__ __forceinline__ float4 zero4() { return make_float4(0.f, 0.f, 0.f, 0.f); }
+__device__ __forceinline__ float4 add4(const float4 a, const float4 b) { return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); }
+
+__device__ __forceinline__ float rnd(const int bf16, float v) { return bf16 ? __bfloat162float(__float2bfloat16_rn(v)) : v; }
+__device__ __forceinline__ float4 rnd4(const int bf16, float4 v) { return bf16 ? make_float4(rnd(1, v.x), rnd(1, v.y), rnd(1, v.z), rnd(1, v.w)) : v; }
+__device__ __forceinline__ float act_fwd(int a, float v) {
+  switch (a) {
+    case 1: return v > 0.f ? v : 0.f;
+    case 2: return tanhf(v);
+    case 3: return 1.f / (1.f + expf(-v));
+    default: return v;
+  }
+}
+__device__ __forceinline__ float4 act_fwd4(int a, float4 v) {
+  if (a == 1) return make_float4(v.x > 0.f ? v.x : 0.f, v.y > 0.f ? v.y : 0.f, v.z > 0.f ? v.z : 0.f, v.w > 0.f ? v.w : 0.f);
+  if (a == 2) return make_float4(tanhf(v.x), tanhf(v.y), tanhf(v.z), tanhf(v.w));
+  if (a == 3) return make_float4(1.f / (1.f + expf(-v.x)), 1.f / (1.f + expf(-v.y)), 1.f / (1.f + expf(-v.z)), 1.f / (1.f + expf(-v.w)));
+  return v;
+}
+__device__ __forceinline__ float act_grad(int a, float y) {
+  switch (a) {
+    case 1: return y > 0.f ? 1.f : 0.f;
+    case 2: return 1.f - y * y;
+    case 3: return y * (1.f - y);
+    default: return 1.f;
+  }
+}
+// n / d for 0 <= n < 200000 and 1 <= d <= 2048 by one multiply-high
+struct FastDiv {
+  unsigned d, M;
+  __device__ explicit FastDiv(int d_) : d((unsigned)d_), M(d_ > 1 ? 0xFFFFFFFFu / (unsigned)d_ + 1u : 0u) {}
+  __device__ __forceinline__ int div(int n) const { return d > 1 ? (int)__umulhi((unsigned)n, M) : n; }
+};
+__host__ __device__ __forceinline__ int pad_ld(int n) { int l = (n + 3) & ~3; while ((l & 7) != 4) l += 4; return l; }      // row stride in shared memory: 4 (mod 8) floats
+
+// Real (row, column) of padded coordinates; -1 where there is only padding.
+__device__ __forceinline__ int real_out(const Mat& m, int po) { const int wp = (m.out_w + 3) & ~3, s = po / wp, j = po - s * wp; return (s < m.nso && j < m.out_w) ? m.row0 + s * m.out_w + j : -1; }
+__device__ __forceinline__ int real_in(const Mat& m, int pi) { const int wp = (m.in_w + 3) & ~3, s = pi / wp, j = pi - s * wp; return (s < m.nsi && j < m.in_w) ? s * m.in_w + j : -1; }
+
+struct OptStep {              // update of parameters from their accumulated gradients: SGD, momentum or Adam on the mean (Sec. 3, App. A)
+  int opt; float step, inv_n, lr, mu, b1, b2, eps, c1, c2; float *om, *ov;
+};
+__device__ __noinline__ OptStep opt_step(float* om, float* ov, long long t0, int n_upd, int upd_t) {
+  OptStep s;
+  s.opt = S.core.opt; s.lr = S.core.lr; s.inv_n = 1.f / (float)n_upd; s.step = S.core.lr * s.inv_n; s.mu = S.core.mu; s.b1 = S.core.beta1; s.b2 = S.core.beta2; s.eps = S.core.eps; s.c1 = s.c2 = 1.f; s.om = om; s.ov = ov;
+  if (s.opt == 2) {
+    const double t = (double)(t0 + upd_t);
+    s.c1 = (float)(1.0 / (1.0 - pow((double)s.b1, t)));
+    s.c2 = (float)(1.0 / (1.0 - pow((double)s.b2, t)));
+  }
+  return s;
+}
+__device__ __noinline__ float opt_moments(const OptStep& s, float w, const float a, const size_t k) {
+  const float g = a * s.inv_n;
+  if (s.opt == 1) {
+    const float v = fmaf(s.mu, s.om[k], g);
+    s.om[k] = v;
+    return fmaf(-s.lr, v, w);
+  }
+  const float m = fmaf(s.b1, s.om[k], (1.f - s.b1) * g), v = fmaf(s.b2, s.ov[k], (1.f - s.b2) * g * g);
+  s.om[k] = m; s.ov[k] = v;
+  return w - s.lr * (m * s.c1) / (sqrtf(v * s.c2) + s.eps);
+}
+__device__ __forceinline__ float opt_one(const OptStep& s, const float w, const float a, const size_t k) { return s.opt == 0 ? fmaf(-s.step, a, w) : opt_moments(s, w, a, k); }
+// Four neighbours of a padded matrix row with moments (padding is left alone); plain SGD needs no index, padding has zero gradients.
+__device__ __noinline__ float4 opt_padded(const OptStep& s, const Mat& m, const int po, const int pi, const float4 w, const float4 a) {
+  IN_SMEM(&m);
+  const int r = po < m.outp ? real_out(m, po) : -1;
+  float v[4] = {w.x, w.y, w.z, w.w};
+  const float g[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+  for (int j = 0; j < 4; j++) {
+    const int q = pi + j < m.inp ? real_in(m, pi + j) : -1;
+    if (r >= 0 && q >= 0) v[j] = opt_moments(s, v[j], g[j], (size_t)r * m.in_real + q);
+  }
+  return make_float4(v[0], v[1], v[2], v[3]);
+}
+__device__ __forceinline__ float4 sgd4(const float step, const float4 w, const float4 a) { return make_float4(fmaf(-step, a.x, w.x), fmaf(-step, a.y, w.y), fmaf(-step, a.z, w.z), fmaf(-step, a.w, w.w)); }
+
+// ---- helper warps: the rows of the coming rounds ------------------------------------------------------------------------
+// Key slots: position in the instance's step table, its end, arena, instance (bit 31: only evaluated), rows before it in the round's
+// list, first entry of the step.
+struct Slots { unsigned *tab, *end, *base4; int* inst; unsigned *pre, *lo; };
+__device__ __forceinline__ Slots slots_at(unsigned char* p, int mak) {
+  unsigned* w = reinterpret_cast<unsigned*>(p);
+  return Slots{w, w + mak, w + 2 * mak, reinterpret_cast<int*>(w + 3 * mak), w + 4 * mak, w + 5 * mak + 1};
+}
+__host__ __device__ __forceinline__ size_t slots_bytes(int mak) { return (((size_t)SLOT_WORDS * mak + 8) * 4 + 63) & ~(size_t)63; }
+
+__device__ __forceinline__ int helper_scan(const int v, int& total) {          // exclusive over the helper threads; ends with a barrier pending
+  const int ht = threadIdx.x - CT, lane = ht & 31, warp = ht >> 5;
+  int s = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) { const int x = __shfl_up_sync(0xffffffffu, s, o); if (lane >= o) s += x; }
+  if (lane == 31) S.warp_sum[warp] = s;
+  bar_helper();
+  const int a = S.warp_sum[0], b = S.warp_sum[1], c = S.warp_sum[2], d = S.warp_sum[3];
+  total = a + b + c + d;
+  return s - v + (warp > 0 ? a : 0) + (warp > 1 ? b : 0) + (warp > 2 ? c : 0);
+}
+
+__device__ __noinline__ void helper_main(const int cta, const int tile, const int shard, unsigned char* smem, const unsigned long long t0) {
+  IN_SMEM(smem);
+  const int ht = threadIdx.x - CT;
+  const Team& T = S.team;
+  const int mak = S.core.mak, passes = (mak + HT - 1) / HT, BM = T.BM, kind = T.kind;
+  const Slots L = slots_at(smem, mak);
+  RowD* const rows = reinterpret_cast<RowD*>(smem + slots_bytes(mak));
+  const unsigned* const tab = S.core.prog.tab[T.cell];
+  const Entry* const ent = S.core.prog.ent[T.cell];
+  const bool backward = kind == LOOKUP_B || kind == LIN_DX || kind == ACC || kind == GRU_DC || kind == GRU_DZR;
+  const bool updates = kind == ACC || kind == LOOKUP_B;          // chunks end where an update falls due
+  const bool leader = tile == 0;
+  const int muf = S.ppt.muf;
+#pragma unroll 1
+  for (int s = ht; s < mak; s += HT) { L.tab[s] = 0; L.end[s] = 0; L.base4[s] = ((unsigned)(s + 1) * (unsigned)S.core.copies - 1u) * S.core.slot4; L.inst[s] = 0; }
+  long long next = 0;
+  int round = 0, active = 0, buf = 0, n_acc = 0, n_updates = 0;
+  unsigned parity = 1;                                            // both chunk buffers start empty
+  unsigned long long node_msgs = 0, n_grads = 0, n_msgs = 0;
+  int max_active = 0;
+  bool finishing = true;
+  unsigned max_rows = 0;
+  long long inf_instances = 0;
+  bar_helper();
+  auto publish = [&](int count, int flags, int n_upd) {
+    if (ht == 0) { Head h; h.round = round; h.count = count; h.flags = flags; h.n_upd = n_upd; h.upd_t = n_updates; h.n_updates = n_updates - ((flags & H_UPDATE) ? 1 : 0); h.total = 0; h.pad = 0; S.hd[buf] = h; }
+    mbar_arrive(&S.full[buf]);                                     // (release: the rows written before are visible to whoever sees the phase)
+    buf ^= 1;
+    if (buf == 0) parity ^= 1;
+  };
+  for (;;) {
+    // ---- keys: finished instances leave, the next ones of the order take their slots -----------------------------------
+    int quota = S.core.pace;
+    for (int p = 0; quota > 0 && (finishing || active < mak) && next < S.core.n_order && p < passes; p++) {
+      const int s = p * HT + ht;
+      const bool idle = s < mak && L.tab[s] == L.end[s];
+      int total = 0;
+      const long long left = S.core.n_order - next;
+      const int rank = helper_scan(idle && left > 0 ? 1 : 0, total);
+      const int admitted = (int)min((long long)min(total, quota), left);
+      if (idle) {
+        if (left > 0 && rank < admitted) {
+          const long long i = S.core.order ? S.core.order[next + rank] : next + rank;
+          const InstHdr h = S.core.prog.hdr[i];
+          const bool ev = S.core.eval || (S.core.inference_only && S.core.inference_only[i]);
+          L.tab[s] = h.tab; L.end[s] = h.tab + (ev ? h.steps_eval : h.steps);
+          const unsigned home = (unsigned)s * (unsigned)S.core.copies * S.core.slot4, b = L.base4[s] + S.core.slot4;      // the key's arenas take turns
+          L.base4[s] = b == home + (unsigned)S.core.copies * S.core.slot4 ? home : b;
+          L.inst[s] = (int)i | (ev && !S.core.eval ? (int)0x80000000 : 0);
+          if (cta == 0) { node_msgs += ev ? h.msgs_eval : h.msgs; inf_instances += ev && !S.core.eval; }
+        }
+      }
+      next += admitted;
+      quota -= admitted;
+      bar_helper();
+    }
+    // ---- rows of this cell in this round ------------------------------------------------------------------------------
+    int N = 0;
+    bool fin = false;
+    active = 0;
+    for (int p = 0; p < passes; p++) {
+      const int s = p * HT + ht;
+      int n = 0;
+      bool on = false;
+      if (s < mak) {
+        const unsigned t = L.tab[s];
+        on = t != L.end[s];
+        if (on && !(backward && L.inst[s] < 0)) {
+          const unsigned a = __ldg(tab + t), b = __ldg(tab + t + 1);
+          n = (int)(b - a);
+          L.lo[s] = a;
+        }
+        if (on) { L.tab[s] = t + 1; fin |= t + 1 == L.end[s]; }
+      }
+      int total;
+      const int ex = helper_scan(n | (on ? 1 << 23 : 0), total) & 0x7fffff;      // (a pass holds at most 128 keys and far fewer than 2^23 rows)
+      if (s < mak) L.pre[s] = (unsigned)(N + ex);
+      N += total & 0x7fffff;
+      active += (unsigned)total >> 23;
+      if (p + 1 < passes) bar_helper();
+    }
+    finishing = bar_helper_or(fin);
+    if (active == 0) break;
+    if (active > max_active) max_active = active;
+    if ((unsigned)N > max_rows) max_rows = (unsigned)N;
+    const int j1 = T.Sh > 1 ? (int)((long long)N * (shard + 1) / T.Sh) : N;
+    int j = T.Sh > 1 ? (int)((long long)N * shard / T.Sh) : 0;
+    bool first = true;
+    do {
+      int cnt = min(BM, j1 - j);
+      bool upd = false;
+      Entry e;
+      int inst = 0;
+      unsigned base4 = 0;
+      bool end_msg = false;
+      if (ht < cnt) {
+        int a = 0, b = mak - 1;                                   // last slot with pre <= j (slots without rows share `pre` with their successor)
+        while (a < b) { const int m = (a + b + 1) >> 1; if ((int)L.pre[m] <= j + ht) a = m; else b = m - 1; }
+        const Entry* src = ent + L.lo[a] + (unsigned)(j + ht - (int)L.pre[a]);
+        const uint4* q = reinterpret_cast<const uint4*>(src);
+        const uint4 w0 = __ldg(q), w1 = __ldg(q + 1), w2 = __ldg(q + 2);
+        reinterpret_cast<uint4*>(&e)[0] = w0; reinterpret_cast<uint4*>(&e)[1] = w1; reinterpret_cast<uint4*>(&e)[2] = w2;
+        inst = L.inst[a]; base4 = L.base4[a];
+        end_msg = (e.meta & E_MSG_END) != 0;
+      }
+      if (updates && n_acc + cnt >= muf) {
+        // the update falls due at the first message boundary at or past the gradient that reaches the threshold
+        if (ht == 0) S.sel = 1 << 30;
+        bar_helper();
+        if (ht < cnt && end_msg && n_acc + ht + 1 >= muf) atomicMin(&S.sel, ht + 1);
+        bar_helper();
+        const int cut = S.sel;
+        if (cut <= cnt) { cnt = cut; upd = true; }
+        bar_helper();
+      }
+      if (leader && ht < cnt && end_msg) n_msgs++;
+      if (updates) n_acc += cnt;
+      int n_upd = 0;
+      if (upd) {
+        n_upd = n_acc; n_acc = 0; n_updates++; n_grads += n_upd;
+        if (leader && ht == 0 && n_updates <= S.ppt.log_cap) S.ppt.update_log[n_updates - 1] = n_upd;
+      }
+      // every row one copy of the whole width, or two side by side?
+      bool copies = true;
+      if (ht < cnt) {
+        const unsigned nt = e.meta & E_NT, all = (unsigned)T.k4;
+        const bool one = nt == 1 && e.t[0].w4 == all, two = nt == 2 && e.t[1].col4 == e.t[0].w4 && e.t[0].w4 + e.t[1].w4 == (int)all;
+        copies = !(e.meta & (E_OVERFLOW | E_DENSE | E_RAW)) && e.t[0].col4 == 0 && (one || two);
+        if (one) e.t[1].col4 = 0xffff;
+      }
+      copies = !bar_helper_or(!copies);
+      if (!mbar_wait(&S.empty[buf], parity, t0, 21)) return;
+      if (ht < cnt) {
+        RowD& r = rows[buf * BM + ht];
+        const unsigned nt = e.meta & E_NT, nx = (e.meta & E_OVERFLOW) ? 0u : kind == LIN_F && T.lstm ? nt + (e.meta >> 16) : nt;
+        uint4 w0, w1, w2;
+        w0.x = e.out4 == NONE ? NONE : e.out4 + base4;
+        w0.y = e.a4 == NONE ? NONE : e.a4 + base4;
+        w0.z = kind == LIN_DX ? e.b4 + base4 : e.b4;
+        w0.w = e.meta;
+        w1.x = e.t[0].src4 + (nx > 0 ? base4 : 0u); w1.y = reinterpret_cast<const unsigned*>(&e.t[0])[1];
+        w1.z = e.t[1].src4 + (nx > 1 ? base4 : 0u); w1.w = reinterpret_cast<const unsigned*>(&e.t[1])[1];
+        w2.x = e.t[2].src4 + (nx > 2 ? base4 : 0u); w2.y = reinterpret_cast<const unsigned*>(&e.t[2])[1];
+        w2.z = e.t[3].src4 + (nx > 3 ? base4 : 0u); w2.w = reinterpret_cast<const unsigned*>(&e.t[3])[1];
+        uint4* d = reinterpret_cast<uint4*>(&r);
+        d[0] = w0; d[1] = w1; d[2] = w2; d[3] = make_uint4((unsigned)inst, base4, 0u, 0u);
+      }
+      j += cnt;
+      const bool last = j >= j1;
+      publish(cnt, (first ? H_FIRST : 0) | (last ? H_LAST : 0) | (upd ? H_UPDATE : 0) | (copies ? H_COPIES : 0), n_upd);
+      first = false;
+      if (last) break;
+    } while (true);
+    round++;
+    bar_helper();                                                 // (the slot tables of this round are used up)
+  }
+  // ---- the end: the leftover gradients are applied once more --------------------------------------------------------------
+  int n_upd = 0;
+  if (updates && n_acc > 0) {
+    n_upd = n_acc; n_updates++; n_grads += n_upd;
+    if (leader && ht == 0 && n_updates <= S.ppt.log_cap) S.ppt.update_log[n_updates - 1] = n_upd;
+  }
+  if (!mbar_wait(&S.empty[buf], parity, t0, 22)) return;
+  publish(0, H_END | (n_upd ? H_UPDATE : 0), n_upd);
+  // ---- statistics ----------------------------------------------------------------------------------------------------------
+  PPTStats& st = *S.ppt.stats;
+  const bool counts_msgs = leader && kind != GRU_C && kind != GRU_DZR && !(kind == ACC && !S.ppt.source_adj);
+  if (counts_msgs && n_msgs) atomicAdd(&st.msgs, n_msgs * (kind == HEAD && !S.core.eval ? 2ull : 1ull));
+  if (leader && ht == 0) {
+    if (updates && !(kind == ACC && T.pad)) { st.n_updates = n_updates; st.n_grads_applied = n_grads; st.log_n = n_updates; }
+    if (!backward && shard == 0) st.max_pending[0] = max_rows;
+    if (backward && kind != ACC) st.max_pending[1] = max_rows;
+  }
+  if (cta == 0) {
+    if (node_msgs) atomicAdd(&S.core.g->node_messages, node_msgs);
+    if (inf_instances) atomicAdd(&S.core.g->inf_instances, (unsigned long long)inf_instances);
+    if (ht == 0) { S.core.g->max_active = max_active; S.core.g->rounds = (unsigned long long)round; }
+  }
+}
+
+// ---- compute warps: waiting, signalling -------------------------------------------------------------------------------------
+// Warp 0: the publishing cell has finished the round `lag` back; the cells this one reads have finished the previous round, everybody the
+// round DRIFT back (arenas, publications and counters are reused after that).  Returns 1 when only the version is there yet (first
+// call: the reload of the weights then overlaps the rest of the wait), 2 when everything is, 0 when the run is being aborted.
+__device__ __noinline__ int wait_round(const int round, const bool rows, const bool first, const unsigned long long t0) {
+  const int lane = threadIdx.x & 31;
+  const Team& T = S.team;
+  const bool versioned = T.acc >= 0 && rows && round >= S.core.lag;
+  int target = -1, n = 0;
+  const unsigned* p = nullptr;
+  bool of_version = false;
+  if (lane < S.core.n_teams) {
+    target = round - DRIFT;
+    if (rows && (T.wait_mask >> lane & 1)) target = round - 1;
+    if (rows && lane == T.acc) { of_version = true; target = max(target, round - S.core.lag); }
+    if (target >= 0) { n = S.team_n[lane] * ((target >> 4) + 1); p = S.core.progress + lane * 16 + (target & 15); }
+  }
+  const unsigned long long* vp = nullptr;
+  const int vr = round - S.core.lag;
+  if (lane == 31 && versioned && first && S.mat.ver) { vp = reinterpret_cast<const unsigned long long*>(S.mat.ver) + (vr & 31); of_version = true; }
+  unsigned long long v = 0;
+  bool ok = true, all = false;
+  if (first && (round & 7) == 7 && lane == 0 && over(t0, 23)) ok = false;
+  for (unsigned it = 1;; it++) {
+    bool ready = true;
+    if (p) ready = (int)ld_acq(p) >= n;
+    if (vp) { v = ld_acq64(vp); ready = (v & 0xffff) == ((unsigned)vr & 0xffffu); }
+    all = __all_sync(0xffffffffu, ready);
+    if (all) break;
+    if (first && versioned && __all_sync(0xffffffffu, ready || !of_version)) break;
+    if ((it & 63u) == 0 && lane == 0 && over(t0, 24)) ok = false;
+    if (!__all_sync(0xffffffffu, ok)) break;
+  }
+  ok = __all_sync(0xffffffffu, ok);
+  if (lane == 31 && first) S.ver = vp ? v : 0ull;
+  if (lane == 0 && !ok) *(volatile int*)&S.stop = 1;
+  return ok ? (all ? 2 : 1) : 0;
+}
+// The chunk loop of a role: body(head, rows) between the waits; returns the final head (flags 0 when the run was aborted).
+// fresh(version) starts the reload of the weights when another version is due; idle(head) runs in rounds without rows.
+struct Nothing { __device__ void operator()(const Head&) const {} __device__ void operator()(unsigned long long) const {} };
+template <class Body, class Fresh = Nothing, class Idle = Nothing>
+__device__ __forceinline__ Head chunk_loop(RowD* rows, const int team, const unsigned long long t0, const Body& body, const Fresh& fresh = Fresh(), const Idle& idle = Idle()) {
+  const int tid = threadIdx.x, warp = tid >> 5;
+  const int BM = S.team.BM;
+  const bool T_publishes = S.team.kind == ACC;
+  unsigned parity = 0;
+  for (int buf = 0;;) {
+    if (!mbar_wait(&S.full[buf], parity, t0, 25)) break;
+    phase(0);
+    const Head h = S.hd[buf];
+    const bool end = h.flags & H_END;
+    if (end && !(h.flags & H_UPDATE)) return h;
+    const bool last = h.flags & H_LAST, any = h.count > 0;
+    if (h.flags & H_FIRST) {
+      if (warp == 0) { const int r = wait_round(h.round, any, true, t0); if ((tid & 31) == 0) S.ok = r; }
+      bar_compute();
+      int ok = S.ok;
+      if (!ok) break;
+      if (any) fresh(S.ver);
+      if (ok == 1) {
+        if (warp == 0) { const int r = wait_round(h.round, any, false, t0); __syncwarp(); if ((tid & 31) == 0) S.ok2 = r; }
+        bar_compute();
+        ok = S.ok2;
+        if (!ok) break;
+      }
+      phase(1);
+    }
+    if (any || end) {                                              // (at the end: the leftover gradients' update)
+      if (tid == 0 && any) { S.batches++; S.batch_rows += h.count; }
+      body(h, rows + buf * BM);
+      if (end) return h;
+    } else if (last) idle(h);
+    if (any || last) bar_compute();                                // results stored, rows used up
+    if (tid == 0) {
+      unsigned* const mine = S.core.progress + team * 16 + (h.round & 15);
+      if (last) { if (any || !(h.flags & H_FIRST) || T_publishes) red_release(mine); else red_relaxed(mine); }      // (nothing to order in a round without rows)
+      mbar_arrive(&S.empty[buf]);
+    }
+    phase(4);
+    buf ^= 1;
+    if (buf == 0) parity ^= 1;
+  }
+  Head none{};
+  return none;
+}
+
+// ---- gathers ---------------------------------------------------------------------------------------------------------------
+// Value of columns 4 c .. 4 c + 3 of a row given by terms.
+__device__ __forceinline__ float4 row_sum(const RowD& r, const int c) {
+  const int nt = r.meta & E_NT;
+  float4 v = zero4();
+  if (r.meta & E_OVERFLOW) {
+    const Term* t = S.core.prog.ov + r.t[0].src4;
+    for (int q = 0; q < nt; q++) {
+      const unsigned d = (unsigned)c - t[q].col4;
+      if (d < t[q].w4) v = add4(v, ldcg4(S.core.arena + r.base4 + t[q].src4 + d));
+    }
+    return v;
+  }
+  float4 w[4];
+#pragma unroll
+  for (int q = 0; q < 4; q++) {
+    w[q] = zero4();
+    const Term t = r.t[q];
+    const unsigned d = (unsigned)c - t.col4;
+    if (q < nt && d < t.w4) w[q] = ldcg4(S.core.arena + t.src4 + d);
+  }
+  return add4(add4(w[0], w[1]), add4(w[2], w[3]));
+}
+__device__ __noinline__ float4 dense4(const int inst, const int c) {
+  const float* x = S.core.dense + (long long)(inst & 0x7fffffff) * S.core.dense_dim + 4 * c;
+  float4 v;
+  v.x = 4 * c < S.core.dense_dim ? __ldg(x) : 0.f; v.y = 4 * c + 1 < S.core.dense_dim ? __ldg(x + 1) : 0.f;
+  v.z = 4 * c + 2 < S.core.dense_dim ? __ldg(x + 2) : 0.f; v.w = 4 * c + 3 < S.core.dense_dim ? __ldg(x + 3) : 0.f;
+  return v;
+}
+// Columns [c0, c0 + nc) (in fours) of the rows' terms into X; copies are asynchronous (cp_wait before the barrier), sums take up to
+// four loads at a time.  Chunks of plain copies (one source, or a Concat of two) have a loop of their own: what a round costs is
+// mostly how many instructions it walks through.
+__device__ __noinline__ void gather_general(const RowD* rows, const int count, const int c0, const int nc, float* X, const int ldx) {
+  IN_SMEM(rows); IN_SMEM(X);
+  const FastDiv dn(nc);
+#pragma unroll 1
+  for (int i = threadIdx.x; i < count * nc; i += CT) {
+    const int b = dn.div(i), k = i - b * nc, c = c0 + k;
+    const RowD& r = rows[b];
+    float* const dst = X + b * ldx + 4 * k;
+    if (r.meta & (E_DENSE | E_RAW)) {
+      if ((S.core.dense_dim & 3) == 0) { if (4 * c < S.core.dense_dim) cp16(dst, S.core.dense + (long long)(r.inst & 0x7fffffff) * S.core.dense_dim + 4 * c); else *reinterpret_cast<float4*>(dst) = zero4(); }
+      else *reinterpret_cast<float4*>(dst) = dense4(r.inst, c);
+    } else *reinterpret_cast<float4*>(dst) = rnd4(S.core.bf16, row_sum(r, c));
+  }
+}
+__device__ __forceinline__ void gather_terms(const Head& h, const RowD* rows, const int c0, const int nc, float* X, const int ldx) {
+  if (!(h.flags & H_COPIES)) { gather_general(rows, h.count, c0, nc, X, ldx); return; }
+  const FastDiv dn(nc);
+  const int n = h.count * nc;
+#pragma unroll 1
+  for (int i = threadIdx.x; i < n; i += CT) {
+    const int b = dn.div(i), k = i - b * nc, c = c0 + k;
+    const uint4 t = *reinterpret_cast<const uint4*>(&rows[b].t[0]);            // {source, columns} twice
+    const bool second = c >= (int)(t.w & 0xffffu);
+    cp16(X + b * ldx + 4 * k, S.core.arena + (second ? t.z + c - (t.w & 0xffffu) : t.x + c));
+  }
+}
+
+// ---- products ---------------------------------------------------------------------------------------------------------------
+// Y[b][o] = sum_k A[b][k] B[o][k]: all in shared memory, k contiguous, row strides of A and B 4 (mod 8) floats, K4 groups of four,
+// nB a multiple of four.  512 threads, no barrier inside.  Three shapes:
+//   gemm_few     up to four rows: a warp per output column, lanes along k
+//   gemm_warps   up to 1,536 outputs: a warp per 4 x 4 outputs, lanes along k, a reduce-scatter of shuffles (short code)
+//   gemm_blocks  8 x 4 outputs per thread, k in up to 32 interleaved slices.  The bound is what shared memory can hand to registers
+//                (a 16-byte load costs four cycles of the SM whatever it hits: 12 loads per 128 multiply-adds).
+__device__ __noinline__ void gemm_warps(const float* __restrict__ A, const int lda, const int nA, const float* __restrict__ B, const int ldb, const int nB, const int K4, float* __restrict__ Y, const int ldy) {
+  IN_SMEM(A); IN_SMEM(B); IN_SMEM(Y);
+  const int lane = threadIdx.x & 31, tB = nB >> 2, tiles = ((nA + 3) >> 2) * tB;
+  const FastDiv dB(tB);
+  const int lda4 = lda >> 2, ldb4 = ldb >> 2;
+#pragma unroll 1
+  for (int t = threadIdx.x >> 5; t < tiles; t += CW) {
+    const int bt = dB.div(t), ot = t - bt * tB;
+    const float4* const a = reinterpret_cast<const float4*>(A) + 4 * bt * lda4;
+    const float4* const w = reinterpret_cast<const float4*>(B) + 4 * ot * ldb4;
+    const int m1 = min(1, nA - 1 - 4 * bt) * lda4, m2 = min(2, nA - 1 - 4 * bt) * lda4, m3 = min(3, nA - 1 - 4 * bt) * lda4;
+    float v[16];
+#pragma unroll
+    for (int i = 0; i < 16; i++) v[i] = 0.f;
+#pragma unroll 1
+    for (int k = lane; k < K4; k += 32) {
+      const float4 x[4] = {a[k], a[m1 + k], a[m2 + k], a[m3 + k]}, y[4] = {w[k], w[ldb4 + k], w[2 * ldb4 + k], w[3 * ldb4 + k]};
+#pragma unroll
+      for (int m = 0; m < 4; m++)
+#pragma unroll
+        for (int j = 0; j < 4; j++) v[4 * m + j] = fmaf(x[m].w, y[j].w, fmaf(x[m].z, y[j].z, fmaf(x[m].y, y[j].y, fmaf(x[m].x, y[j].x, v[4 * m + j]))));
+    }
+    int at = 0;
+#pragma unroll
+    for (int s = 0; s < 4; s++) {
+      const int H = 8 >> s;
+      const bool up = (lane >> s) & 1;
+#pragma unroll
+      for (int i = 0; i < H; i++) {
+        const float give = up ? v[i] : v[i + H], keep = up ? v[i + H] : v[i];
+        v[i] = keep + __shfl_xor_sync(0xffffffffu, give, 1 << s);
+      }
+      at += up ? H : 0;
+    }
+    v[0] += __shfl_xor_sync(0xffffffffu, v[0], 16);
+    const int b = 4 * bt + (at >> 2);
+    if (lane < 16 && b < nA) Y[b * ldy + 4 * ot + (at & 3)] = v[0];
+  }
+}
+template <int TA>
+__device__ __noinline__ void gemm_blocks(const float* __restrict__ A, const int lda, const int nA, const float* __restrict__ B, const int ldb, const int nB, const int K4, float* __restrict__ Y, const int ldy) {
+  IN_SMEM(A); IN_SMEM(B); IN_SMEM(Y);
+  constexpr int V = TA * 4;
+  const int tid = threadIdx.x;
+  const int tA = (nA + TA - 1) / TA, tB = nB >> 2, n_tiles = tA * tB;
+  int sh = 0;
+  while (sh < 5 && (n_tiles << (sh + 1)) <= CT && (4 << sh) <= K4) sh++;
+  const int nsl = 1 << sh, per_pass = CT >> sh, ks = tid & (nsl - 1);
+  const FastDiv dB(tB);
+  const float4* const A4 = reinterpret_cast<const float4*>(A);
+  const float4* const B4 = reinterpret_cast<const float4*>(B);
+  const int lda4 = lda >> 2, ldb4 = ldb >> 2;
+#pragma unroll 1
+  for (int t0 = 0; t0 < n_tiles; t0 += per_pass) {
+    const int ti = t0 + (tid >> sh);
+    const bool valid = ti < n_tiles;
+    if (!__any_sync(0xffffffffu, valid)) break;
+    const int bt = valid ? dB.div(ti) : 0, ot = valid ? ti - bt * tB : 0;
+    int a[TA];
+#pragma unroll
+    for (int m = 0; m < TA; m++) a[m] = min(TA * bt + m, nA - 1) * lda4;
+    const int w0 = 4 * ot * ldb4;
+    float v[V];
+#pragma unroll
+    for (int i = 0; i < V; i++) v[i] = 0.f;
+#pragma unroll 1
+    for (int k4 = valid ? ks : K4; k4 < K4; k4 += nsl) {
+      const float4 y[4] = {B4[w0 + k4], B4[w0 + ldb4 + k4], B4[w0 + 2 * ldb4 + k4], B4[w0 + 3 * ldb4 + k4]};
+#pragma unroll
+      for (int m = 0; m < TA; m++) {
+        const float4 x = A4[a[m] + k4];
+#pragma unroll
+        for (int j = 0; j < 4; j++) {
+          v[4 * m + j] = fmaf(x.x, y[j].x, v[4 * m + j]); v[4 * m + j] = fmaf(x.y, y[j].y, v[4 * m + j]);
+          v[4 * m + j] = fmaf(x.z, y[j].z, v[4 * m + j]); v[4 * m + j] = fmaf(x.w, y[j].w, v[4 * m + j]);
+        }
+      }
+    }
+    int base = 0;
+    bool mine = valid;
+#pragma unroll
+    for (int s = 0; s < 5; s++)
+      if (s < sh) {
+        const int H = V >> (s + 1);
+        const bool up = (ks >> s) & 1;
+        if (H > 0) {
+#pragma unroll
+          for (int i = 0; i < H; i++) {
+            const float give = up ? v[i] : v[i + H], keep = up ? v[i + H] : v[i];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, give, 1 << s);
+          }
+          base += up ? H : 0;
+        } else {
+          v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1 << s);
+          mine = mine && !up;
+        }
+      }
+    if (!mine) continue;
+    const int left = V >> sh;
+    if (left >= 4) {
+#pragma unroll
+      for (int i = 0; i < V; i += 4)
+        if (i < left) { const int b = TA * bt + ((base + i) >> 2); if (b < nA) *reinterpret_cast<float4*>(Y + b * ldy + 4 * ot) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]); }
+    } else {
+      const int b = TA * bt + (base >> 2), o = 4 * ot + (base & 3);
+      if (b < nA) { Y[b * ldy + o] = v[0]; if (left == 2) Y[b * ldy + o + 1] = v[1]; }
+    }
+  }
+}
+__device__ __noinline__ void gemm_few(const float* __restrict__ A, const int lda, const int nA, const float* __restrict__ B, const int ldb, const int nB, const int K4, float* __restrict__ Y, const int ldy) {
+  IN_SMEM(A); IN_SMEM(B); IN_SMEM(Y);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const float4* const A4 = reinterpret_cast<const float4*>(A);
+  const float4* const B4 = reinterpret_cast<const float4*>(B);
+  const int ldb4 = ldb >> 2, l1 = nA > 1 ? lda >> 2 : 0, l2 = nA > 2 ? 2 * (lda >> 2) : 0, l3 = nA > 3 ? 3 * (lda >> 2) : 0;
+#pragma unroll 1
+  for (int o = warp; o < nB; o += CW) {
+    float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
+    auto dot = [](const float4 w, const float4 x, float s) { s = fmaf(x.x, w.x, s); s = fmaf(x.y, w.y, s); s = fmaf(x.z, w.z, s); return fmaf(x.w, w.w, s); };
+#pragma unroll 2
+    for (int k4 = lane; k4 < K4; k4 += 32) {
+      const float4 w = B4[o * ldb4 + k4];
+      a0 = dot(w, A4[k4], a0);
+      if (nA > 1) { a1 = dot(w, A4[l1 + k4], a1); a2 = dot(w, A4[l2 + k4], a2); a3 = dot(w, A4[l3 + k4], a3); }
+    }
+    // lanes 0-15 keep rows 0, 1, lanes 16-31 rows 2, 3; then one row per group of eight lanes
+    const bool hi = lane & 16, mid = lane & 8;
+    float s0 = hi ? a2 : a0, s1 = hi ? a3 : a1;
+    s0 += __shfl_xor_sync(0xffffffffu, hi ? a0 : a2, 16);
+    s1 += __shfl_xor_sync(0xffffffffu, hi ? a1 : a3, 16);
+    float v = mid ? s1 : s0;
+    v += __shfl_xor_sync(0xffffffffu, mid ? s0 : s1, 8);
+    v += __shfl_xor_sync(0xffffffffu, v, 4);
+    v += __shfl_xor_sync(0xffffffffu, v, 2);
+    v += __shfl_xor_sync(0xffffffffu, v, 1);
+    const int b = (hi ? 2 : 0) + (mid ? 1 : 0);
+    if ((lane & 7) == 0 && b < nA) Y[b * ldy + o] = v;
+  }
+}
+__device__ __forceinline__ void gemm(const float* A, const int lda, const int nA, const float* B, const int ldb, const int nB, const int K4, float* Y, const int ldy) {
+  if (nA <= 4) gemm_few(A, lda, nA, B, ldb, nB, K4, Y, ldy);
+  else if (nA * nB <= 1536) gemm_warps(A, lda, nA, B, ldb, nB, K4, Y, ldy);
+  else gemm_blocks<8>(A, lda, nA, B, ldb, nB, K4, Y, ldy);
+}
+
+// ---- weights ---------------------------------------------------------------------------------------------------------------
+// Rows rr = g * jn + jj of a tile (gate g, padded output column g * gate_width + j0 + jj), all input columns, into Ws[rr][ld].
+// Version 0 is the parameter array itself (first_rows, at the start of a run), later ones are the published copies.
+__device__ __noinline__ void first_rows(const Mat& m, const int G, const int gw, const int j0, const int jn, float* Ws, const int ld, float* bs) {
+  IN_SMEM(&m); IN_SMEM(Ws); IN_SMEM(bs);
+#pragma unroll 1
+  for (int i = threadIdx.x; i < G * jn * m.inp; i += CT) {
+    const int rr = i / m.inp, k = i - rr * m.inp, g = rr / jn, ro = real_out(m, g * gw + j0 + rr - g * jn), ri = real_in(m, k);
+    Ws[rr * ld + k] = (ro >= 0 && ri >= 0) ? m.W[(size_t)ro * m.in_real + ri] : 0.f;
+  }
+#pragma unroll 1
+  for (int i = threadIdx.x; i < G * jn; i += CT) { const int g = i / jn, ro = real_out(m, g * gw + j0 + i - g * jn); bs[i] = ro >= 0 ? m.b[ro] : 0.f; }
+}
+__device__ __noinline__ void load_rows(const Mat& m, const unsigned pub, const int G, const int gw, const int j0, const int jn, float* Ws, const int ld, float* bs) {
+  IN_SMEM(&m); IN_SMEM(Ws); IN_SMEM(bs);
+  const float* Wp = m.Wp + (size_t)(pub % PUB) * m.outp * m.inp;
+  const float* bp = m.bp + (size_t)(pub % PUB) * m.outp;
+  const int n4 = m.inp >> 2, lane = threadIdx.x & 31;
+#pragma unroll 1
+  for (int rr = threadIdx.x >> 5; rr < G * jn; rr += CW) {       // a warp per row
+    const int g = G > 1 ? rr / jn : 0;
+    const float* src = Wp + (size_t)(g * gw + j0 + rr - g * jn) * m.inp;
+#pragma unroll 1
+    for (int k = lane; k < n4; k += 32) cp16(Ws + rr * ld + 4 * k, src + 4 * k);
+    if (lane == 0) bs[rr] = __ldcg(bp + g * gw + j0 + rr - g * jn);
+  }
+}
+// Input columns [c0, c0 + cn) for all outputs, transposed: Wt[c][ld].
+__device__ __noinline__ void first_cols(const Mat& m, const int c0, const int cn, float* Wt, const int ld) {
+  IN_SMEM(&m); IN_SMEM(Wt);
+#pragma unroll 1
+  for (int i = threadIdx.x; i < cn * m.outp; i += CT) {
+    const int o = i / cn, c = i - o * cn, ro = real_out(m, o), ri = real_in(m, c0 + c);
+    Wt[c * ld + o] = (ro >= 0 && ri >= 0) ? m.W[(size_t)ro * m.in_real + ri] : 0.f;
+  }
+}
+__device__ __noinline__ void load_cols(const Mat& m, const unsigned pub, const int c0, const int cn, float* Wt, const int ld) {
+  IN_SMEM(&m); IN_SMEM(Wt);
+  const float* Wp = m.WTp + (size_t)(pub % PUB) * m.outp * m.inp;
+  const int n4 = m.outp >> 2, lane = threadIdx.x & 31;
+#pragma unroll 1
+  for (int c = threadIdx.x >> 5; c < cn; c += CW)
+#pragma unroll 1
+    for (int k = lane; k < n4; k += 32) cp16(Wt + c * ld + 4 * k, Wp + (size_t)(c0 + c) * m.outp + 4 * k);
+}
+__device__ __forceinline__ unsigned pub_of(const unsigned long long ver) { return (unsigned)(ver >> 16) & 0xffffu; }
+
+__device__ __forceinline__ float sigm(float v) { return 1.f / (1.f + expf(-v)); }
+__device__ __forceinline__ float4 term4(const RowD& r, const int first, const int n, const int c) {     // columns of terms [first, first + n): copies
+  float4 v = zero4();
+#pragma unroll
+  for (int q = 0; q < 4; q++) {
+    const Term t = r.t[q];
+    const unsigned d = (unsigned)c - t.col4;
+    if (q >= first && q < first + n && d < t.w4) v = ldcg4(S.core.arena + t.src4 + d);
+  }
+  return v;
+}
+
+// ---- forward cell ----------------------------------------------------------------------------------------------------------
+// A tile holds R columns of every gate group (G = 1 for a Linear node, 2 for a GRU's z and r, 3 or 5 for an LSTM's gates) for all
+// inputs; a shard takes its part of the round's rows.  Bound by the latency of gather -> product -> store at the usual 10-60 rows.
+enum { F_PLAIN, F_TENSOR, F_ZR, F_C, F_LSTM };      // (a function per variant: a round runs through its code once, so it has to be short)
+template <int MODE>
+__device__ __noinline__ void forward_main(const int team, const int tile, float* smem, RowD* rows, const unsigned long long t0) {
+  IN_SMEM(smem);  IN_SMEM(rows);
+  const Team& T = S.team; const Mat& m = S.mat;
+  constexpr int kind = MODE == F_ZR ? GRU_ZR : MODE == F_C ? GRU_C : LIN_F;
+  const int tid = threadIdx.x, G = MODE == F_ZR ? 2 : MODE == F_LSTM ? T.G : 1, H4 = T.H4, gw = 4 * H4, bf16 = S.core.bf16;
+  const int j0 = tile * T.R, jn = min(T.R, gw - j0), nB = G * jn, K = m.inp, ld = pad_ld(K), n4 = K >> 2;
+  constexpr bool tcm = MODE == F_TENSOR, lstm = MODE == F_LSTM;
+  const int NTC = (T.BM + 15) & ~15, YP = pad_ld(nB);
+  const size_t w_floats = tcm ? (size_t)tc::M * K / 2 : (size_t)G * T.R * ld, x_floats = tcm ? (size_t)NTC * K / 2 : (size_t)T.BM * ld;
+  float *Ws = smem, *bs = Ws + w_floats, *Xs = bs + ((G * T.R + 3) & ~3), *Ys = Xs + x_floats, *Zs = Ys + (size_t)T.BM * YP;      // Zs: a GRU's z and h columns
+  unsigned char *const Wb = reinterpret_cast<unsigned char*>(Ws), *const Xb = reinterpret_cast<unsigned char*>(Xs);
+  unsigned have = 0;
+  const FastDiv dj4(max(jn >> 2, 1));
+  auto fill_w = [&](const unsigned pub) {
+    const float* W = pub ? m.Wp + (size_t)(pub % PUB) * m.outp * m.inp : m.W;        // (the sizes of a tensor-core node need no padding)
+    tc::fill_operand(Wb, nB, K, [&](const int r) { return W + (size_t)(j0 + r) * K; }, tid, CT);
+    const float* b = pub ? m.bp + (size_t)(pub % PUB) * m.outp : m.b;
+#pragma unroll 1
+    for (int i = tid; i < nB; i += CT) bs[i] = __ldcg(b + j0 + i);
+    tc::fence_operands();
+  };
+  if (tcm) {
+#pragma unroll 1
+    for (size_t i = tid; i < w_floats; i += CT) Ws[i] = 0.f;
+#pragma unroll 1
+    for (size_t i = tid; i < x_floats; i += CT) Xs[i] = 0.f;
+    bar_compute();
+    fill_w(0);
+  } else first_rows(m, G, gw, j0, jn, Ws, ld, bs);
+  unsigned tc_parity = 0;
+  bar_compute();
+  chunk_loop(rows, team, t0, [&](const Head& h, const RowD* R) {
+    const int count = h.count;
+    const int version = (int)(S.ver >> 32);
+    if constexpr (tcm) {
+      // the batch as the second operand: payload rows, rounded when they were emitted, stored as bfloat16
+      const int K8 = K >> 3, items = ((count + 7) >> 3) * K8 * 8;
+      constexpr int U = 4;
+      const FastDiv d8(K8);
+      for (int i0 = tid; i0 < items; i0 += U * CT) {
+        float4 a[U], b[U];
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+          const int i = i0 + u * CT, g8 = d8.div(i >> 3), r = g8 * 8 + (i & 7), k8 = (i >> 3) - g8 * K8;
+          a[u] = b[u] = zero4();
+          if (i < items && r < count) { const int nt = R[r].meta & E_NT; a[u] = term4(R[r], 0, nt, 2 * k8); b[u] = term4(R[r], 0, nt, 2 * k8 + 1); }
+        }
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+          const int i = i0 + u * CT, g8 = d8.div(i >> 3), r = g8 * 8 + (i & 7), k8 = (i >> 3) - g8 * K8;
+          if (i < items) tc::store8(Xb, r, 8 * k8, K, a[u], b[u]);
+        }
+      }
+      tc::fence_operands();
+      if (count <= tc::SMALL_ROWS) for (int i = tid; i < count * YP; i += CT) Ys[i] = 0.f;
+      bar_compute();
+      if (count <= tc::SMALL_ROWS) {
+        tc::small_product(Wb, Xb, K, count, Ys, YP, tid);
+      } else {
+        if (tid == 0) { tc::issue(S.tmem, Wb, Xb, K, NTC, smem_u32(&S.tc_mbar)); S.tc_batches++; }
+        const bool done = mbar_wait(&S.tc_mbar, tc_parity, t0, 26);
+        if (!done) for (unsigned extra = 0; extra < (1u << 16) && !mbar_try(&S.tc_mbar, tc_parity); extra++) {}      // what was issued still writes the accumulator
+        tc_parity ^= 1;
+        if (__all_sync(0xffffffffu, done)) tc::read_accumulator(S.tmem, NTC, count, Ys, YP, nB);
+      }
+      bar_compute();
+      const FastDiv dr(nB >> 2);
+#pragma unroll 1
+      for (int i = tid; i < count * (nB >> 2); i += CT) {
+        const int b = dr.div(i), k = i - b * (nB >> 2);
+        S.core.arena[R[b].out4 + (j0 >> 2) + k] = rnd4(bf16, act_fwd4(T.act, add4(*reinterpret_cast<const float4*>(Ys + b * YP + 4 * k), *reinterpret_cast<const float4*>(bs + 4 * k))));
+      }
+      if (tile == 0 && !S.core.eval) for (int b = tid; b < count; b += CT) S.core.arena[R[b].out4 + H4] = make_float4(__int_as_float(version), 0.f, 0.f, 0.f);
+      return;
+    }
+    gather_terms(h, R, 0, n4, Xs, ld);
+    if (kind == GRU_C)                                          // z and h of this tile's columns
+#pragma unroll 1
+      for (int i = tid; i < count * (jn >> 2); i += CT) {
+        const int b = dj4.div(i), k = i - b * (jn >> 2);
+        cp16(Zs + b * 2 * jn + 4 * k, S.core.arena + R[b].out4 + 2 * H4 + (j0 >> 2) + k);
+        cp16(Zs + b * 2 * jn + jn + 4 * k, S.core.arena + R[b].out4 + H4 + (j0 >> 2) + k);
+      }
+    cp_wait();
+    bar_compute();
+    phase(2);
+    gemm(Xs, ld, count, Ws, ld, nB, n4, Ys, YP);
+    bar_compute();
+    phase(3);
+    const int ow = m.out_w, w4 = jn >> 2;
+    if constexpr (MODE == F_PLAIN) {                              // one output per thread: the activation's code once
+      const FastDiv dj(jn);
+#pragma unroll 1
+      for (int i = tid; i < count * jn; i += CT) {
+        const int b = dj.div(i), o = i - b * jn;
+        reinterpret_cast<float*>(S.core.arena + R[b].out4)[j0 + o] = j0 + o < ow ? rnd(bf16, act_fwd(T.act, Ys[b * YP + o] + bs[o])) : 0.f;
+      }
+    }
+    if constexpr (MODE != F_PLAIN) {
+#pragma unroll 1
+    for (int i = tid; i < count * w4; i += CT) {
+      const int b = dj4.div(i), k = i - b * w4, c4 = (j0 >> 2) + k;
+      const RowD& r = R[b];
+      float4* const out = S.core.arena + r.out4;
+      const float4* const y4 = reinterpret_cast<const float4*>(Ys + b * YP + 4 * k);
+      const float4* const b4 = reinterpret_cast<const float4*>(bs + 4 * k);
+      const int past = 4 * c4 + 4 - ow;                          // columns past the width (padding) stay zero
+      auto clip = [&](float4 v) { if (past > 0) { v.w = 0.f; if (past > 1) v.z = 0.f; if (past > 2) v.y = 0.f; if (past > 3) v.x = 0.f; } return v; };
+      if (kind == GRU_ZR) {
+        const float4 z = clip(act_fwd4(3, add4(y4[0], b4[0]))), rr = clip(act_fwd4(3, add4(y4[w4], b4[w4])));
+        const float4 hh = *reinterpret_cast<const float4*>(Xs + b * ld + gw + 4 * c4);
+        out[2 * H4 + c4] = z; out[3 * H4 + c4] = rr;
+        out[4 * H4 + c4] = make_float4(rr.x * hh.x, rr.y * hh.y, rr.z * hh.z, rr.w * hh.w);
+        continue;
+      }
+      if (kind == GRU_C) {
+        const float4 cc = clip(act_fwd4(2, add4(y4[0], b4[0])));
+        const float4 z = *reinterpret_cast<const float4*>(Zs + b * 2 * jn + 4 * k), hh = *reinterpret_cast<const float4*>(Zs + b * 2 * jn + jn + 4 * k);
+        out[5 * H4 + c4] = cc;
+        out[6 * H4 + c4] = rnd4(bf16, make_float4((1.f - z.x) * hh.x + z.x * cc.x, (1.f - z.y) * hh.y + z.y * cc.y, (1.f - z.z) * hh.z + z.z * cc.z, (1.f - z.w) * hh.w + z.w * cc.w));
+        continue;
+      }
+      // LSTM gates: c = s(i) tanh(u) [+ s(fL) cL + s(fR) cR], h = s(o) tanh(c)
+      const bool branch = T.lstm == 5;
+      auto pre = [&](const int g) { return rnd4(bf16, add4(y4[g * w4], b4[g * w4])); };
+      const float4 gi = act_fwd4(3, pre(0)), gu = act_fwd4(2, pre(branch ? 4 : 2)), go = act_fwd4(3, pre(branch ? 3 : 1));
+      float4 c = make_float4(gi.x * gu.x, gi.y * gu.y, gi.z * gu.z, gi.w * gu.w);
+      if (!S.core.eval) { out[c4] = gi; out[(branch ? 3 : 1) * H4 + c4] = go; out[(branch ? 4 : 2) * H4 + c4] = gu; }
+      if (branch) {
+        const int nt = r.meta & E_NT, nc = r.meta >> 16;
+        const float4 cl = term4(r, nt, nc, c4), cr = term4(r, nt, nc, H4 + c4), fl = act_fwd4(3, pre(1)), fr = act_fwd4(3, pre(2));
+        c = make_float4(c.x + fl.x * cl.x + fr.x * cr.x, c.y + fl.y * cl.y + fr.y * cr.y, c.z + fl.z * cl.z + fr.z * cr.z, c.w + fl.w * cl.w + fr.w * cr.w);
+        if (!S.core.eval) { out[H4 + c4] = fl; out[2 * H4 + c4] = fr; out[7 * H4 + 1 + c4] = cl; out[8 * H4 + 1 + c4] = cr; }
+      }
+      const float4 tc4 = act_fwd4(2, c);
+      out[T.lstm * H4 + c4] = rnd4(bf16, clip(make_float4(go.x * tc4.x, go.y * tc4.y, go.z * tc4.z, go.w * tc4.w)));
+      out[(T.lstm + 1) * H4 + c4] = rnd4(bf16, clip(c));
+    }
+    }
+    // a summed input is kept for the accumulator (every tile a share of the columns); so is a GRU's
+    if (kind == GRU_ZR || (T.keep && !S.core.eval)) {
+      const int share = (n4 + T.T - 1) / T.T, k0 = tile * share, kn = min(share, n4 - k0);
+#pragma unroll 1
+      for (int i = tid; i < count * share; i += CT) {
+        const int b = i / share, k = i - b * share;
+        if (k < kn) S.core.arena[(kind == GRU_ZR ? R[b].out4 : R[b].a4) + k0 + k] = *reinterpret_cast<const float4*>(Xs + b * ld + 4 * (k0 + k));
+      }
+    }
+    if (tile == 0 && !S.core.eval && kind != GRU_ZR) {
+      const unsigned at = kind == GRU_C ? 7u * H4 : lstm ? (unsigned)(T.lstm + 2) * H4 : (unsigned)H4;
+#pragma unroll 1
+      for (int b = tid; b < count; b += CT) S.core.arena[R[b].out4 + at] = make_float4(__int_as_float(version), 0.f, 0.f, 0.f);
+    }
+  }, [&](const unsigned long long ver) {
+    const unsigned pub = pub_of(ver);
+    if (pub == have) return;
+    have = pub;
+    if (tcm) fill_w(pub); else load_rows(m, pub, G, gw, j0, jn, Ws, ld, bs);
+  });
+}
+
+// ---- input-gradient cell ---------------------------------------------------------------------------------------------------
+// A tile holds R input columns of the matrix for all outputs.  The pre-activation gradients of a row are formed while the row
+// is gathered (every tile stores its share of them for the accumulator) and multiplied with the transposed weights.
+enum { B_PLAIN, B_DC, B_DZR, B_LSTM };
+template <int MODE>
+__device__ __noinline__ void input_grad_main(const int team, const int tile, float* smem, RowD* rows, const unsigned long long t0) {
+  IN_SMEM(smem);  IN_SMEM(rows);
+  const Team& T = S.team; const Mat& m = S.mat;
+  constexpr int kind = MODE == B_DC ? GRU_DC : MODE == B_DZR ? GRU_DZR : LIN_DX;
+  const int tid = threadIdx.x, H4 = T.H4, bf16 = S.core.bf16;
+  const int c0 = tile * T.R, cn = min(T.R, m.inp - c0), K = m.outp, ld = pad_ld(K), n4 = K >> 2;
+  const int YP = pad_ld(cn);
+  float *Wt = smem, *Gs = Wt + (size_t)T.R * ld, *Ys = Gs + (size_t)T.BM * ld;
+  const FastDiv dc4(max(cn >> 2, 1));
+  first_cols(m, c0, cn, Wt, ld);
+  unsigned have = 0;
+  constexpr bool lstm = MODE == B_LSTM;
+  const bool branch = lstm && T.lstm == 5;
+  const int w4 = lstm ? H4 : n4;
+  const FastDiv dw(w4);
+  const int in4 = m.inp >> 2;
+  bar_compute();
+  chunk_loop(rows, team, t0, [&](const Head& h, const RowD* R) {
+    const int count = h.count;
+#pragma unroll 1
+    for (int i = tid; i < count * w4; i += CT) {
+      const int b = dw.div(i), c = i - b * w4;
+      const RowD& r = R[b];
+      const bool mine = c % T.T == tile;
+      float4 d;
+      if (kind == LIN_DX && !lstm) {
+        const float4 y = T.act ? ldcg4(S.core.arena + r.a4 + c) : zero4();
+        const float4 g = rnd4(bf16, row_sum(r, c));
+        d = T.act ? make_float4(g.x * act_grad(T.act, y.x), g.y * act_grad(T.act, y.y), g.z * act_grad(T.act, y.z), g.w * act_grad(T.act, y.w)) : g;
+        if (mine) S.core.arena[r.b4 + c] = d;
+      } else if (kind == GRU_DC) {
+        const float4* f = S.core.arena + r.out4 + c;
+        float4* q = S.core.arena + r.a4 + c;
+        const float4 hh = ldcg4(f + H4), z = ldcg4(f + 2 * H4), cc = ldcg4(f + 5 * H4), g = rnd4(bf16, row_sum(r, c));
+        d = make_float4(g.x * z.x * (1.f - cc.x * cc.x), g.y * z.y * (1.f - cc.y * cc.y), g.z * z.z * (1.f - cc.z * cc.z), g.w * z.w * (1.f - cc.w * cc.w));
+        if (mine) {
+          q[0] = g;
+          q[H4] = make_float4(g.x * (cc.x - hh.x) * z.x * (1.f - z.x), g.y * (cc.y - hh.y) * z.y * (1.f - z.y), g.z * (cc.z - hh.z) * z.z * (1.f - z.z), g.w * (cc.w - hh.w) * z.w * (1.f - z.w));
+          q[3 * H4] = d;
+        }
+      } else if (kind == GRU_DZR) {
+        float4* q = S.core.arena + r.a4;
+        if (c < H4) d = ldcg4(q + H4 + c);
+        else {
+          const int k = c - H4;
+          const float4 u = ldcg4(q + 5 * H4 + k), hh = ldcg4(S.core.arena + r.out4 + H4 + k), rr = ldcg4(S.core.arena + r.out4 + 3 * H4 + k);
+          d = make_float4(u.x * hh.x * rr.x * (1.f - rr.x), u.y * hh.y * rr.y * (1.f - rr.y), u.z * hh.z * rr.z * (1.f - rr.z), u.w * hh.w * rr.w * (1.f - rr.w));
+          if (mine) q[2 * H4 + k] = d;
+        }
+      } else {                                                    // LSTM gates: all gates of four columns
+        const float4* f = S.core.arena + r.a4 + c;
+        const float4 gh4 = rnd4(bf16, row_sum(r, c)), gc4 = rnd4(bf16, row_sum(r, H4 + c));
+        const int L = T.lstm;
+        const float4 i4 = ldcg4(f), o4 = ldcg4(f + (branch ? 3 : 1) * H4), u4 = ldcg4(f + (branch ? 4 : 2) * H4);
+        float4 fl4 = zero4(), fr4 = zero4(), cl4 = zero4(), cr4 = zero4();
+        if (branch) { fl4 = ldcg4(f + H4); fr4 = ldcg4(f + 2 * H4); cl4 = ldcg4(f + (L + 2) * H4 + 1); cr4 = ldcg4(f + (L + 3) * H4 + 1); }
+        float out[7][4];
+        const float* pi = &i4.x; const float* po = &o4.x; const float* pu = &u4.x; const float* pfl = &fl4.x; const float* pfr = &fr4.x;
+        const float* pcl = &cl4.x; const float* pcr = &cr4.x; const float* pgh = &gh4.x; const float* pgc = &gc4.x;
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+          const float ii = pi[q], oo = po[q], uu = pu[q], fl = pfl[q], fr = pfr[q];
+          const bool on = 4 * c + q < m.out_w;
+          const float tcv = tanhf(ii * uu + fl * pcl[q] + fr * pcr[q]), dc = pgc[q] + pgh[q] * oo * (1.f - tcv * tcv);
+          out[0][q] = on ? rnd(bf16, dc * uu * ii * (1.f - ii)) : 0.f;
+          out[1][q] = on ? rnd(bf16, dc * pcl[q] * fl * (1.f - fl)) : 0.f;
+          out[2][q] = on ? rnd(bf16, dc * pcr[q] * fr * (1.f - fr)) : 0.f;
+          out[3][q] = on ? rnd(bf16, pgh[q] * tcv * oo * (1.f - oo)) : 0.f;
+          out[4][q] = on ? rnd(bf16, dc * ii * (1.f - uu * uu)) : 0.f;
+          out[5][q] = on ? rnd(bf16, dc * fl) : 0.f;
+          out[6][q] = on ? rnd(bf16, dc * fr) : 0.f;
+        }
+        float4* const dp = S.core.arena + r.out4 + in4 + c;
+        int g = 0;
+#pragma unroll
+        for (int k = 0; k < 5; k++)
+          if (branch || k == 0 || k > 2) {
+            const float4 v = make_float4(out[k][0], out[k][1], out[k][2], out[k][3]);
+            *reinterpret_cast<float4*>(Gs + b * ld + 4 * (g * H4 + c)) = v;
+            if (mine) dp[g * H4] = v;
+            g++;
+          }
+        if (branch && mine) { dp[L * H4] = make_float4(out[5][0], out[5][1], out[5][2], out[5][3]); dp[(L + 1) * H4] = make_float4(out[6][0], out[6][1], out[6][2], out[6][3]); }
+        continue;
+      }
+      *reinterpret_cast<float4*>(Gs + b * ld + 4 * c) = d;
+    }
+    cp_wait();
+    bar_compute();
+    phase(2);
+    gemm(Gs, ld, count, Wt, ld, cn, n4, Ys, YP);
+    bar_compute();
+    const int w4c = cn >> 2;
+#pragma unroll 1
+    for (int i = tid; i < count * w4c; i += CT) {
+      const int b = dc4.div(i), k = i - b * w4c, c4 = (c0 >> 2) + k;
+      const RowD& r = R[b];
+      float4 v = *reinterpret_cast<const float4*>(Ys + b * YP + 4 * k);
+      if (kind == LIN_DX) { S.core.arena[r.out4 + c4] = rnd4(bf16, v); continue; }
+      float4* q = S.core.arena + r.a4;
+      if (kind == GRU_DC) { q[4 * H4 + c4] = v; continue; }
+      const float4 u = ldcg4(q + 4 * H4 + c4);                    // the other half of the cell's input gradient
+      if (c4 < H4) v = add4(v, u);
+      else {
+        const int h4 = c4 - H4;
+        const float4 rr = ldcg4(S.core.arena + r.out4 + 3 * H4 + h4), z = ldcg4(S.core.arena + r.out4 + 2 * H4 + h4), g = ldcg4(q + h4);
+        v = make_float4(v.x + u.x * rr.x + g.x * (1.f - z.x), v.y + u.y * rr.y + g.y * (1.f - z.y), v.z + u.z * rr.z + g.z * (1.f - z.z), v.w + u.w * rr.w + g.w * (1.f - z.w));
+      }
+      q[6 * H4 + c4] = rnd4(bf16, v);
+    }
+    phase(3);
+  }, [&](const unsigned long long ver) {
+    const unsigned pub = pub_of(ver);
+    if (pub != have) { have = pub; load_cols(m, pub, c0, cn, Wt, ld); }
+  });
+}
+
+// ---- accumulator cell ------------------------------------------------------------------------------------------------------
+// A tile owns Ro x Ci of the matrix: master weights in shared memory, gradient sums in registers.  The warps form a WO x WI grid of
+// rectangles of 8 LO x 4 LI (32 lanes of 8 x 4 sums each) times WS slices of the rows; at an update the slices meet in shared memory
+// (64 KB whatever the grid) and every slice moves its share of the weights.
+__device__ __noinline__ void accumulate_main(const int team, const int tile, float* smem, RowD* rows, const unsigned long long t0) {
+  IN_SMEM(smem);  IN_SMEM(rows);
+  const Team& T = S.team; const Mat& m = S.mat;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int Ro = T.R, Ci = T.C, WO = T.WO, WI = T.WI, NR = WO * WI, WS = CW / NR, LO = T.LO, LI = 32 / LO;
+  const int ti = (m.inp + Ci - 1) / Ci, to = tile / ti, o0 = to * Ro, i0 = (tile - to * ti) * Ci;
+  const int ro = min(Ro, m.outp - o0), ci = min(Ci, m.inp - i0);
+  const int ldd = Ro + 4, ldx = Ci + 4, ldw = Ci + 4;
+  float *Wm = smem, *red = Wm + (size_t)Ro * ldw, *Dg = red + (WS > 1 ? ACC_RED : 0), *Xg = Dg + (size_t)T.BM * ldd, *bm = Xg + (size_t)T.BM * ldx, *bred = bm + Ro;   // bred: WS x Ro floats
+  const bool biased = i0 == 0;
+#pragma unroll 1
+  for (int i = tid; i < Ro * Ci; i += CT) {
+    const int o = i / Ci, c = i - o * Ci, r = o < ro ? real_out(m, o0 + o) : -1, k = c < ci ? real_in(m, i0 + c) : -1;
+    Wm[o * ldw + c] = (r >= 0 && k >= 0) ? m.W[(size_t)r * m.in_real + k] : 0.f;
+  }
+#pragma unroll 1
+  for (int i = tid; i < Ro; i += CT) { const int r = i < ro ? real_out(m, o0 + i) : -1; bm[i] = r >= 0 ? m.b[r] : 0.f; }
+#pragma unroll 1
+  for (int i = tid; i < T.BM * (ldd + ldx); i += CT) Dg[i] = 0.f;           // columns past the matrix stay zero
+  const int ws = warp / NR, wr = warp - ws * NR, wo = wr / WI, wi = wr - wo * WI;
+  const int lo = lane / LI, li = lane - lo * LI;
+  const int ob = (wo * LO + lo) * 8, ib = (wi * LI + li) * 4;
+  const bool summing = biased && wi == 0 && li == 0;                        // these lanes also add up their rows' gradients (bias)
+  float acc[8][4], bacc[8];
+#pragma unroll
+  for (int k = 0; k < 8; k++) {
+    bacc[k] = 0.f;
+#pragma unroll
+    for (int j = 0; j < 4; j++) acc[k][j] = 0.f;
+  }
+  unsigned pubs = 0;
+  int updates = 0;
+  bool dirty = false;
+  const int d4 = ro >> 2, x4 = ci >> 2;
+  const FastDiv dd(d4), dx(x4);
+  const bool leader = tile == 0;
+  unsigned long long* const ver = reinterpret_cast<unsigned long long*>(m.ver);
+  bar_compute();
+  // theta <- theta - step(A / n); the accumulators start over
+  auto update = [&](const int n_upd, const int upd_t) {
+    const OptStep os = opt_step(m.om, m.ov, m.opt_t0, n_upd, upd_t);
+    float4* const r4 = reinterpret_cast<float4*>(red);
+    if (summing) {
+#pragma unroll
+      for (int k = 0; k < 8; k++) { bred[ws * Ro + ob + k] = bacc[k]; bacc[k] = 0.f; }
+    }
+    if (WS > 1) {
+#pragma unroll
+      for (int k = 0; k < 8; k++)
+        if ((WS >= 8 ? k : (k * WS) >> 3) != ws) r4[((ws * NR + wr) * 8 + k) * 32 + lane] = make_float4(acc[k][0], acc[k][1], acc[k][2], acc[k][3]);
+    }
+    bar_compute();
+#pragma unroll
+    for (int k = 0; k < 8; k++) {
+      if ((WS >= 8 ? k : (k * WS) >> 3) == ws) {                // this slice's share of the rows
+        float4 a = make_float4(acc[k][0], acc[k][1], acc[k][2], acc[k][3]);
+#pragma unroll 1
+        for (int s = 0; s < WS; s++) if (s != ws) a = add4(a, r4[((s * NR + wr) * 8 + k) * 32 + lane]);
+        float4* const w4 = reinterpret_cast<float4*>(Wm + (ob + k) * ldw + ib);
+        *w4 = os.opt == 0 ? sgd4(os.step, *w4, a) : opt_padded(os, m, o0 + ob + k, i0 + ib, *w4, a);
+      }
+#pragma unroll
+      for (int j = 0; j < 4; j++) acc[k][j] = 0.f;
+    }
+    if (biased)
+#pragma unroll 1
+      for (int i = tid; i < ro; i += CT) {
+        float a = 0.f;
+        for (int s = 0; s < WS; s++) a += bred[s * Ro + i];
+        const int r = real_out(m, o0 + i);
+        if (r >= 0) bm[i] = opt_one(os, bm[i], a, (size_t)m.nW + r);
+      }
+    bar_compute();
+  };
+  auto stamp = [&](const Head& h) { if (leader && tid == 0) *reinterpret_cast<volatile unsigned long long*>(ver + (h.round & 31)) = ((unsigned long long)(unsigned)updates << 32) | ((unsigned long long)(pubs & 0xffffu) << 16) | ((unsigned)h.round & 0xffffu); };
+  const Head end = chunk_loop(rows, team, t0, [&](const Head& h, const RowD* R) {
+    const int count = h.count;
+#pragma unroll 1
+    for (int i = tid; i < count * d4; i += CT) {
+      const int b = dd.div(i), k = i - b * d4, c = (o0 >> 2) + k;
+      const RowD& r = R[b];
+      if (!(r.meta & E_RAW)) { cp16(Dg + b * ldd + 4 * k, S.core.arena + r.out4 + c); continue; }
+      const float4 y = ldcg4(S.core.arena + r.a4 + c), g = rnd4(S.core.bf16, row_sum(r, c));
+      *reinterpret_cast<float4*>(Dg + b * ldd + 4 * k) = make_float4(g.x * act_grad(T.act, y.x), g.y * act_grad(T.act, y.y), g.z * act_grad(T.act, y.z), g.w * act_grad(T.act, y.w));
+    }
+    gather_terms(h, R, i0 >> 2, x4, Xg, ldx);
+    if (leader && warp == CW - 1) {                              // staleness: updates of the node since the forward pass (Sec. 3)
+#pragma unroll 1
+      for (int b0 = 0; b0 < count; b0 += 32) {
+        const int b = b0 + lane;
+        int stale = -1;
+        if (b < count && (R[b].meta & E_MSG_END)) {
+          stale = 0;
+          if (R[b].a4 != NONE) { const float4 v = ldcg4(S.core.arena + R[b].a4 + ((R[b].meta & E_RAW) ? (m.outp >> 2) : 0)); stale = max(0, h.n_updates - __float_as_int(v.x)); }
+        }
+        const unsigned same = __match_any_sync(0xffffffffu, stale);
+        if (stale >= 0 && (same & ((1u << lane) - 1u)) == 0) { atomicAdd(&S.stale_hist[min(stale, 63)], __popc(same)); atomicMax(&S.max_stale, stale); }
+      }
+    }
+    cp_wait();
+    bar_compute();
+    phase(2);
+#pragma unroll 2
+    for (int b = ws; b < count; b += WS) {
+      const float4 da = *reinterpret_cast<const float4*>(Dg + b * ldd + ob), db = *reinterpret_cast<const float4*>(Dg + b * ldd + ob + 4);
+      const float4 x = *reinterpret_cast<const float4*>(Xg + b * ldx + ib);
+      const float d[8] = {da.x, da.y, da.z, da.w, db.x, db.y, db.z, db.w};
+#pragma unroll
+      for (int k = 0; k < 8; k++) {
+        acc[k][0] = fmaf(d[k], x.x, acc[k][0]); acc[k][1] = fmaf(d[k], x.y, acc[k][1]);
+        acc[k][2] = fmaf(d[k], x.z, acc[k][2]); acc[k][3] = fmaf(d[k], x.w, acc[k][3]);
+      }
+      if (summing) {
+#pragma unroll
+        for (int k = 0; k < 8; k++) bacc[k] += d[k];
+      }
+    }
+    phase(3);
+    if (h.flags & H_UPDATE) { update(h.n_upd, h.upd_t); dirty = true; updates = h.upd_t; phase(5); }
+    if (!(h.flags & H_LAST)) return;
+    if (dirty) {                                                // publish: for the forward tiles, and transposed for the input-gradient tiles
+      pubs++;
+      dirty = false;
+      float* const Wp = m.Wp + (size_t)(pubs % PUB) * m.outp * m.inp; float* const WT = m.WTp + (size_t)(pubs % PUB) * m.outp * m.inp;
+#pragma unroll 1
+      for (int i = tid; i < ro * x4; i += CT) { const int o = dx.div(i), c = i - o * x4; *reinterpret_cast<float4*>(Wp + (size_t)(o0 + o) * m.inp + i0 + 4 * c) = *reinterpret_cast<const float4*>(Wm + o * ldw + 4 * c); }
+      if (T.G)
+#pragma unroll 1
+        for (int i = tid; i < d4 * x4; i += CT) {
+          const int c = dd.div(i), o = 4 * (i - c * d4);
+          const float* w = Wm + o * ldw + 4 * c;
+          const float4 a = *reinterpret_cast<const float4*>(w), b = *reinterpret_cast<const float4*>(w + ldw), e = *reinterpret_cast<const float4*>(w + 2 * ldw), f = *reinterpret_cast<const float4*>(w + 3 * ldw);
+          float* t = WT + (size_t)(i0 + 4 * c) * m.outp + o0 + o;
+          *reinterpret_cast<float4*>(t) = make_float4(a.x, b.x, e.x, f.x); *reinterpret_cast<float4*>(t + m.outp) = make_float4(a.y, b.y, e.y, f.y);
+          *reinterpret_cast<float4*>(t + 2 * (size_t)m.outp) = make_float4(a.z, b.z, e.z, f.z); *reinterpret_cast<float4*>(t + 3 * (size_t)m.outp) = make_float4(a.w, b.w, e.w, f.w);
+        }
+      if (biased) for (int i = tid; i < ro; i += CT) m.bp[(size_t)(pubs % PUB) * m.outp + o0 + i] = bm[i];
+    }
+    stamp(h);
+  }, Nothing(), stamp);                                         // (a round without rows: the version stays)
+  if (!(end.flags & H_END)) return;
+#pragma unroll 1
+  for (int i = tid; i < ro * ci; i += CT) {
+    const int o = i / ci, c = i - o * ci, r = real_out(m, o0 + o), k = real_in(m, i0 + c);
+    if (r >= 0 && k >= 0) m.W[(size_t)r * m.in_real + k] = Wm[o * ldw + c];
+  }
+  if (biased) for (int i = tid; i < ro; i += CT) { const int r = real_out(m, o0 + i); if (r >= 0) m.b[r] = bm[i]; }
+}
+
+// ---- loss head ---------------------------------------------------------------------------------------------------------------
+// A Linear node that feeds a Loss: a CTA holds the whole (small) matrix and takes a share of the rows through forward, Loss, and
+// the input gradient of the message the Loss answers with.
+__device__ __noinline__ void head_main(const int team, float* smem, RowD* rows, const unsigned long long t0) {
+  IN_SMEM(smem);  IN_SMEM(rows);
+  const Team& T = S.team; const Mat& m = S.mat;
+  const int tid = threadIdx.x, K = m.inp, ld = pad_ld(K), n4 = K >> 2, outp = m.outp, out = m.out_w, YP = pad_ld(outp), bf16 = S.core.bf16, d4 = outp >> 2;
+  float *Ws = smem, *bs = Ws + (size_t)outp * ld, *Xs = bs + outp, *Ys = Xs + (size_t)T.BM * ld, *Ds = Ys + (size_t)T.BM * YP;
+  first_rows(m, 1, outp, 0, outp, Ws, ld, bs);
+  unsigned have = 0;
+  double loss_sum = 0.0, inf_sum = 0.0;
+  unsigned long long correct = 0, preds = 0, inf_correct = 0, inf_preds = 0;
+  const int G = out <= 8 ? 8 : out <= 16 ? 16 : 32, per_pass = CT / G, lj = tid & (G - 1);
+  const FastDiv dn4(n4);
+  const bool ce = S.ppt.loss_type == LOSS_CE;
+  bar_compute();
+  chunk_loop(rows, team, t0, [&](const Head& h, const RowD* R) {
+    const int count = h.count;
+    gather_terms(h, R, 0, n4, Xs, ld);
+    cp_wait();
+    bar_compute();
+    phase(2);
+    gemm(Xs, ld, count, Ws, ld, outp, n4, Ys, YP);
+    bar_compute();
+    phase(3);
+    // the Loss on G lanes per row, lane lj holding outputs lj, lj + G, ...: maximum and arg-max (lowest index on ties), sum of
+    // exponentials, the label's output
+#pragma unroll 1
+    for (int m0 = 0; m0 < count; m0 += per_pass) {
+      const int b = m0 + tid / G;
+      const bool live = b < count;
+      const RowD& r = R[live ? b : 0];
+      const unsigned label_bits = r.b4;
+      float* const y = Ys + (live ? b : 0) * YP;
+      float* const d = Ds + (live ? b : 0) * YP;
+      const bool inf = r.inst < 0;
+      float mx = -3.4e38f, loss = 0.f;
+      int arg = 0x7fffffff;
+      if (live) for (int j = lj; j < out; j += G) { const float v = rnd(bf16, act_fwd(T.act, y[j] + bs[j])); y[j] = v; if (v > mx) { mx = v; arg = j; } }
+      if (ce) {
+        for (int o = G >> 1; o; o >>= 1) {
+          const float om = __shfl_xor_sync(0xffffffffu, mx, o, G); const int oa = __shfl_xor_sync(0xffffffffu, arg, o, G);
+          if (om > mx || (om == mx && oa < arg)) { mx = om; arg = oa; }
+        }
+        float sum = 0.f, ylab = 0.f;
+        if (live) for (int j = lj; j < out; j += G) { sum += expf(y[j] - mx); if (j == (int)label_bits) ylab = y[j]; }
+        for (int o = G >> 1; o; o >>= 1) { sum += __shfl_xor_sync(0xffffffffu, sum, o, G); ylab += __shfl_xor_sync(0xffffffffu, ylab, o, G); }
+        const float lse = mx + logf(sum);
+        loss = lse - ylab;
+        if (live) for (int j = lj; j < outp; j += G) d[j] = j < out ? rnd(bf16, expf(y[j] - lse) - (j == (int)label_bits ? 1.f : 0.f)) * act_grad(T.act, y[j]) : 0.f;
+        if (live && lj == 0) { if (inf) { inf_correct += arg == (int)label_bits; inf_preds++; } else { correct += arg == (int)label_bits; preds++; } }
+      } else if (live) {
+        const float e = y[0] - __uint_as_float(label_bits);
+        loss = e * e;
+#pragma unroll 1
+        for (int j = lj; j < outp; j += G) d[j] = j == 0 ? rnd(bf16, 2.f * e) * act_grad(T.act, y[0]) : 0.f;
+      }
+      if (live && lj == 0) {
+        atomicAdd(S.core.loss_out + (r.inst & 0x7fffffff), loss);
+        if (inf) inf_sum += loss; else loss_sum += loss;
+      }
+    }
+    if (S.core.eval) return;
+    bar_compute();
+    phase(5);
+#pragma unroll 1
+    for (int i = tid; i < count * d4; i += CT) { const int b = i / d4, k = i - b * d4; if (R[b].inst >= 0) S.core.arena[R[b].a4 + k] = *reinterpret_cast<const float4*>(Ds + b * YP + 4 * k); }
+    // dx = D W: four columns per thread, a strip of the rows
+    if (!S.ppt.source_adj) {
+      const int strips = n4 < CT ? CT / n4 : 1;
+#pragma unroll 1
+      for (int k0 = 0; k0 < n4; k0 += CT) {
+        const int st = n4 < CT ? dn4.div(tid) : 0, k = n4 < CT ? tid - st * n4 : k0 + tid;
+        if (st >= strips || k >= n4) continue;
+#pragma unroll 1
+        for (int b = st; b < count; b += strips) {
+          if (R[b].inst < 0) continue;
+          float4 v = zero4();
+#pragma unroll 4
+          for (int j = 0; j < out; j++) {
+            const float dj = Ds[b * YP + j];
+            const float4 w = *reinterpret_cast<const float4*>(Ws + j * ld + 4 * k);
+            v.x = fmaf(dj, w.x, v.x); v.y = fmaf(dj, w.y, v.y); v.z = fmaf(dj, w.z, v.z); v.w = fmaf(dj, w.w, v.w);
+          }
+          S.core.arena[R[b].out4 + k] = rnd4(bf16, v);
+        }
+      }
+    }
+    if (T.G)                                                     // a summed input is kept for the accumulator
+#pragma unroll 1
+      for (int i = tid; i < count * n4; i += CT) { const int b = dn4.div(i), k = i - b * n4; if (R[b].inst >= 0) S.core.arena[R[b].a4 + d4 + k] = *reinterpret_cast<const float4*>(Xs + b * ld + 4 * k); }
+  }, [&](const unsigned long long ver) {
+    const unsigned pub = pub_of(ver);
+    if (pub != have) { have = pub; load_rows(m, pub, 1, outp, 0, outp, Ws, ld, bs); }
+  });
+  Globals* g = S.core.g;
+  for (int o = 16; o; o >>= 1) {
+    loss_sum += __shfl_xor_sync(0xffffffffu, loss_sum, o); inf_sum += __shfl_xor_sync(0xffffffffu, inf_sum, o);
+    correct += __shfl_xor_sync(0xffffffffu, correct, o); preds += __shfl_xor_sync(0xffffffffu, preds, o);
+    inf_correct += __shfl_xor_sync(0xffffffffu, inf_correct, o); inf_preds += __shfl_xor_sync(0xffffffffu, inf_preds, o);
+  }
+  if ((tid & 31) == 0) {
+    if (loss_sum != 0.0) atomicAdd(&g->total_loss, loss_sum);
+    if (inf_sum != 0.0) atomicAdd(&g->inf_loss, inf_sum);
+    if (correct) atomicAdd(&g->correct, correct);
+    if (preds) atomicAdd(&g->n_pred, preds);
+    if (inf_correct) atomicAdd(&g->inf_correct, inf_correct);
+    if (inf_preds) atomicAdd(&g->inf_pred, inf_preds);
+  }
+}
+
+// ---- embedding table -----------------------------------------------------------------------------------------------------------
+__device__ __noinline__ void lookup_main(const int team, RowD* rows, const unsigned long long t0) {
+  IN_SMEM(rows);
+  const int tid = threadIdx.x, out = S.ppt.out_dim, o4 = S.ppt.out4;
+  const FastDiv d4(o4);
+  const float* const W = S.ppt.W;
+  const bool wide = (out & 3) == 0;
+  chunk_loop(rows, team, t0, [&](const Head& h, const RowD* R) {
+#pragma unroll 2
+    for (int i = tid; i < h.count * o4; i += CT) {
+      const int b = d4.div(i), k = i - b * o4;
+      const float* e = W + (size_t)R[b].b4 * out + 4 * k;
+      float4 v;
+      if (wide) v = __ldcg(reinterpret_cast<const float4*>(e));
+      else { v.x = __ldcg(e); v.y = 4 * k + 1 < out ? __ldcg(e + 1) : 0.f; v.z = 4 * k + 2 < out ? __ldcg(e + 2) : 0.f; v.w = 4 * k + 3 < out ? __ldcg(e + 3) : 0.f; }
+      S.core.arena[R[b].out4 + k] = rnd4(S.core.bf16, v);
+    }
+  });
+}
+// A small table (its sums fit in shared memory): a thread owns columns and adds up its slice of the rows in a copy of the sums of
+// its own, several loads in flight.  Zipf-like ids pile up on a few rows, so the work is dealt by row, not by id.
+__device__ __noinline__ void lookup_grad_small_main(const int team, float* smem, RowD* rows, const unsigned long long t0) {
+  IN_SMEM(smem); IN_SMEM(rows);
+  const int tid = threadIdx.x, out = S.ppt.out_dim, ids = S.ppt.in_dim, cols = (out + 31) & ~31, slices = S.team.R;
+  const PptRun& P = S.ppt;
+  const int sl = tid / cols, c = tid - sl * cols;
+  float* const own = smem + (size_t)sl * ids * out + c;
+  const bool on = sl < slices && c < out;
+  int* const flag = reinterpret_cast<int*>(smem + (size_t)slices * ids * out);      // rows with gradients since the last update
+  const FastDiv dout(out);
+  for (int i = tid; i < slices * ids * out + ids; i += CT) smem[i] = 0.f;
+  bar_compute();
+  chunk_loop(rows, team, t0, [&](const Head& h, const RowD* R) {
+    if (on) {
+      const float* const arena = reinterpret_cast<const float*>(S.core.arena);
+      if (h.flags & H_COPIES) {
+#pragma unroll 4
+        for (int b = sl; b < h.count; b += slices) own[R[b].b4 * out] += __ldcg(arena + (size_t)R[b].t[0].src4 * 4 + c);
+      } else {
+#pragma unroll 1
+        for (int b = sl; b < h.count; b += 2 * slices) {
+          float g[2] = {0.f, 0.f};
+#pragma unroll
+          for (int q = 0; q < 2; q++) {
+            if (b + q * slices >= h.count) continue;
+            const RowD& r = R[b + q * slices];
+            const int nt = r.meta & E_NT, cc = c >> 2;
+            if (r.meta & E_OVERFLOW) { const float4 v = row_sum(r, cc); g[q] = (c & 3) == 0 ? v.x : (c & 3) == 1 ? v.y : (c & 3) == 2 ? v.z : v.w; continue; }
+#pragma unroll
+            for (int k = 0; k < 4; k++) { const Term t = r.t[k]; const unsigned d = (unsigned)cc - t.col4; if (k < nt && d < t.w4) g[q] += __ldcg(arena + (size_t)(t.src4 + d) * 4 + (c & 3)); }
+          }
+#pragma unroll
+          for (int q = 0; q < 2; q++) if (b + q * slices < h.count) own[R[b + q * slices].b4 * out] += rnd(S.core.bf16, g[q]);
+        }
+      }
+    }
+    for (int b = tid; b < h.count; b += CT) flag[R[b].b4] = 1;
+    if (h.flags & H_UPDATE) {
+      const OptStep os = opt_step(P.om, P.ov, P.opt_t0, h.n_upd, h.upd_t);
+      bar_compute();
+#pragma unroll 1
+      for (int i = tid; i < ids * out; i += CT) {
+        float a = 0.f;
+        for (int s = 0; s < slices; s++) { float* q = smem + (size_t)s * ids * out + i; a += *q; *q = 0.f; }
+        if (flag[dout.div(i)]) P.W[i] = opt_one(os, P.W[i], a, i);      // (the other rows keep their weights and moments)
+      }
+      bar_compute();
+      for (int i = tid; i < ids; i += CT) flag[i] = 0;
+      bar_compute();
+    }
+  });
+}
+// A large table: rows are dealt to the tiles by id; a piece of 128 columns of a row always belongs to the same warp of the tile and a
+// column to the same lane, so that a thread's adds and its own later reads are in order without fences or barriers.  A warp lists the
+// pieces it has touched since the last update (the list's overflow in device memory) and moves exactly those.
+__device__ __noinline__ void lookup_grad_main(const int team, const int tile, float* smem, RowD* rows, const unsigned long long t0) {
+  IN_SMEM(smem); IN_SMEM(rows);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, out = S.ppt.out_dim, o4 = S.ppt.out4, NTL = S.team.T;
+  const PptRun& P = S.ppt;
+  const int segs = (o4 + 31) >> 5, ids = (P.in_dim + NTL - 1) / NTL;
+  int* const near_list = reinterpret_cast<int*>(smem) + warp * NEAR;
+  int* const far_list = P.touched_list + ((size_t)tile * CW + warp) * ((size_t)ids * segs / CW + segs + 1);
+  const bool wide = (out & 3) == 0;
+  int touched = 0;                                               // (the same in all lanes)
+  auto update = [&](const int n_upd, const int upd_t) {
+    const OptStep os = opt_step(P.om, P.ov, P.opt_t0, n_upd, upd_t);
+#pragma unroll 1
+    for (int k0 = 0; k0 < touched; k0 += 2) {                    // two pieces' loads in flight
+      float a[2][4], w[2][4];
+      size_t r0[2];
+      int cq[2];
+#pragma unroll
+      for (int u = 0; u < 2; u++) {
+        const int k = min(k0 + u, touched - 1), piece = k < NEAR ? near_list[k] : far_list[k], local = piece / segs, c = (piece - local * segs) * 32 + lane;
+        r0[u] = ((size_t)local * NTL + tile) * out + 4 * c;
+        cq[u] = k0 + u < touched ? out - 4 * c : 0;
+        if (wide && cq[u] > 0) {
+          asm volatile("ld.relaxed.gpu.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(a[u][0]), "=f"(a[u][1]), "=f"(a[u][2]), "=f"(a[u][3]) : "l"(P.A + r0[u]) : "memory");
+          const float4 x = *reinterpret_cast<const float4*>(P.W + r0[u]);
+          w[u][0] = x.x; w[u][1] = x.y; w[u][2] = x.z; w[u][3] = x.w;
+        } else
+#pragma unroll
+          for (int q = 0; q < 4; q++)
+            if (q < cq[u]) { asm volatile("ld.relaxed.gpu.global.f32 %0, [%1];" : "=f"(a[u][q]) : "l"(P.A + r0[u] + q) : "memory"); w[u][q] = P.W[r0[u] + q]; }
+      }
+#pragma unroll
+      for (int u = 0; u < 2; u++)
+#pragma unroll
+        for (int q = 0; q < 4; q++)
+          if (q < cq[u]) {
+            P.W[r0[u] + q] = opt_one(os, w[u][q], a[u][q], r0[u] + q);
+            asm volatile("st.relaxed.gpu.global.f32 [%0], %1;" :: "l"(P.A + r0[u] + q), "f"(0.f) : "memory");
+          }
+    }
+    touched = 0;
+    __syncwarp();
+  };
+  chunk_loop(rows, team, t0, [&](const Head& h, const RowD* R) {
+#pragma unroll 1
+    for (int b0 = 0; b0 < h.count; b0 += 32) {
+      const unsigned id = R[min(b0 + lane, h.count - 1)].b4;
+      const int local = b0 + lane < h.count && (int)(id % (unsigned)NTL) == tile ? (int)(id / (unsigned)NTL) : -1;
+      if (!__any_sync(0xffffffffu, local >= 0)) continue;
+#pragma unroll 1
+      for (int q = 0; q < segs; q++) {
+        const int c = 32 * q + lane;
+        unsigned mine = __ballot_sync(0xffffffffu, local >= 0 && (local * segs + q) % CW == warp);
+        while (mine) {
+          // all rows of one id (a piece), four loads in flight, one add
+          const int id0 = __shfl_sync(0xffffffffu, local, __ffs((int)mine) - 1);
+          unsigned same = __ballot_sync(0xffffffffu, local == id0) & mine;
+          mine &= ~same;
+          float4 g = zero4();
+#pragma unroll 1
+          while (same) {
+            float4 v[4];
+#pragma unroll
+            for (int k = 0; k < 4; k++) {
+              v[k] = zero4();
+              const int l = same ? __ffs((int)same) - 1 : -1;
+              same &= same - 1;
+              if (l < 0 || c >= o4) continue;
+              const RowD& r = R[b0 + l];
+              v[k] = rnd4(S.core.bf16, h.flags & H_COPIES ? ldcg4(S.core.arena + r.t[0].src4 + c) : row_sum(r, c));
+            }
+            g = add4(g, add4(add4(v[0], v[1]), add4(v[2], v[3])));
+          }
+          float* const a = P.A + ((size_t)id0 * NTL + tile) * out + 4 * c;
+          if (c < o4) {
+            if (wide) asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" :: "l"(a), "f"(g.x), "f"(g.y), "f"(g.z), "f"(g.w) : "memory");
+            else {
+              const float v[4] = {g.x, g.y, g.z, g.w};
+#pragma unroll
+              for (int k = 0; k < 4; k++) if (4 * c + k < out) asm volatile("red.relaxed.gpu.global.add.f32 [%0], %1;" :: "l"(a + k), "f"(v[k]) : "memory");
+            }
+          }
+          const int piece = id0 * segs + q;
+          bool have = false;
+          for (int k = lane; k < touched; k += 32) have |= (k < NEAR ? near_list[k] : far_list[k]) == piece;
+          if (!__any_sync(0xffffffffu, have)) {
+            if (lane == 0) { if (touched < NEAR) near_list[touched] = piece; else far_list[touched] = piece; }
+            touched++;
+            __syncwarp();
+          }
+        }
+      }
+    }
+    if (h.flags & H_UPDATE) update(h.n_upd, h.upd_t);
+  });
+}
+
+// ---- the kernel -------------------------------------------------------------------------------------------------------------------
+extern "C" __global__ void __launch_bounds__(NT, 1) ampnet_engine_scheduled(const __grid_constant__ Run C) {
+  extern __shared__ __align__(128) unsigned char smem[];
+  const unsigned long long t0 = gtime();
+  const int tid = threadIdx.x, cta = blockIdx.x;
+  int team = 0;
+  while (team + 1 < C.core.n_teams && C.teams[team + 1].first <= cta) team++;
+  const int idx = cta - C.teams[team].first;
+  for (unsigned k = tid; k < sizeof(Team) / 4; k += NT) reinterpret_cast<unsigned*>(&S.team)[k] = reinterpret_cast<const unsigned*>(&C.teams[team])[k];
+  const int mi = C.teams[team].mat;
+  if (mi >= 0) for (unsigned k = tid; k < sizeof(Mat) / 4; k += NT) reinterpret_cast<unsigned*>(&S.mat)[k] = reinterpret_cast<const unsigned*>(&C.mats[mi])[k];
+  const int pi = C.teams[team].ppt;
+  for (unsigned k = tid; k < sizeof(PptRun) / 4; k += NT) reinterpret_cast<unsigned*>(&S.ppt)[k] = reinterpret_cast<const unsigned*>(&C.ppts[pi])[k];
+  for (unsigned k = tid; k < sizeof(Core) / 4; k += NT) reinterpret_cast<unsigned*>(&S.core)[k] = reinterpret_cast<const unsigned*>(&C.core)[k];
+  if (tid < MAX_CELLS) S.team_n[tid] = tid < C.core.n_teams ? C.teams[tid].n : 0;
+  if (tid < 64) S.stale_hist[tid] = 0;
+  if (tid == 0) {
+    for (int k = 0; k < 2; k++) { mbar_init(&S.full[k], HT); mbar_init(&S.empty[k], 1); }
+    mbar_init(&S.tc_mbar, 1);
+    for (int k = 0; k < N_PHASES; k++) S.phase[k] = 0;
+    S.mark = clock64();
+    S.stop = 0; S.ok = 1; S.ver = 0; S.batches = S.batch_rows = S.tc_batches = 0; S.max_stale = 0;
+    if (mi < 0) S.mat.ver = nullptr;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncthreads();
+  const bool tcm = S.team.bf16_tc != 0;
+  if (tcm) {
+    if (tid < 32) tc::tmem_alloc(&S.tmem);
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  }
+  const int T = S.team.T, tile = idx % T, shard = idx / T;
+  RowD* const rows = reinterpret_cast<RowD*>(smem + slots_bytes(C.core.mak));
+  float* const work = reinterpret_cast<float*>(rows + 2 * S.team.BM);
+  if (tid >= CT) helper_main(cta, tile, shard, smem, t0);
+  else switch (S.team.kind) {
+    case LIN_F:
+      if (S.team.bf16_tc) forward_main<F_TENSOR>(team, tile, work, rows, t0);
+      else if (S.team.lstm) forward_main<F_LSTM>(team, tile, work, rows, t0);
+      else forward_main<F_PLAIN>(team, tile, work, rows, t0);
+      break;
+    case GRU_ZR: forward_main<F_ZR>(team, tile, work, rows, t0); break;
+    case GRU_C: forward_main<F_C>(team, tile, work, rows, t0); break;
+    case LIN_DX: if (S.team.lstm) input_grad_main<B_LSTM>(team, tile, work, rows, t0); else input_grad_main<B_PLAIN>(team, tile, work, rows, t0); break;
+    case GRU_DC: input_grad_main<B_DC>(team, tile, work, rows, t0); break;
+    case GRU_DZR: input_grad_main<B_DZR>(team, tile, work, rows, t0); break;
+    case ACC: accumulate_main(team, tile, work, rows, t0); break;
+    case HEAD: head_main(team, work, rows, t0); break;
+    case LOOKUP_F: lookup_main(team, rows, t0); break;
+    case LOOKUP_B: if (S.team.R) lookup_grad_small_main(team, work, rows, t0); else lookup_grad_main(team, tile, work, rows, t0); break;
+  }
+  __syncthreads();
+  if (idx == 0 && tid < N_PHASES) C.core.phases[team * N_PHASES + tid] = S.phase[tid];
+  // micro-batches, staleness
+  PPTStats& st = *S.ppt.stats;
+  const int kind = S.team.kind;
+  if (tid == 0 && tile == 0 && (kind == LIN_F || kind == GRU_ZR || kind == HEAD || kind == LOOKUP_F || kind == LOOKUP_B || kind == LIN_DX || kind == GRU_DC || (kind == ACC && S.ppt.source_adj))) {
+    atomicAdd(&st.batches, S.batches); atomicAdd(&st.batch_rows, S.batch_rows);
+    if (S.tc_batches) atomicAdd(&st.tc_batches, S.tc_batches);
+  }
+  if (tile == 0 && kind == ACC && S.team.pad == 0) {
+    if (tid < 64) st.stale_hist[tid] = S.stale_hist[tid];
+    if (tid == 0) st.max_staleness = S.max_stale;
+  }
+  if (tcm && tid < 32) tc::tmem_free(S.tmem);
+}
+
+// ---- host hooks ---------------------------------------------------------------------------------------------------------------
+size_t smem_bytes(const Team& t, const Mat& m, int mak) {
+  const size_t head = slots_bytes(mak) + 2 * (size_t)t.BM * sizeof(RowD);
+  const size_t ldi = pad_ld(m.inp), ldo = pad_ld(m.outp), BM = t.BM;
+  size_t f = 0;
+  switch (t.kind) {
+    case LIN_F: case GRU_ZR: case GRU_C:
+      if (t.bf16_tc) f = (size_t)tc::M * m.inp / 2 + tc::M + ((BM + 15) & ~(size_t)15) * m.inp / 2 + BM * pad_ld(tc::M);
+      else f = (size_t)t.G * t.R * ldi + ((t.G * t.R + 3) & ~3) + BM * ldi + BM * pad_ld(t.G * t.R) + (t.kind == GRU_C ? BM * 2 * t.R : 0);
+      break;
+    case LIN_DX: case GRU_DC: case GRU_DZR: f = (size_t)t.R * ldo + BM * ldo + BM * pad_ld(t.R); break;
+    case ACC: f = (size_t)t.R * (t.C + 4) + (t.WO * t.WI < CW ? ACC_RED : 0) + BM * (t.R + 4 + t.C + 4) + t.R + (size_t)(CW / (t.WO * t.WI)) * t.R; break;
+    case LOOKUP_B: f = t.R ? (size_t)(t.R + 1) * t.C : CW * NEAR; break;      // (small table: R copies of C sums)
+    case HEAD: f = (size_t)m.outp * ldi + m.outp + BM * ldi + 2 * BM * pad_ld(m.outp); break;
+    default: break;
+  }
+  return head + f * sizeof(float) + 256;
+}
+int max_keys() { return 2048; }
+size_t static_smem() {
+  cudaFuncAttributes fa{};
+  return cudaFuncGetAttributes(&fa, ampnet_engine_scheduled) == cudaSuccess ? fa.sharedSizeBytes : 4096;
+}
+cudaError_t launch(const Run* run, int n_ctas, size_t smem, cudaStream_t st) {
+  static size_t set[64] = {};
+  int dev = 0;
+  cudaGetDevice(&dev);
+  if (dev < 0 || dev >= 64 || set[dev] < smem) {
+    const cudaError_t e = cudaFuncSetAttribute(ampnet_engine_scheduled, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    if (dev >= 0 && dev < 64) set[dev] = smem;
+  }
+  void* args[] = {const_cast<Run*>(run)};
+  return cudaLaunchCooperativeKernel((void*)ampnet_engine_scheduled, dim3(n_ctas), dim3(NT), args, smem, st);
+}
+
+}  // namespace wave

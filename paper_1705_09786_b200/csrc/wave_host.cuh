@@ -1,0 +1,589 @@
+// Host side of the scheduled engine (wave.h): which graphs it takes, encoding of loaded instances, placement and launch.
+// Included by ampnet.cu, inside its anonymous namespace.
+#pragma once
+
+
+static int pad4i(int v) { return (v + 3) & ~3; }
+
+// Padded layouts: a payload row is nseg segments of w columns, each padded to four floats (nseg = 1 where w needs no padding);
+// nseg 0: any (a zero payload).
+struct Lay { int nseg, w; bool operator==(const Lay& o) const { return nseg == o.nseg && w == o.w; } };
+static Lay lay(int nseg, int w) { return w % 4 == 0 ? Lay{1, nseg * w} : Lay{nseg, w}; }
+
+// Graphs the engine takes: a Loss is fed by a Linear node, a dense row feeds a Linear node, tokens feed a Lookup, an LSTM gate
+// node is fed by a Linear node of its own, and the padded layouts of joined payloads agree.
+using wave::WaveCell; using wave::WaveMat; using wave::WaveModel; using wave::WaveData; using wave::WaveTeam; using wave::WavePlan;
+
+static bool wave_model(const std::vector<DevNode>& nodes, const std::vector<int>& sources, int it_count, bool bf16, WaveModel& M, const std::vector<int>& ppt_nodes) {
+  using namespace wave;
+  const int n = (int)nodes.size(), np = (int)ppt_nodes.size();
+  M = WaveModel{};
+  if (n > ENC_MAX_NODES || np > ENC_MAX_PPTS) return false;
+  (void)bf16;
+  std::vector<Lay> L(n, Lay{-1, 0});            // -1: not known yet
+  std::vector<char> sums(n, 0);
+  for (int pass = 0; pass < 2 * n + 4; pass++)
+    for (int i = 0; i < n; i++) {
+      const DevNode& h = nodes[i];
+      Lay in{-1, 0};
+      bool s = false;
+      for (int k = 0; k < h.n_pred; k++) {
+        const Lay a = L[h.pred_node[k]];
+        s |= sums[h.pred_node[k]] != 0;
+        if (a.nseg <= 0) { if (a.nseg == 0 && in.nseg < 0) in = a; continue; }
+        if (in.nseg > 0 && !(in == a) && h.type != NPT_LSTM) return false;
+        if (h.type != NPT_LSTM || k == 0) in = a;
+      }
+      switch (h.type) {
+        case SOURCE: L[i] = Lay{0, 0}; break;
+        case LINEAR: case LOOKUP: case GRUCELL: L[i] = lay(1, h.out_dim); break;
+        case NPT_LSTM: L[i] = lay(2, h.out_dim / 2); break;
+        case CONCAT:
+          if (in.nseg > 0 && !(in == lay(1, h.in_dim))) return false;
+          L[i] = lay(h.fn_arg, h.in_dim); sums[i] = s; break;
+        case SPLIT:
+          if (in.nseg > 0 && !(in == lay(h.fn_arg, h.out_dim))) return false;
+          L[i] = lay(1, h.out_dim); sums[i] = s; break;
+        case NPT_SUMROWS: L[i] = in; sums[i] = 1; break;
+        default: L[i] = in; sums[i] = s; break;
+      }
+    }
+  EncModel& E = M.enc;
+  E.n_nodes = n; E.n_ppts = np; E.n_sources = (int)sources.size(); E.IT = it_count;
+  for (size_t k = 0; k < sources.size(); k++) E.sources[k] = sources[k];
+  for (int s : sources) {
+    const DevNode &h = nodes[s], &t = nodes[h.succ_node[0]];
+    if (h.fn == 1 && t.type != LINEAR) return false;
+    if (h.fn != 1 && h.fn != 3 && t.type != LOOKUP) return false;
+    if (h.fn == 3 && t.type == LINEAR) return false;
+  }
+  for (int i = 0; i < n; i++) {
+    const DevNode& h = nodes[i];
+    EncNode& N = E.nodes[i];
+    N = EncNode{};
+    N.type = h.type; N.fn = h.fn; N.fn_arg = h.fn_arg; N.n_succ = h.n_succ; N.n_pred = h.n_pred; N.ppt = h.ppt;
+    for (int k = 0; k < MAX_PORTS; k++) { N.succ_node[k] = (signed char)h.succ_node[k]; N.succ_port[k] = (signed char)h.succ_port[k]; N.pred_node[k] = (signed char)h.pred_node[k]; N.pred_port[k] = (signed char)h.pred_port[k]; }
+    if (h.type == CONCAT) N.w4 = pad4i(h.in_dim) / 4;
+    if (h.type == SPLIT) N.w4 = pad4i(h.out_dim) / 4;
+    if ((h.type == LOSS_CE || h.type == LOSS_MSE) && nodes[h.pred_node[0]].type != LINEAR) return false;
+    if (h.type == NPT_LSTM && (nodes[h.pred_node[0]].type != LINEAR || sums[h.pred_node[0]])) return false;
+  }
+  auto cell = [&](int kind, int p, int mat, int delay, bool fwd) { M.cells.push_back(WaveCell{kind, p, mat, delay, fwd}); return (int)M.cells.size() - 1; };
+  auto matrix = [&](int p, int row0, int nso, int out_w, int nsi, int in_w) {
+    M.mats.push_back(WaveMat{p, row0, out_w, nso, in_w, nsi, nso * pad4i(out_w), nsi * pad4i(in_w)});
+    return (int)M.mats.size() - 1;
+  };
+  for (int p = 0; p < np; p++) {
+    const int i = ppt_nodes[p];
+    const DevNode& h = nodes[i];
+    EncPpt& P = E.ppts[p];
+    P = EncPpt{};
+    for (int k = 0; k < 6; k++) P.cell[k] = -1;
+    P.kind = h.type; P.node = i; P.head = P.lstm = -1; P.source_adj = h.flags & 1;
+    P.out4 = pad4i(h.out_dim) / 4;
+    const Lay in = L[h.pred_node[0]];
+    P.xstore = h.type == LINEAR && sums[h.pred_node[0]];
+    if (h.type == LOOKUP) {
+      P.src_fn = nodes[h.pred_node[0]].fn;
+      P.cell[0] = cell(LOOKUP_F, p, -1, 0, true);
+      P.cell[1] = cell(LOOKUP_B, p, -1, 0, false);
+      continue;
+    }
+    if (h.type == GRUCELL) {
+      if (in.nseg > 0 && !(in == lay(2, h.out_dim))) return false;
+      P.in4 = 2 * P.out4;
+      const int zr = matrix(p, 0, 2, h.out_dim, 2, h.out_dim), c = matrix(p, 2 * h.out_dim, 1, h.out_dim, 2, h.out_dim);
+      P.cell[0] = cell(GRU_ZR, p, zr, 0, true);
+      P.cell[1] = cell(GRU_C, p, c, 1, true);
+      P.cell[2] = cell(GRU_DC, p, c, 0, false);
+      P.cell[3] = cell(GRU_DZR, p, zr, 1, false);
+      P.cell[4] = cell(ACC, p, c, 1, false);
+      P.cell[5] = cell(ACC, p, zr, 2, false);
+      continue;
+    }
+    const DevNode& s = nodes[h.succ_node[0]];
+    Lay il = in;
+    if (il.nseg <= 0) il = lay(1, h.in_dim);
+    if (il.nseg * il.w != h.in_dim) return false;
+    P.in4 = il.nseg * pad4i(il.w) / 4;
+    int mat;
+    if (s.type == NPT_LSTM) {
+      if (P.source_adj || P.xstore) return false;
+      P.lstm = h.succ_node[0];
+      const int gates = s.fn == 1 ? 3 : 5, H = s.out_dim / 2;
+      if (h.succ_port[0] != 0 || h.act != 0) return false;
+      mat = matrix(p, 0, gates, H, il.nseg, il.w);
+      P.out4 = pad4i(H) / 4;
+      P.gates4 = gates * P.out4;
+    } else mat = matrix(p, 0, 1, h.out_dim, il.nseg, il.w);
+    if (s.type == LOSS_CE || s.type == LOSS_MSE) {
+      P.head = h.succ_node[0];
+      P.cell[0] = cell(HEAD, p, mat, 0, true);
+      P.cell[1] = cell(ACC, p, mat, 1, false);
+    } else {
+      P.cell[0] = cell(LIN_F, p, mat, 0, true);
+      if (!P.source_adj) P.cell[1] = cell(LIN_DX, p, mat, 0, false);
+      P.cell[2] = cell(ACC, p, mat, P.source_adj ? 0 : 1, false);
+    }
+  }
+  // (teams poll with a lane each, one lane is left for the version word)
+  if (M.cells.size() > 31 || M.mats.size() > 24) return false;
+  E.n_cells = (int)M.cells.size();
+  for (int c = 0; c < E.n_cells; c++) { E.delay[c] = (unsigned char)M.cells[c].delay; E.forward[c] = M.cells[c].forward; }
+  // producers of every node's input and gradient: through the parameter-free nodes to the next parameterised ones
+  auto out_cell = [&](int p) { const EncPpt& P = E.ppts[p]; return P.kind == GRUCELL ? P.cell[1] : P.cell[0]; };
+  auto grad_cell = [&](int p) { const EncPpt& P = E.ppts[p]; return P.kind == GRUCELL ? P.cell[3] : P.head >= 0 ? P.cell[0] : P.kind == LOOKUP ? -1 : P.cell[1]; };
+  M.fwd_mask.assign(np, 0); M.bwd_mask.assign(np, 0);
+  for (int p = 0; p < np; p++) {
+    const DevNode& h = nodes[ppt_nodes[p]];
+    for (int dir = 0; dir < 2; dir++) {
+      std::vector<int> todo;
+      std::vector<char> seen(n, 0);
+      if (dir == 0) { for (int k = 0; k < h.n_pred; k++) todo.push_back(h.pred_node[k]); if (E.ppts[p].lstm >= 0) { const DevNode& l = nodes[E.ppts[p].lstm]; for (int k = 1; k < l.n_pred; k++) todo.push_back(l.pred_node[k]); } }
+      else { const DevNode& e = E.ppts[p].lstm >= 0 ? nodes[E.ppts[p].lstm] : h; for (int k = 0; k < e.n_succ; k++) todo.push_back(e.succ_node[k]); }
+      while (!todo.empty()) {
+        const int v = todo.back(); todo.pop_back();
+        if (v < 0 || seen[v]) continue;
+        seen[v] = 1;
+        const DevNode& x = nodes[v];
+        int q = x.ppt;
+        if (x.type == NPT_LSTM) q = nodes[x.pred_node[0]].ppt;
+        if (q >= 0) {
+          const int c = dir == 0 ? out_cell(q) : grad_cell(q);
+          if (c >= 0) (dir == 0 ? M.fwd_mask : M.bwd_mask)[p] |= 1u << c;
+          continue;
+        }
+        if (dir == 0) for (int k = 0; k < x.n_pred; k++) todo.push_back(x.pred_node[k]);
+        else for (int k = 0; k < x.n_succ; k++) todo.push_back(x.succ_node[k]);
+      }
+    }
+  }
+  M.ok = true;
+  return true;
+}
+
+// Sizes that depend on the loaded data: key spaces, scratch of an encoding warp.
+static void wave_sizes(WaveModel& M, const std::vector<DevNode>& nodes, const HostDataset& D) {
+  using namespace wave;
+  EncModel& E = M.enc;
+  unsigned long long w = 0, rows = 64, front = 64;
+  const unsigned long long IT = E.IT;
+  for (int i = 0; i < E.n_nodes; i++) {
+    const DevNode& h = nodes[i];
+    EncNode& N = E.nodes[i];
+    N.U = h.U_in; N.J = 0;
+    bool counted = true;
+    switch (h.type) {
+      case CONCAT: N.U = h.U_out; N.J = h.fn_arg; break;
+      case BCAST: case SPLIT: N.J = h.fn_arg; break;
+      case GROUP: N.U = h.U_out; N.J = h.rows_out; break;
+      case UNGROUP: N.J = h.rows_in; break;
+      case FLATMAP: N.J = D.maxOut; break;
+      case NPT_LSTM: N.J = 2; break;
+      case PHI: case NPT_SUMROWS: break;
+      default: counted = false;
+    }
+    const unsigned long long keys = IT * N.U;
+    N.ref_off = (unsigned)w; w += keys * N.J;
+    N.cnt_off = (unsigned)w; if (counted) w += keys;
+    rows += IT * std::max((unsigned long long)h.U_in * h.rows_in, (unsigned long long)h.U_out * h.rows_out) * (2 + std::max(h.n_succ, h.n_pred));
+    if (h.ppt >= 0) { EncPpt& P = E.ppts[h.ppt]; P.U = h.U_in; P.save_off = (unsigned)w; w += keys * 3; front += 3ull * h.U_in; }
+  }
+  E.table_words = (unsigned)((w + 3) & ~3ull);
+  bool forks = false;
+  for (int i = 0; i < E.n_nodes; i++) forks |= nodes[i].type == UNGROUP || nodes[i].type == GROUP || nodes[i].type == FLATMAP;
+  E.stack_cap = forks ? 1024 : 256;
+  E.front_cap = (unsigned)front; E.row_cap = (unsigned)rows; E.term_cap = (unsigned)(3 * rows);
+  unsigned long long messages = 4;
+  for (int c = 0; c < E.n_cells; c++) E.bound[c] = 0;
+  for (int p = 0; p < E.n_ppts; p++) {
+    const DevNode& h = nodes[E.ppts[p].node];
+    const unsigned long long b = IT * h.U_in * h.rows_in;
+    for (int k = 0; k < 6; k++) if (E.ppts[p].cell[k] >= 0) E.bound[E.ppts[p].cell[k]] = (unsigned)std::min<unsigned long long>(b, 1u << 30);
+    messages += 2 * IT * h.U_in;
+  }
+  E.steps_cap = (unsigned)std::min<unsigned long long>(messages + 4, 60000);
+  E.scratch_words = (unsigned)(((unsigned long long)E.table_words + 12ull * front + 6ull * rows + 2ull * rows + 31) & ~31ull);
+  E.near_scratch = (size_t)E.scratch_words * 4 + E.stack_cap * 16 <= 100 * 1024;
+}
+
+// ---- encoding of a loaded split (at the end of ampnet_load_instances) -------------------------------------------------------
+
+static ampnet_status_t wave_encode(ampnet_graph* g, HostDataset& D, WaveModel& M, WaveData& W, void** scratch, size_t* scratch_cap) {
+  using namespace wave;
+  W = WaveData{};
+  const long long n = D.n;
+  if (!M.ok || n < 1 || n > (1ll << 30)) return AMPNET_OK;
+  wave_sizes(M, g->hnodes, D);
+  for (auto& h : g->hnodes) if (h.U_in > 65535 || h.U_out > 65535) return AMPNET_OK;      // (positions travel in sixteen bits)
+  if ((unsigned long long)M.enc.scratch_words * 4 > (1ull << 30)) return AMPNET_OK;
+  const EncModel& E = M.enc;
+  // warps per block: with the scratch in shared memory as many as fit there (an SM holds 16 of them by registers)
+  const size_t warp_bytes = (size_t)E.scratch_words * 4;
+  int per = encode_warps_per_block();
+  if (E.near_scratch) per = (int)std::max<size_t>(1, std::min<size_t>(per, (size_t)(200 * 1024) / (warp_bytes + E.stack_cap * 16)));
+  if (n < (long long)g->n_sms * per) per = 1;
+  long long blocks = (n + per - 1) / per;
+  EncTotals init{};
+  init.steps_min = init.steps_eval_min = 0xffffffffu;
+  size_t bytes = 0;
+  auto take = [&](size_t b) { const size_t at = bytes; bytes += (b + 255) & ~(size_t)255; return at; };
+  std::vector<size_t> tab_at(E.n_cells), ent_at(E.n_cells);
+  // a handful of small instances: one pass, each with room for the most it can need
+  unsigned long long room = 0;
+  bool sums = false;
+  for (int c = 0; c < E.n_cells; c++) room += (unsigned long long)n * (E.bound[c] * sizeof(Entry) + E.steps_cap * 4ull);
+  for (auto& h : g->hnodes) sums |= h.type == NPT_SUMROWS || h.type == FLATMAP || (h.type == CONCAT && h.fn_arg > 4) || (h.type == BCAST && h.fn_arg > 4);
+  if (E.near_scratch && !sums && room <= (8ull << 20)) {
+    const size_t tot_at = take(sizeof(EncTotals)), hdr_at = take((size_t)n * sizeof(InstHdr));
+    for (int c = 0; c < E.n_cells; c++) { tab_at[c] = take(((size_t)n * E.steps_cap + 2) * 4); ent_at[c] = take((size_t)n * E.bound[c] * sizeof(Entry)); }
+    char* mem = (char*)dev_alloc(g, bytes);
+    if (!mem) return set_err(g, AMPNET_ENOMEM, "device allocation of %zu bytes (message programs) failed", bytes);
+    D.allocs.push_back(mem);
+    EncTotals* totals = (EncTotals*)(mem + tot_at);
+    W.prog.hdr = (InstHdr*)(mem + hdr_at);
+    for (int c = 0; c < E.n_cells; c++) { W.prog.tab[c] = (const unsigned*)(mem + tab_at[c]); W.prog.ent[c] = (const Entry*)(mem + ent_at[c]); }
+    CUDA_TRY(g, cudaMemcpyAsync(totals, &init, sizeof init, cudaMemcpyHostToDevice, g->stream));
+    CUDA_TRY(g, encode_bounded(&E, D.dev, (int)blocks, per, W.prog, totals, g->stream));
+    CUDA_TRY(g, cudaMemcpyAsync(&W.tot, totals, sizeof W.tot, cudaMemcpyDeviceToHost, g->stream));
+    CUDA_TRY(g, cudaStreamSynchronize(g->stream));
+    W.ok = W.tot.status == 0;
+    return AMPNET_OK;
+  }
+  blocks = std::min<long long>(blocks, 8ll * g->n_sms);
+  size_t need = 256;
+  if (!E.near_scratch) {
+    blocks = std::min<long long>(blocks, 4ll * g->n_sms);
+    blocks = std::min<long long>(blocks, std::max<long long>(1, (long long)((512ull << 20) / (warp_bytes * per))));
+    need = (size_t)blocks * per * warp_bytes;
+  }
+  if (need > *scratch_cap) {
+    dev_free(g, *scratch);
+    *scratch = dev_alloc(g, need);
+    *scratch_cap = *scratch ? need : 0;
+    if (!*scratch) return set_err(g, AMPNET_ENOMEM, "device allocation of %zu bytes (encoder) failed", need);
+  }
+  const size_t hdr_b = (size_t)n * sizeof(InstHdr), cnt_b = (size_t)E.n_cells * n * 4, tot_b = sizeof(EncTotals);
+  char* meta = (char*)dev_alloc(g, hdr_b + ((cnt_b + 255) & ~(size_t)255) + tot_b + 256);
+  if (!meta) return set_err(g, AMPNET_ENOMEM, "device allocation (program headers) failed");
+  D.allocs.push_back(meta);
+  InstHdr* hdr = (InstHdr*)meta;
+  unsigned* counts = (unsigned*)(meta + hdr_b);
+  EncTotals* totals = (EncTotals*)(meta + hdr_b + ((cnt_b + 255) & ~(size_t)255));
+  CUDA_TRY(g, cudaMemcpyAsync(totals, &init, sizeof init, cudaMemcpyHostToDevice, g->stream));
+  if (!E.near_scratch) CUDA_TRY(g, cudaMemset2DAsync(*scratch, warp_bytes, 0, (size_t)E.table_words * 4, (size_t)blocks * per, g->stream));
+  CUDA_TRY(g, encode_count(&E, D.dev, (unsigned*)*scratch, (int)blocks, per, hdr, counts, totals, g->stream));
+  CUDA_TRY(g, encode_scan(counts, hdr, n, E.n_cells, totals, g->stream));
+  CUDA_TRY(g, cudaMemcpyAsync(&W.tot, totals, sizeof W.tot, cudaMemcpyDeviceToHost, g->stream));
+  CUDA_TRY(g, cudaStreamSynchronize(g->stream));
+  if (getenv("AMPNET_DEBUG")) {
+    fprintf(stderr, "[ampnet] programs: status %d, %u steps table, arena %u x 16 B, steps min %u (eval %u) mean %.1f, overflow terms %u, entries", W.tot.status, W.tot.tab, W.tot.arena4_max,
+            W.tot.steps_min, W.tot.steps_eval_min, (double)W.tot.steps_sum / n, W.tot.ov);
+    for (int c = 0; c < E.n_cells; c++) fprintf(stderr, " %u", W.tot.entries[c]);
+    fprintf(stderr, "\n");
+  }
+  if (W.tot.status != 0) return AMPNET_OK;       // (a structure beyond the encoder's bounds: the interpreter engine runs it)
+  for (int c = 0; c < E.n_cells; c++) { tab_at[c] = take(((size_t)W.tot.tab + 2) * 4); ent_at[c] = take((size_t)W.tot.entries[c] * sizeof(Entry)); }
+  const size_t ov_at = take((size_t)W.tot.ov * sizeof(Term));
+  char* mem = (char*)dev_alloc(g, bytes);
+  if (!mem) return set_err(g, AMPNET_ENOMEM, "device allocation of %zu bytes (message programs) failed", bytes);
+  D.allocs.push_back(mem);
+  W.prog.hdr = hdr;
+  for (int c = 0; c < E.n_cells; c++) { W.prog.tab[c] = (const unsigned*)(mem + tab_at[c]); W.prog.ent[c] = (const Entry*)(mem + ent_at[c]); }
+  W.prog.ov = (const Term*)(mem + ov_at);
+  CUDA_TRY(g, encode_emit(&E, D.dev, (unsigned*)*scratch, (int)blocks, per, W.prog, counts, (Term*)(mem + ov_at), totals, g->stream));
+  W.ok = true;
+  return AMPNET_OK;
+}
+
+// ---- placement -----------------------------------------------------------------------------------------------------------------
+// Every cell gets the CTAs that bring its estimated time per round down, the slowest cell first, until the SMs are dealt out or
+// nothing gains.  The estimate (in cycles) counts the latency of a gather, its bytes, the multiply-adds at the rate the
+// products reach, the reload of updated weights and, for accumulators, the merge at updates.
+
+static bool wave_best(const WaveModel& M, int c, int ctas, double rows, double msgs_per_update, bool eval, size_t budget, int mak, bool bf16, bool use_tc, const ampnet_graph* g, WaveTeam& best) {
+  using namespace wave;
+  const WaveCell& K = M.cells[c];
+  const EncPpt& P = M.enc.ppts[K.ppt];
+  const DevNode& h = g->hnodes[P.node];
+  Team t{};
+  t.kind = K.kind; t.ppt = K.ppt; t.mat = K.mat; t.cell = c; t.acc = -1; t.T = t.Sh = t.n = 1; t.G = 1; t.act = h.type == LINEAR ? h.act : 0;
+  t.H4 = pad4i(h.type == LINEAR && P.lstm >= 0 ? g->hnodes[P.lstm].out_dim / 2 : h.out_dim) / 4;
+  t.keep = P.xstore;
+  t.lstm = P.lstm >= 0 ? (g->hnodes[P.lstm].fn == 1 ? 3 : 5) : 0;
+  t.k4 = P.kind == LOOKUP || K.kind == LIN_DX || K.kind == GRU_DC ? t.H4 * (t.lstm ? 2 : 1) : P.in4;      // what the cell's rows are made of: gradients or inputs
+  Mat m{};
+  if (K.mat >= 0) { const WaveMat& w = M.mats[K.mat]; m.outp = w.outp; m.inp = w.inp; m.out_w = w.out_w; m.nso = w.nso; m.in_w = w.in_w; m.nsi = w.nsi; }
+  const double upd = eval ? 0.0 : std::min(1.0, rows / std::max(1.0, msgs_per_update));      // rounds with new weights
+  bool found = false;
+  auto offer = [&](Team x, double cycles) {
+    static const int caps[] = {128, 96, 64, 48, 32, 24, 16, 8};
+    for (int bm : caps) {
+      if (bm > 32 && bm >= 2 * rows / x.Sh + 32) continue;              // (no more staging than a round needs)
+      if (x.bf16_tc && bm > 64) continue;
+      x.BM = bm;
+      if (smem_bytes(x, m, mak) > budget) continue;
+      const double chunks = std::max(1.0, rows / x.Sh / bm);
+      cycles += 900.0 * (chunks - 1.0);
+      if (!found || cycles < best.cycles * 0.995) { best.t = x; best.cycles = cycles; found = true; }
+      return;
+    }
+  };
+  const double lat = 700, bpc = 36, fma = 128 * 0.42;
+  int env_rows = 0, env_cols = 0;
+  if (const char* e = getenv("AMPNET_DIRECT_ROWS")) env_rows = std::max(1, atoi(e));
+  if (const char* e = getenv("AMPNET_DIRECT_COLS")) env_cols = std::max(4, atoi(e));
+  switch (K.kind) {
+    case LIN_F: case GRU_ZR: case GRU_C: {
+      t.G = K.kind == GRU_ZR ? 2 : t.lstm ? t.lstm : 1;
+      const int gw = 4 * t.H4;
+      const bool tc = bf16 && use_tc && K.kind == LIN_F && !t.lstm && h.out_dim % 64 == 0 && h.in_dim % 16 == 0 && m.inp == h.in_dim;
+      for (int T = 1; T <= std::min(ctas, gw / 4); T++) {
+        Team x = t;
+        x.R = tc ? 64 : pad4i((gw + T - 1) / T);
+        if (env_rows && !tc) x.R = std::min(gw, pad4i(env_rows));
+        x.T = (gw + x.R - 1) / x.R;
+        if (x.T > ctas) continue;
+        if (x.T != T && !tc && !env_rows) continue;
+        x.bf16_tc = tc;
+        x.Sh = std::max(1, std::min(ctas / x.T, (int)std::ceil(rows)));
+        x.n = x.T * x.Sh;
+        const double rs = std::max(1.0, rows / x.Sh), outs = x.R * x.G;
+        const double g_cyc = lat + (rs * m.inp * 4.0 + upd * outs * m.inp * 4.0) / bpc;
+        const double k_cyc = tc ? 600 + rs * m.inp / 64.0 : 250 + std::max(4.0, rs) * outs * m.inp / fma;
+        offer(x, g_cyc + k_cyc + 200 + (t.lstm ? 300 : 0));
+        if (tc || env_rows) break;
+      }
+      break;
+    }
+    case LIN_DX: case GRU_DC: case GRU_DZR:
+      for (int T = 1; T <= std::min(ctas, m.inp / 4); T++) {
+        Team x = t;
+        x.R = pad4i((m.inp + T - 1) / T);
+        if (env_cols) x.R = std::min(m.inp, pad4i(env_cols));
+        x.T = (m.inp + x.R - 1) / x.R;
+        if (x.T > ctas) { if (env_cols) break; continue; }
+        if (x.T != T && !env_cols) continue;
+        x.Sh = std::max(1, std::min(ctas / x.T, (int)std::ceil(rows)));
+        x.n = x.T * x.Sh;
+        const double rs = std::max(1.0, rows / x.Sh);
+        const double g_cyc = 1.3 * lat + (rs * m.outp * 4.0 * 3.2 + upd * x.R * m.outp * 4.0) / bpc;
+        offer(x, g_cyc + 250 + std::max(4.0, rs) * x.R * m.outp / fma + 200);
+        if (env_cols) break;
+      }
+      break;
+    case ACC:
+      for (int LO = 1; LO <= 8; LO *= 2)
+        for (int WO = 1; WO <= 16; WO *= 2)
+          for (int WI = 1; WO * WI <= 16; WI *= 2) {
+            Team x = t;
+            x.LO = LO; x.WO = WO; x.WI = WI; x.R = WO * 8 * LO; x.C = WI * 4 * (32 / LO);
+            if (x.R > 512) continue;
+            x.T = ((m.outp + x.R - 1) / x.R) * ((m.inp + x.C - 1) / x.C);
+            if (x.T > ctas) continue;
+            x.n = x.T;
+            const double area = (double)x.R * x.C, ws = 16.0 / (WO * WI);
+            offer(x, lat + rows * (std::min(x.R, m.outp) + std::min(x.C, m.inp)) * 4.0 / bpc + rows * area / (128 * 0.5) + upd * (400 + area * (2 * ws + 3) / 100.0));
+          }
+      break;
+    case HEAD:
+      for (int n = 1; n <= std::min(ctas, std::max(1, (int)rows)); n++) {
+        Team x = t;
+        x.Sh = x.n = n; x.G = P.xstore; x.R = 0;
+        const double rs = std::max(1.0, rows / n);
+        offer(x, lat + (rs * m.inp * 4.0 + upd * m.outp * m.inp * 4.0) / bpc + 900 + 3.0 * rs * m.inp * m.outp / (128 * 0.25));
+      }
+      break;
+    case LOOKUP_F:
+      for (int n = 1; n <= std::min(ctas, std::max(1, (int)rows)); n++) {
+        Team x = t;
+        x.Sh = x.n = n;
+        offer(x, lat + rows / n * h.out_dim * 4.0 * 2 / bpc);
+      }
+      break;
+    default: {    // LOOKUP_B: the sums of a small table in shared memory, otherwise rows dealt to tiles by id
+      const int cols = (h.out_dim + 31) & ~31;
+      if (cols <= 512 && (long long)h.in_dim * h.out_dim * 4 <= 48 * 1024) {
+        Team x = t;
+        x.R = 512 / cols; x.C = h.in_dim * h.out_dim;
+        while (x.R > 1 && (long long)x.R * x.C * 4 > 128 * 1024) x.R--;
+        offer(x, 2500 + rows / x.R * 250 + upd * (1500 + (double)x.C * x.R / 40.0));
+        break;
+      }
+      for (int n = 1; n <= std::min(ctas, std::max(1, h.in_dim / 8)); n++) {
+        Team x = t;
+        x.T = x.n = n;
+        offer(x, 3000 + rows * 15.0 + rows / n * 150.0 + upd * (2500 + std::min(msgs_per_update, (double)h.in_dim) / n * 150.0));
+      }
+    }
+  }
+  return found;
+}
+
+
+static WavePlan wave_place(const ampnet_graph* g, const WaveModel& M, const WaveData& W, int mak, int muf, bool eval, long long n_order, long long n_loaded, int n_ctas) {
+  using namespace wave;
+  WavePlan P;
+  if (!M.ok || !W.ok || mak > max_keys() || n_loaded < 1) return P;
+  const unsigned dmin = std::max(1u, eval ? W.tot.steps_eval_min : std::min(W.tot.steps_min, W.tot.steps_eval_min));
+  P.copies = 1 + (int)((DRIFT + dmin - 1) / dmin);
+  if ((unsigned long long)mak * P.copies * (W.tot.arena4_max + 8ull) > 0xf0000000ull) return P;      // (offsets are 32 bits of 16 bytes)
+  static const size_t fixed = static_smem();
+  const size_t budget = (size_t)g->max_smem - fixed - 1024;
+  bool use_tc = true;
+  if (const char* e = getenv("AMPNET_TENSOR_CORES")) use_tc = atoi(e) != 0;
+  const double steps = (double)(eval ? W.tot.steps_eval_sum : W.tot.steps_sum);
+  const double keys = (double)std::max<long long>(1, std::min<long long>(mak, n_order));
+  std::vector<int> cells;
+  for (int c = 0; c < (int)M.cells.size(); c++) if (!eval || M.cells[c].forward) cells.push_back(c);
+  const int nc = (int)cells.size();
+  std::vector<int> got(nc, 0);
+  P.teams.resize(nc);
+  auto rows_of = [&](int c) { return keys * W.tot.entries[c] / std::max(1.0, steps); };
+  auto muf_of = [&](int c) { const int o = g->nodes[M.enc.ppts[M.cells[c].ppt].node].muf_override; return (double)(o > 0 ? o : muf); };
+  auto best = [&](int k, int n, WaveTeam& t) { return wave_best(M, cells[k], n, rows_of(cells[k]), muf_of(cells[k]), eval, budget, mak, g->payload_bf16, use_tc, g, t); };
+  int used = 0;
+  for (int k = 0; k < nc; k++) {
+    int n = 1;
+    while (n <= n_ctas && !best(k, n, P.teams[k])) n++;
+    if (n > n_ctas) { if (getenv("AMPNET_DEBUG")) fprintf(stderr, "[ampnet] cell %d does not fit\n", cells[k]); return P; }
+    got[k] = P.teams[k].t.n; used += got[k];
+  }
+  if (used > n_ctas) { if (getenv("AMPNET_DEBUG")) fprintf(stderr, "[ampnet] %d CTAs needed\n", used); return P; }
+  std::vector<char> stuck(nc, 0);
+  for (;;) {
+    int worst = -1;
+    for (int k = 0; k < nc; k++) if (!stuck[k] && (worst < 0 || P.teams[k].cycles > P.teams[worst].cycles)) worst = k;
+    if (worst < 0) break;
+    // the next larger count that gains at least 2 % (tile counts move in steps)
+    bool grown = false;
+    for (int n = got[worst] + 1; n <= got[worst] + (n_ctas - used) && n <= got[worst] + 16; n++) {
+      WaveTeam t;
+      if (!best(worst, n, t) || t.t.n <= got[worst] || t.cycles > P.teams[worst].cycles * 0.98) continue;
+      used += t.t.n - got[worst]; got[worst] = t.t.n; P.teams[worst] = t;
+      grown = true;
+      break;
+    }
+    if (!grown) stuck[worst] = 1;
+  }
+  // team indices: accumulators publish to the readers of their matrix; who waits for whom
+  std::vector<int> team_of(M.cells.size(), -1);
+  for (int k = 0; k < nc; k++) team_of[cells[k]] = k;
+  auto to_teams = [&](unsigned mask) { unsigned r = 0; for (int c = 0; c < (int)M.cells.size(); c++) if ((mask >> c & 1) && team_of[c] >= 0) r |= 1u << team_of[c]; return r; };
+  int first = 0;
+  for (int k = 0; k < nc; k++) {
+    Team& t = P.teams[k].t;
+    const int c = cells[k], p = t.ppt;
+    const EncPpt& E = M.enc.ppts[p];
+    t.first = first; first += t.n;
+    if (!eval && t.kind != ACC && t.mat >= 0)
+      for (int j = 0; j < nc; j++) if (P.teams[j].t.kind == ACC && P.teams[j].t.mat == t.mat) t.acc = j;
+    if (!eval && t.kind == LOOKUP_F) t.acc = team_of[E.cell[1]];
+    unsigned mask = 0;
+    switch (t.kind) {
+      case LIN_F: case HEAD: case GRU_ZR: mask = M.fwd_mask[p]; break;
+      case GRU_C: mask = 1u << E.cell[0]; break;
+      case LIN_DX: case LOOKUP_B: case GRU_DC: mask = M.bwd_mask[p]; break;
+      case GRU_DZR: mask = 1u << E.cell[2]; break;
+      case ACC: mask = E.kind == GRUCELL ? 1u << (c == E.cell[4] ? E.cell[2] : E.cell[3]) : E.head >= 0 ? 1u << E.cell[0] : E.source_adj ? M.bwd_mask[p] : 1u << E.cell[1]; break;
+      default: break;
+    }
+    t.wait_mask = to_teams(mask);
+    if (t.kind == ACC) { t.G = 0; for (int j = 0; j < nc; j++) { const Team& u = P.teams[j].t; if (u.mat == t.mat && (u.kind == LIN_DX || u.kind == GRU_DC || u.kind == GRU_DZR)) t.G = 1; } }      // the transposed copy is read
+    if (t.kind == ACC && E.kind == GRUCELL && c == E.cell[5]) t.pad = 1;      // (the node's statistics come from the other one)
+    Mat m{};
+    if (t.mat >= 0) { m.outp = M.mats[t.mat].outp; m.inp = M.mats[t.mat].inp; }
+    P.smem = std::max(P.smem, smem_bytes(t, m, mak));
+  }
+  P.n_ctas = first;
+  // Instances of one size would move in lockstep, all of them in the same cell at a time: once a round's rows are more than a
+  // cell's fixed costs hide, admissions are spread over the steps of an instance.
+  double entries = 0;
+  for (int c : cells) entries += W.tot.entries[c];
+  // An instance that is a chain (a dense row, a list: about one message at a time) gains nothing from more company than keeps
+  // the rounds' fixed costs shared, and its gradients only get staler: four such instances start per round.
+  P.pace = mak;
+  double forward_rows = 0;
+  for (int c : cells) if (M.cells[c].forward && M.cells[c].kind != LOOKUP_F && M.cells[c].kind != GRU_C) forward_rows += W.tot.entries[c];
+  if (!eval && forward_rows < 1.5 * steps) P.pace = std::min(mak, 4);
+  else if (keys * entries / std::max(1.0, steps) >= 64.0) P.pace = (int)std::max(1.0, std::ceil(keys * (double)n_loaded / std::max(1.0, steps)));
+  P.ok = true;
+  return P;
+}
+
+// ---- a run -----------------------------------------------------------------------------------------------------------------------
+// Carves the run's scratch from the handle's arenas (dry: sizes only) and fills the kernel's argument.  What the host reads
+// back and what must start at zero lies together at the front of the control arena.
+struct WaveScratch { size_t zero_bytes, read_bytes, stats_at, loss_at, node_msgs_at, phases_at; };
+static WaveScratch wave_carve(ampnet_graph* g, HostDataset& D, const WaveModel& M, const WaveData& W, const WavePlan& P, int mak, int eval, const ampnet_run_cfg_t* cfg,
+                              long long n_order, bool dry, wave::Run& R) {
+  using namespace wave;
+  DeviceArena &C = g->ctl, &B = g->bulk;
+  C.used = B.used = 0;
+  C.base = dry ? nullptr : (char*)g->ctl_mem; B.base = dry ? nullptr : (char*)g->bulk_mem;
+  g->leftover_regions.clear();
+  g->zero_regions.clear();
+  const size_t np = g->ppts.size();
+  WaveScratch S{};
+  R = Run{};
+  R.core.g = C.take<Globals>(1);
+  PPTStats* stats = C.take<PPTStats>(np);
+  S.stats_at = C.used - np * sizeof(PPTStats);
+  g->d_node_msgs = C.take<unsigned long long>(g->hnodes.size() * 2);
+  S.node_msgs_at = C.used - g->hnodes.size() * 2 * sizeof(unsigned long long);
+  R.core.phases = C.take<unsigned long long>(MAX_CELLS * N_PHASES);
+  S.phases_at = C.used - MAX_CELLS * N_PHASES * sizeof(unsigned long long);
+  const size_t nl = (size_t)std::max<long long>(D.n, 1);
+  R.core.loss_out = C.take<float>(nl);
+  S.loss_at = C.used - nl * sizeof(float);
+  S.read_bytes = C.used;
+  R.core.progress = C.take<unsigned>(MAX_CELLS * 16);
+  g->d_stats.assign(np, nullptr);
+  g->d_update_log.assign(np, nullptr);
+  R.core.n_teams = (int)P.teams.size(); R.n_mats = (int)M.mats.size(); R.n_ppts = (int)np; R.core.n_ctas = P.n_ctas;
+  for (int k = 0; k < R.core.n_teams; k++) R.teams[k] = P.teams[k].t;
+  for (int k = 0; k < R.n_mats; k++) {
+    const WaveMat& w = M.mats[k];
+    const HostPPT& H = g->ppts[w.ppt];
+    Mat& m = R.mats[k];
+    m.W = H.W; m.b = H.b; m.om = H.om; m.ov = H.ov; m.nW = (long long)H.nW; m.opt_t0 = H.opt_t;
+    m.row0 = w.row0; m.in_real = H.in; m.out_w = w.out_w; m.nso = w.nso; m.in_w = w.in_w; m.nsi = w.nsi; m.outp = w.outp; m.inp = w.inp;
+    if (eval) continue;
+    const size_t area = (size_t)w.outp * w.inp;
+    m.Wp = B.take<float>(PUB * area); m.WTp = B.take<float>(PUB * area); m.bp = B.take<float>((size_t)PUB * w.outp);
+    m.ver = reinterpret_cast<unsigned*>(C.take<unsigned long long>(32));
+  }
+  for (size_t p = 0; p < np; p++) {
+    const HostPPT& H = g->ppts[p];
+    const EncPpt& E = M.enc.ppts[p];
+    PptRun& Q = R.ppts[p];
+    const int o = g->nodes[H.node].muf_override;
+    Q.kind = H.kind; Q.node = H.node; Q.act = g->hnodes[H.node].act; Q.muf = o > 0 ? o : (cfg ? cfg->min_update_frequency : 1);
+    Q.loss_type = E.head >= 0 ? g->hnodes[E.head].type : -1; Q.source_adj = E.source_adj && E.head < 0;
+    Q.stats = stats ? stats + p : nullptr;
+    Q.in_dim = H.in; Q.out_dim = H.out; Q.out4 = pad4i(H.out) / 4;
+    Q.W = H.W; Q.om = H.om; Q.ov = H.ov; Q.opt_t0 = H.opt_t;
+    g->d_stats[p] = Q.stats;
+    if (eval) continue;
+    Q.update_log = B.take<int>(g->update_log_cap); Q.log_cap = g->update_log_cap;
+    g->d_update_log[p] = Q.update_log;
+    if (H.kind == LOOKUP) {
+      auto zeroed = [&](size_t n_floats) { float* a = B.take<float>(n_floats); if (!dry) g->zero_regions.push_back({a, n_floats * sizeof(float)}); return a; };
+      int T = 1;
+      for (auto& t : P.teams) if (t.t.kind == LOOKUP_B && t.t.ppt == (int)p) T = t.t.T;
+      Q.A = zeroed(H.nW);
+      const size_t segs = (size_t)(Q.out4 + 31) / 32, ids = (size_t)(H.in + T - 1) / T;      // a list per tile and warp
+      Q.touched_list = B.take<int>((size_t)T * 16 * (ids * segs / 16 + segs + 1));
+    }
+  }
+  S.zero_bytes = C.used;
+  R.core.prog = W.prog;
+  R.core.copies = P.copies; R.core.slot4 = (W.tot.arena4_max + 7) & ~7u;
+  R.core.arena = B.take<float4>((size_t)mak * R.core.copies * R.core.slot4 + 8);
+  R.core.n_order = n_order;
+  R.core.dense = D.dev.dense; R.core.dense_dim = D.dense_dim;
+  R.core.mak = mak; R.core.eval = eval; R.core.bf16 = g->payload_bf16 ? 1 : 0; R.core.lag = mak == 1 ? 1 : 2; R.core.pace = P.pace;
+  R.core.lr = cfg ? cfg->lr : 0.f; R.core.opt = g->opt; R.core.mu = g->opt_mu; R.core.beta1 = g->opt_beta1; R.core.beta2 = g->opt_beta2; R.core.eps = g->opt_eps;
+  R.core.timeout_ns = (unsigned long long)((cfg && cfg->timeout_s > 0 ? cfg->timeout_s : 120.0) * 1e9);
+  return S;
+}
