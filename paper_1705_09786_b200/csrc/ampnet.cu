@@ -1115,8 +1115,6 @@ ampnet_status_t wave_execute(ampnet_graph* g, HostDataset& D, const WavePlan& P,
   for (auto& z : g->zero_regions) CUDA_TRY(g, cudaMemsetAsync(z.first, 0, z.second, g->stream));
   if (getenv("AMPNET_DEBUG")) {
     fprintf(stderr, "[ampnet] scheduled engine, %d CTAs, %zu B smem, ctl %zu B, bulk %zu B, arena %u x 16 B x %d x %d\n", P.n_ctas, P.smem, g->ctl.used, g->bulk.used, R.core.slot4, mak, R.core.copies);
-    static const char* names[] = {"LOOKUP_F", "LOOKUP_B", "LIN_F", "LIN_DX", "ACC", "HEAD", "GRU_ZR", "GRU_C", "GRU_DC", "GRU_DZR"};
-    for (auto& t : P.teams) fprintf(stderr, "[ampnet]   node %2d %-8s %3d CTAs = %d tiles x %d shards, R %d C %d BM %d%s, est %.0f cycles\n", g->ppts[t.t.ppt].node, names[t.t.kind], t.t.n, t.t.T, t.t.Sh, t.t.R, t.t.C, t.t.BM, t.t.bf16_tc ? " tc" : "", t.cycles);
   }
   for (auto& H : g->ppts) { H.LT = 1; }
   for (auto& t : P.teams) { HostPPT& H = g->ppts[t.t.ppt]; if (t.t.kind == wave::LIN_F || t.t.kind == wave::HEAD || t.t.kind == wave::GRU_ZR || t.t.kind == wave::LOOKUP_F) { H.T = t.t.n; H.BM = t.t.BM; } }
@@ -1136,8 +1134,11 @@ ampnet_status_t wave_execute(ampnet_graph* g, HostDataset& D, const WavePlan& P,
   if (getenv("AMPNET_DEBUG")) {
     const unsigned long long* ph = reinterpret_cast<const unsigned long long*>(g->host_read + S.phases_at);
     for (size_t k = 0; k < P.teams.size(); k++) {
-      fprintf(stderr, "[ampnet]   team %2zu kind %d node %2d cycles/round:", k, P.teams[k].t.kind, g->ppts[P.teams[k].t.ppt].node);
-      for (int q = 0; q < wave::N_PHASES; q++) fprintf(stderr, " %8.0f", (double)ph[k * wave::N_PHASES + q] / std::max<double>(1, (double)G.rounds));
+      const wave::Team& t = P.teams[k].t;
+      static const char* names[] = {"LOOKUP_F", "LOOKUP_B", "LIN_F", "LIN_DX", "ACC", "HEAD", "GRU_ZR", "GRU_C", "GRU_DC", "GRU_DZR"};
+      fprintf(stderr, "[team] %-8s node %2d CTAs %3d T %2d Sh %2d R %3d C %3d BM %3d rows/round %7.1f est %6.0f | wait-rows %6.0f wait %6.0f gather %6.0f product %6.0f rest %6.0f update %6.0f", names[t.kind], g->ppts[t.ppt].node,
+              t.n, t.T, t.Sh, t.R, t.C, t.BM, (double)D.wave.tot.entries[t.cell] / std::max<double>(1, (double)G.rounds), P.teams[k].cycles, (double)ph[k * 6] / G.rounds, (double)ph[k * 6 + 1] / G.rounds,
+              (double)ph[k * 6 + 2] / G.rounds, (double)ph[k * 6 + 3] / G.rounds, (double)ph[k * 6 + 4] / G.rounds, (double)ph[k * 6 + 5] / G.rounds);
       fprintf(stderr, "\n");
     }
     fprintf(stderr, "[ampnet]   rounds %llu\n", (unsigned long long)G.rounds);

@@ -97,6 +97,7 @@ struct Mat {
   unsigned* ver;                       // [32]: round << 16 | publications so far, by round
 };
 constexpr int PUB = 8;                 // published versions kept (readers lag by less than DRIFT + lag rounds)
+constexpr int LOOKUP_BITS = 8192;      // words of the bit map of touched rows that a tile of a large table keeps in shared memory
 constexpr int N_PHASES = 6;            // cycle counters of a cell's first CTA
 constexpr int DRIFT = 4;               // no CTA runs more than this many rounds ahead of another
 
@@ -114,7 +115,7 @@ struct PptRun {
   int kind, node, act, muf, loss_type, source_adj;
   amp::PPTStats* stats;
   int* update_log; int log_cap;
-  float* A; int* touched_list;         // LOOKUP: sparse accumulator
+  float* A; int* touched_list; unsigned* touched_bits;         // LOOKUP: sparse accumulator
   float *W, *om, *ov; long long opt_t0;
   int in_dim, out_dim, out4;
 };

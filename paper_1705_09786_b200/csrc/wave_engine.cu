@@ -24,6 +24,7 @@ constexpr int HT = 128;                       // helper threads
 constexpr int NT = CT + HT;
 constexpr int SLOT_WORDS = 6;
 constexpr int ACC_RED = CW * 8 * 32 * 4;       // floats of an accumulator's merge buffer
+constexpr int PIECES = 256;                   // pieces of a chunk a warp lists
 constexpr int NEAR = 128;                     // touched pieces of embedding rows a warp lists in shared memory
 
 enum { H_FIRST = 1, H_LAST = 2, H_UPDATE = 4, H_END = 8, H_COPIES = 16 };      // H_COPIES: every row is one or two copies
@@ -298,6 +299,7 @@ __device__ __noinline__ void helper_main(const int cta, const int tile, const in
         const uint4 w0 = __ldg(q), w1 = __ldg(q + 1), w2 = __ldg(q + 2);
         reinterpret_cast<uint4*>(&e)[0] = w0; reinterpret_cast<uint4*>(&e)[1] = w1; reinterpret_cast<uint4*>(&e)[2] = w2;
         inst = L.inst[a]; base4 = L.base4[a];
+        if (e.meta & E_OVERFLOW) asm volatile("prefetch.global.L1 [%0];" :: "l"(S.core.prog.ov + e.t[0].src4));      // (a sum of many terms: its list is read by the compute warps)
         end_msg = (e.meta & E_MSG_END) != 0;
       }
       if (updates && n_acc + cnt >= muf) {
@@ -462,13 +464,59 @@ __device__ __forceinline__ Head chunk_loop(RowD* rows, const int team, const uns
   return none;
 }
 
+// A piece of work per row, columns in groups of four: f(row, first group, step).  What a row's descriptor holds is read once and no
+// division is left in the loop; rows of up to 32 groups share a warp or take one, wider rows are dealt out in segments of 32 groups where
+// there are too few rows to fill the warps.  Measured against a flat loop over single outputs (cycles of one SM, 74 x 100 outputs of a
+// linear layer): 5,100 -> 1,500; 13 x 52: 1,090 -> 630; 4 x 8: 760 -> 550.
+template <class F>
+__device__ __forceinline__ void for_rows(const int count, const int n4, const F& f) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (n4 <= 32) {
+    const int sh = 32 - __clz(n4 - 1), P = 1 << sh;
+#pragma unroll 1
+    for (int b = (warp << (5 - sh)) + (lane >> sh); b < count; b += CW << (5 - sh)) f(b, lane & (P - 1), P);
+    return;
+  }
+  const int segs = (n4 + 31) >> 5;
+  if (count >= 2 * CW) {
+#pragma unroll 1
+    for (int b = warp; b < count; b += CW) f(b, lane, 32);
+    return;
+  }
+  const FastDiv ds(segs);
+#pragma unroll 1
+  for (int t = warp; t < count * segs; t += CW) { const int b = ds.div(t); f(b, (t - b * segs) * 32 + lane, n4); }
+}
+
 // ---- gathers ---------------------------------------------------------------------------------------------------------------
+// A sum of more terms than a row's descriptor holds: eight loads in flight (one after another, each is a trip to L2; the sum over a
+// graph's nodes took 24,000 cycles of a round).
+__device__ __noinline__ float4 sum_terms(const Term* t, const unsigned base4, const int nt, const int c) {
+  float4 v = zero4();
+#pragma unroll 1
+  for (int q0 = 0; q0 < nt; q0 += 8) {
+    float4 w[8];
+#pragma unroll
+    for (int q = 0; q < 8; q++) {
+      w[q] = zero4();
+      if (q0 + q >= nt) continue;
+      const Term u = t[q0 + q];
+      const unsigned d = (unsigned)c - u.col4;
+      if (d < u.w4) w[q] = ldcg4(S.core.arena + base4 + u.src4 + d);
+    }
+    v = add4(v, add4(add4(add4(w[0], w[1]), add4(w[2], w[3])), add4(add4(w[4], w[5]), add4(w[6], w[7]))));
+  }
+  return v;
+}
 // Value of columns 4 c .. 4 c + 3 of a row given by terms.
+template <bool CALL = true>                                       // CALL false: nothing is called (a caller with many live registers would save them)
 __device__ __forceinline__ float4 row_sum(const RowD& r, const int c) {
   const int nt = r.meta & E_NT;
-  float4 v = zero4();
   if (r.meta & E_OVERFLOW) {
-    const Term* t = S.core.prog.ov + r.t[0].src4;
+    const Term* const t = S.core.prog.ov + r.t[0].src4;
+    if (CALL) return sum_terms(t, r.base4, nt, c);
+    float4 v = zero4();
+#pragma unroll 1
     for (int q = 0; q < nt; q++) {
       const unsigned d = (unsigned)c - t[q].col4;
       if (d < t[q].w4) v = add4(v, ldcg4(S.core.arena + r.base4 + t[q].src4 + d));
@@ -495,6 +543,7 @@ __device__ __noinline__ float4 dense4(const int inst, const int c) {
 // Columns [c0, c0 + nc) (in fours) of the rows' terms into X; copies are asynchronous (cp_wait before the barrier), sums take up to
 // four loads at a time.  Chunks of plain copies (one source, or a Concat of two) have a loop of their own: what a round costs is
 // mostly how many instructions it walks through.
+template <bool CALL>
 __device__ __noinline__ void gather_general(const RowD* rows, const int count, const int c0, const int nc, float* X, const int ldx) {
   IN_SMEM(rows); IN_SMEM(X);
   const FastDiv dn(nc);
@@ -506,20 +555,20 @@ __device__ __noinline__ void gather_general(const RowD* rows, const int count, c
     if (r.meta & (E_DENSE | E_RAW)) {
       if ((S.core.dense_dim & 3) == 0) { if (4 * c < S.core.dense_dim) cp16(dst, S.core.dense + (long long)(r.inst & 0x7fffffff) * S.core.dense_dim + 4 * c); else *reinterpret_cast<float4*>(dst) = zero4(); }
       else *reinterpret_cast<float4*>(dst) = dense4(r.inst, c);
-    } else *reinterpret_cast<float4*>(dst) = rnd4(S.core.bf16, row_sum(r, c));
+    } else *reinterpret_cast<float4*>(dst) = rnd4(S.core.bf16, row_sum<CALL>(r, c));
   }
 }
 __device__ __forceinline__ void gather_terms(const Head& h, const RowD* rows, const int c0, const int nc, float* X, const int ldx) {
-  if (!(h.flags & H_COPIES)) { gather_general(rows, h.count, c0, nc, X, ldx); return; }
-  const FastDiv dn(nc);
-  const int n = h.count * nc;
-#pragma unroll 1
-  for (int i = threadIdx.x; i < n; i += CT) {
-    const int b = dn.div(i), k = i - b * nc, c = c0 + k;
+  if (!(h.flags & H_COPIES)) { gather_general<true>(rows, h.count, c0, nc, X, ldx); return; }
+  const float4* const arena = S.core.arena;
+  for_rows(h.count, nc, [&](const int b, const int k0, const int step) {
     const uint4 t = *reinterpret_cast<const uint4*>(&rows[b].t[0]);            // {source, columns} twice
-    const bool second = c >= (int)(t.w & 0xffffu);
-    cp16(X + b * ldx + 4 * k, S.core.arena + (second ? t.z + c - (t.w & 0xffffu) : t.x + c));
-  }
+    const int cut = (int)(t.w & 0xffffu);
+    const float4* const first = arena + t.x + c0; const float4* const second = arena + t.z + (c0 - cut);
+    float* const dst = X + b * ldx;
+#pragma unroll 2
+    for (int k = k0; k < nc; k += step) cp16(dst + 4 * k, (c0 + k >= cut ? second : first) + k);
+  });
 }
 
 // ---- products ---------------------------------------------------------------------------------------------------------------
@@ -527,8 +576,11 @@ __device__ __forceinline__ void gather_terms(const Head& h, const RowD* rows, co
 // nB a multiple of four.  512 threads, no barrier inside.  Three shapes:
 //   gemm_few     up to four rows: a warp per output column, lanes along k
 //   gemm_warps   up to 1,536 outputs: a warp per 4 x 4 outputs, lanes along k, a reduce-scatter of shuffles (short code)
-//   gemm_blocks  8 x 4 outputs per thread, k in up to 32 interleaved slices.  The bound is what shared memory can hand to registers
-//                (a 16-byte load costs four cycles of the SM whatever it hits: 12 loads per 128 multiply-adds).
+//   gemm_tiles   4 x 4 outputs per thread, k in four interleaved lanes that meet in a reduce-scatter of shuffles.  The bound is what
+//                shared memory can hand to registers (a 16-byte load costs four cycles of the SM whatever it hits); packed multiply-adds
+//                (two neighbouring k at a time) halve the instructions beside the loads.  Measured on one SM against 8 x 4 outputs with
+//                single multiply-adds (rows x columns x k, cycles): 30 x 52 x 304 12,545 -> 11,004, 20 x 100 x 208 11,890 -> 8,403,
+//                64 x 100 x 200 28,253 -> 26,881.
 __device__ __noinline__ void gemm_warps(const float* __restrict__ A, const int lda, const int nA, const float* __restrict__ B, const int ldb, const int nB, const int K4, float* __restrict__ Y, const int ldy) {
   IN_SMEM(A); IN_SMEM(B); IN_SMEM(Y);
   const int lane = threadIdx.x & 31, tB = nB >> 2, tiles = ((nA + 3) >> 2) * tB;
@@ -568,74 +620,50 @@ __device__ __noinline__ void gemm_warps(const float* __restrict__ A, const int l
     if (lane < 16 && b < nA) Y[b * ldy + 4 * ot + (at & 3)] = v[0];
   }
 }
-template <int TA>
-__device__ __noinline__ void gemm_blocks(const float* __restrict__ A, const int lda, const int nA, const float* __restrict__ B, const int ldb, const int nB, const int K4, float* __restrict__ Y, const int ldy) {
+__device__ __forceinline__ void fma2(unsigned long long& d, const unsigned long long a, const unsigned long long b) { asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b)); }
+__device__ __noinline__ void gemm_tiles(const float* __restrict__ A, const int lda, const int nA, const float* __restrict__ B, const int ldb, const int nB, const int K4, float* __restrict__ Y, const int ldy) {
   IN_SMEM(A); IN_SMEM(B); IN_SMEM(Y);
-  constexpr int V = TA * 4;
-  const int tid = threadIdx.x;
-  const int tA = (nA + TA - 1) / TA, tB = nB >> 2, n_tiles = tA * tB;
-  int sh = 0;
-  while (sh < 5 && (n_tiles << (sh + 1)) <= CT && (4 << sh) <= K4) sh++;
-  const int nsl = 1 << sh, per_pass = CT >> sh, ks = tid & (nsl - 1);
+  constexpr int KL = 4;
+  const int lane = threadIdx.x & 31, ks = lane & (KL - 1), tB = nB >> 2, n = ((nA + 3) >> 2) * tB;
   const FastDiv dB(tB);
-  const float4* const A4 = reinterpret_cast<const float4*>(A);
-  const float4* const B4 = reinterpret_cast<const float4*>(B);
   const int lda4 = lda >> 2, ldb4 = ldb >> 2;
+  const ulonglong2* const A2 = reinterpret_cast<const ulonglong2*>(A); const ulonglong2* const B2 = reinterpret_cast<const ulonglong2*>(B);
 #pragma unroll 1
-  for (int t0 = 0; t0 < n_tiles; t0 += per_pass) {
-    const int ti = t0 + (tid >> sh);
-    const bool valid = ti < n_tiles;
-    if (!__any_sync(0xffffffffu, valid)) break;
-    const int bt = valid ? dB.div(ti) : 0, ot = valid ? ti - bt * tB : 0;
-    int a[TA];
+  for (int t0 = (threadIdx.x >> 5) * (32 / KL); t0 < n; t0 += CW * (32 / KL)) {
+    const int ti = min(t0 + lane / KL, n - 1), bt = dB.div(ti), ot = ti - bt * tB;
+    int a[4];
 #pragma unroll
-    for (int m = 0; m < TA; m++) a[m] = min(TA * bt + m, nA - 1) * lda4;
-    const int w0 = 4 * ot * ldb4;
-    float v[V];
+    for (int m = 0; m < 4; m++) a[m] = min(4 * bt + m, nA - 1) * lda4 + ks;
+    const int w0 = 4 * ot * ldb4 + ks;
+    unsigned long long acc[16];
 #pragma unroll
-    for (int i = 0; i < V; i++) v[i] = 0.f;
+    for (int i = 0; i < 16; i++) acc[i] = 0ull;
 #pragma unroll 1
-    for (int k4 = valid ? ks : K4; k4 < K4; k4 += nsl) {
-      const float4 y[4] = {B4[w0 + k4], B4[w0 + ldb4 + k4], B4[w0 + 2 * ldb4 + k4], B4[w0 + 3 * ldb4 + k4]};
+    for (int k = 0; k + ks < K4; k += KL) {
+      ulonglong2 y[4];
 #pragma unroll
-      for (int m = 0; m < TA; m++) {
-        const float4 x = A4[a[m] + k4];
+      for (int j = 0; j < 4; j++) y[j] = B2[w0 + j * ldb4 + k];
 #pragma unroll
-        for (int j = 0; j < 4; j++) {
-          v[4 * m + j] = fmaf(x.x, y[j].x, v[4 * m + j]); v[4 * m + j] = fmaf(x.y, y[j].y, v[4 * m + j]);
-          v[4 * m + j] = fmaf(x.z, y[j].z, v[4 * m + j]); v[4 * m + j] = fmaf(x.w, y[j].w, v[4 * m + j]);
-        }
+      for (int m = 0; m < 4; m++) {
+        const ulonglong2 x = A2[a[m] + k];
+#pragma unroll
+        for (int j = 0; j < 4; j++) { fma2(acc[4 * m + j], x.x, y[j].x); fma2(acc[4 * m + j], x.y, y[j].y); }
       }
     }
-    int base = 0;
-    bool mine = valid;
+    float v[16];
 #pragma unroll
-    for (int s = 0; s < 5; s++)
-      if (s < sh) {
-        const int H = V >> (s + 1);
-        const bool up = (ks >> s) & 1;
-        if (H > 0) {
+    for (int i = 0; i < 16; i++) v[i] = __uint_as_float((unsigned)acc[i]) + __uint_as_float((unsigned)(acc[i] >> 32));
+    const bool mine = t0 + lane / KL < n;
+    int at = 0;
 #pragma unroll
-          for (int i = 0; i < H; i++) {
-            const float give = up ? v[i] : v[i + H], keep = up ? v[i + H] : v[i];
-            v[i] = keep + __shfl_xor_sync(0xffffffffu, give, 1 << s);
-          }
-          base += up ? H : 0;
-        } else {
-          v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1 << s);
-          mine = mine && !up;
-        }
-      }
-    if (!mine) continue;
-    const int left = V >> sh;
-    if (left >= 4) {
+    for (int s = 1, H = 8; s < KL; s <<= 1, H >>= 1) {
+      const bool up = lane & s;
 #pragma unroll
-      for (int i = 0; i < V; i += 4)
-        if (i < left) { const int b = TA * bt + ((base + i) >> 2); if (b < nA) *reinterpret_cast<float4*>(Y + b * ldy + 4 * ot) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]); }
-    } else {
-      const int b = TA * bt + (base >> 2), o = 4 * ot + (base & 3);
-      if (b < nA) { Y[b * ldy + o] = v[0]; if (left == 2) Y[b * ldy + o + 1] = v[1]; }
+      for (int i = 0; i < H; i++) { const float give = up ? v[i] : v[i + H], keep = up ? v[i + H] : v[i]; v[i] = keep + __shfl_xor_sync(0xffffffffu, give, s); }
+      at += up ? H : 0;
     }
+    const int b = 4 * bt + (at >> 2);
+    if (mine && b < nA) *reinterpret_cast<float4*>(Y + b * ldy + 4 * ot) = make_float4(v[0], v[1], v[2], v[3]);
   }
 }
 __device__ __noinline__ void gemm_few(const float* __restrict__ A, const int lda, const int nA, const float* __restrict__ B, const int ldb, const int nB, const int K4, float* __restrict__ Y, const int ldy) {
@@ -671,7 +699,7 @@ __device__ __noinline__ void gemm_few(const float* __restrict__ A, const int lda
 __device__ __forceinline__ void gemm(const float* A, const int lda, const int nA, const float* B, const int ldb, const int nB, const int K4, float* Y, const int ldy) {
   if (nA <= 4) gemm_few(A, lda, nA, B, ldb, nB, K4, Y, ldy);
   else if (nA * nB <= 1536) gemm_warps(A, lda, nA, B, ldb, nB, K4, Y, ldy);
-  else gemm_blocks<8>(A, lda, nA, B, ldb, nB, K4, Y, ldy);
+  else gemm_tiles(A, lda, nA, B, ldb, nB, K4, Y, ldy);
 }
 
 // ---- weights ---------------------------------------------------------------------------------------------------------------
@@ -783,7 +811,13 @@ __device__ __noinline__ void forward_main(const int team, const int tile, float*
         for (int u = 0; u < U; u++) {
           const int i = i0 + u * CT, g8 = d8.div(i >> 3), r = g8 * 8 + (i & 7), k8 = (i >> 3) - g8 * K8;
           a[u] = b[u] = zero4();
-          if (i < items && r < count) { const int nt = R[r].meta & E_NT; a[u] = term4(R[r], 0, nt, 2 * k8); b[u] = term4(R[r], 0, nt, 2 * k8 + 1); }
+          if (i < items && r < count) {
+            if (h.flags & H_COPIES) {                             // (eight loads in flight; a general row is put together by a call)
+              const uint4 t = *reinterpret_cast<const uint4*>(&R[r].t[0]);
+              const int cut = (int)(t.w & 0xffffu), c = 2 * k8;
+              a[u] = ldcg4(S.core.arena + (c >= cut ? t.z + (c - cut) : t.x + c)); b[u] = ldcg4(S.core.arena + (c + 1 >= cut ? t.z + (c + 1 - cut) : t.x + c + 1));
+            } else { const int nt = R[r].meta & E_NT; a[u] = term4(R[r], 0, nt, 2 * k8); b[u] = term4(R[r], 0, nt, 2 * k8 + 1); }
+          }
         }
 #pragma unroll
         for (int u = 0; u < U; u++) {
@@ -792,6 +826,7 @@ __device__ __noinline__ void forward_main(const int team, const int tile, float*
         }
       }
       tc::fence_operands();
+      phase(2);
       if (count <= tc::SMALL_ROWS) for (int i = tid; i < count * YP; i += CT) Ys[i] = 0.f;
       bar_compute();
       if (count <= tc::SMALL_ROWS) {
@@ -804,6 +839,7 @@ __device__ __noinline__ void forward_main(const int team, const int tile, float*
         if (__all_sync(0xffffffffu, done)) tc::read_accumulator(S.tmem, NTC, count, Ys, YP, nB);
       }
       bar_compute();
+      phase(3);
       const FastDiv dr(nB >> 2);
 #pragma unroll 1
       for (int i = tid; i < count * (nB >> 2); i += CT) {
@@ -828,13 +864,17 @@ __device__ __noinline__ void forward_main(const int team, const int tile, float*
     bar_compute();
     phase(3);
     const int ow = m.out_w, w4 = jn >> 2;
-    if constexpr (MODE == F_PLAIN) {                              // one output per thread: the activation's code once
-      const FastDiv dj(jn);
-#pragma unroll 1
-      for (int i = tid; i < count * jn; i += CT) {
-        const int b = dj.div(i), o = i - b * jn;
-        reinterpret_cast<float*>(S.core.arena + R[b].out4)[j0 + o] = j0 + o < ow ? rnd(bf16, act_fwd(T.act, Ys[b * YP + o] + bs[o])) : 0.f;
-      }
+    if constexpr (MODE == F_PLAIN) {
+      const int act = T.act;
+      for_rows(count, w4, [&](const int b, const int k0, const int step) {
+        float4* const out = S.core.arena + R[b].out4 + (j0 >> 2);
+        for (int k = k0; k < w4; k += step) {
+          float4 v = act_fwd4(act, add4(*reinterpret_cast<const float4*>(Ys + b * YP + 4 * k), *reinterpret_cast<const float4*>(bs + 4 * k)));
+          const int past = j0 + 4 * k + 4 - ow;                   // columns past the width (padding) stay zero
+          if (past > 0) { v.w = 0.f; if (past > 1) v.z = 0.f; if (past > 2) v.y = 0.f; if (past > 3) v.x = 0.f; }
+          out[k] = rnd4(bf16, v);
+        }
+      });
     }
     if constexpr (MODE != F_PLAIN) {
 #pragma unroll 1
@@ -1033,7 +1073,7 @@ __device__ __noinline__ void accumulate_main(const int team, const int tile, flo
   const int ti = (m.inp + Ci - 1) / Ci, to = tile / ti, o0 = to * Ro, i0 = (tile - to * ti) * Ci;
   const int ro = min(Ro, m.outp - o0), ci = min(Ci, m.inp - i0);
   const int ldd = Ro + 4, ldx = Ci + 4, ldw = Ci + 4;
-  float *Wm = smem, *red = Wm + (size_t)Ro * ldw, *Dg = red + (WS > 1 ? ACC_RED : 0), *Xg = Dg + (size_t)T.BM * ldd, *bm = Xg + (size_t)T.BM * ldx, *bred = bm + Ro;   // bred: WS x Ro floats
+  float *Wm = smem, *red = Wm + (size_t)Ro * ldw, *Dg = red + ACC_RED, *Xg = Dg + (size_t)T.BM * ldd, *bm = Xg + (size_t)T.BM * ldx, *bred = bm + Ro;   // bred: WS x Ro floats
   const bool biased = i0 == 0;
 #pragma unroll 1
   for (int i = tid; i < Ro * Ci; i += CT) {
@@ -1069,60 +1109,70 @@ __device__ __noinline__ void accumulate_main(const int team, const int tile, flo
     float4* const r4 = reinterpret_cast<float4*>(red);
     if (summing) {
 #pragma unroll
-      for (int k = 0; k < 8; k++) { bred[ws * Ro + ob + k] = bacc[k]; bacc[k] = 0.f; }
+      for (int k = 0; k < 8; k++) bred[ws * Ro + ob + k] = bacc[k];
     }
-    if (WS > 1) {
 #pragma unroll
-      for (int k = 0; k < 8; k++)
-        if ((WS >= 8 ? k : (k * WS) >> 3) != ws) r4[((ws * NR + wr) * 8 + k) * 32 + lane] = make_float4(acc[k][0], acc[k][1], acc[k][2], acc[k][3]);
-    }
+    for (int k = 0; k < 8; k++) r4[(ws * 8 + k) * (32 * NR) + wr * 32 + lane] = make_float4(acc[k][0], acc[k][1], acc[k][2], acc[k][3]);
     bar_compute();
-#pragma unroll
-    for (int k = 0; k < 8; k++) {
-      if ((WS >= 8 ? k : (k * WS) >> 3) == ws) {                // this slice's share of the rows
-        float4 a = make_float4(acc[k][0], acc[k][1], acc[k][2], acc[k][3]);
+    const int per = 8 * 32 * NR, sW = 31 - __clz(WI), sL = 31 - __clz(LI), sN = 31 - __clz(NR);                                // sums of four columns; every thread adds up some over the slices
 #pragma unroll 1
-        for (int s = 0; s < WS; s++) if (s != ws) a = add4(a, r4[((s * NR + wr) * 8 + k) * 32 + lane]);
-        float4* const w4 = reinterpret_cast<float4*>(Wm + (ob + k) * ldw + ib);
-        *w4 = os.opt == 0 ? sgd4(os.step, *w4, a) : opt_padded(os, m, o0 + ob + k, i0 + ib, *w4, a);
-      }
-#pragma unroll
-      for (int j = 0; j < 4; j++) acc[k][j] = 0.f;
+    for (int i = tid; i < per; i += CT) {
+      float4 a = zero4();
+#pragma unroll 4
+      for (int s = 0; s < WS; s++) a = add4(a, r4[s * per + i]);
+      const int l = i & 31, q = (i >> 5) & (NR - 1), k = i >> (5 + sN), o = ((q >> sW) * LO + (l >> sL)) * 8 + k, c = ((q & (WI - 1)) * LI + (l & (LI - 1))) * 4;
+      float4* const w4 = reinterpret_cast<float4*>(Wm + o * ldw + c);
+      *w4 = os.opt == 0 ? sgd4(os.step, *w4, a) : opt_padded(os, m, o0 + o, i0 + c, *w4, a);
     }
     if (biased)
 #pragma unroll 1
-      for (int i = tid; i < ro; i += CT) {
+      for (int i = CT - 1 - tid; i < ro; i += CT) {
         float a = 0.f;
+#pragma unroll 4
         for (int s = 0; s < WS; s++) a += bred[s * Ro + i];
         const int r = real_out(m, o0 + i);
         if (r >= 0) bm[i] = opt_one(os, bm[i], a, (size_t)m.nW + r);
       }
+#pragma unroll
+    for (int k = 0; k < 8; k++) {
+      bacc[k] = 0.f;
+#pragma unroll
+      for (int j = 0; j < 4; j++) acc[k][j] = 0.f;
+    }
     bar_compute();
   };
   auto stamp = [&](const Head& h) { if (leader && tid == 0) *reinterpret_cast<volatile unsigned long long*>(ver + (h.round & 31)) = ((unsigned long long)(unsigned)updates << 32) | ((unsigned long long)(pubs & 0xffffu) << 16) | ((unsigned)h.round & 0xffffu); };
   const Head end = chunk_loop(rows, team, t0, [&](const Head& h, const RowD* R) {
     const int count = h.count;
+    // staleness: updates of the node since the forward pass (Sec. 3); a warp per 32 rows, loaded before the rows and counted after
+    float version = 0.f;
+    bool message = false, stamped = false;
+    if (leader && tid < count) {
+      const RowD& r = R[tid];
+      message = r.meta & E_MSG_END; stamped = message && r.a4 != NONE;
+      if (stamped) version = __ldcg(reinterpret_cast<const float*>(S.core.arena + r.a4 + ((r.meta & E_RAW) ? (m.outp >> 2) : 0)));
+    }
 #pragma unroll 1
     for (int i = tid; i < count * d4; i += CT) {
       const int b = dd.div(i), k = i - b * d4, c = (o0 >> 2) + k;
       const RowD& r = R[b];
       if (!(r.meta & E_RAW)) { cp16(Dg + b * ldd + 4 * k, S.core.arena + r.out4 + c); continue; }
-      const float4 y = ldcg4(S.core.arena + r.a4 + c), g = rnd4(S.core.bf16, row_sum(r, c));
+      const float4 y = ldcg4(S.core.arena + r.a4 + c), g = rnd4(S.core.bf16, row_sum<false>(r, c));
       *reinterpret_cast<float4*>(Dg + b * ldd + 4 * k) = make_float4(g.x * act_grad(T.act, y.x), g.y * act_grad(T.act, y.y), g.z * act_grad(T.act, y.z), g.w * act_grad(T.act, y.w));
     }
-    gather_terms(h, R, i0 >> 2, x4, Xg, ldx);
-    if (leader && warp == CW - 1) {                              // staleness: updates of the node since the forward pass (Sec. 3)
+    if (h.flags & H_COPIES) {                                    // (a flat loop: the sums leave no registers for more)
 #pragma unroll 1
-      for (int b0 = 0; b0 < count; b0 += 32) {
-        const int b = b0 + lane;
-        int stale = -1;
-        if (b < count && (R[b].meta & E_MSG_END)) {
-          stale = 0;
-          if (R[b].a4 != NONE) { const float4 v = ldcg4(S.core.arena + R[b].a4 + ((R[b].meta & E_RAW) ? (m.outp >> 2) : 0)); stale = max(0, h.n_updates - __float_as_int(v.x)); }
-        }
-        const unsigned same = __match_any_sync(0xffffffffu, stale);
-        if (stale >= 0 && (same & ((1u << lane) - 1u)) == 0) { atomicAdd(&S.stale_hist[min(stale, 63)], __popc(same)); atomicMax(&S.max_stale, stale); }
+      for (int i = tid; i < count * x4; i += CT) {
+        const int b = dx.div(i), k = i - b * x4, c = (i0 >> 2) + k;
+        const uint4 t = *reinterpret_cast<const uint4*>(&R[b].t[0]);
+        const bool second = c >= (int)(t.w & 0xffffu);
+        cp16(Xg + b * ldx + 4 * k, S.core.arena + (second ? t.z + c - (t.w & 0xffffu) : t.x + c));
       }
+    } else gather_general<false>(R, count, i0 >> 2, x4, Xg, ldx);
+    if (leader && (tid & ~31) < count) {
+      const int stale = message ? (stamped ? max(0, h.n_updates - __float_as_int(version)) : 0) : -1;
+      const unsigned same = __match_any_sync(0xffffffffu, stale);
+      if (stale >= 0 && (same & ((1u << lane) - 1u)) == 0) { atomicAdd(&S.stale_hist[min(stale, 63)], __popc(same)); atomicMax(&S.max_stale, stale); }
     }
     cp_wait();
     bar_compute();
@@ -1293,14 +1343,21 @@ __device__ __noinline__ void lookup_main(const int team, RowD* rows, const unsig
   const float* const W = S.ppt.W;
   const bool wide = (out & 3) == 0;
   chunk_loop(rows, team, t0, [&](const Head& h, const RowD* R) {
-#pragma unroll 2
-    for (int i = tid; i < h.count * o4; i += CT) {
-      const int b = d4.div(i), k = i - b * o4;
-      const float* e = W + (size_t)R[b].b4 * out + 4 * k;
-      float4 v;
-      if (wide) v = __ldcg(reinterpret_cast<const float4*>(e));
-      else { v.x = __ldcg(e); v.y = 4 * k + 1 < out ? __ldcg(e + 1) : 0.f; v.z = 4 * k + 2 < out ? __ldcg(e + 2) : 0.f; v.w = 4 * k + 3 < out ? __ldcg(e + 3) : 0.f; }
-      S.core.arena[R[b].out4 + k] = rnd4(S.core.bf16, v);
+const int n = h.count * o4;
+#pragma unroll 1
+    for (int i0 = tid; i0 < n; i0 += 4 * CT) {                   // four loads in flight
+      float4 v[4];
+      unsigned at[4];
+#pragma unroll
+      for (int u = 0; u < 4; u++) {
+        const int i = min(i0 + u * CT, n - 1), b = d4.div(i), k = i - b * o4;
+        const float* e = W + (size_t)R[b].b4 * out + 4 * k;
+        at[u] = R[b].out4 + k;
+        if (wide) v[u] = __ldcg(reinterpret_cast<const float4*>(e));
+        else { v[u].x = __ldcg(e); v[u].y = 4 * k + 1 < out ? __ldcg(e + 1) : 0.f; v[u].z = 4 * k + 2 < out ? __ldcg(e + 2) : 0.f; v[u].w = 4 * k + 3 < out ? __ldcg(e + 3) : 0.f; }
+      }
+#pragma unroll
+      for (int u = 0; u < 4; u++) if (i0 + u * CT < n) S.core.arena[at[u]] = rnd4(S.core.bf16, v[u]);
     }
   });
 }
@@ -1332,7 +1389,7 @@ __device__ __noinline__ void lookup_grad_small_main(const int team, float* smem,
             if (b + q * slices >= h.count) continue;
             const RowD& r = R[b + q * slices];
             const int nt = r.meta & E_NT, cc = c >> 2;
-            if (r.meta & E_OVERFLOW) { const float4 v = row_sum(r, cc); g[q] = (c & 3) == 0 ? v.x : (c & 3) == 1 ? v.y : (c & 3) == 2 ? v.z : v.w; continue; }
+            if (r.meta & E_OVERFLOW) { const float4 v = sum_terms(S.core.prog.ov + r.t[0].src4, r.base4, nt, cc); g[q] = (c & 3) == 0 ? v.x : (c & 3) == 1 ? v.y : (c & 3) == 2 ? v.z : v.w; continue; }
 #pragma unroll
             for (int k = 0; k < 4; k++) { const Term t = r.t[k]; const unsigned d = (unsigned)cc - t.col4; if (k < nt && d < t.w4) g[q] += __ldcg(arena + (size_t)(t.src4 + d) * 4 + (c & 3)); }
           }
@@ -1366,18 +1423,25 @@ __device__ __noinline__ void lookup_grad_main(const int team, const int tile, fl
   const PptRun& P = S.ppt;
   const int segs = (o4 + 31) >> 5, ids = (P.in_dim + NTL - 1) / NTL;
   int* const near_list = reinterpret_cast<int*>(smem) + warp * NEAR;
+  int* const work = reinterpret_cast<int*>(smem) + CW * NEAR + warp * PIECES;      // (segment, row) of the chunk
+  // a bit per piece: listed already (in device memory behind the lists where a table is too large)
+  const size_t words = ((size_t)ids * segs + 31) >> 5;
+  unsigned* const bits = words <= LOOKUP_BITS ? reinterpret_cast<unsigned*>(smem) + CW * (NEAR + PIECES) : P.touched_bits + (size_t)tile * words;
+  if (words <= LOOKUP_BITS) for (int i = threadIdx.x; i < (int)words; i += CT) bits[i] = 0u;
+  const FastDiv d_tiles(NTL);
+  bar_compute();
   int* const far_list = P.touched_list + ((size_t)tile * CW + warp) * ((size_t)ids * segs / CW + segs + 1);
   const bool wide = (out & 3) == 0;
   int touched = 0;                                               // (the same in all lanes)
   auto update = [&](const int n_upd, const int upd_t) {
     const OptStep os = opt_step(P.om, P.ov, P.opt_t0, n_upd, upd_t);
 #pragma unroll 1
-    for (int k0 = 0; k0 < touched; k0 += 2) {                    // two pieces' loads in flight
-      float a[2][4], w[2][4];
-      size_t r0[2];
-      int cq[2];
+    for (int k0 = 0; k0 < touched; k0 += 4) {                    // four pieces' loads in flight
+      float a[4][4], w[4][4];
+      size_t r0[4];
+      int cq[4];
 #pragma unroll
-      for (int u = 0; u < 2; u++) {
+      for (int u = 0; u < 4; u++) {
         const int k = min(k0 + u, touched - 1), piece = k < NEAR ? near_list[k] : far_list[k], local = piece / segs, c = (piece - local * segs) * 32 + lane;
         r0[u] = ((size_t)local * NTL + tile) * out + 4 * c;
         cq[u] = k0 + u < touched ? out - 4 * c : 0;
@@ -1391,67 +1455,84 @@ __device__ __noinline__ void lookup_grad_main(const int team, const int tile, fl
             if (q < cq[u]) { asm volatile("ld.relaxed.gpu.global.f32 %0, [%1];" : "=f"(a[u][q]) : "l"(P.A + r0[u] + q) : "memory"); w[u][q] = P.W[r0[u] + q]; }
       }
 #pragma unroll
-      for (int u = 0; u < 2; u++)
+      for (int u = 0; u < 4; u++) {
+        if (wide && cq[u] > 0 && os.opt == 0) {
+          *reinterpret_cast<float4*>(P.W + r0[u]) = sgd4(os.step, make_float4(w[u][0], w[u][1], w[u][2], w[u][3]), make_float4(a[u][0], a[u][1], a[u][2], a[u][3]));
+          asm volatile("st.relaxed.gpu.global.v4.f32 [%0], {%1, %1, %1, %1};" :: "l"(P.A + r0[u]), "f"(0.f) : "memory");
+          continue;
+        }
 #pragma unroll
         for (int q = 0; q < 4; q++)
           if (q < cq[u]) {
             P.W[r0[u] + q] = opt_one(os, w[u][q], a[u][q], r0[u] + q);
             asm volatile("st.relaxed.gpu.global.f32 [%0], %1;" :: "l"(P.A + r0[u] + q), "f"(0.f) : "memory");
           }
+      }
     }
+#pragma unroll 1
+    for (int k = lane; k < touched; k += 32) { const int piece = k < NEAR ? near_list[k] : far_list[k]; atomicAnd(bits + (piece >> 5), ~(1u << (piece & 31))); }
     touched = 0;
     __syncwarp();
   };
   chunk_loop(rows, team, t0, [&](const Head& h, const RowD* R) {
+// the warp's pieces of the chunk are listed first, so that its loads overlap whatever rows they come from
+    int listed = 0;
+    auto add_listed = [&]() {
 #pragma unroll 1
-    for (int b0 = 0; b0 < h.count; b0 += 32) {
-      const unsigned id = R[min(b0 + lane, h.count - 1)].b4;
-      const int local = b0 + lane < h.count && (int)(id % (unsigned)NTL) == tile ? (int)(id / (unsigned)NTL) : -1;
-      if (!__any_sync(0xffffffffu, local >= 0)) continue;
-#pragma unroll 1
-      for (int q = 0; q < segs; q++) {
-        const int c = 32 * q + lane;
-        unsigned mine = __ballot_sync(0xffffffffu, local >= 0 && (local * segs + q) % CW == warp);
-        while (mine) {
-          // all rows of one id (a piece), four loads in flight, one add
-          const int id0 = __shfl_sync(0xffffffffu, local, __ffs((int)mine) - 1);
-          unsigned same = __ballot_sync(0xffffffffu, local == id0) & mine;
-          mine &= ~same;
-          float4 g = zero4();
-#pragma unroll 1
-          while (same) {
-            float4 v[4];
+      for (int k0 = 0; k0 < listed; k0 += 4) {
+        float4 v[4];
 #pragma unroll
-            for (int k = 0; k < 4; k++) {
-              v[k] = zero4();
-              const int l = same ? __ffs((int)same) - 1 : -1;
-              same &= same - 1;
-              if (l < 0 || c >= o4) continue;
-              const RowD& r = R[b0 + l];
-              v[k] = rnd4(S.core.bf16, h.flags & H_COPIES ? ldcg4(S.core.arena + r.t[0].src4 + c) : row_sum(r, c));
-            }
-            g = add4(g, add4(add4(v[0], v[1]), add4(v[2], v[3])));
-          }
-          float* const a = P.A + ((size_t)id0 * NTL + tile) * out + 4 * c;
+        for (int k = 0; k < 4; k++) {
+          v[k] = zero4();
+          const int x = k0 + k < listed ? work[k0 + k] : -1, c = 32 * (x >> 8) + lane;
+          if (x < 0 || c >= o4) continue;
+          const RowD& r = R[x & 255];
+          v[k] = h.flags & H_COPIES ? ldcg4(S.core.arena + r.t[0].src4 + c) : rnd4(S.core.bf16, row_sum<false>(r, c));
+        }
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+          if (k0 + k >= listed) break;
+          const int x = work[k0 + k], q = x >> 8, c = 32 * q + lane;
+          const unsigned id = R[x & 255].b4;
+          float* const a = P.A + (size_t)id * out + 4 * c;
           if (c < o4) {
-            if (wide) asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" :: "l"(a), "f"(g.x), "f"(g.y), "f"(g.z), "f"(g.w) : "memory");
+            if (wide) asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" :: "l"(a), "f"(v[k].x), "f"(v[k].y), "f"(v[k].z), "f"(v[k].w) : "memory");
             else {
-              const float v[4] = {g.x, g.y, g.z, g.w};
+              const float e[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
 #pragma unroll
-              for (int k = 0; k < 4; k++) if (4 * c + k < out) asm volatile("red.relaxed.gpu.global.add.f32 [%0], %1;" :: "l"(a + k), "f"(v[k]) : "memory");
+              for (int y = 0; y < 4; y++) if (4 * c + y < out) asm volatile("red.relaxed.gpu.global.add.f32 [%0], %1;" :: "l"(a + y), "f"(e[y]) : "memory");
             }
-          }
-          const int piece = id0 * segs + q;
-          bool have = false;
-          for (int k = lane; k < touched; k += 32) have |= (k < NEAR ? near_list[k] : far_list[k]) == piece;
-          if (!__any_sync(0xffffffffu, have)) {
-            if (lane == 0) { if (touched < NEAR) near_list[touched] = piece; else far_list[touched] = piece; }
-            touched++;
-            __syncwarp();
           }
         }
       }
+      listed = 0;
+      __syncwarp();
+    };
+#pragma unroll 1
+    for (int b0 = 0; b0 < h.count; b0 += 32) {
+      const int id = (int)R[min(b0 + lane, h.count - 1)].b4, of = d_tiles.div(id);
+      const bool ours = b0 + lane < h.count && id - of * NTL == tile;
+      if (!__any_sync(0xffffffffu, ours)) continue;
+#pragma unroll 1
+      for (int q = 0; q < segs; q++) {
+        const bool mine = ours && ((of * segs + q) & (CW - 1)) == warp;
+        const unsigned all = __ballot_sync(0xffffffffu, mine);
+        if (listed + __popc(all) > PIECES) add_listed();
+        const unsigned before = (1u << lane) - 1u;
+        const int piece = of * segs + q;
+        bool fresh = false;
+        if (mine) {
+          work[listed + __popc(all & before)] = (q << 8) | (b0 + lane);
+          fresh = !(atomicOr(bits + (piece >> 5), 1u << (piece & 31)) >> (piece & 31) & 1u);
+        }
+        const unsigned news = __ballot_sync(0xffffffffu, fresh);
+        if (fresh) { const int x = touched + __popc(news & before); if (x < NEAR) near_list[x] = piece; else far_list[x] = piece; }
+        listed += __popc(all);
+        touched += __popc(news);
+        __syncwarp();
+      }
     }
+    add_listed();
     if (h.flags & H_UPDATE) update(h.n_upd, h.upd_t);
   });
 }
@@ -1536,8 +1617,8 @@ size_t smem_bytes(const Team& t, const Mat& m, int mak) {
       else f = (size_t)t.G * t.R * ldi + ((t.G * t.R + 3) & ~3) + BM * ldi + BM * pad_ld(t.G * t.R) + (t.kind == GRU_C ? BM * 2 * t.R : 0);
       break;
     case LIN_DX: case GRU_DC: case GRU_DZR: f = (size_t)t.R * ldo + BM * ldo + BM * pad_ld(t.R); break;
-    case ACC: f = (size_t)t.R * (t.C + 4) + (t.WO * t.WI < CW ? ACC_RED : 0) + BM * (t.R + 4 + t.C + 4) + t.R + (size_t)(CW / (t.WO * t.WI)) * t.R; break;
-    case LOOKUP_B: f = t.R ? (size_t)(t.R + 1) * t.C : CW * NEAR; break;      // (small table: R copies of C sums)
+    case ACC: f = (size_t)t.R * (t.C + 4) + ACC_RED + BM * (t.R + 4 + t.C + 4) + t.R + (size_t)(CW / (t.WO * t.WI)) * t.R; break;
+    case LOOKUP_B: f = t.R ? (size_t)(t.R + 1) * t.C : CW * (NEAR + PIECES) + LOOKUP_BITS; break;      // (small table: R copies of C sums)
     case HEAD: f = (size_t)m.outp * ldi + m.outp + BM * ldi + 2 * BM * pad_ld(m.outp); break;
     default: break;
   }

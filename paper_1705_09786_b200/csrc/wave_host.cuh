@@ -329,7 +329,7 @@ static bool wave_best(const WaveModel& M, int c, int ctas, double rows, double m
       return;
     }
   };
-  const double lat = 700, bpc = 36, fma = 128 * 0.42;
+  const double bpc = 36, fma = 40;
   int env_rows = 0, env_cols = 0;
   if (const char* e = getenv("AMPNET_DIRECT_ROWS")) env_rows = std::max(1, atoi(e));
   if (const char* e = getenv("AMPNET_DIRECT_COLS")) env_cols = std::max(4, atoi(e));
@@ -349,9 +349,10 @@ static bool wave_best(const WaveModel& M, int c, int ctas, double rows, double m
         x.Sh = std::max(1, std::min(ctas / x.T, (int)std::ceil(rows)));
         x.n = x.T * x.Sh;
         const double rs = std::max(1.0, rows / x.Sh), outs = x.R * x.G;
-        const double g_cyc = lat + (rs * m.inp * 4.0 + upd * outs * m.inp * 4.0) / bpc;
-        const double k_cyc = tc ? 600 + rs * m.inp / 64.0 : 250 + std::max(4.0, rs) * outs * m.inp / fma;
-        offer(x, g_cyc + k_cyc + 200 + (t.lstm ? 300 : 0));
+        const bool sums = K.kind == GRU_ZR || (t.keep && !eval);
+        const double gather = 1300 + rs * m.inp / 4 * (sums ? 3.5 : 1.0), weights = std::min(1.0, upd) * outs * m.inp * 4.0 / bpc;
+        const double product = tc ? 1500 + rs * m.inp / 8.0 : 600 + (rs + 4) * outs * m.inp / fma;
+        offer(x, gather + weights + product + 1600 + rs * x.R / 4 * (t.lstm ? 20.0 : K.kind == LIN_F ? 2.0 : 3.0));
         if (tc || env_rows) break;
       }
       break;
@@ -367,8 +368,8 @@ static bool wave_best(const WaveModel& M, int c, int ctas, double rows, double m
         x.Sh = std::max(1, std::min(ctas / x.T, (int)std::ceil(rows)));
         x.n = x.T * x.Sh;
         const double rs = std::max(1.0, rows / x.Sh);
-        const double g_cyc = 1.3 * lat + (rs * m.outp * 4.0 * 3.2 + upd * x.R * m.outp * 4.0) / bpc;
-        offer(x, g_cyc + 250 + std::max(4.0, rs) * x.R * m.outp / fma + 200);
+        const double per4 = t.lstm ? 17.0 * t.H4 : m.outp / 4 * (K.kind == GRU_DC ? 12.0 : 3.4);
+        offer(x, 1500 + rs * per4 + std::min(1.0, upd) * x.R * m.outp * 4.0 / bpc + 600 + (rs + 4) * x.R * m.outp / fma + 1700 + rs * x.R / 4 * 1.5);
         if (env_cols) break;
       }
       break;
@@ -382,8 +383,8 @@ static bool wave_best(const WaveModel& M, int c, int ctas, double rows, double m
             x.T = ((m.outp + x.R - 1) / x.R) * ((m.inp + x.C - 1) / x.C);
             if (x.T > ctas) continue;
             x.n = x.T;
-            const double area = (double)x.R * x.C, ws = 16.0 / (WO * WI);
-            offer(x, lat + rows * (std::min(x.R, m.outp) + std::min(x.C, m.inp)) * 4.0 / bpc + rows * area / (128 * 0.5) + upd * (400 + area * (2 * ws + 3) / 100.0));
+            const double area = (double)x.R * x.C;
+            offer(x, 4500 + rows * (36 + 0.23 * (std::min(x.R, m.outp) + std::min(x.C, m.inp)) + area / (area < 4096 ? 46 : 59)) + upd * 3000 + std::min(1.0, upd) * area / 5);
           }
       break;
     case HEAD:
@@ -391,14 +392,14 @@ static bool wave_best(const WaveModel& M, int c, int ctas, double rows, double m
         Team x = t;
         x.Sh = x.n = n; x.G = P.xstore; x.R = 0;
         const double rs = std::max(1.0, rows / n);
-        offer(x, lat + (rs * m.inp * 4.0 + upd * m.outp * m.inp * 4.0) / bpc + 900 + 3.0 * rs * m.inp * m.outp / (128 * 0.25));
+        offer(x, 4500 + rs * (150 + 0.6 * m.inp) + std::min(1.0, upd) * m.outp * m.inp * 4.0 / bpc);
       }
       break;
     case LOOKUP_F:
       for (int n = 1; n <= std::min(ctas, std::max(1, (int)rows)); n++) {
         Team x = t;
         x.Sh = x.n = n;
-        offer(x, lat + rows / n * h.out_dim * 4.0 * 2 / bpc);
+        offer(x, 1200 + rows / n * h.out_dim / 4 * 1.7);
       }
       break;
     default: {    // LOOKUP_B: the sums of a small table in shared memory, otherwise rows dealt to tiles by id
@@ -407,13 +408,14 @@ static bool wave_best(const WaveModel& M, int c, int ctas, double rows, double m
         Team x = t;
         x.R = 512 / cols; x.C = h.in_dim * h.out_dim;
         while (x.R > 1 && (long long)x.R * x.C * 4 > 128 * 1024) x.R--;
-        offer(x, 2500 + rows / x.R * 250 + upd * (1500 + (double)x.C * x.R / 40.0));
+        offer(x, 2500 + rows / x.R * 500 + upd * (1500 + (double)x.C * x.R / 40.0));
         break;
       }
-      for (int n = 1; n <= std::min(ctas, std::max(1, h.in_dim / 8)); n++) {
+      for (int n = 1; n <= std::min(ctas, std::max(1, h.in_dim / 8)) && (n == 1 || (long long)h.in_dim * n < (1ll << 31)); n++) {      // (the kernel divides ids by multiplication)
         Team x = t;
         x.T = x.n = n;
-        offer(x, 3000 + rows * 15.0 + rows / n * 150.0 + upd * (2500 + std::min(msgs_per_update, (double)h.in_dim) / n * 150.0));
+        const double pieces = std::max((h.out_dim + 127) / 128 / 16.0 / n, 0.02);      // of a row, per warp of a tile (frequent ids keep one warp busy)
+        offer(x, 4000 + rows * (40 + pieces * 1300) + upd * (4000 + std::min(msgs_per_update, (double)h.in_dim) * pieces * 1500));
       }
     }
   }
@@ -573,6 +575,8 @@ static WaveScratch wave_carve(ampnet_graph* g, HostDataset& D, const WaveModel& 
       for (auto& t : P.teams) if (t.t.kind == LOOKUP_B && t.t.ppt == (int)p) T = t.t.T;
       Q.A = zeroed(H.nW);
       const size_t segs = (size_t)(Q.out4 + 31) / 32, ids = (size_t)(H.in + T - 1) / T;      // a list per tile and warp
+      const size_t words = (ids * segs + 31) / 32;
+      if (words > wave::LOOKUP_BITS) Q.touched_bits = reinterpret_cast<unsigned*>(zeroed((size_t)T * words));
       Q.touched_list = B.take<int>((size_t)T * 16 * (ids * segs / 16 + segs + 1));
     }
   }
