@@ -117,9 +117,9 @@ struct ampnet_graph {
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   wave::WaveModel wave;                 // scheduled engine: the graph's cells and encoder tables
   void* enc_scratch = nullptr; size_t enc_scratch_cap = 0;
-  char* stage = nullptr; size_t stage_used = 0;              // pinned: small arrays on their way to the device, where their addresses go
+  char* stage = nullptr; size_t stage_used = 0;              // small arrays on their way to the device, where their addresses go
   std::vector<std::pair<const void**, size_t>> staged;
-  char* host_read = nullptr; size_t host_read_cap = 0;       // pinned: what a run reads back
+  char* host_read = nullptr; size_t host_read_cap = 0;       // what a run reads back
 };
 
 // FP32 FMA issue rate of the device, measured: every thread runs 16 independent FMA chains from registers.
@@ -1050,12 +1050,14 @@ ampnet_status_t ensure_arenas(ampnet_graph* g, size_t ctl_need, size_t bulk_need
   return AMPNET_OK;
 }
 
-// Pinned memory for what a run reads back; sized when instances are loaded, so that no run allocates it.
+// Memory for what a run reads back; sized when instances are loaded, so that no run allocates it.  (Ordinary memory: these are copies of
+// some kilobytes, and pinning a buffer costs a handle 2-10 ms when it opens and closes.)
 ampnet_status_t ensure_host_read(ampnet_graph* g, size_t bytes) {
   if (bytes <= g->host_read_cap) return AMPNET_OK;
-  if (g->host_read) cudaFreeHost(g->host_read);
-  g->host_read = nullptr; g->host_read_cap = 0;
-  CUDA_TRY(g, cudaMallocHost((void**)&g->host_read, bytes));
+  free(g->host_read);
+  g->host_read_cap = 0;
+  g->host_read = (char*)malloc(bytes);
+  if (!g->host_read) return set_err(g, AMPNET_ENOMEM, "out of memory");
   g->host_read_cap = bytes;
   return AMPNET_OK;
 }
@@ -1326,8 +1328,8 @@ void ampnet_graph_destroy(ampnet_graph_t* g) {
   dev_free(g, g->ctl_alloc);
   dev_free(g, g->bulk_mem);
   dev_free(g, g->enc_scratch);
-  if (g->host_read) cudaFreeHost(g->host_read);
-  if (g->stage) cudaFreeHost(g->stage);
+  free(g->host_read);
+  free(g->stage);
   if (g->ev0) cudaEventDestroy(g->ev0);
   if (g->ev1) cudaEventDestroy(g->ev1);
   delete g;
@@ -1418,7 +1420,7 @@ ampnet_status_t ampnet_load_instances(ampnet_graph_t* g, int32_t split, const am
   CUDA_TRY(g, cudaStreamSynchronize(g->stream));
   free_dataset(g, g->data[split]);
   g->staged.clear(); g->stage_used = 0;
-  if (!g->stage) CUDA_TRY(g, cudaMallocHost((void**)&g->stage, STAGE_BYTES));
+  if (!g->stage && !(g->stage = (char*)malloc(STAGE_BYTES))) return set_err(g, AMPNET_ENOMEM, "out of memory");
   HostDataset& D = g->data[split];
   const long long n = in->n_instances;
   D.kind = in->kind; D.n = n;

@@ -27,7 +27,9 @@ constexpr int ACC_RED = CW * 8 * 32 * 4;       // floats of an accumulator's mer
 constexpr int PIECES = 256;                   // pieces of a chunk a warp lists
 constexpr int NEAR = 128;                     // touched pieces of embedding rows a warp lists in shared memory
 
-enum { H_FIRST = 1, H_LAST = 2, H_UPDATE = 4, H_END = 8, H_COPIES = 16 };      // H_COPIES: every row is one or two copies
+enum { H_FIRST = 1, H_LAST = 2, H_UPDATE = 4, H_END = 8, H_COPIES = 16, H_LONG = 32 };      // H_COPIES: every row is one or two copies; H_LONG: a row has more terms than its descriptor holds
+// A loop that may call sum_terms keeps nothing in flight across the call, so loops over rows exist twice.
+template <bool V> struct Flag { static constexpr bool value = V; };
 struct __align__(16) RowD { unsigned out4, a4, b4, meta; Term t[4]; int inst; unsigned base4; unsigned pad[2]; };
 struct Head { int round, count, flags, n_upd, upd_t, n_updates, total, pad; };
 
@@ -328,6 +330,7 @@ __device__ __noinline__ void helper_main(const int cta, const int tile, const in
         if (one) e.t[1].col4 = 0xffff;
       }
       copies = !bar_helper_or(!copies);
+      const bool over = !copies && bar_helper_or(ht < cnt && (e.meta & E_OVERFLOW));
       if (!mbar_wait(&S.empty[buf], parity, t0, 21)) return;
       if (ht < cnt) {
         RowD& r = rows[buf * BM + ht];
@@ -346,7 +349,7 @@ __device__ __noinline__ void helper_main(const int cta, const int tile, const in
       }
       j += cnt;
       const bool last = j >= j1;
-      publish(cnt, (first ? H_FIRST : 0) | (last ? H_LAST : 0) | (upd ? H_UPDATE : 0) | (copies ? H_COPIES : 0), n_upd);
+      publish(cnt, (first ? H_FIRST : 0) | (last ? H_LAST : 0) | (upd ? H_UPDATE : 0) | (copies ? H_COPIES : 0) | (over ? H_LONG : 0), n_upd);
       first = false;
       if (last) break;
     } while (true);
@@ -559,7 +562,7 @@ __device__ __noinline__ void gather_general(const RowD* rows, const int count, c
   }
 }
 __device__ __forceinline__ void gather_terms(const Head& h, const RowD* rows, const int c0, const int nc, float* X, const int ldx) {
-  if (!(h.flags & H_COPIES)) { gather_general<true>(rows, h.count, c0, nc, X, ldx); return; }
+  if (!(h.flags & H_COPIES)) { if (h.flags & H_LONG) gather_general<true>(rows, h.count, c0, nc, X, ldx); else gather_general<false>(rows, h.count, c0, nc, X, ldx); return; }
   const float4* const arena = S.core.arena;
   for_rows(h.count, nc, [&](const int b, const int k0, const int step) {
     const uint4 t = *reinterpret_cast<const uint4*>(&rows[b].t[0]);            // {source, columns} twice
@@ -805,26 +808,29 @@ __device__ __noinline__ void forward_main(const int team, const int tile, float*
       const int K8 = K >> 3, items = ((count + 7) >> 3) * K8 * 8;
       constexpr int U = 4;
       const FastDiv d8(K8);
-      for (int i0 = tid; i0 < items; i0 += U * CT) {
-        float4 a[U], b[U];
+      auto fill_x = [&](auto of_copies) {
+#pragma unroll 1
+        for (int i0 = tid; i0 < items; i0 += U * CT) {
+          float4 a[U], b[U];
 #pragma unroll
-        for (int u = 0; u < U; u++) {
-          const int i = i0 + u * CT, g8 = d8.div(i >> 3), r = g8 * 8 + (i & 7), k8 = (i >> 3) - g8 * K8;
-          a[u] = b[u] = zero4();
-          if (i < items && r < count) {
-            if (h.flags & H_COPIES) {                             // (eight loads in flight; a general row is put together by a call)
+          for (int u = 0; u < U; u++) {
+            const int i = i0 + u * CT, g8 = d8.div(i >> 3), r = g8 * 8 + (i & 7), c = 2 * ((i >> 3) - g8 * K8);
+            a[u] = b[u] = zero4();
+            if (i >= items || r >= count) continue;
+            if constexpr (decltype(of_copies)::value) {
               const uint4 t = *reinterpret_cast<const uint4*>(&R[r].t[0]);
-              const int cut = (int)(t.w & 0xffffu), c = 2 * k8;
+              const int cut = (int)(t.w & 0xffffu);
               a[u] = ldcg4(S.core.arena + (c >= cut ? t.z + (c - cut) : t.x + c)); b[u] = ldcg4(S.core.arena + (c + 1 >= cut ? t.z + (c + 1 - cut) : t.x + c + 1));
-            } else { const int nt = R[r].meta & E_NT; a[u] = term4(R[r], 0, nt, 2 * k8); b[u] = term4(R[r], 0, nt, 2 * k8 + 1); }
+            } else { const int nt = R[r].meta & E_NT; a[u] = term4(R[r], 0, nt, c); b[u] = term4(R[r], 0, nt, c + 1); }
+          }
+#pragma unroll
+          for (int u = 0; u < U; u++) {
+            const int i = i0 + u * CT, g8 = d8.div(i >> 3), r = g8 * 8 + (i & 7), k8 = (i >> 3) - g8 * K8;
+            if (i < items) tc::store8(Xb, r, 8 * k8, K, a[u], b[u]);
           }
         }
-#pragma unroll
-        for (int u = 0; u < U; u++) {
-          const int i = i0 + u * CT, g8 = d8.div(i >> 3), r = g8 * 8 + (i & 7), k8 = (i >> 3) - g8 * K8;
-          if (i < items) tc::store8(Xb, r, 8 * k8, K, a[u], b[u]);
-        }
-      }
+      };
+      if (h.flags & H_COPIES) fill_x(Flag<true>()); else fill_x(Flag<false>());
       tc::fence_operands();
       phase(2);
       if (count <= tc::SMALL_ROWS) for (int i = tid; i < count * YP; i += CT) Ys[i] = 0.f;
@@ -963,6 +969,8 @@ __device__ __noinline__ void input_grad_main(const int team, const int tile, flo
   bar_compute();
   chunk_loop(rows, team, t0, [&](const Head& h, const RowD* R) {
     const int count = h.count;
+    auto gather = [&](auto is_long) {
+    constexpr bool LONG = decltype(is_long)::value;
 #pragma unroll 1
     for (int i = tid; i < count * w4; i += CT) {
       const int b = dw.div(i), c = i - b * w4;
@@ -971,13 +979,13 @@ __device__ __noinline__ void input_grad_main(const int team, const int tile, flo
       float4 d;
       if (kind == LIN_DX && !lstm) {
         const float4 y = T.act ? ldcg4(S.core.arena + r.a4 + c) : zero4();
-        const float4 g = rnd4(bf16, row_sum(r, c));
+        const float4 g = rnd4(bf16, row_sum<LONG>(r, c));
         d = T.act ? make_float4(g.x * act_grad(T.act, y.x), g.y * act_grad(T.act, y.y), g.z * act_grad(T.act, y.z), g.w * act_grad(T.act, y.w)) : g;
         if (mine) S.core.arena[r.b4 + c] = d;
       } else if (kind == GRU_DC) {
         const float4* f = S.core.arena + r.out4 + c;
         float4* q = S.core.arena + r.a4 + c;
-        const float4 hh = ldcg4(f + H4), z = ldcg4(f + 2 * H4), cc = ldcg4(f + 5 * H4), g = rnd4(bf16, row_sum(r, c));
+        const float4 hh = ldcg4(f + H4), z = ldcg4(f + 2 * H4), cc = ldcg4(f + 5 * H4), g = rnd4(bf16, row_sum<LONG>(r, c));
         d = make_float4(g.x * z.x * (1.f - cc.x * cc.x), g.y * z.y * (1.f - cc.y * cc.y), g.z * z.z * (1.f - cc.z * cc.z), g.w * z.w * (1.f - cc.w * cc.w));
         if (mine) {
           q[0] = g;
@@ -995,7 +1003,7 @@ __device__ __noinline__ void input_grad_main(const int team, const int tile, flo
         }
       } else {                                                    // LSTM gates: all gates of four columns
         const float4* f = S.core.arena + r.a4 + c;
-        const float4 gh4 = rnd4(bf16, row_sum(r, c)), gc4 = rnd4(bf16, row_sum(r, H4 + c));
+        const float4 gh4 = rnd4(bf16, row_sum<LONG>(r, c)), gc4 = rnd4(bf16, row_sum<LONG>(r, H4 + c));
         const int L = T.lstm;
         const float4 i4 = ldcg4(f), o4 = ldcg4(f + (branch ? 3 : 1) * H4), u4 = ldcg4(f + (branch ? 4 : 2) * H4);
         float4 fl4 = zero4(), fr4 = zero4(), cl4 = zero4(), cr4 = zero4();
@@ -1031,6 +1039,8 @@ __device__ __noinline__ void input_grad_main(const int team, const int tile, flo
       }
       *reinterpret_cast<float4*>(Gs + b * ld + 4 * c) = d;
     }
+    };
+    if (kind != GRU_DZR && (h.flags & H_LONG)) gather(Flag<true>()); else gather(Flag<false>());
     cp_wait();
     bar_compute();
     phase(2);
