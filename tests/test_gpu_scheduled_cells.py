@@ -1,0 +1,64 @@
+"""Cells of the scheduled engine at the sizes where their tiles, chunks and tables can go wrong, against the CPU oracle."""
+import numpy as np
+import pytest
+
+from workloads import ir, data, params as wp
+
+pytestmark = pytest.mark.gpu
+
+CASES = [
+    # widths that are no multiple of four, one row per round, the smallest layers
+    ("mlp", (61, 37, 3), 9, 1, 0.05, None),
+    ("mlp", (5, 3, 2), 3, 2, 0.05, None),
+    # more rows per round than a chunk holds; tiles of four rows with remainders; moments on padded matrices
+    ("mlp", (61, 258, 7), 301, 150, 0.05, None),
+    ("mlp", (61, 37, 3), 40, 33, 0.005, "adam"),
+    ("rnn", (14, 33, 33, 10), 90, 70, 0.02, None),
+    ("rnn", (14, 33, 33, 10), 30, 8, 0.005, "momentum"),
+    # a table whose sums fit in shared memory, one that is dealt to tiles (two column segments), one whose bit map does not fit
+    ("tree", (60, 36, 21, 5), 40, 32, 0.02, None),
+    ("tree", (5000, 132, 36, 5), 70, 64, 0.02, None),
+    ("tree", (600000, 4, 12, 3), 6, 2, 0.02, None),
+    # sums of more terms than a row's descriptor holds; both LSTM cells
+    ("ggnn", (15, 25, 3), 40, 33, 1e-5, None),
+    ("tree_lstm", (5000, 36, 21, 5), 30, 16, 0.02, "momentum"),
+]
+
+
+def _case(family, size, n):
+    if family == "mlp":
+        return ir.mlp(size), data.mlp_instances(n=n, dim=size[0], classes=size[-1])
+    if family == "rnn":
+        return ir.rnn(size[0], size[1], size[2], size[3]), data.list_instances(n=n)
+    if family == "ggnn":
+        return ir.ggnn(size[0], size[1], size[2], readout=size[1]), data.graph_instances(n=n, steps=size[2])
+    return (ir.tree if family == "tree" else ir.tree_lstm)(*size), data.tree_instances(n=n, vocab=size[0], classes=size[3])
+
+
+@pytest.mark.parametrize("family,size,n,mak,lr,kind", CASES)
+def test_epochs_of_one_update_match_oracle(oracle_mod, family, size, n, mak, lr, kind):
+    """Two epochs whose only update is the flush at their end (so that the schedule cannot matter) and an evaluation: the second
+    epoch reads what the first one wrote back.  Losses are sums of at most a few thousand single-precision terms (an error of
+    2^-24 sqrt(terms), under 1e-5 of the loss, with a floor of 2e-6 for the log-sum-exp); a parameter moves by the mean gradient,
+    whose error is of the same order, so it stays within 1e-4 of the tensor's largest entry (twice these after an update)."""
+    import paper_1705_09786_b200 as amp
+    g, inst = _case(family, size, n)
+    p = wp.init_params(g)
+    sides = []
+    for s in (oracle_mod.Oracle(g), amp.Engine(g)):
+        s.load_instances(inst)
+        s.load_instances(inst, split=1)
+        s.set_params(p)
+        if kind:
+            s.set_optimizer(kind=kind, momentum=0.8, beta1=0.85, beta2=0.99, eps=1e-6)
+        sides.append(s)
+    o, e = sides
+    for epoch in range(2):
+        _, oloss = o.run_epoch(mak=1, muf=1 << 30, lr=lr)
+        st, eloss = e.run_epoch(mak=mak, muf=1 << 30, lr=lr, timeout_s=60)
+        np.testing.assert_allclose(eloss, oloss, rtol=(1 + epoch) * 1e-5, atol=(1 + epoch) * 2e-6)
+        ep, op = e.get_params(), o.get_params()
+        for k in op:
+            assert np.abs(ep[k] - op[k]).max() <= (1 + epoch) * 1e-4 * np.abs(op[k]).max(), (epoch, g.names[k[0]], k[1])
+    np.testing.assert_allclose(e.eval(split=1, mak=mak)[2], o.eval(split=1)[2], rtol=3e-5, atol=6e-6)
+    e.close()
