@@ -217,11 +217,15 @@ static ampnet_status_t wave_encode(ampnet_graph* g, HostDataset& D, WaveModel& M
   wave_sizes(M, g->hnodes, D);
   for (auto& h : g->hnodes) if (h.U_in > 65535 || h.U_out > 65535) return AMPNET_OK;      // (positions travel in sixteen bits)
   if ((unsigned long long)M.enc.scratch_words * 4 > (1ull << 30)) return AMPNET_OK;
-  const EncModel& E = M.enc;
-  // warps per block: with the scratch in shared memory as many as fit there (an SM holds 16 of them by registers)
-  const size_t warp_bytes = (size_t)E.scratch_words * 4;
+  // Warps per block: with the scratch in shared memory as many as fit there.  An instance is one long chain of dependent steps, so a large
+  // split wants warps more than it wants near memory (an SM holds 16 by registers): 20,000 lists of 26 KB scratch 8.5 -> 4.8 ms.
+  const size_t warp_bytes = (size_t)M.enc.scratch_words * 4, near_bytes = warp_bytes + M.enc.stack_cap * 16;
   int per = encode_warps_per_block();
-  if (E.near_scratch) per = (int)std::max<size_t>(1, std::min<size_t>(per, (size_t)(200 * 1024) / (warp_bytes + E.stack_cap * 16)));
+  const int near_per = (int)std::max<size_t>(1, std::min<size_t>(per, (size_t)(200 * 1024) / near_bytes));
+  const long long near_warps = (long long)((size_t)(220 * 1024) / near_bytes);      // of an SM
+  if (near_warps < 16 && n > 2 * g->n_sms * std::max(1ll, near_warps)) M.enc.near_scratch = false;
+  const EncModel& E = M.enc;
+  if (E.near_scratch) per = near_per;
   if (n < (long long)g->n_sms * per) per = 1;
   long long blocks = (n + per - 1) / per;
   EncTotals init{};
@@ -254,7 +258,7 @@ static ampnet_status_t wave_encode(ampnet_graph* g, HostDataset& D, WaveModel& M
   size_t need = 256;
   if (!E.near_scratch) {
     blocks = std::min<long long>(blocks, 4ll * g->n_sms);
-    blocks = std::min<long long>(blocks, std::max<long long>(1, (long long)((512ull << 20) / (warp_bytes * per))));
+    blocks = std::min<long long>(blocks, std::max<long long>(1, (long long)((2048ull << 20) / (warp_bytes * per))));
     need = (size_t)blocks * per * warp_bytes;
   }
   if (need > *scratch_cap) {
@@ -293,6 +297,11 @@ static ampnet_status_t wave_encode(ampnet_graph* g, HostDataset& D, WaveModel& M
   W.prog.ov = (const Term*)(mem + ov_at);
   CUDA_TRY(g, encode_emit(&E, D.dev, (unsigned*)*scratch, (int)blocks, per, W.prog, counts, (Term*)(mem + ov_at), totals, g->stream));
   W.ok = true;
+  if (*scratch_cap > (64ull << 20)) {                            // (given back: a handle keeps what small splits need)
+    CUDA_TRY(g, cudaStreamSynchronize(g->stream));
+    dev_free(g, *scratch);
+    *scratch = nullptr; *scratch_cap = 0;
+  }
   return AMPNET_OK;
 }
 
