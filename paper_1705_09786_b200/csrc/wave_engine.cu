@@ -16,8 +16,19 @@
 #include "tc_tile.cuh"
 #include "wave.h"
 
+#ifdef WAVE_FORWARD
+#define ENGINE_KERNEL ampnet_engine_scheduled_forward
+#define EVALUATING true
+#define ENGINE_NAMESPACE forward
+#else
+#define ENGINE_KERNEL ampnet_engine_scheduled
+#define EVALUATING false
+#define ENGINE_NAMESPACE training
+#endif
+
 namespace wave {
 using namespace amp;
+namespace ENGINE_NAMESPACE {
 
 constexpr int CT = 512, CW = CT / 32;         // compute threads
 constexpr int HT = 128;                       // helper threads
@@ -242,12 +253,12 @@ __device__ __noinline__ void helper_main(const int cta, const int tile, const in
         if (left > 0 && rank < admitted) {
           const long long i = S.core.order ? S.core.order[next + rank] : next + rank;
           const InstHdr h = S.core.prog.hdr[i];
-          const bool ev = S.core.eval || (S.core.inference_only && S.core.inference_only[i]);
+          const bool ev = EVALUATING || (S.core.inference_only && S.core.inference_only[i]);
           L.tab[s] = h.tab; L.end[s] = h.tab + (ev ? h.steps_eval : h.steps);
           const unsigned home = (unsigned)s * (unsigned)S.core.copies * S.core.slot4, b = L.base4[s] + S.core.slot4;      // the key's arenas take turns
           L.base4[s] = b == home + (unsigned)S.core.copies * S.core.slot4 ? home : b;
-          L.inst[s] = (int)i | (ev && !S.core.eval ? (int)0x80000000 : 0);
-          if (cta == 0) { node_msgs += ev ? h.msgs_eval : h.msgs; inf_instances += ev && !S.core.eval; }
+          L.inst[s] = (int)i | (ev && !EVALUATING ? (int)0x80000000 : 0);
+          if (cta == 0) { node_msgs += ev ? h.msgs_eval : h.msgs; inf_instances += ev && !EVALUATING; }
         }
       }
       next += admitted;
@@ -367,7 +378,7 @@ __device__ __noinline__ void helper_main(const int cta, const int tile, const in
   // ---- statistics ----------------------------------------------------------------------------------------------------------
   PPTStats& st = *S.ppt.stats;
   const bool counts_msgs = leader && kind != GRU_C && kind != GRU_DZR && !(kind == ACC && !S.ppt.source_adj);
-  if (counts_msgs && n_msgs) atomicAdd(&st.msgs, n_msgs * (kind == HEAD && !S.core.eval ? 2ull : 1ull));
+  if (counts_msgs && n_msgs) atomicAdd(&st.msgs, n_msgs * (kind == HEAD && !EVALUATING ? 2ull : 1ull));
   if (leader && ht == 0) {
     if (updates && !(kind == ACC && T.pad)) { st.n_updates = n_updates; st.n_grads_applied = n_grads; st.log_n = n_updates; }
     if (!backward && shard == 0) st.max_pending[0] = max_rows;
@@ -624,9 +635,9 @@ __device__ __noinline__ void gemm_warps(const float* __restrict__ A, const int l
   }
 }
 __device__ __forceinline__ void fma2(unsigned long long& d, const unsigned long long a, const unsigned long long b) { asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b)); }
+template <int KL>
 __device__ __noinline__ void gemm_tiles(const float* __restrict__ A, const int lda, const int nA, const float* __restrict__ B, const int ldb, const int nB, const int K4, float* __restrict__ Y, const int ldy) {
   IN_SMEM(A); IN_SMEM(B); IN_SMEM(Y);
-  constexpr int KL = 4;
   const int lane = threadIdx.x & 31, ks = lane & (KL - 1), tB = nB >> 2, n = ((nA + 3) >> 2) * tB;
   const FastDiv dB(tB);
   const int lda4 = lda >> 2, ldb4 = ldb >> 2;
@@ -665,8 +676,11 @@ __device__ __noinline__ void gemm_tiles(const float* __restrict__ A, const int l
       for (int i = 0; i < H; i++) { const float give = up ? v[i] : v[i + H], keep = up ? v[i + H] : v[i]; v[i] = keep + __shfl_xor_sync(0xffffffffu, give, s); }
       at += up ? H : 0;
     }
-    const int b = 4 * bt + (at >> 2);
-    if (mine && b < nA) *reinterpret_cast<float4*>(Y + b * ldy + 4 * ot) = make_float4(v[0], v[1], v[2], v[3]);
+    const int b = 4 * bt + (at >> 2), o = 4 * ot + (at & 3);
+    if (!mine || b >= nA) continue;
+    if constexpr (KL == 4) *reinterpret_cast<float4*>(Y + b * ldy + o) = make_float4(v[0], v[1], v[2], v[3]);
+    else if constexpr (KL == 8) *reinterpret_cast<float2*>(Y + b * ldy + o) = make_float2(v[0], v[1]);
+    else Y[b * ldy + o] = v[0];
   }
 }
 __device__ __noinline__ void gemm_few(const float* __restrict__ A, const int lda, const int nA, const float* __restrict__ B, const int ldb, const int nB, const int K4, float* __restrict__ Y, const int ldy) {
@@ -700,9 +714,21 @@ __device__ __noinline__ void gemm_few(const float* __restrict__ A, const int lda
   }
 }
 __device__ __forceinline__ void gemm(const float* A, const int lda, const int nA, const float* B, const int ldb, const int nB, const int K4, float* Y, const int ldy) {
-  if (nA <= 4) gemm_few(A, lda, nA, B, ldb, nB, K4, Y, ldy);
-  else if (nA * nB <= 1536) gemm_warps(A, lda, nA, B, ldb, nB, K4, Y, ldy);
-  else gemm_tiles(A, lda, nA, B, ldb, nB, K4, Y, ldy);
+  if (nA <= 4) { gemm_few(A, lda, nA, B, ldb, nB, K4, Y, ldy); return; }
+#ifdef WAVE_FORWARD
+  // a round of an evaluation has some ten rows per CTA: as many k lanes as keep the threads busy (tree 9.75 -> 8.9 ms, graph net 14.6 ->
+  // 13.4).  Training keeps to two shapes: with more, the register allocation of its other cells lost more than the products gained.
+  const int tiles = ((nA + 3) >> 2) * (nB >> 2);
+  if (tiles > 16) {
+    if (tiles <= 32) gemm_tiles<16>(A, lda, nA, B, ldb, nB, K4, Y, ldy);
+    else if (tiles <= 64) gemm_tiles<8>(A, lda, nA, B, ldb, nB, K4, Y, ldy);
+    else gemm_tiles<4>(A, lda, nA, B, ldb, nB, K4, Y, ldy);
+    return;
+  }
+#else
+  if (nA * nB > 1536) { gemm_tiles<4>(A, lda, nA, B, ldb, nB, K4, Y, ldy); return; }
+#endif
+  gemm_warps(A, lda, nA, B, ldb, nB, K4, Y, ldy);
 }
 
 // ---- weights ---------------------------------------------------------------------------------------------------------------
@@ -852,7 +878,7 @@ __device__ __noinline__ void forward_main(const int team, const int tile, float*
         const int b = dr.div(i), k = i - b * (nB >> 2);
         S.core.arena[R[b].out4 + (j0 >> 2) + k] = rnd4(bf16, act_fwd4(T.act, add4(*reinterpret_cast<const float4*>(Ys + b * YP + 4 * k), *reinterpret_cast<const float4*>(bs + 4 * k))));
       }
-      if (tile == 0 && !S.core.eval) for (int b = tid; b < count; b += CT) S.core.arena[R[b].out4 + H4] = make_float4(__int_as_float(version), 0.f, 0.f, 0.f);
+      if (tile == 0 && !EVALUATING) for (int b = tid; b < count; b += CT) S.core.arena[R[b].out4 + H4] = make_float4(__int_as_float(version), 0.f, 0.f, 0.f);
       return;
     }
     gather_terms(h, R, 0, n4, Xs, ld);
@@ -911,12 +937,12 @@ __device__ __noinline__ void forward_main(const int team, const int tile, float*
       auto pre = [&](const int g) { return rnd4(bf16, add4(y4[g * w4], b4[g * w4])); };
       const float4 gi = act_fwd4(3, pre(0)), gu = act_fwd4(2, pre(branch ? 4 : 2)), go = act_fwd4(3, pre(branch ? 3 : 1));
       float4 c = make_float4(gi.x * gu.x, gi.y * gu.y, gi.z * gu.z, gi.w * gu.w);
-      if (!S.core.eval) { out[c4] = gi; out[(branch ? 3 : 1) * H4 + c4] = go; out[(branch ? 4 : 2) * H4 + c4] = gu; }
+      if (!EVALUATING) { out[c4] = gi; out[(branch ? 3 : 1) * H4 + c4] = go; out[(branch ? 4 : 2) * H4 + c4] = gu; }
       if (branch) {
         const int nt = r.meta & E_NT, nc = r.meta >> 16;
         const float4 cl = term4(r, nt, nc, c4), cr = term4(r, nt, nc, H4 + c4), fl = act_fwd4(3, pre(1)), fr = act_fwd4(3, pre(2));
         c = make_float4(c.x + fl.x * cl.x + fr.x * cr.x, c.y + fl.y * cl.y + fr.y * cr.y, c.z + fl.z * cl.z + fr.z * cr.z, c.w + fl.w * cl.w + fr.w * cr.w);
-        if (!S.core.eval) { out[H4 + c4] = fl; out[2 * H4 + c4] = fr; out[7 * H4 + 1 + c4] = cl; out[8 * H4 + 1 + c4] = cr; }
+        if (!EVALUATING) { out[H4 + c4] = fl; out[2 * H4 + c4] = fr; out[7 * H4 + 1 + c4] = cl; out[8 * H4 + 1 + c4] = cr; }
       }
       const float4 tc4 = act_fwd4(2, c);
       out[T.lstm * H4 + c4] = rnd4(bf16, clip(make_float4(go.x * tc4.x, go.y * tc4.y, go.z * tc4.z, go.w * tc4.w)));
@@ -924,7 +950,7 @@ __device__ __noinline__ void forward_main(const int team, const int tile, float*
     }
     }
     // a summed input is kept for the accumulator (every tile a share of the columns); so is a GRU's
-    if (kind == GRU_ZR || (T.keep && !S.core.eval)) {
+    if (kind == GRU_ZR || (T.keep && !EVALUATING)) {
       const int share = (n4 + T.T - 1) / T.T, k0 = tile * share, kn = min(share, n4 - k0);
 #pragma unroll 1
       for (int i = tid; i < count * share; i += CT) {
@@ -932,7 +958,7 @@ __device__ __noinline__ void forward_main(const int team, const int tile, float*
         if (k < kn) S.core.arena[(kind == GRU_ZR ? R[b].out4 : R[b].a4) + k0 + k] = *reinterpret_cast<const float4*>(Xs + b * ld + 4 * (k0 + k));
       }
     }
-    if (tile == 0 && !S.core.eval && kind != GRU_ZR) {
+    if (tile == 0 && !EVALUATING && kind != GRU_ZR) {
       const unsigned at = kind == GRU_C ? 7u * H4 : lstm ? (unsigned)(T.lstm + 2) * H4 : (unsigned)H4;
 #pragma unroll 1
       for (int b = tid; b < count; b += CT) S.core.arena[R[b].out4 + at] = make_float4(__int_as_float(version), 0.f, 0.f, 0.f);
@@ -1296,7 +1322,7 @@ __device__ __noinline__ void head_main(const int team, float* smem, RowD* rows, 
         if (inf) inf_sum += loss; else loss_sum += loss;
       }
     }
-    if (S.core.eval) return;
+    if (EVALUATING) return;
     bar_compute();
     phase(5);
 #pragma unroll 1
@@ -1548,7 +1574,7 @@ __device__ __noinline__ void lookup_grad_main(const int team, const int tile, fl
 }
 
 // ---- the kernel -------------------------------------------------------------------------------------------------------------------
-extern "C" __global__ void __launch_bounds__(NT, 1) ampnet_engine_scheduled(const __grid_constant__ Run C) {
+extern "C" __global__ void __launch_bounds__(NT, 1) ENGINE_KERNEL(const __grid_constant__ Run C) {
   extern __shared__ __align__(128) unsigned char smem[];
   const unsigned long long t0 = gtime();
   const int tid = threadIdx.x, cta = blockIdx.x;
@@ -1592,13 +1618,15 @@ extern "C" __global__ void __launch_bounds__(NT, 1) ampnet_engine_scheduled(cons
       break;
     case GRU_ZR: forward_main<F_ZR>(team, tile, work, rows, t0); break;
     case GRU_C: forward_main<F_C>(team, tile, work, rows, t0); break;
+    case HEAD: head_main(team, work, rows, t0); break;
+    case LOOKUP_F: lookup_main(team, rows, t0); break;
+#ifndef WAVE_FORWARD
     case LIN_DX: if (S.team.lstm) input_grad_main<B_LSTM>(team, tile, work, rows, t0); else input_grad_main<B_PLAIN>(team, tile, work, rows, t0); break;
     case GRU_DC: input_grad_main<B_DC>(team, tile, work, rows, t0); break;
     case GRU_DZR: input_grad_main<B_DZR>(team, tile, work, rows, t0); break;
     case ACC: accumulate_main(team, tile, work, rows, t0); break;
-    case HEAD: head_main(team, work, rows, t0); break;
-    case LOOKUP_F: lookup_main(team, rows, t0); break;
     case LOOKUP_B: if (S.team.R) lookup_grad_small_main(team, work, rows, t0); else lookup_grad_main(team, tile, work, rows, t0); break;
+#endif
   }
   __syncthreads();
   if (idx == 0 && tid < N_PHASES) C.core.phases[team * N_PHASES + tid] = S.phase[tid];
@@ -1617,6 +1645,24 @@ extern "C" __global__ void __launch_bounds__(NT, 1) ampnet_engine_scheduled(cons
 }
 
 // ---- host hooks ---------------------------------------------------------------------------------------------------------------
+cudaError_t launch(const Run* run, int n_ctas, size_t smem, cudaStream_t st) {
+  static size_t set[64] = {};
+  int dev = 0;
+  cudaGetDevice(&dev);
+  if (dev < 0 || dev >= 64 || set[dev] < smem) {
+    const cudaError_t e = cudaFuncSetAttribute(ENGINE_KERNEL, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    if (dev >= 0 && dev < 64) set[dev] = smem;
+  }
+  void* args[] = {const_cast<Run*>(run)};
+  return cudaLaunchCooperativeKernel((void*)ENGINE_KERNEL, dim3(n_ctas), dim3(NT), args, smem, st);
+}
+}  // namespace ENGINE_NAMESPACE
+
+#ifndef WAVE_FORWARD
+namespace forward { cudaError_t launch(const Run* run, int n_ctas, size_t smem, cudaStream_t st); }      // wave_forward.cu
+cudaError_t launch(const Run* run, int n_ctas, size_t smem, cudaStream_t st) { return run->core.eval ? forward::launch(run, n_ctas, smem, st) : training::launch(run, n_ctas, smem, st); }
+using namespace training;
 size_t smem_bytes(const Team& t, const Mat& m, int mak) {
   const size_t head = slots_bytes(mak) + 2 * (size_t)t.BM * sizeof(RowD);
   const size_t ldi = pad_ld(m.inp), ldo = pad_ld(m.outp), BM = t.BM;
@@ -1639,17 +1685,6 @@ size_t static_smem() {
   cudaFuncAttributes fa{};
   return cudaFuncGetAttributes(&fa, ampnet_engine_scheduled) == cudaSuccess ? fa.sharedSizeBytes : 4096;
 }
-cudaError_t launch(const Run* run, int n_ctas, size_t smem, cudaStream_t st) {
-  static size_t set[64] = {};
-  int dev = 0;
-  cudaGetDevice(&dev);
-  if (dev < 0 || dev >= 64 || set[dev] < smem) {
-    const cudaError_t e = cudaFuncSetAttribute(ampnet_engine_scheduled, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    if (dev >= 0 && dev < 64) set[dev] = smem;
-  }
-  void* args[] = {const_cast<Run*>(run)};
-  return cudaLaunchCooperativeKernel((void*)ampnet_engine_scheduled, dim3(n_ctas), dim3(NT), args, smem, st);
-}
+#endif
 
 }  // namespace wave
