@@ -20,6 +20,10 @@
 #define ENGINE_KERNEL ampnet_engine_scheduled_forward
 #define EVALUATING true
 #define ENGINE_NAMESPACE forward
+#elif defined(WAVE_MOMENTS)
+#define ENGINE_KERNEL ampnet_engine_scheduled_moments
+#define EVALUATING false
+#define ENGINE_NAMESPACE moments
 #else
 #define ENGINE_KERNEL ampnet_engine_scheduled
 #define EVALUATING false
@@ -29,6 +33,13 @@
 namespace wave {
 using namespace amp;
 namespace ENGINE_NAMESPACE {
+#ifdef WAVE_MOMENTS
+constexpr bool SGD = false;
+#define OPT_STEP_INLINE __noinline__
+#else
+constexpr bool SGD = true;                    // (momentum and Adam: wave_moments.cu)
+#define OPT_STEP_INLINE __forceinline__
+#endif
 
 constexpr int CT = 512, CW = CT / 32;         // compute threads
 constexpr int HT = 128;                       // helper threads
@@ -44,7 +55,11 @@ template <bool V> struct Flag { static constexpr bool value = V; };
 struct __align__(16) RowD { unsigned out4, a4, b4, meta; Term t[4]; int inst; unsigned base4; unsigned pad[2]; };
 struct Head { int round, count, flags, n_upd, upd_t, n_updates, total, pad; };
 
+// Geometry of an accumulator's tile (floats and fours; smem offsets in floats; s*: powers of two).  It is read from shared memory in every
+// section of a chunk: kept in registers it drives the gradient sums out of them.
+struct AccGeo { int ro, ci, o0, i0, d4, x4, ldd, ldx, ldw, sN, sW, sL, red, dg, xg, bm, bred, Ro; unsigned ddM, dxM; };
 struct Shared {
+  AccGeo ag;
   Core core; Team team; Mat mat; PptRun ppt;
   Head hd[2];
   unsigned long long full[2], empty[2], tc_mbar;
@@ -138,6 +153,7 @@ __device__ __forceinline__ float act_grad(int a, float y) {
 // n / d for 0 <= n < 200000 and 1 <= d <= 2048 by one multiply-high
 struct FastDiv {
   unsigned d, M;
+  __device__ FastDiv(unsigned d_, unsigned M_) : d(d_), M(M_) {}
   __device__ explicit FastDiv(int d_) : d((unsigned)d_), M(d_ > 1 ? 0xFFFFFFFFu / (unsigned)d_ + 1u : 0u) {}
   __device__ __forceinline__ int div(int n) const { return d > 1 ? (int)__umulhi((unsigned)n, M) : n; }
 };
@@ -150,10 +166,10 @@ __device__ __forceinline__ int real_in(const Mat& m, int pi) { const int wp = (m
 struct OptStep {              // update of parameters from their accumulated gradients: SGD, momentum or Adam on the mean (Sec. 3, App. A)
   int opt; float step, inv_n, lr, mu, b1, b2, eps, c1, c2; float *om, *ov;
 };
-__device__ __noinline__ OptStep opt_step(float* om, float* ov, long long t0, int n_upd, int upd_t) {
+__device__ OPT_STEP_INLINE OptStep opt_step(float* om, float* ov, long long t0, int n_upd, int upd_t) {
   OptStep s;
-  s.opt = S.core.opt; s.lr = S.core.lr; s.inv_n = 1.f / (float)n_upd; s.step = S.core.lr * s.inv_n; s.mu = S.core.mu; s.b1 = S.core.beta1; s.b2 = S.core.beta2; s.eps = S.core.eps; s.c1 = s.c2 = 1.f; s.om = om; s.ov = ov;
-  if (s.opt == 2) {
+  s.opt = SGD ? 0 : S.core.opt; s.lr = S.core.lr; s.inv_n = 1.f / (float)n_upd; s.step = S.core.lr * s.inv_n; s.mu = S.core.mu; s.b1 = S.core.beta1; s.b2 = S.core.beta2; s.eps = S.core.eps; s.c1 = s.c2 = 1.f; s.om = om; s.ov = ov;
+  if (!SGD && s.opt == 2) {
     const double t = (double)(t0 + upd_t);
     s.c1 = (float)(1.0 / (1.0 - pow((double)s.b1, t)));
     s.c2 = (float)(1.0 / (1.0 - pow((double)s.b2, t)));
@@ -171,7 +187,7 @@ __device__ __noinline__ float opt_moments(const OptStep& s, float w, const float
   s.om[k] = m; s.ov[k] = v;
   return w - s.lr * (m * s.c1) / (sqrtf(v * s.c2) + s.eps);
 }
-__device__ __forceinline__ float opt_one(const OptStep& s, const float w, const float a, const size_t k) { return s.opt == 0 ? fmaf(-s.step, a, w) : opt_moments(s, w, a, k); }
+__device__ __forceinline__ float opt_one(const OptStep& s, const float w, const float a, const size_t k) { return SGD || s.opt == 0 ? fmaf(-s.step, a, w) : opt_moments(s, w, a, k); }
 // Four neighbours of a padded matrix row with moments (padding is left alone); plain SGD needs no index, padding has zero gradients.
 __device__ __noinline__ float4 opt_padded(const OptStep& s, const Mat& m, const int po, const int pi, const float4 w, const float4 a) {
   IN_SMEM(&m);
@@ -1104,26 +1120,28 @@ __device__ __noinline__ void input_grad_main(const int team, const int tile, flo
 __device__ __noinline__ void accumulate_main(const int team, const int tile, float* smem, RowD* rows, const unsigned long long t0) {
   IN_SMEM(smem);  IN_SMEM(rows);
   const Team& T = S.team; const Mat& m = S.mat;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int Ro = T.R, Ci = T.C, WO = T.WO, WI = T.WI, NR = WO * WI, WS = CW / NR, LO = T.LO, LI = 32 / LO;
-  const int ti = (m.inp + Ci - 1) / Ci, to = tile / ti, o0 = to * Ro, i0 = (tile - to * ti) * Ci;
-  const int ro = min(Ro, m.outp - o0), ci = min(Ci, m.inp - i0);
-  const int ldd = Ro + 4, ldx = Ci + 4, ldw = Ci + 4;
-  float *Wm = smem, *red = Wm + (size_t)Ro * ldw, *Dg = red + ACC_RED, *Xg = Dg + (size_t)T.BM * ldd, *bm = Xg + (size_t)T.BM * ldx, *bred = bm + Ro;   // bred: WS x Ro floats
-  const bool biased = i0 == 0;
+  const int tid = threadIdx.x;
+  {
+    const int Ro = T.R, Ci = T.C, ti = (m.inp + Ci - 1) / Ci, to = tile / ti, o0 = to * Ro, i0 = (tile - to * ti) * Ci, ro = min(Ro, m.outp - o0), ci = min(Ci, m.inp - i0);
+    const int ldd = Ro + 4, ldx = Ci + 4, ldw = Ci + 4, dg = Ro * ldw + ACC_RED, xg = dg + T.BM * ldd, bm = xg + T.BM * ldx;
+    if (tid == 0) {
+      AccGeo z;
+      z.ro = ro; z.ci = ci; z.o0 = o0; z.i0 = i0; z.d4 = ro >> 2; z.x4 = ci >> 2; z.ldd = ldd; z.ldx = ldx; z.ldw = ldw;
+      z.sN = 31 - __clz(T.WO * T.WI); z.sW = 31 - __clz(T.WI); z.sL = 31 - __clz(32 / T.LO);
+      z.red = Ro * ldw; z.dg = dg; z.xg = xg; z.bm = bm; z.bred = bm + Ro; z.Ro = Ro;
+      z.ddM = FastDiv(ro >> 2).M; z.dxM = FastDiv(ci >> 2).M;
+      S.ag = z;
+    }
 #pragma unroll 1
-  for (int i = tid; i < Ro * Ci; i += CT) {
-    const int o = i / Ci, c = i - o * Ci, r = o < ro ? real_out(m, o0 + o) : -1, k = c < ci ? real_in(m, i0 + c) : -1;
-    Wm[o * ldw + c] = (r >= 0 && k >= 0) ? m.W[(size_t)r * m.in_real + k] : 0.f;
+    for (int i = tid; i < Ro * Ci; i += CT) {
+      const int o = i / Ci, c = i - o * Ci, r = o < ro ? real_out(m, o0 + o) : -1, k = c < ci ? real_in(m, i0 + c) : -1;
+      smem[o * ldw + c] = (r >= 0 && k >= 0) ? m.W[(size_t)r * m.in_real + k] : 0.f;
+    }
+#pragma unroll 1
+    for (int i = tid; i < Ro; i += CT) { const int r = i < ro ? real_out(m, o0 + i) : -1; smem[bm + i] = r >= 0 ? m.b[r] : 0.f; }
+#pragma unroll 1
+    for (int i = tid; i < T.BM * (ldd + ldx); i += CT) smem[dg + i] = 0.f;      // columns past the matrix stay zero
   }
-#pragma unroll 1
-  for (int i = tid; i < Ro; i += CT) { const int r = i < ro ? real_out(m, o0 + i) : -1; bm[i] = r >= 0 ? m.b[r] : 0.f; }
-#pragma unroll 1
-  for (int i = tid; i < T.BM * (ldd + ldx); i += CT) Dg[i] = 0.f;           // columns past the matrix stay zero
-  const int ws = warp / NR, wr = warp - ws * NR, wo = wr / WI, wi = wr - wo * WI;
-  const int lo = lane / LI, li = lane - lo * LI;
-  const int ob = (wo * LO + lo) * 8, ib = (wi * LI + li) * 4;
-  const bool summing = biased && wi == 0 && li == 0;                        // these lanes also add up their rows' gradients (bias)
   float acc[8][4], bacc[8];
 #pragma unroll
   for (int k = 0; k < 8; k++) {
@@ -1134,106 +1152,128 @@ __device__ __noinline__ void accumulate_main(const int team, const int tile, flo
   unsigned pubs = 0;
   int updates = 0;
   bool dirty = false;
-  const int d4 = ro >> 2, x4 = ci >> 2;
-  const FastDiv dd(d4), dx(x4);
-  const bool leader = tile == 0;
-  unsigned long long* const ver = reinterpret_cast<unsigned long long*>(m.ver);
+  const volatile AccGeo& Z = S.ag;
   bar_compute();
-  // theta <- theta - step(A / n); the accumulators start over
-  auto update = [&](const int n_upd, const int upd_t) {
-    const OptStep os = opt_step(m.om, m.ov, m.opt_t0, n_upd, upd_t);
-    float4* const r4 = reinterpret_cast<float4*>(red);
-    if (summing) {
-#pragma unroll
-      for (int k = 0; k < 8; k++) bred[ws * Ro + ob + k] = bacc[k];
-    }
-#pragma unroll
-    for (int k = 0; k < 8; k++) r4[(ws * 8 + k) * (32 * NR) + wr * 32 + lane] = make_float4(acc[k][0], acc[k][1], acc[k][2], acc[k][3]);
-    bar_compute();
-    const int per = 8 * 32 * NR, sW = 31 - __clz(WI), sL = 31 - __clz(LI), sN = 31 - __clz(NR);                                // sums of four columns; every thread adds up some over the slices
-#pragma unroll 1
-    for (int i = tid; i < per; i += CT) {
-      float4 a = zero4();
-#pragma unroll 4
-      for (int s = 0; s < WS; s++) a = add4(a, r4[s * per + i]);
-      const int l = i & 31, q = (i >> 5) & (NR - 1), k = i >> (5 + sN), o = ((q >> sW) * LO + (l >> sL)) * 8 + k, c = ((q & (WI - 1)) * LI + (l & (LI - 1))) * 4;
-      float4* const w4 = reinterpret_cast<float4*>(Wm + o * ldw + c);
-      *w4 = os.opt == 0 ? sgd4(os.step, *w4, a) : opt_padded(os, m, o0 + o, i0 + c, *w4, a);
-    }
-    if (biased)
-#pragma unroll 1
-      for (int i = CT - 1 - tid; i < ro; i += CT) {
-        float a = 0.f;
-#pragma unroll 4
-        for (int s = 0; s < WS; s++) a += bred[s * Ro + i];
-        const int r = real_out(m, o0 + i);
-        if (r >= 0) bm[i] = opt_one(os, bm[i], a, (size_t)m.nW + r);
-      }
-#pragma unroll
-    for (int k = 0; k < 8; k++) {
-      bacc[k] = 0.f;
-#pragma unroll
-      for (int j = 0; j < 4; j++) acc[k][j] = 0.f;
-    }
-    bar_compute();
+  auto stamp = [&](const Head& h) {
+    if (tile == 0 && tid == 0) *(reinterpret_cast<volatile unsigned long long*>(m.ver) + (h.round & 31)) = ((unsigned long long)(unsigned)updates << 32) | ((unsigned long long)(pubs & 0xffffu) << 16) | ((unsigned)h.round & 0xffffu);
   };
-  auto stamp = [&](const Head& h) { if (leader && tid == 0) *reinterpret_cast<volatile unsigned long long*>(ver + (h.round & 31)) = ((unsigned long long)(unsigned)updates << 32) | ((unsigned long long)(pubs & 0xffffu) << 16) | ((unsigned)h.round & 0xffffu); };
   const Head end = chunk_loop(rows, team, t0, [&](const Head& h, const RowD* R) {
     const int count = h.count;
-    // staleness: updates of the node since the forward pass (Sec. 3); a warp per 32 rows, loaded before the rows and counted after
-    float version = 0.f;
-    bool message = false, stamped = false;
-    if (leader && tid < count) {
-      const RowD& r = R[tid];
-      message = r.meta & E_MSG_END; stamped = message && r.a4 != NONE;
-      if (stamped) version = __ldcg(reinterpret_cast<const float*>(S.core.arena + r.a4 + ((r.meta & E_RAW) ? (m.outp >> 2) : 0)));
-    }
-#pragma unroll 1
-    for (int i = tid; i < count * d4; i += CT) {
-      const int b = dd.div(i), k = i - b * d4, c = (o0 >> 2) + k;
-      const RowD& r = R[b];
-      if (!(r.meta & E_RAW)) { cp16(Dg + b * ldd + 4 * k, S.core.arena + r.out4 + c); continue; }
-      const float4 y = ldcg4(S.core.arena + r.a4 + c), g = rnd4(S.core.bf16, row_sum<false>(r, c));
-      *reinterpret_cast<float4*>(Dg + b * ldd + 4 * k) = make_float4(g.x * act_grad(T.act, y.x), g.y * act_grad(T.act, y.y), g.z * act_grad(T.act, y.z), g.w * act_grad(T.act, y.w));
-    }
-    if (h.flags & H_COPIES) {                                    // (a flat loop: the sums leave no registers for more)
-#pragma unroll 1
-      for (int i = tid; i < count * x4; i += CT) {
-        const int b = dx.div(i), k = i - b * x4, c = (i0 >> 2) + k;
-        const uint4 t = *reinterpret_cast<const uint4*>(&R[b].t[0]);
-        const bool second = c >= (int)(t.w & 0xffffu);
-        cp16(Xg + b * ldx + 4 * k, S.core.arena + (second ? t.z + c - (t.w & 0xffffu) : t.x + c));
+    {
+      const int d4 = Z.d4, x4 = Z.x4, ldd = Z.ldd, ldx = Z.ldx, o4 = Z.o0 >> 2, i4 = Z.i0 >> 2;
+      float* const Dg = smem + Z.dg; float* const Xg = smem + Z.xg;
+      // staleness: updates of the node since the forward pass (Sec. 3); a warp per 32 rows, loaded before the rows and counted after
+      float version = 0.f;
+      bool message = false, stamped = false;
+      if (tile == 0 && tid < count) {
+        const RowD& r = R[tid];
+        message = r.meta & E_MSG_END; stamped = message && r.a4 != NONE;
+        if (stamped) version = __ldcg(reinterpret_cast<const float*>(S.core.arena + r.a4 + ((r.meta & E_RAW) ? (m.outp >> 2) : 0)));
       }
-    } else gather_general<false>(R, count, i0 >> 2, x4, Xg, ldx);
-    if (leader && (tid & ~31) < count) {
-      const int stale = message ? (stamped ? max(0, h.n_updates - __float_as_int(version)) : 0) : -1;
-      const unsigned same = __match_any_sync(0xffffffffu, stale);
-      if (stale >= 0 && (same & ((1u << lane) - 1u)) == 0) { atomicAdd(&S.stale_hist[min(stale, 63)], __popc(same)); atomicMax(&S.max_stale, stale); }
+      const FastDiv dd((unsigned)d4, Z.ddM);
+#pragma unroll 1
+      for (int i = tid; i < count * d4; i += CT) {
+        const int b = dd.div(i), k = i - b * d4, c = o4 + k;
+        const RowD& r = R[b];
+        if (!(r.meta & E_RAW)) { cp16(Dg + b * ldd + 4 * k, S.core.arena + r.out4 + c); continue; }
+        const float4 y = ldcg4(S.core.arena + r.a4 + c), g = rnd4(S.core.bf16, row_sum<false>(r, c));
+        *reinterpret_cast<float4*>(Dg + b * ldd + 4 * k) = make_float4(g.x * act_grad(T.act, y.x), g.y * act_grad(T.act, y.y), g.z * act_grad(T.act, y.z), g.w * act_grad(T.act, y.w));
+      }
+      if (h.flags & H_COPIES) {                                  // (a flat loop: the sums leave no registers for more)
+        const FastDiv dx((unsigned)x4, Z.dxM);
+#pragma unroll 1
+        for (int i = tid; i < count * x4; i += CT) {
+          const int b = dx.div(i), k = i - b * x4, c = i4 + k;
+          const uint4 t = *reinterpret_cast<const uint4*>(&R[b].t[0]);
+          const bool second = c >= (int)(t.w & 0xffffu);
+          cp16(Xg + b * ldx + 4 * k, S.core.arena + (second ? t.z + c - (t.w & 0xffffu) : t.x + c));
+        }
+      } else gather_general<false>(R, count, i4, x4, Xg, ldx);
+      if (tile == 0 && (tid & ~31) < count) {
+        const int stale = message ? (stamped ? max(0, h.n_updates - __float_as_int(version)) : 0) : -1;
+        const unsigned same = __match_any_sync(0xffffffffu, stale);
+        if (stale >= 0 && (same & ((1u << (tid & 31)) - 1u)) == 0) { atomicAdd(&S.stale_hist[min(stale, 63)], __popc(same)); atomicMax(&S.max_stale, stale); }
+      }
     }
     cp_wait();
     bar_compute();
     phase(2);
+    {
+      const int sN = Z.sN, sW = Z.sW, sL = Z.sL, ldd = Z.ldd, ldx = Z.ldx, w = tid >> 5, l = tid & 31, WS = CW >> sN, wr = w & ((1 << sN) - 1), wi = wr & ((1 << sW) - 1), li = l & ((1 << sL) - 1);
+      const float* const Dt = smem + Z.dg + (((wr >> sW) << (5 - sL)) + (l >> sL)) * 8; const float* const Xt = smem + Z.xg + ((wi << sL) + li) * 4;
+      const bool summing = Z.i0 == 0 && wi == 0 && li == 0;      // these lanes also add up their rows' gradients (bias)
 #pragma unroll 2
-    for (int b = ws; b < count; b += WS) {
-      const float4 da = *reinterpret_cast<const float4*>(Dg + b * ldd + ob), db = *reinterpret_cast<const float4*>(Dg + b * ldd + ob + 4);
-      const float4 x = *reinterpret_cast<const float4*>(Xg + b * ldx + ib);
-      const float d[8] = {da.x, da.y, da.z, da.w, db.x, db.y, db.z, db.w};
+      for (int b = w >> sN; b < count; b += WS) {
+        const float4 da = *reinterpret_cast<const float4*>(Dt + b * ldd), db = *reinterpret_cast<const float4*>(Dt + b * ldd + 4);
+        const float4 x = *reinterpret_cast<const float4*>(Xt + b * ldx);
+        const float d[8] = {da.x, da.y, da.z, da.w, db.x, db.y, db.z, db.w};
 #pragma unroll
-      for (int k = 0; k < 8; k++) {
-        acc[k][0] = fmaf(d[k], x.x, acc[k][0]); acc[k][1] = fmaf(d[k], x.y, acc[k][1]);
-        acc[k][2] = fmaf(d[k], x.z, acc[k][2]); acc[k][3] = fmaf(d[k], x.w, acc[k][3]);
-      }
-      if (summing) {
+        for (int k = 0; k < 8; k++) {
+          acc[k][0] = fmaf(d[k], x.x, acc[k][0]); acc[k][1] = fmaf(d[k], x.y, acc[k][1]);
+          acc[k][2] = fmaf(d[k], x.z, acc[k][2]); acc[k][3] = fmaf(d[k], x.w, acc[k][3]);
+        }
+        if (summing) {
 #pragma unroll
-        for (int k = 0; k < 8; k++) bacc[k] += d[k];
+          for (int k = 0; k < 8; k++) bacc[k] += d[k];
+        }
       }
     }
     phase(3);
-    if (h.flags & H_UPDATE) { update(h.n_upd, h.upd_t); dirty = true; updates = h.upd_t; phase(5); }
+    if (h.flags & H_UPDATE) {                                    // theta <- theta - step(A / n); the sums start over
+      const int sN = Z.sN, sW = Z.sW, sL = Z.sL, ldw = Z.ldw, WS = CW >> sN, NR = 1 << sN, WI = 1 << sW, LI = 1 << sL, sO = 5 - sL, Ro = Z.Ro;
+      float4* const r4 = reinterpret_cast<float4*>(smem + Z.red);
+      float* const bm = smem + Z.bm; float* const bred = smem + Z.bred;
+      {
+        const int w = tid >> 5, l = tid & 31, ws = w >> sN, wr = w & (NR - 1), wi = wr & (WI - 1), li = l & (LI - 1);
+        if (Z.i0 == 0 && wi == 0 && li == 0) {
+          float* const q = bred + ws * Ro + (((wr >> sW) << sO) + (l >> sL)) * 8;
+#pragma unroll
+          for (int k = 0; k < 8; k++) q[k] = bacc[k];
+        }
+        float4* const q = r4 + ((ws * 8) << (5 + sN)) + wr * 32 + l;
+#pragma unroll
+        for (int k = 0; k < 8; k++) q[k << (5 + sN)] = make_float4(acc[k][0], acc[k][1], acc[k][2], acc[k][3]);
+      }
+      bar_compute();
+      const OptStep os = opt_step(m.om, m.ov, m.opt_t0, h.n_upd, h.upd_t);
+      const int per = 256 << sN, o0 = Z.o0, i0 = Z.i0;           // sums of four columns; every thread adds up some over the slices
+#pragma unroll 1
+      for (int i = tid; i < per; i += CT) {
+        float4 a = zero4();
+#pragma unroll 4
+        for (int s = 0; s < WS; s++) a = add4(a, r4[s * per + i]);
+        const int l = i & 31, q = (i >> 5) & (NR - 1), k = i >> (5 + sN), o = (((q >> sW) << sO) + (l >> sL)) * 8 + k, c = (((q & (WI - 1)) << sL) + (l & (LI - 1))) * 4;
+        float4* const w4 = reinterpret_cast<float4*>(smem + o * ldw + c);
+        *w4 = SGD || os.opt == 0 ? sgd4(os.step, *w4, a) : opt_padded(os, m, o0 + o, i0 + c, *w4, a);
+      }
+      if (i0 == 0) {
+        const int ro = Z.ro;
+#pragma unroll 1
+        for (int i = CT - 1 - tid; i < ro; i += CT) {
+          float a = 0.f;
+#pragma unroll 4
+          for (int s = 0; s < WS; s++) a += bred[s * Ro + i];
+          const int r = real_out(m, o0 + i);
+          if (r >= 0) bm[i] = opt_one(os, bm[i], a, (size_t)m.nW + r);
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < 8; k++) {
+        bacc[k] = 0.f;
+#pragma unroll
+        for (int j = 0; j < 4; j++) acc[k][j] = 0.f;
+      }
+      bar_compute();
+      dirty = true; updates = h.upd_t;
+      phase(5);
+    }
     if (!(h.flags & H_LAST)) return;
     if (dirty) {                                                // publish: for the forward tiles, and transposed for the input-gradient tiles
       pubs++;
       dirty = false;
+      const int x4 = Z.x4, d4 = Z.d4, ro = Z.ro, o0 = Z.o0, i0 = Z.i0, ldw = Z.ldw;
+      const FastDiv dd((unsigned)d4, Z.ddM), dx((unsigned)x4, Z.dxM);
+      const float* const Wm = smem; const float* const bm = smem + Z.bm;
       float* const Wp = m.Wp + (size_t)(pubs % PUB) * m.outp * m.inp; float* const WT = m.WTp + (size_t)(pubs % PUB) * m.outp * m.inp;
 #pragma unroll 1
       for (int i = tid; i < ro * x4; i += CT) { const int o = dx.div(i), c = i - o * x4; *reinterpret_cast<float4*>(Wp + (size_t)(o0 + o) * m.inp + i0 + 4 * c) = *reinterpret_cast<const float4*>(Wm + o * ldw + 4 * c); }
@@ -1247,17 +1287,18 @@ __device__ __noinline__ void accumulate_main(const int team, const int tile, flo
           *reinterpret_cast<float4*>(t) = make_float4(a.x, b.x, e.x, f.x); *reinterpret_cast<float4*>(t + m.outp) = make_float4(a.y, b.y, e.y, f.y);
           *reinterpret_cast<float4*>(t + 2 * (size_t)m.outp) = make_float4(a.z, b.z, e.z, f.z); *reinterpret_cast<float4*>(t + 3 * (size_t)m.outp) = make_float4(a.w, b.w, e.w, f.w);
         }
-      if (biased) for (int i = tid; i < ro; i += CT) m.bp[(size_t)(pubs % PUB) * m.outp + o0 + i] = bm[i];
+      if (i0 == 0) for (int i = tid; i < ro; i += CT) m.bp[(size_t)(pubs % PUB) * m.outp + o0 + i] = bm[i];
     }
     stamp(h);
   }, Nothing(), stamp);                                         // (a round without rows: the version stays)
   if (!(end.flags & H_END)) return;
+  const int ro = Z.ro, ci = Z.ci, o0 = Z.o0, i0 = Z.i0, ldw = Z.ldw;
 #pragma unroll 1
   for (int i = tid; i < ro * ci; i += CT) {
     const int o = i / ci, c = i - o * ci, r = real_out(m, o0 + o), k = real_in(m, i0 + c);
-    if (r >= 0 && k >= 0) m.W[(size_t)r * m.in_real + k] = Wm[o * ldw + c];
+    if (r >= 0 && k >= 0) m.W[(size_t)r * m.in_real + k] = smem[o * ldw + c];
   }
-  if (biased) for (int i = tid; i < ro; i += CT) { const int r = real_out(m, o0 + i); if (r >= 0) m.b[r] = bm[i]; }
+  if (i0 == 0) for (int i = tid; i < ro; i += CT) { const int r = real_out(m, o0 + i); if (r >= 0) m.b[r] = smem[Z.bm + i]; }
 }
 
 // ---- loss head ---------------------------------------------------------------------------------------------------------------
@@ -1492,7 +1533,7 @@ __device__ __noinline__ void lookup_grad_main(const int team, const int tile, fl
       }
 #pragma unroll
       for (int u = 0; u < 4; u++) {
-        if (wide && cq[u] > 0 && os.opt == 0) {
+        if (wide && cq[u] > 0 && (SGD || os.opt == 0)) {
           *reinterpret_cast<float4*>(P.W + r0[u]) = sgd4(os.step, make_float4(w[u][0], w[u][1], w[u][2], w[u][3]), make_float4(a[u][0], a[u][1], a[u][2], a[u][3]));
           asm volatile("st.relaxed.gpu.global.v4.f32 [%0], {%1, %1, %1, %1};" :: "l"(P.A + r0[u]), "f"(0.f) : "memory");
           continue;
@@ -1659,9 +1700,12 @@ cudaError_t launch(const Run* run, int n_ctas, size_t smem, cudaStream_t st) {
 }
 }  // namespace ENGINE_NAMESPACE
 
-#ifndef WAVE_FORWARD
+#if !defined(WAVE_FORWARD) && !defined(WAVE_MOMENTS)
 namespace forward { cudaError_t launch(const Run* run, int n_ctas, size_t smem, cudaStream_t st); }      // wave_forward.cu
-cudaError_t launch(const Run* run, int n_ctas, size_t smem, cudaStream_t st) { return run->core.eval ? forward::launch(run, n_ctas, smem, st) : training::launch(run, n_ctas, smem, st); }
+namespace moments { cudaError_t launch(const Run* run, int n_ctas, size_t smem, cudaStream_t st); }      // wave_moments.cu
+cudaError_t launch(const Run* run, int n_ctas, size_t smem, cudaStream_t st) {
+  return run->core.eval ? forward::launch(run, n_ctas, smem, st) : run->core.opt ? moments::launch(run, n_ctas, smem, st) : training::launch(run, n_ctas, smem, st);
+}
 using namespace training;
 size_t smem_bytes(const Team& t, const Mat& m, int mak) {
   const size_t head = slots_bytes(mak) + 2 * (size_t)t.BM * sizeof(RowD);
