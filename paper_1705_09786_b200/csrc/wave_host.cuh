@@ -393,7 +393,7 @@ static bool wave_best(const WaveModel& M, int c, int ctas, double rows, double m
             if (x.T > ctas) continue;
             x.n = x.T;
             const double area = (double)x.R * x.C;
-            offer(x, 4500 + rows * (36 + 0.23 * (std::min(x.R, m.outp) + std::min(x.C, m.inp)) + area / (area < 4096 ? 46 : 59)) + upd * 3000 + std::min(1.0, upd) * area / 5);
+            offer(x, 4000 + rows * (24 + 0.23 * (std::min(x.R, m.outp) + std::min(x.C, m.inp)) + area / (area < 4096 ? 46 : 59)) + upd * 2200 + std::min(1.0, upd) * area / 5);
           }
       break;
     case HEAD:
