@@ -281,7 +281,7 @@ __device__ __noinline__ void helper_main(const int cta, const int tile, const in
       quota -= admitted;
       bar_helper();
     }
-    // ---- rows of this cell in this round ------------------------------------------------------------------------------
+    // ---- the cell's rows of the coming round ------------------------------------------------------------------------------
     int N = 0;
     bool fin = false;
     active = 0;
@@ -381,7 +381,7 @@ __device__ __noinline__ void helper_main(const int cta, const int tile, const in
       if (last) break;
     } while (true);
     round++;
-    bar_helper();                                                 // (the slot tables of this round are used up)
+    bar_helper();                                                 // (the slot tables are used up)
   }
   // ---- the end: the leftover gradients are applied once more --------------------------------------------------------------
   int n_upd = 0;
