@@ -64,7 +64,7 @@ struct Shared {
   Head hd[2];
   unsigned long long full[2], empty[2], tc_mbar;
   unsigned tmem;
-  int stop, ok, ok2;
+  int stop, ok, ok2, helper_ok[2];
   unsigned long long ver;                      // what the ACC team had published `lag` rounds ago: updates << 32 | publications << 16 | round
   int warp_sum[4], sel;
   unsigned long long batches, batch_rows, msgs, tc_batches;
@@ -225,6 +225,14 @@ __device__ __forceinline__ int helper_scan(const int v, int& total) {          /
   return s - v + (warp > 0 ? a : 0) + (warp > 1 ? b : 0) + (warp > 2 ? c : 0);
 }
 
+// One helper warp waits until the compute warps have used a chunk buffer up; the others learn the outcome behind the next barrier.
+// (No thread may give up on its own: the ones that saw the buffer free would wait for it at their next counted barrier for good.
+// Two words, by buffer: the next chunk's outcome is written while slow warps may still read this one's.)
+__device__ __forceinline__ void buffer_free(const int buf, const unsigned parity, const unsigned long long t0, const int where) {
+  const bool ok = __all_sync(0xffffffffu, mbar_wait(&S.empty[buf], parity, t0, where));
+  if ((threadIdx.x & 31) == 0) S.helper_ok[buf] = ok;
+}
+
 __device__ __noinline__ void helper_main(const int cta, const int tile, const int shard, unsigned char* smem, const unsigned long long t0) {
   IN_SMEM(smem);
   const int ht = threadIdx.x - CT;
@@ -356,9 +364,10 @@ __device__ __noinline__ void helper_main(const int cta, const int tile, const in
         copies = !(e.meta & (E_OVERFLOW | E_DENSE | E_RAW)) && e.t[0].col4 == 0 && (one || two);
         if (one) e.t[1].col4 = 0xffff;
       }
+      if (ht < 32) buffer_free(buf, parity, t0, 21);
       copies = !bar_helper_or(!copies);
+      if (!S.helper_ok[buf]) return;
       const bool over = !copies && bar_helper_or(ht < cnt && (e.meta & E_OVERFLOW));
-      if (!mbar_wait(&S.empty[buf], parity, t0, 21)) return;
       if (ht < cnt) {
         RowD& r = rows[buf * BM + ht];
         const unsigned nt = e.meta & E_NT, nx = (e.meta & E_OVERFLOW) ? 0u : kind == LIN_F && T.lstm ? nt + (e.meta >> 16) : nt;
@@ -389,7 +398,9 @@ __device__ __noinline__ void helper_main(const int cta, const int tile, const in
     n_upd = n_acc; n_updates++; n_grads += n_upd;
     if (leader && ht == 0 && n_updates <= S.ppt.log_cap) S.ppt.update_log[n_updates - 1] = n_upd;
   }
-  if (!mbar_wait(&S.empty[buf], parity, t0, 22)) return;
+  if (ht < 32) buffer_free(buf, parity, t0, 22);
+  bar_helper();
+  if (!S.helper_ok[buf]) return;
   publish(0, H_END | (n_upd ? H_UPDATE : 0), n_upd);
   // ---- statistics ----------------------------------------------------------------------------------------------------------
   PPTStats& st = *S.ppt.stats;
@@ -455,17 +466,23 @@ __device__ __forceinline__ Head chunk_loop(RowD* rows, const int team, const uns
   const bool T_publishes = S.team.kind == ACC;
   unsigned parity = 0;
   for (int buf = 0;;) {
-    if (!mbar_wait(&S.full[buf], parity, t0, 25)) break;
+    // Whether the run goes on is warp 0's word, read behind a barrier: a warp that left alone would leave the others at their next one.
+    const bool mine = mbar_wait(&S.full[buf], parity, t0, 25);
     phase(0);
-    const Head h = S.hd[buf];
+    Head h = S.hd[buf];                                            // (complete if this thread saw the phase; otherwise read again below)
+    if (warp == 0) {
+      int r = __all_sync(0xffffffffu, mine) ? 2 : 0;
+      if (r && (h.flags & H_FIRST)) r = wait_round(h.round, h.count > 0, true, t0);
+      if ((tid & 31) == 0) S.ok = r;
+    }
+    bar_compute();
+    int ok = S.ok;
+    if (!ok) break;
+    if (!mine) h = S.hd[buf];
     const bool end = h.flags & H_END;
     if (end && !(h.flags & H_UPDATE)) return h;
     const bool last = h.flags & H_LAST, any = h.count > 0;
     if (h.flags & H_FIRST) {
-      if (warp == 0) { const int r = wait_round(h.round, any, true, t0); if ((tid & 31) == 0) S.ok = r; }
-      bar_compute();
-      int ok = S.ok;
-      if (!ok) break;
       if (any) fresh(S.ver);
       if (ok == 1) {
         if (warp == 0) { const int r = wait_round(h.round, any, false, t0); __syncwarp(); if ((tid & 31) == 0) S.ok2 = r; }

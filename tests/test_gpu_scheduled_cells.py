@@ -62,3 +62,28 @@ def test_epochs_of_one_update_match_oracle(oracle_mod, family, size, n, mak, lr,
             assert np.abs(ep[k] - op[k]).max() <= (1 + epoch) * 1e-4 * np.abs(op[k]).max(), (epoch, g.names[k[0]], k[1])
     np.testing.assert_allclose(e.eval(split=1, mak=mak)[2], o.eval(split=1)[2], rtol=3e-5, atol=6e-6)
     e.close()
+
+
+@pytest.mark.parametrize("family,size,n,mak,bf16", [("mlp", (61, 258, 7), 400, 16, False), ("tree", (60, 36, 21, 5), 150, 64, False),
+                                                    ("tree", (500, 64, 64, 5), 60, 32, True), ("ggnn", (15, 25, 3), 150, 64, False)])
+def test_runs_that_give_up_end_and_leave_the_handle_usable(family, size, n, mak, bf16):
+    """Time budgets that run out at different points of an epoch: the call returns (AMPNET_ETIMEOUT, or a result if the epoch was
+    faster), whichever of a CTA's warps were waiting for each other, and the next epoch on the handle is complete."""
+    import paper_1705_09786_b200 as amp
+    g, inst = _case(family, size, n)
+    p = wp.init_params(g)
+    e = amp.Engine(g, payload_bf16=bf16)
+    e.load_instances(inst)
+    gave_up = 0
+    for budget in (5e-6, 2e-5, 5e-5, 1e-4, 2e-4, 4e-4, 8e-4):
+        e.set_params(p)
+        try:
+            e.run_epoch(mak=mak, muf=20, lr=1e-4, timeout_s=budget)
+        except amp.AmpnetError as err:
+            assert err.status == 4
+            gave_up += 1
+    assert gave_up >= 1
+    e.set_params(p)
+    st, loss = e.run_epoch(mak=mak, muf=20, lr=1e-4, timeout_s=60)
+    assert st.instances == inst.n and np.isfinite(loss).all()
+    e.close()
