@@ -16,6 +16,7 @@
 #include "../../include/ampnet.h"
 #include "engine.cuh"
 #include "wave.h"
+#include "wave_sizes.h"
 
 using namespace amp;
 

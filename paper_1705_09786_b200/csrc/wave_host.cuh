@@ -162,51 +162,6 @@ static bool wave_model(const std::vector<DevNode>& nodes, const std::vector<int>
   return true;
 }
 
-// Sizes that depend on the loaded data: key spaces, scratch of an encoding warp.
-static void wave_sizes(WaveModel& M, const std::vector<DevNode>& nodes, const HostDataset& D) {
-  using namespace wave;
-  EncModel& E = M.enc;
-  unsigned long long w = 0, rows = 64, front = 64;
-  const unsigned long long IT = E.IT;
-  for (int i = 0; i < E.n_nodes; i++) {
-    const DevNode& h = nodes[i];
-    EncNode& N = E.nodes[i];
-    N.U = h.U_in; N.J = 0;
-    bool counted = true;
-    switch (h.type) {
-      case CONCAT: N.U = h.U_out; N.J = h.fn_arg; break;
-      case BCAST: case SPLIT: N.J = h.fn_arg; break;
-      case GROUP: N.U = h.U_out; N.J = h.rows_out; break;
-      case UNGROUP: N.J = h.rows_in; break;
-      case FLATMAP: N.J = D.maxOut; break;
-      case NPT_LSTM: N.J = 2; break;
-      case PHI: case NPT_SUMROWS: break;
-      default: counted = false;
-    }
-    const unsigned long long keys = IT * N.U;
-    N.ref_off = (unsigned)w; w += keys * N.J;
-    N.cnt_off = (unsigned)w; if (counted) w += keys;
-    rows += IT * std::max((unsigned long long)h.U_in * h.rows_in, (unsigned long long)h.U_out * h.rows_out) * (2 + std::max(h.n_succ, h.n_pred));
-    if (h.ppt >= 0) { EncPpt& P = E.ppts[h.ppt]; P.U = h.U_in; P.save_off = (unsigned)w; w += keys * 3; front += 3ull * h.U_in; }
-  }
-  E.table_words = (unsigned)((w + 3) & ~3ull);
-  bool forks = false;
-  for (int i = 0; i < E.n_nodes; i++) forks |= nodes[i].type == UNGROUP || nodes[i].type == GROUP || nodes[i].type == FLATMAP;
-  E.stack_cap = forks ? 1024 : 256;
-  E.front_cap = (unsigned)front; E.row_cap = (unsigned)rows; E.term_cap = (unsigned)(3 * rows);
-  unsigned long long messages = 4;
-  for (int c = 0; c < E.n_cells; c++) E.bound[c] = 0;
-  for (int p = 0; p < E.n_ppts; p++) {
-    const DevNode& h = nodes[E.ppts[p].node];
-    const unsigned long long b = IT * h.U_in * h.rows_in;
-    for (int k = 0; k < 6; k++) if (E.ppts[p].cell[k] >= 0) E.bound[E.ppts[p].cell[k]] = (unsigned)std::min<unsigned long long>(b, 1u << 30);
-    messages += 2 * IT * h.U_in;
-  }
-  E.steps_cap = (unsigned)std::min<unsigned long long>(messages + 4, 60000);
-  E.scratch_words = (unsigned)(((unsigned long long)E.table_words + 12ull * front + 6ull * rows + 2ull * rows + 31) & ~31ull);
-  E.near_scratch = (size_t)E.scratch_words * 4 + E.stack_cap * 16 <= 100 * 1024;
-}
-
 // ---- encoding of a loaded split (at the end of ampnet_load_instances) -------------------------------------------------------
 
 static ampnet_status_t wave_encode(ampnet_graph* g, HostDataset& D, WaveModel& M, WaveData& W, void** scratch, size_t* scratch_cap) {
@@ -214,9 +169,7 @@ static ampnet_status_t wave_encode(ampnet_graph* g, HostDataset& D, WaveModel& M
   W = WaveData{};
   const long long n = D.n;
   if (!M.ok || n < 1 || n > (1ll << 30)) return AMPNET_OK;
-  wave_sizes(M, g->hnodes, D);
-  for (auto& h : g->hnodes) if (h.U_in > 65535 || h.U_out > 65535) return AMPNET_OK;      // (positions travel in sixteen bits)
-  if ((unsigned long long)M.enc.scratch_words * 4 > (1ull << 30)) return AMPNET_OK;
+  if (!encoder_sizes(M.enc, g->hnodes, D.maxOut)) return AMPNET_OK;
   // Warps per block: with the scratch in shared memory as many as fit there.  An instance is one long chain of dependent steps, so a large
   // split wants warps more than it wants near memory (an SM holds 16 by registers): 20,000 lists of 26 KB scratch 8.5 -> 4.8 ms.
   const size_t warp_bytes = (size_t)M.enc.scratch_words * 4, near_bytes = warp_bytes + M.enc.stack_cap * 16;
