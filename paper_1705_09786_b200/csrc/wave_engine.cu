@@ -360,7 +360,8 @@ __device__ __noinline__ void helper_main(const int cta, const int tile, const in
       bool copies = true;
       if (ht < cnt) {
         const unsigned nt = e.meta & E_NT, all = (unsigned)T.k4;
-        const bool one = nt == 1 && e.t[0].w4 == all, two = nt == 2 && e.t[1].col4 == e.t[0].w4 && e.t[0].w4 + e.t[1].w4 == (int)all;
+        // (the second term of a single copy is free to say so, unless the children's cells of an LSTM gate row begin there)
+        const bool one = nt == 1 && e.t[0].w4 == all && (e.meta >> 16) == 0, two = nt == 2 && e.t[1].col4 == e.t[0].w4 && e.t[0].w4 + e.t[1].w4 == (int)all;
         copies = !(e.meta & (E_OVERFLOW | E_DENSE | E_RAW)) && e.t[0].col4 == 0 && (one || two);
         if (one) e.t[1].col4 = 0xffff;
       }

@@ -87,3 +87,36 @@ def test_runs_that_give_up_end_and_leave_the_handle_usable(family, size, n, mak,
     st, loss = e.run_epoch(mak=mak, muf=20, lr=1e-4, timeout_s=60)
     assert st.instances == inst.n and np.isfinite(loss).all()
     e.close()
+
+
+def _epochs_match(oracle_mod, g, inst, mak, lr, payload_bf16=False, loss_rtol=1e-5, loss_atol=2e-6, param_rtol=1e-4, param_floor=1e-30):
+    """Two epochs whose only update is their flush, then an evaluation, against the oracle; the engine comes back open."""
+    import paper_1705_09786_b200 as amp
+    p = wp.init_params(g)
+    o, e = oracle_mod.Oracle(g, payload_bf16=payload_bf16), amp.Engine(g, payload_bf16=payload_bf16)
+    for s in (o, e):
+        s.load_instances(inst)
+        s.load_instances(inst, split=1)
+        s.set_params(p)
+    for epoch in range(2):
+        _, oloss = o.run_epoch(mak=1, muf=1 << 30, lr=lr)
+        _, eloss = e.run_epoch(mak=mak, muf=1 << 30, lr=lr, timeout_s=60)
+        np.testing.assert_allclose(eloss, oloss, rtol=(1 + epoch) * loss_rtol, atol=(1 + epoch) * loss_atol)
+        ep, op = e.get_params(), o.get_params()
+        for k in op:
+            assert np.abs(ep[k] - op[k]).max() <= (1 + epoch) * param_rtol * max(np.abs(op[k]).max(), param_floor), (epoch, g.names[k[0]], k[1])
+    np.testing.assert_allclose(e.eval(split=1, mak=mak)[2], o.eval(split=1)[2], rtol=3 * loss_rtol, atol=3 * loss_atol)
+    return e
+
+
+@pytest.mark.parametrize("width", [20, 37])
+def test_branch_gates_fed_by_one_copy_match_oracle(oracle_mod, width):
+    """A Linear between the children's Concat and the branch gates: the gates' input is a single row, behind which the row's
+    descriptor holds the children's cells."""
+    g = ir.tree_lstm(60, 36, 20, 5)
+    cat, gates = g.index("concat_h"), g.index("branch_gates")
+    g._nodes[gates] = (ir.LINEAR, width, 5 * 20) + g._nodes[gates][3:]
+    mix = g.node("mix", ir.LINEAR, 2 * 20, width, act=ir.ACT_TANH)
+    g._edges = [(s, sp, mix if s == cat else d, dp) for s, sp, d, dp in g._edges]
+    g.edge(mix, gates)
+    _epochs_match(oracle_mod, g, data.tree_instances(n=40, vocab=60), 16, 0.02).close()
