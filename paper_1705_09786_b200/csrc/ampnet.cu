@@ -581,6 +581,8 @@ ampnet_status_t place(ampnet_graph* g, int n_ctas, int max_batch_rows, std::vect
   return AMPNET_OK;
 }
 
+bool single_row_graph(ampnet_graph* g, const HostDataset& D);
+
 #include "wave_host.cuh"
 
 // ---- direct-delivery engine: which graphs it takes, and its placement -------------------------------------
@@ -592,6 +594,9 @@ bool direct_candidate(ampnet_graph* g, const HostDataset& D, int det) {
   if (det) return false;
   if (const char* e = getenv("AMPNET_ENGINE")) if (!strcmp(e, "classic")) return false;
   if (const char* e = getenv("AMPNET_TUNE")) if (atoi(e) & (16 | 32 | 8)) return false;
+  return single_row_graph(g, D);
+}
+bool single_row_graph(ampnet_graph* g, const HostDataset& D) {
   if (D.kind == 3) return false;
   const int n = (int)g->hnodes.size();
   int max_nodes = 0, max_ppts = 0, max_landings = 0, batch_rows = 0;

@@ -155,7 +155,7 @@ struct WaveModel {
   std::vector<unsigned> fwd_mask, bwd_mask;      // per parameterised node: cells that produce its input / its gradient
 };
 struct WaveData {
-  bool ok = false;
+  bool ok = false, tc = false;         // tc: forward products may run on the tensor cores
   long long load_id = 0;
   Program prog{};
   EncTotals tot{};

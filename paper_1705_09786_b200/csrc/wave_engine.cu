@@ -881,7 +881,10 @@ __device__ __noinline__ void forward_main(const int team, const int tile, float*
               const uint4 t = *reinterpret_cast<const uint4*>(&R[r].t[0]);
               const int cut = (int)(t.w & 0xffffu);
               a[u] = ldcg4(S.core.arena + (c >= cut ? t.z + (c - cut) : t.x + c)); b[u] = ldcg4(S.core.arena + (c + 1 >= cut ? t.z + (c + 1 - cut) : t.x + c + 1));
-            } else { const int nt = R[r].meta & E_NT; a[u] = term4(R[r], 0, nt, c); b[u] = term4(R[r], 0, nt, c + 1); }
+            } else if (R[r].meta & E_DENSE) {                   // (a dense row of K values, K a multiple of sixteen)
+              const float4* const x = reinterpret_cast<const float4*>(S.core.dense + (long long)(R[r].inst & 0x7fffffff) * K) + c;
+              a[u] = __ldg(x); b[u] = __ldg(x + 1);
+            } else { a[u] = row_sum<false>(R[r], c); b[u] = row_sum<false>(R[r], c + 1); }
           }
 #pragma unroll
           for (int u = 0; u < U; u++) {

@@ -168,6 +168,7 @@ static ampnet_status_t wave_encode(ampnet_graph* g, HostDataset& D, WaveModel& M
   using namespace wave;
   W = WaveData{};
   const long long n = D.n;
+  W.tc = g->payload_bf16 && single_row_graph(g, D);
   if (!M.ok || n < 1 || n > (1ll << 30)) return AMPNET_OK;
   if (!encoder_sizes(M.enc, g->hnodes, D.maxOut)) return AMPNET_OK;
   // Warps per block: with the scratch in shared memory as many as fit there.  An instance is one long chain of dependent steps, so a large
@@ -263,7 +264,7 @@ static ampnet_status_t wave_encode(ampnet_graph* g, HostDataset& D, WaveModel& M
 // nothing gains.  The estimate (in cycles) counts the latency of a gather, its bytes, the multiply-adds at the rate the
 // products reach, the reload of updated weights and, for accumulators, the merge at updates.
 
-static bool wave_best(const WaveModel& M, int c, int ctas, double rows, double msgs_per_update, bool eval, size_t budget, int mak, bool bf16, bool use_tc, const ampnet_graph* g, WaveTeam& best) {
+static bool wave_best(const WaveModel& M, int c, int ctas, double rows, double msgs_per_update, bool eval, size_t budget, int mak, bool use_tc, const ampnet_graph* g, WaveTeam& best) {
   using namespace wave;
   const WaveCell& K = M.cells[c];
   const EncPpt& P = M.enc.ppts[K.ppt];
@@ -299,7 +300,9 @@ static bool wave_best(const WaveModel& M, int c, int ctas, double rows, double m
     case LIN_F: case GRU_ZR: case GRU_C: {
       t.G = K.kind == GRU_ZR ? 2 : t.lstm ? t.lstm : 1;
       const int gw = 4 * t.H4;
-      const bool tc = bf16 && use_tc && K.kind == LIN_F && !t.lstm && h.out_dim % 64 == 0 && h.in_dim % 16 == 0 && m.inp == h.in_dim;
+      // Tensor cores, whose operands are bfloat16: where the payloads are, and only in graphs of single-row messages; the others (graph nets,
+      // grouped leaves, gates) keep their weights in 32 bits.  A summed input is kept for the accumulator by the other variant alone.
+      const bool tc = use_tc && K.kind == LIN_F && !t.lstm && !t.keep && h.out_dim % 64 == 0 && h.in_dim % 16 == 0 && m.inp == h.in_dim;
       for (int T = 1; T <= std::min(ctas, gw / 4); T++) {
         Team x = t;
         x.R = tc ? 64 : pad4i((gw + T - 1) / T);
@@ -394,8 +397,8 @@ static WavePlan wave_place(const ampnet_graph* g, const WaveModel& M, const Wave
   if ((unsigned long long)mak * P.copies * (W.tot.arena4_max + 8ull) > 0xf0000000ull) return P;      // (offsets are 32 bits of 16 bytes)
   static const size_t fixed = static_smem();
   const size_t budget = (size_t)g->max_smem - fixed - 1024;
-  bool use_tc = true;
-  if (const char* e = getenv("AMPNET_TENSOR_CORES")) use_tc = atoi(e) != 0;
+  bool use_tc = W.tc;
+  if (const char* e = getenv("AMPNET_TENSOR_CORES")) use_tc &= atoi(e) != 0;
   const double steps = (double)(eval ? W.tot.steps_eval_sum : W.tot.steps_sum);
   const double keys = (double)std::max<long long>(1, std::min<long long>(mak, n_order));
   std::vector<int> cells;
@@ -405,7 +408,7 @@ static WavePlan wave_place(const ampnet_graph* g, const WaveModel& M, const Wave
   P.teams.resize(nc);
   auto rows_of = [&](int c) { return keys * W.tot.entries[c] / std::max(1.0, steps); };
   auto muf_of = [&](int c) { const int o = g->nodes[M.enc.ppts[M.cells[c].ppt].node].muf_override; return (double)(o > 0 ? o : muf); };
-  auto best = [&](int k, int n, WaveTeam& t) { return wave_best(M, cells[k], n, rows_of(cells[k]), muf_of(cells[k]), eval, budget, mak, g->payload_bf16, use_tc, g, t); };
+  auto best = [&](int k, int n, WaveTeam& t) { return wave_best(M, cells[k], n, rows_of(cells[k]), muf_of(cells[k]), eval, budget, mak, use_tc, g, t); };
   int used = 0;
   for (int k = 0; k < nc; k++) {
     int n = 1;

@@ -120,3 +120,41 @@ def test_branch_gates_fed_by_one_copy_match_oracle(oracle_mod, width):
     g._edges = [(s, sp, mix if s == cat else d, dp) for s, sp, d, dp in g._edges]
     g.edge(mix, gates)
     _epochs_match(oracle_mod, g, data.tree_instances(n=40, vocab=60), 16, 0.02).close()
+
+
+# bf16 runs at sizes the tensor-core tiles take (outputs a multiple of 64, inputs of 16): dense rows, copies, and the graphs whose weights
+# stay in 32 bits (messages that land at more than two places, matrix messages, gates)
+BF16_CASES = [("mlp", (64, 128, 64, 10), 1200, 1024, 0.05, ("linear1", "linear2")), ("mlp", (784, 256, 10), 90, 4, 0.05, ()),
+              ("rnn", (14, 64, 64, 10), 1200, 1024, 0.02, ("linear1",)), ("concat", (32, 64, 5), 200, 64, 0.02, ()),
+              ("ggnn", (15, 64, 3), 60, 33, 1e-5, ()), ("tree_lstm", (60, 64, 64, 5), 30, 16, 0.02, ())]
+
+
+def _wide_concat(dim, width, classes):
+    """A dense row through one Linear and a Bcast into the five parts of a Concat."""
+    g = ir.IRGraph("concat")
+    src = g.node("src", ir.SOURCE, out_dim=dim, fn=ir.SRC_DENSE_ROW)
+    first = g.node("first", ir.LINEAR, dim, 16, act=ir.ACT_TANH, flags=ir.FLAG_SOURCE_ADJACENT)
+    bc = g.node("bcast", ir.BCAST, 16, 16, fn_arg=5)
+    cat = g.node("concat", ir.CONCAT, 16, 80, fn=ir.CONCAT_BY_EDGE, fn_arg=5)
+    mix = g.node("mix", ir.LINEAR, 80, width, act=ir.ACT_TANH)
+    head = g.node("head", ir.LINEAR, width, classes)
+    loss = g.node("loss", ir.LOSS_CE, classes, 0, fn=ir.LABEL_PER_INSTANCE)
+    g.edge(src, first)
+    g.edge(first, bc)
+    for k in range(5):
+        g.edge(bc, cat, k, k)
+    g.edge(cat, mix)
+    g.edge(mix, head)
+    g.edge(head, loss)
+    return g
+
+
+@pytest.mark.parametrize("family,size,n,mak,lr,tensor", BF16_CASES)
+def test_bf16_epochs_at_tensor_core_sizes_match_oracle(oracle_mod, family, size, n, mak, lr, tensor):
+    """Asynchronous bf16 training and evaluation; the tolerances are the ones the oracle's own rounding gap gives (test_oracle_pins.py).
+    With many keys, evaluation has more than four rows a round and a tile: the nodes named must have run on the tensor cores, and no other."""
+    from test_oracle_pins import BF16_TOL
+    g, inst = (_wide_concat(*size), data.mlp_instances(n=n, dim=size[0], classes=size[-1])) if family == "concat" else _case(family, size, n)
+    e = _epochs_match(oracle_mod, g, inst, mak, lr, payload_bf16=True, **BF16_TOL)
+    assert tuple(g.names[i] for i in g.ppt_nodes() if e.micro_batch_split(i)[1] > 0) == tensor
+    e.close()
