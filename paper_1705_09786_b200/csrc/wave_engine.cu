@@ -842,10 +842,8 @@ __device__ __noinline__ void forward_main(const int team, const int tile, float*
   unsigned char *const Wb = reinterpret_cast<unsigned char*>(Ws), *const Xb = reinterpret_cast<unsigned char*>(Xs);
   unsigned have = 0;
   const FastDiv dj4(max(jn >> 2, 1));
-  auto fill_w = [&](const unsigned pub) {
-    const float* W = pub ? m.Wp + (size_t)(pub % PUB) * m.outp * m.inp : m.W;        // (the sizes of a tensor-core node need no padding)
+  auto fill_w = [&](const float* W, const float* b) {              // (the sizes of a tensor-core node need no padding)
     tc::fill_operand(Wb, nB, K, [&](const int r) { return W + (size_t)(j0 + r) * K; }, tid, CT);
-    const float* b = pub ? m.bp + (size_t)(pub % PUB) * m.outp : m.b;
 #pragma unroll 1
     for (int i = tid; i < nB; i += CT) bs[i] = __ldcg(b + j0 + i);
     tc::fence_operands();
@@ -856,7 +854,7 @@ __device__ __noinline__ void forward_main(const int team, const int tile, float*
 #pragma unroll 1
     for (size_t i = tid; i < x_floats; i += CT) Xs[i] = 0.f;
     bar_compute();
-    fill_w(0);
+    fill_w(m.W, m.b);                                              // version 0, which no publication number stands for: they wrap at 2^16
   } else first_rows(m, G, gw, j0, jn, Ws, ld, bs);
   unsigned tc_parity = 0;
   bar_compute();
@@ -1004,7 +1002,7 @@ __device__ __noinline__ void forward_main(const int team, const int tile, float*
     const unsigned pub = pub_of(ver);
     if (pub == have) return;
     have = pub;
-    if (tcm) fill_w(pub); else load_rows(m, pub, G, gw, j0, jn, Ws, ld, bs);
+    if (tcm) fill_w(m.Wp + (size_t)(pub % PUB) * m.outp * m.inp, m.bp + (size_t)(pub % PUB) * m.outp); else load_rows(m, pub, G, gw, j0, jn, Ws, ld, bs);
   });
 }
 
