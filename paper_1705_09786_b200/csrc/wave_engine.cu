@@ -356,12 +356,12 @@ __device__ __noinline__ void helper_main(const int cta, const int tile, const in
         n_upd = n_acc; n_acc = 0; n_updates++; n_grads += n_upd;
         if (leader && ht == 0 && n_updates <= S.ppt.log_cap) S.ppt.update_log[n_updates - 1] = n_upd;
       }
-      // every row one copy of the whole width, or two side by side?
+      // every row one copy of the whole width, or two side by side?  (embedding gradients are added a column at a time: one copy, or a sum)
       bool copies = true;
       if (ht < cnt) {
         const unsigned nt = e.meta & E_NT, all = (unsigned)T.k4;
         // (the second term of a single copy is free to say so, unless the children's cells of an LSTM gate row begin there)
-        const bool one = nt == 1 && e.t[0].w4 == all && (e.meta >> 16) == 0, two = nt == 2 && e.t[1].col4 == e.t[0].w4 && e.t[0].w4 + e.t[1].w4 == (int)all;
+        const bool one = nt == 1 && e.t[0].w4 == all && (e.meta >> 16) == 0, two = kind != LOOKUP_B && nt == 2 && e.t[1].col4 == e.t[0].w4 && e.t[0].w4 + e.t[1].w4 == (int)all;
         copies = !(e.meta & (E_OVERFLOW | E_DENSE | E_RAW)) && e.t[0].col4 == 0 && (one || two);
         if (one) e.t[1].col4 = 0xffff;
       }

@@ -180,3 +180,25 @@ def test_published_weights_are_read_past_the_sixteen_bits_of_their_count():
     assert e.node_stats(g.index("linear1"))["n_updates"] == n
     assert loss[2000:].max() < 0.01, np.argmax(loss[2000:]) + 2000
     e.close()
+
+
+@pytest.mark.parametrize("vocab,width,bf16", [(14, 12, False), (5000, 68, False), (5000, 4, True)])
+def test_split_embedding_rows_match_oracle(oracle_mod, vocab, width, bf16):
+    """A Split behind the Lookup: the gradient of an embedding row is two copies side by side, for a table whose sums fit in shared memory
+    and for ones dealt to tiles."""
+    from test_oracle_pins import BF16_TOL
+    g = ir.IRGraph("split_rows")
+    src = g.node("src", ir.SOURCE, fn=ir.SRC_TOKENS)
+    look = g.node("lookup", ir.LOOKUP, vocab, 2 * width, flags=ir.FLAG_SOURCE_ADJACENT)
+    sp = g.node("split", ir.SPLIT, 2 * width, width, fn_arg=2)
+    g.edge(src, look)
+    g.edge(look, sp)
+    for k in range(2):
+        head = g.node(f"head{k}", ir.LINEAR, width, 5)
+        loss = g.node(f"loss{k}", ir.LOSS_CE, 5, 0, fn=ir.LABEL_PER_INSTANCE)
+        g.edge(sp, head, k, 0)
+        g.edge(head, loss)
+    n, rng = 90, np.random.default_rng(7)
+    inst = data.Instances(ir.KIND_SEQUENCES, n)                     # one token each: one loss per head
+    inst.offsets, inst.tokens, inst.labels_i = np.arange(n + 1), rng.integers(0, min(vocab, 40), n), rng.integers(0, 5, n)
+    _epochs_match(oracle_mod, g, inst.finalize(), 32, 0.5, payload_bf16=bf16, **(BF16_TOL if bf16 else {})).close()
