@@ -202,3 +202,35 @@ def test_split_embedding_rows_match_oracle(oracle_mod, vocab, width, bf16):
     inst = data.Instances(ir.KIND_SEQUENCES, n)                     # one token each: one loss per head
     inst.offsets, inst.tokens, inst.labels_i = np.arange(n + 1), rng.integers(0, min(vocab, 40), n), rng.integers(0, 5, n)
     _epochs_match(oracle_mod, g, inst.finalize(), 32, 0.5, payload_bf16=bf16, **(BF16_TOL if bf16 else {})).close()
+
+
+@pytest.mark.parametrize("vocab,width,muf", [(14, 256, 3), (14, 512, 40), (3000, 256, 2), (3000, 512, 30)])
+def test_embedding_rows_are_read_whole(vocab, width, muf):
+    """Every column of an embedding row, and of the weights of the layer behind it, starts with the same value and gets the same gradient
+    in the same order, so at every version they are the same bits.  A message that took a part of a row before and a part after an update
+    would leave columns of the layer's weights different for good."""
+    import paper_1705_09786_b200 as amp
+    g = ir.IRGraph("rows")
+    src = g.node("src", ir.SOURCE, fn=ir.SRC_TOKENS)
+    look = g.node("lookup", ir.LOOKUP, vocab, width, flags=ir.FLAG_SOURCE_ADJACENT)
+    head = g.node("head", ir.LINEAR, width, 5)
+    loss = g.node("loss", ir.LOSS_CE, 5, 0, fn=ir.LABEL_PER_INSTANCE)
+    g.edge(src, look)
+    g.edge(look, head)
+    g.edge(head, loss)
+    n, rng = 6000, np.random.default_rng(8)
+    inst = data.Instances(ir.KIND_SEQUENCES, n)
+    inst.offsets, inst.tokens, inst.labels_i = np.arange(n + 1), rng.integers(0, 6, n), rng.integers(0, 5, n)
+    p = wp.init_params(g)
+    for k in ((look, 0), (head, 0)):
+        p[k] = np.repeat(p[k][:, :1], width, axis=1)
+    e = amp.Engine(g)
+    e.load_instances(inst.finalize())
+    e.set_params(p)
+    _, losses = e.run_epoch(mak=64, muf=muf, lr=0.01, timeout_s=60)
+    assert np.isfinite(losses).all() and e.node_stats(look)["n_updates"] >= n // muf // 2
+    after = e.get_params()
+    for k in ((look, 0), (head, 0)):
+        assert np.abs(after[k][:6] - p[k][:6]).max() > 0
+        np.testing.assert_array_equal(after[k], np.repeat(after[k][:, :1], width, axis=1))
+    e.close()
