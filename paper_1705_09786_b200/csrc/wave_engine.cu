@@ -64,7 +64,7 @@ struct Shared {
   Head hd[2];
   unsigned long long full[2], empty[2], tc_mbar;
   unsigned tmem;
-  int stop, ok, ok2, helper_ok[2];
+  int stop, helper_stop, ok, ok2;
   unsigned long long ver;                      // what the ACC team had published `lag` rounds ago: updates << 32 | publications << 16 | round
   int warp_sum[4], sel;
   unsigned long long batches, batch_rows, msgs, tc_batches;
@@ -113,12 +113,25 @@ __device__ __forceinline__ bool over(const unsigned long long t0, int where) {
   fail(S.core.g, ST_TIMEOUT, S.ppt.node, where);
   return true;
 }
-// Waits for a phase of a shared-memory barrier; false when the run is being aborted.
+// Waits for a phase of a shared-memory barrier that hardware completes; false when the run is being aborted.
 __device__ __forceinline__ bool mbar_wait(unsigned long long* b, unsigned parity, const unsigned long long t0, int where) {
   for (unsigned it = 1;; it++) {
     if (mbar_try(b, parity)) return true;
-    if ((it & 255u) == 0 && (*(volatile int*)&S.stop || over(t0, where))) { *(volatile int*)&S.stop = 1; return false; }
+    if ((it & 255u) == 0 && over(t0, where)) return false;
   }
+}
+// Who may give up.  The waits for other CTAs are all in the compute warps' wait_round, whose outcome reaches the sixteen warps behind one
+// barrier; when it says so they leave together and set S.stop, and the helpers leave together at the end of their round.  In between
+// the two groups wait for nobody but each other, and no thread draws a conclusion of its own from such a wait: one that left alone would
+// leave its group at the next counted barrier.  (The limits are for a run whose own logic is broken.)
+constexpr unsigned long long CHUNK_WAIT_NS = 20ull * 1000 * 1000 * 1000;
+__device__ __forceinline__ void chunk_full(unsigned long long* b, unsigned parity, const unsigned long long t0) {
+  for (unsigned it = 1; !mbar_try(b, parity); it++)
+    if ((it & 0xfffu) == 0 && gtime() - t0 > S.core.timeout_ns + CHUNK_WAIT_NS) { fail(S.core.g, ST_TIMEOUT, S.ppt.node, 25); return; }
+}
+__device__ __forceinline__ void chunk_empty(unsigned long long* b, unsigned parity, const unsigned long long t0) {      // or nobody uses chunks any more
+  for (unsigned it = 1; !mbar_try(b, parity); it++)
+    if ((it & 63u) == 0 && (*(volatile int*)&S.stop || gtime() - t0 > S.core.timeout_ns + CHUNK_WAIT_NS)) return;
 }
 __device__ __forceinline__ void cp16(float* dst, const void* src) { asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(smem_u32(dst)), "l"(src) : "memory"); }
 __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
@@ -223,14 +236,6 @@ __device__ __forceinline__ int helper_scan(const int v, int& total) {          /
   const int a = S.warp_sum[0], b = S.warp_sum[1], c = S.warp_sum[2], d = S.warp_sum[3];
   total = a + b + c + d;
   return s - v + (warp > 0 ? a : 0) + (warp > 1 ? b : 0) + (warp > 2 ? c : 0);
-}
-
-// One helper warp waits until the compute warps have used a chunk buffer up; the others learn the outcome behind the next barrier.
-// (No thread may give up on its own: the ones that saw the buffer free would wait for it at their next counted barrier for good.
-// Two words, by buffer: the next chunk's outcome is written while slow warps may still read this one's.)
-__device__ __forceinline__ void buffer_free(const int buf, const unsigned parity, const unsigned long long t0, const int where) {
-  const bool ok = __all_sync(0xffffffffu, mbar_wait(&S.empty[buf], parity, t0, where));
-  if ((threadIdx.x & 31) == 0) S.helper_ok[buf] = ok;
 }
 
 __device__ __noinline__ void helper_main(const int cta, const int tile, const int shard, unsigned char* smem, const unsigned long long t0) {
@@ -365,10 +370,9 @@ __device__ __noinline__ void helper_main(const int cta, const int tile, const in
         copies = !(e.meta & (E_OVERFLOW | E_DENSE | E_RAW)) && e.t[0].col4 == 0 && (one || two);
         if (one) e.t[1].col4 = 0xffff;
       }
-      if (ht < 32) buffer_free(buf, parity, t0, 21);
       copies = !bar_helper_or(!copies);
-      if (!S.helper_ok[buf]) return;
       const bool over = !copies && bar_helper_or(ht < cnt && (e.meta & E_OVERFLOW));
+      chunk_empty(&S.empty[buf], parity, t0);
       if (ht < cnt) {
         RowD& r = rows[buf * BM + ht];
         const unsigned nt = e.meta & E_NT, nx = (e.meta & E_OVERFLOW) ? 0u : kind == LIN_F && T.lstm ? nt + (e.meta >> 16) : nt;
@@ -391,7 +395,9 @@ __device__ __noinline__ void helper_main(const int cta, const int tile, const in
       if (last) break;
     } while (true);
     round++;
+    if (ht == 0) S.helper_stop = *(volatile int*)&S.stop;
     bar_helper();                                                 // (the slot tables are used up)
+    if (S.helper_stop) return;
   }
   // ---- the end: the leftover gradients are applied once more --------------------------------------------------------------
   int n_upd = 0;
@@ -399,9 +405,7 @@ __device__ __noinline__ void helper_main(const int cta, const int tile, const in
     n_upd = n_acc; n_updates++; n_grads += n_upd;
     if (leader && ht == 0 && n_updates <= S.ppt.log_cap) S.ppt.update_log[n_updates - 1] = n_upd;
   }
-  if (ht < 32) buffer_free(buf, parity, t0, 22);
-  bar_helper();
-  if (!S.helper_ok[buf]) return;
+  chunk_empty(&S.empty[buf], parity, t0);
   publish(0, H_END | (n_upd ? H_UPDATE : 0), n_upd);
   // ---- statistics ----------------------------------------------------------------------------------------------------------
   PPTStats& st = *S.ppt.stats;
@@ -454,7 +458,6 @@ __device__ __noinline__ int wait_round(const int round, const bool rows, const b
   }
   ok = __all_sync(0xffffffffu, ok);
   if (lane == 31 && first) S.ver = vp ? v : 0ull;
-  if (lane == 0 && !ok) *(volatile int*)&S.stop = 1;
   return ok ? (all ? 2 : 1) : 0;
 }
 // Before an embedding cell changes rows of its table in round r.  A row has one copy, so a reader beside the update would get half of it
@@ -468,7 +471,7 @@ __device__ __forceinline__ void wait_readers(const Head& h, const unsigned long 
     const unsigned* const p = S.core.progress + reader * 16 + (target & 15);
     const int n = S.team_n[reader] * ((target >> 4) + 1);
     for (unsigned it = 1; (int)ld_acq(p) < n; it++)
-      if ((it & 63u) == 0 && over(t0, 27)) { *(volatile int*)&S.stop = 1; break; }
+      if ((it & 63u) == 0 && over(t0, 27)) break;
   }
   __syncwarp();
 }
@@ -482,23 +485,17 @@ __device__ __forceinline__ Head chunk_loop(RowD* rows, const int team, const uns
   const bool T_publishes = S.team.kind == ACC;
   unsigned parity = 0;
   for (int buf = 0;;) {
-    // Whether the run goes on is warp 0's word, read behind a barrier: a warp that left alone would leave the others at their next one.
-    const bool mine = mbar_wait(&S.full[buf], parity, t0, 25);
+    chunk_full(&S.full[buf], parity, t0);
     phase(0);
-    Head h = S.hd[buf];                                            // (complete if this thread saw the phase; otherwise read again below)
-    if (warp == 0) {
-      int r = __all_sync(0xffffffffu, mine) ? 2 : 0;
-      if (r && (h.flags & H_FIRST)) r = wait_round(h.round, h.count > 0, true, t0);
-      if ((tid & 31) == 0) S.ok = r;
-    }
-    bar_compute();
-    int ok = S.ok;
-    if (!ok) break;
-    if (!mine) h = S.hd[buf];
+    const Head h = S.hd[buf];
     const bool end = h.flags & H_END;
     if (end && !(h.flags & H_UPDATE)) return h;
     const bool last = h.flags & H_LAST, any = h.count > 0;
     if (h.flags & H_FIRST) {
+      if (warp == 0) { const int r = wait_round(h.round, any, true, t0); if ((tid & 31) == 0) S.ok = r; }
+      bar_compute();
+      int ok = S.ok;
+      if (!ok) break;
       if (any) fresh(S.ver);
       if (ok == 1) {
         if (warp == 0) { const int r = wait_round(h.round, any, false, t0); __syncwarp(); if ((tid & 31) == 0) S.ok2 = r; }
@@ -523,6 +520,7 @@ __device__ __forceinline__ Head chunk_loop(RowD* rows, const int team, const uns
     buf ^= 1;
     if (buf == 0) parity ^= 1;
   }
+  if (tid == 0) *(volatile int*)&S.stop = 1;
   Head none{};
   return none;
 }
