@@ -837,6 +837,26 @@ __device__ __forceinline__ float4 term4(const RowD& r, const int first, const in
   return v;
 }
 
+// Rows of any kind as the second operand of a tensor-core product (dense rows have K values, K a multiple of sixteen).  A function of its
+// own: inside the cell it costs the chunks of plain copies 5,000 of 230,000 cycles a round of the wide tree.
+__device__ __noinline__ void tensor_rows_general(const RowD* R, const int count, unsigned char* Xb, const int K) {
+  IN_SMEM(R); IN_SMEM(Xb);
+  const int K8 = K >> 3, items = ((count + 7) >> 3) * K8 * 8;
+  const FastDiv d8(K8);
+#pragma unroll 1
+  for (int i = threadIdx.x; i < items; i += CT) {
+    const int g8 = d8.div(i >> 3), r = g8 * 8 + (i & 7), k8 = (i >> 3) - g8 * K8, c = 2 * k8;
+    float4 a = zero4(), b = zero4();
+    if (r < count) {
+      if (R[r].meta & E_DENSE) {
+        const float4* const x = reinterpret_cast<const float4*>(S.core.dense + (long long)(R[r].inst & 0x7fffffff) * K) + c;
+        a = __ldg(x); b = __ldg(x + 1);
+      } else { a = row_sum<false>(R[r], c); b = row_sum<false>(R[r], c + 1); }
+    }
+    tc::store8(Xb, r, 8 * k8, K, a, b);
+  }
+}
+
 // ---- forward cell ----------------------------------------------------------------------------------------------------------
 // A tile holds R columns of every gate group (G = 1 for a Linear node, 2 for a GRU's z and r, 3 or 5 for an LSTM's gates) for all
 // inputs; a shard takes its part of the round's rows.  Bound by the latency of gather -> product -> store at the usual 10-60 rows.
@@ -879,7 +899,7 @@ __device__ __noinline__ void forward_main(const int team, const int tile, float*
       const int K8 = K >> 3, items = ((count + 7) >> 3) * K8 * 8;
       constexpr int U = 4;
       const FastDiv d8(K8);
-      auto fill_x = [&](auto of_copies) {
+      if (h.flags & H_COPIES) {
 #pragma unroll 1
         for (int i0 = tid; i0 < items; i0 += U * CT) {
           float4 a[U], b[U];
@@ -888,14 +908,9 @@ __device__ __noinline__ void forward_main(const int team, const int tile, float*
             const int i = i0 + u * CT, g8 = d8.div(i >> 3), r = g8 * 8 + (i & 7), c = 2 * ((i >> 3) - g8 * K8);
             a[u] = b[u] = zero4();
             if (i >= items || r >= count) continue;
-            if constexpr (decltype(of_copies)::value) {
-              const uint4 t = *reinterpret_cast<const uint4*>(&R[r].t[0]);
-              const int cut = (int)(t.w & 0xffffu);
-              a[u] = ldcg4(S.core.arena + (c >= cut ? t.z + (c - cut) : t.x + c)); b[u] = ldcg4(S.core.arena + (c + 1 >= cut ? t.z + (c + 1 - cut) : t.x + c + 1));
-            } else if (R[r].meta & E_DENSE) {                   // (a dense row of K values, K a multiple of sixteen)
-              const float4* const x = reinterpret_cast<const float4*>(S.core.dense + (long long)(R[r].inst & 0x7fffffff) * K) + c;
-              a[u] = __ldg(x); b[u] = __ldg(x + 1);
-            } else { a[u] = row_sum<false>(R[r], c); b[u] = row_sum<false>(R[r], c + 1); }
+            const uint4 t = *reinterpret_cast<const uint4*>(&R[r].t[0]);
+            const int cut = (int)(t.w & 0xffffu);
+            a[u] = ldcg4(S.core.arena + (c >= cut ? t.z + (c - cut) : t.x + c)); b[u] = ldcg4(S.core.arena + (c + 1 >= cut ? t.z + (c + 1 - cut) : t.x + c + 1));
           }
 #pragma unroll
           for (int u = 0; u < U; u++) {
@@ -903,8 +918,7 @@ __device__ __noinline__ void forward_main(const int team, const int tile, float*
             if (i < items) tc::store8(Xb, r, 8 * k8, K, a[u], b[u]);
           }
         }
-      };
-      if (h.flags & H_COPIES) fill_x(Flag<true>()); else fill_x(Flag<false>());
+      } else tensor_rows_general(R, count, Xb, K);
       tc::fence_operands();
       phase(2);
       if (count <= tc::SMALL_ROWS) for (int i = tid; i < count * YP; i += CT) Ys[i] = 0.f;
