@@ -69,7 +69,7 @@ struct EncModel {
   unsigned near_scratch;               // the scratch is small enough for shared memory
   unsigned bound[MAX_CELLS], steps_cap;       // most entries of a cell, most steps, of one instance
 };
-struct EncTotals { unsigned entries[MAX_CELLS]; unsigned tab, ov, ov_used, arena4_max; unsigned steps_min, steps_eval_min; unsigned long long steps_sum, steps_eval_sum; int status; };
+struct EncTotals { unsigned entries[MAX_CELLS]; unsigned tab, ov_used, arena4_max; unsigned steps_min, steps_eval_min; unsigned long long ov, steps_sum, steps_eval_sum; int status; };
 
 struct Program {                       // device pointers of an encoded split
   InstHdr* hdr;

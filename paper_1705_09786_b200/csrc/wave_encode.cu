@@ -32,6 +32,15 @@ __device__ __forceinline__ unsigned warp_excl(unsigned v, unsigned& total) {
   return s - v;
 }
 
+__device__ __forceinline__ unsigned long long warp_excl64(unsigned long long v, unsigned long long& total) {
+  const int lane = threadIdx.x & 31;
+  unsigned long long s = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) { const unsigned long long x = __shfl_up_sync(FULL, s, o); if (lane >= o) s += x; }
+  total = __shfl_sync(FULL, s, 31);
+  return s - v;
+}
+
 template <bool EMIT>
 struct Encoder {
   const EncModel& M; const DevInst& I; unsigned* const scr; Item* const stack; unsigned* const cur;
@@ -634,7 +643,7 @@ struct Encoder {
 
 __device__ void summarise(EncTotals* totals, const InstHdr& H, unsigned arena4, unsigned n_ov, int status, int left) {
   if (status || left) atomicCAS(&totals->status, 0, status ? status : -1);               // every message must be answered
-  if (n_ov) atomicAdd(&totals->ov, n_ov);
+  if (n_ov) atomicAdd(&totals->ov, (unsigned long long)n_ov);
   atomicMax(&totals->arena4_max, arena4);
   atomicMin(&totals->steps_min, (unsigned)H.steps); atomicMin(&totals->steps_eval_min, (unsigned)H.steps_eval);
   atomicAdd(&totals->steps_sum, (unsigned long long)H.steps); atomicAdd(&totals->steps_eval_sum, (unsigned long long)H.steps_eval);
@@ -696,25 +705,27 @@ __global__ void __launch_bounds__(EW * 32) encode_kernel(const __grid_constant__
 
 // Exclusive prefix sums over the instances, a block per cell (the last one: the instances' first table entries).
 __global__ void __launch_bounds__(1024) scan_kernel(unsigned* counts, InstHdr* hdr, const long long n, const int n_cells, EncTotals* totals) {
-  __shared__ unsigned part[32];
-  __shared__ unsigned block_total;
+  __shared__ unsigned long long part[32], block_total;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, c = blockIdx.x;
-  unsigned carry = 0;
+  unsigned long long carry = 0;                                // (sums beyond 32 bits void the program: offsets have no more)
   for (long long i0 = 0; i0 < n; i0 += 1024) {
     const long long i = i0 + tid;
     const unsigned v = i >= n ? 0u : c < n_cells ? counts[(size_t)c * n + i] : hdr[i].steps + 1u;
-    unsigned total, all;
-    const unsigned ex = warp_excl(v, total);
+    unsigned long long total, all;                             // (a block's thousand counts may pass 32 bits between them)
+    const unsigned long long ex = warp_excl64(v, total);
     if (lane == 31) part[warp] = total;
     __syncthreads();
-    if (warp == 0) { const unsigned p = warp_excl(part[lane], all); part[lane] = p; if (lane == 0) block_total = all; }
+    if (warp == 0) { const unsigned long long p = warp_excl64(part[lane], all); part[lane] = p; if (lane == 0) block_total = all; }
     __syncthreads();
-    const unsigned out = carry + part[warp] + ex;
+    const unsigned out = (unsigned)(carry + part[warp] + ex);
     if (i < n) { if (c < n_cells) counts[(size_t)c * n + i] = out; else hdr[i].tab = out; }
     carry += block_total;
     __syncthreads();
   }
-  if (tid == 0) { if (c < n_cells) totals->entries[c] = carry; else totals->tab = carry; }
+  if (tid == 0) {
+    if (c < n_cells) totals->entries[c] = (unsigned)carry; else totals->tab = (unsigned)carry;
+    if (carry > 0xffffffffull) atomicCAS(&totals->status, 0, ST_OVERFLOW);
+  }
 }
 
 }  // namespace

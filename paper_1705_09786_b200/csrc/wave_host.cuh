@@ -235,12 +235,12 @@ static ampnet_status_t wave_encode(ampnet_graph* g, HostDataset& D, WaveModel& M
   CUDA_TRY(g, cudaMemcpyAsync(&W.tot, totals, sizeof W.tot, cudaMemcpyDeviceToHost, g->stream));
   CUDA_TRY(g, cudaStreamSynchronize(g->stream));
   if (getenv("AMPNET_DEBUG")) {
-    fprintf(stderr, "[ampnet] programs: status %d, %u steps table, arena %u x 16 B, steps min %u (eval %u) mean %.1f, overflow terms %u, entries", W.tot.status, W.tot.tab, W.tot.arena4_max,
+    fprintf(stderr, "[ampnet] programs: status %d, %u steps table, arena %u x 16 B, steps min %u (eval %u) mean %.1f, overflow terms %llu, entries", W.tot.status, W.tot.tab, W.tot.arena4_max,
             W.tot.steps_min, W.tot.steps_eval_min, (double)W.tot.steps_sum / n, W.tot.ov);
     for (int c = 0; c < E.n_cells; c++) fprintf(stderr, " %u", W.tot.entries[c]);
     fprintf(stderr, "\n");
   }
-  if (W.tot.status != 0) return AMPNET_OK;       // (a structure beyond the encoder's bounds: the interpreter engine runs it)
+  if (W.tot.status != 0 || W.tot.ov > 0xffffffffull) return AMPNET_OK;       // (a structure beyond the encoder's bounds: the interpreter engine runs it)
   for (int c = 0; c < E.n_cells; c++) { tab_at[c] = take(((size_t)W.tot.tab + 2) * 4); ent_at[c] = take((size_t)W.tot.entries[c] * sizeof(Entry)); }
   const size_t ov_at = take((size_t)W.tot.ov * sizeof(Term));
   char* mem = (char*)dev_alloc(g, bytes);

@@ -1,4 +1,6 @@
 """Cells of the scheduled engine at the sizes where their tiles, chunks and tables can go wrong, against the CPU oracle."""
+import os
+
 import numpy as np
 import pytest
 
@@ -234,3 +236,55 @@ def test_embedding_rows_are_read_whole(vocab, width, muf):
         assert np.abs(after[k][:6] - p[k][:6]).max() > 0
         np.testing.assert_array_equal(after[k], np.repeat(after[k][:, :1], width, axis=1))
     e.close()
+
+
+SCAN_PROGRAM = r"""
+#include "wave_encode.cu"
+extern "C" int scan(unsigned* counts, wave::InstHdr* hdr, long long n, int n_cells, wave::EncTotals* totals, unsigned* entries, unsigned* tab, int* status) {
+  if (wave::encode_scan(counts, hdr, n, n_cells, totals, 0) != cudaSuccess) return 1;
+  wave::EncTotals h;
+  if (cudaMemcpy(&h, totals, sizeof h, cudaMemcpyDeviceToHost) != cudaSuccess) return 2;
+  for (int c = 0; c < n_cells; c++) entries[c] = h.entries[c];
+  *tab = h.tab; *status = h.status;
+  return 0;
+}
+extern "C" int totals_bytes() { return sizeof(wave::EncTotals); }
+"""
+
+
+@pytest.fixture(scope="module")
+def scan_lib(tmp_path_factory):
+    import ctypes
+    import subprocess
+
+    from paper_1705_09786_b200 import build
+    d = tmp_path_factory.mktemp("scan")
+    (d / "scan.cu").write_text(SCAN_PROGRAM)
+    subprocess.check_call([os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc"), "-gencode", "arch=compute_100a,code=sm_100a", "-std=c++17", "-O1", "-Xcompiler", "-fPIC",
+                           "-shared", "-I", os.path.dirname(build.SRC), "-o", str(d / "scan.so"), str(d / "scan.cu")])
+    return ctypes.CDLL(str(d / "scan.so"))
+
+
+@pytest.mark.parametrize("n,each,fits", [(1, 5, True), (1025, 4190210, True), (1025, 4190213, False), (5000, 1 << 20, False), (3, 0xffffffff, False)])
+def test_program_offsets_beyond_32_bits_void_the_program(scan_lib, n, each, fits):
+    """The offsets of the instances' programs are prefix sums of 32 bits: sums that do not fit are reported, not wrapped around."""
+    import ctypes
+
+    import torch
+    lib = scan_lib
+    cells = 2
+    counts = torch.full((cells, n), each - (1 << 32) if each >= 1 << 31 else each, dtype=torch.int32, device="cuda")
+    counts[1] = 1
+    hdr = torch.zeros((n, 4), dtype=torch.int32, device="cuda")         # no steps: one table entry each
+    totals = torch.zeros(lib.totals_bytes(), dtype=torch.uint8, device="cuda")
+    torch.cuda.synchronize()
+    entries, tab, status = (ctypes.c_uint * cells)(), ctypes.c_uint(), ctypes.c_int()
+    assert lib.scan(ctypes.c_void_p(counts.data_ptr()), ctypes.c_void_p(hdr.data_ptr()), ctypes.c_longlong(n), cells, ctypes.c_void_p(totals.data_ptr()), entries,
+                    ctypes.byref(tab), ctypes.byref(status)) == 0
+    assert (status.value == 0) == fits == (n * each < 1 << 32)
+    assert entries[1] == n and tab.value == n
+    if fits:
+        assert entries[0] == n * each
+        want = np.arange(n, dtype=np.uint64) * each
+        np.testing.assert_array_equal(counts[0].cpu().numpy().astype(np.uint32), want.astype(np.uint32))
+        np.testing.assert_array_equal(hdr[:, 0].cpu().numpy(), np.arange(n))
