@@ -175,7 +175,7 @@ void* dev_alloc(ampnet_graph* g, size_t bytes) {
   if (bytes == 0) bytes = 256;
   if (g->alloc.alloc) return g->alloc.alloc(g->alloc.ctx, bytes);
   void* p = nullptr;
-  if (cudaMalloc(&p, bytes) != cudaSuccess) return nullptr;
+  if (cudaMalloc(&p, bytes) != cudaSuccess) { cudaGetLastError(); return nullptr; }      // (the caller reports it or does without)
   return p;
 }
 void dev_free(ampnet_graph* g, void* p) {
@@ -1161,7 +1161,7 @@ ampnet_status_t wave_execute(ampnet_graph* g, HostDataset& D, const WavePlan& P,
 
 ampnet_status_t execute(ampnet_graph* g, int split, int mak, int det, int eval, const ampnet_run_cfg_t* cfg,
                         ampnet_epoch_stats_t* out, float* per_instance_loss, double* accuracy,
-                        const uint8_t* inference_only = nullptr, ampnet_inference_stats_t* inference = nullptr) {
+                        const uint8_t* inference_only = nullptr, ampnet_inference_stats_t* inference = nullptr, bool scheduled = true) {
   HostDataset& D = g->data[split];
   if (!D.loaded) return set_err(g, AMPNET_ESTATE, "no instances loaded for split %d", split);
   if (mak < 1) return set_err(g, AMPNET_EINVAL, "max_active_keys must be >= 1");
@@ -1179,10 +1179,12 @@ ampnet_status_t execute(ampnet_graph* g, int split, int mak, int det, int eval, 
   CUDA_TRY(g, cudaSetDevice(g->device));
   g->have_run = false;                // planning re-targets the statistics pointers: the previous run's are gone from here on
   WavePlan wp;
-  if (wave_takes(g, D, mak, det, eval, cfg, n_order, wp)) return wave_execute(g, D, wp, mak, eval, cfg, order, n_order, out, per_instance_loss, accuracy, inference_only, inference);
+  ampnet_status_t st = AMPNET_ENOMEM;
+  if (scheduled && wave_takes(g, D, mak, det, eval, cfg, n_order, wp)) st = wave_execute(g, D, wp, mak, eval, cfg, order, n_order, out, per_instance_loss, accuracy, inference_only, inference);
+  if (st != AMPNET_ENOMEM) return st;                             // (without the memory for its arenas, the other engines' may still be there)
   RunPlan R;
   if (dbg) fprintf(stderr, "[ampnet] planning\n");
-  ampnet_status_t st = plan_run(g, split, mak, det, eval, cfg, n_order, true, R);
+  st = plan_run(g, split, mak, det, eval, cfg, n_order, true, R);
   if (st != AMPNET_OK) return st;
   const size_t order_bytes = order ? (size_t)n_order * sizeof(long long) : 0;
   const size_t mask_bytes = inference_only ? (size_t)D.n : 0;
@@ -1783,24 +1785,32 @@ extern "C" ampnet_status_t ampnet_run_epoch_static(ampnet_graph_t* g, const ampn
     CUDA_TRY(g, cudaGetSymbolAddress(&ptr, g_static_scratch));
     g_static_scratch_addr[g->device] = ptr;
   }
-  // size the run state without touching any memory, and refuse what does not fit
+  // size the run state without touching any memory: the scheduled engine's, then the other engines', and refuse what does not fit
   const long long n_order = cfg->order ? cfg->n_order : D.n;
-  RunPlan plan;
+  const size_t order_bytes = cfg->order ? (size_t)std::max<long long>(n_order, 0) * sizeof(long long) : 0;
+  size_t ctl_need = 0, bulk_need = 0;
+  auto fits = [&] {                   // the very sizes execute() will ask ensure_arenas() for
+    ctl_need = ((g->ctl.used + ARENA_SLACK + 255) & ~(size_t)255);
+    bulk_need = g->bulk.used + order_bytes + BULK_EXTRA + ARENA_SLACK;
+    return ctl_need + bulk_need <= (size_t)AMPNET_STATIC_SCRATCH_BYTES;
+  };
   g->have_run = false;                // the dry plan re-targets the statistics pointers of the previous run
   ampnet_status_t st = AMPNET_OK;
   WavePlan wp;
-  if (wave_takes(g, D, cfg->max_active_keys, cfg->deterministic ? 1 : 0, 0, cfg, n_order, wp)) {
+  bool scheduled = wave_takes(g, D, cfg->max_active_keys, cfg->deterministic ? 1 : 0, 0, cfg, n_order, wp);
+  if (scheduled) {
     wave::Run R;
     wave_carve(g, D, g->wave, D.wave, wp, cfg->max_active_keys, 0, cfg, n_order, true, R);
-  } else st = plan_run(g, 0, cfg->max_active_keys, cfg->deterministic ? 1 : 0, 0, cfg, n_order, true, plan);
-  if (st != AMPNET_OK) return st;
-  const size_t order_bytes = cfg->order ? (size_t)std::max<long long>(n_order, 0) * sizeof(long long) : 0;
-  // the very sizes execute() will ask ensure_arenas() for
-  const size_t ctl_need = ((g->ctl.used + ARENA_SLACK + 255) & ~(size_t)255);
-  const size_t bulk_need = g->bulk.used + order_bytes + BULK_EXTRA + ARENA_SLACK;
-  if (ctl_need + bulk_need > (size_t)AMPNET_STATIC_SCRATCH_BYTES)
-    return set_err(g, AMPNET_EINVAL, "this run needs %zu bytes of scratch but the static scratch holds %zu: lower "
-                   "max_active_keys or use ampnet_run_epoch", ctl_need + bulk_need, (size_t)AMPNET_STATIC_SCRATCH_BYTES);
+    scheduled = fits();
+  }
+  if (!scheduled) {
+    RunPlan plan;
+    st = plan_run(g, 0, cfg->max_active_keys, cfg->deterministic ? 1 : 0, 0, cfg, n_order, true, plan);
+    if (st != AMPNET_OK) return st;
+    if (!fits())
+      return set_err(g, AMPNET_EINVAL, "this run needs %zu bytes of scratch but the static scratch holds %zu: lower "
+                     "max_active_keys or use ampnet_run_epoch", ctl_need + bulk_need, (size_t)AMPNET_STATIC_SCRATCH_BYTES);
+  }
   // lend the static array to the handle for the duration of this call
   void *own_ctl = g->ctl_mem, *own_bulk = g->bulk_mem;
   const size_t own_ctl_cap = g->ctl_cap, own_bulk_cap = g->bulk_cap;
@@ -1808,7 +1818,7 @@ extern "C" ampnet_status_t ampnet_run_epoch_static(ampnet_graph_t* g, const ampn
   g->ctl_mem = base; g->ctl_cap = ctl_need;
   g->bulk_mem = base + ctl_need; g->bulk_cap = (size_t)AMPNET_STATIC_SCRATCH_BYTES - ctl_need;
   g->arenas_lent = true;
-  st = execute(g, 0, cfg->max_active_keys, cfg->deterministic ? 1 : 0, 0, cfg, out, per_instance_loss, nullptr);
+  st = execute(g, 0, cfg->max_active_keys, cfg->deterministic ? 1 : 0, 0, cfg, out, per_instance_loss, nullptr, nullptr, nullptr, scheduled);
   g->arenas_lent = false;
   g->ctl_mem = own_ctl; g->ctl_cap = own_ctl_cap; g->bulk_mem = own_bulk; g->bulk_cap = own_bulk_cap;
   g->leftover_regions.clear();      // they described the lent memory

@@ -163,6 +163,8 @@ static bool wave_model(const std::vector<DevNode>& nodes, const std::vector<int>
 }
 
 // ---- encoding of a loaded split (at the end of ampnet_load_instances) -------------------------------------------------------
+// What cannot be encoded (a structure beyond the encoder's bounds, or no memory for its scratch or the programs) stays with the other
+// engines: the split is loaded all the same, and holds nothing of the attempt.
 
 static ampnet_status_t wave_encode(ampnet_graph* g, HostDataset& D, WaveModel& M, WaveData& W, void** scratch, size_t* scratch_cap) {
   using namespace wave;
@@ -171,6 +173,21 @@ static ampnet_status_t wave_encode(ampnet_graph* g, HostDataset& D, WaveModel& M
   W.tc = g->payload_bf16 && single_row_graph(g, D);
   if (!M.ok || n < 1 || n > (1ll << 30)) return AMPNET_OK;
   if (!encoder_sizes(M.enc, g->hnodes, D.maxOut)) return AMPNET_OK;
+  const size_t held = D.allocs.size();
+  auto release_scratch = [&] {                                   // (a handle keeps what small splits need)
+    if (*scratch_cap <= (64ull << 20)) return;
+    dev_free(g, *scratch);
+    *scratch = nullptr; *scratch_cap = 0;
+  };
+  auto not_taken = [&](const char* why, size_t bytes) {          // (the stream has been waited for)
+    if (getenv("AMPNET_DEBUG")) fprintf(stderr, "[ampnet] instances not encoded: %s (%zu bytes)\n", why, bytes);
+    while (D.allocs.size() > held) { dev_free(g, D.allocs.back()); D.allocs.pop_back(); }
+    release_scratch();
+    const bool tc = W.tc;
+    W = WaveData{};
+    W.tc = tc;
+    return AMPNET_OK;
+  };
   // Warps per block: with the scratch in shared memory as many as fit there.  An instance is one long chain of dependent steps, so a large
   // split wants warps more than it wants near memory (an SM holds 16 by registers): 20,000 lists of 26 KB scratch 8.5 -> 4.8 ms.
   const size_t warp_bytes = (size_t)M.enc.scratch_words * 4, near_bytes = warp_bytes + M.enc.stack_cap * 16;
@@ -196,7 +213,7 @@ static ampnet_status_t wave_encode(ampnet_graph* g, HostDataset& D, WaveModel& M
     const size_t tot_at = take(sizeof(EncTotals)), hdr_at = take((size_t)n * sizeof(InstHdr));
     for (int c = 0; c < E.n_cells; c++) { tab_at[c] = take(((size_t)n * E.steps_cap + 2) * 4); ent_at[c] = take((size_t)n * E.bound[c] * sizeof(Entry)); }
     char* mem = (char*)dev_alloc(g, bytes);
-    if (!mem) return set_err(g, AMPNET_ENOMEM, "device allocation of %zu bytes (message programs) failed", bytes);
+    if (!mem) return not_taken("no memory for the programs", bytes);
     D.allocs.push_back(mem);
     EncTotals* totals = (EncTotals*)(mem + tot_at);
     W.prog.hdr = (InstHdr*)(mem + hdr_at);
@@ -205,7 +222,8 @@ static ampnet_status_t wave_encode(ampnet_graph* g, HostDataset& D, WaveModel& M
     CUDA_TRY(g, encode_bounded(&E, D.dev, (int)blocks, per, W.prog, totals, g->stream));
     CUDA_TRY(g, cudaMemcpyAsync(&W.tot, totals, sizeof W.tot, cudaMemcpyDeviceToHost, g->stream));
     CUDA_TRY(g, cudaStreamSynchronize(g->stream));
-    W.ok = W.tot.status == 0;
+    if (W.tot.status != 0) return not_taken("beyond the encoder's bounds", bytes);
+    W.ok = true;
     return AMPNET_OK;
   }
   blocks = std::min<long long>(blocks, 8ll * g->n_sms);
@@ -219,11 +237,12 @@ static ampnet_status_t wave_encode(ampnet_graph* g, HostDataset& D, WaveModel& M
     dev_free(g, *scratch);
     *scratch = dev_alloc(g, need);
     *scratch_cap = *scratch ? need : 0;
-    if (!*scratch) return set_err(g, AMPNET_ENOMEM, "device allocation of %zu bytes (encoder) failed", need);
+    if (!*scratch) return not_taken("no memory for the encoder", need);
   }
   const size_t hdr_b = (size_t)n * sizeof(InstHdr), cnt_b = (size_t)E.n_cells * n * 4, tot_b = sizeof(EncTotals);
-  char* meta = (char*)dev_alloc(g, hdr_b + ((cnt_b + 255) & ~(size_t)255) + tot_b + 256);
-  if (!meta) return set_err(g, AMPNET_ENOMEM, "device allocation (program headers) failed");
+  const size_t meta_b = hdr_b + ((cnt_b + 255) & ~(size_t)255) + tot_b + 256;
+  char* meta = (char*)dev_alloc(g, meta_b);
+  if (!meta) return not_taken("no memory for the program headers", meta_b);
   D.allocs.push_back(meta);
   InstHdr* hdr = (InstHdr*)meta;
   unsigned* counts = (unsigned*)(meta + hdr_b);
@@ -240,21 +259,20 @@ static ampnet_status_t wave_encode(ampnet_graph* g, HostDataset& D, WaveModel& M
     for (int c = 0; c < E.n_cells; c++) fprintf(stderr, " %u", W.tot.entries[c]);
     fprintf(stderr, "\n");
   }
-  if (W.tot.status != 0 || W.tot.ov > 0xffffffffull) return AMPNET_OK;       // (a structure beyond the encoder's bounds: the interpreter engine runs it)
+  if (W.tot.status != 0 || W.tot.ov > 0xffffffffull) return not_taken("beyond the encoder's bounds", need);
   for (int c = 0; c < E.n_cells; c++) { tab_at[c] = take(((size_t)W.tot.tab + 2) * 4); ent_at[c] = take((size_t)W.tot.entries[c] * sizeof(Entry)); }
   const size_t ov_at = take((size_t)W.tot.ov * sizeof(Term));
   char* mem = (char*)dev_alloc(g, bytes);
-  if (!mem) return set_err(g, AMPNET_ENOMEM, "device allocation of %zu bytes (message programs) failed", bytes);
+  if (!mem) return not_taken("no memory for the programs", bytes);
   D.allocs.push_back(mem);
   W.prog.hdr = hdr;
   for (int c = 0; c < E.n_cells; c++) { W.prog.tab[c] = (const unsigned*)(mem + tab_at[c]); W.prog.ent[c] = (const Entry*)(mem + ent_at[c]); }
   W.prog.ov = (const Term*)(mem + ov_at);
   CUDA_TRY(g, encode_emit(&E, D.dev, (unsigned*)*scratch, (int)blocks, per, W.prog, counts, (Term*)(mem + ov_at), totals, g->stream));
   W.ok = true;
-  if (*scratch_cap > (64ull << 20)) {                            // (given back: a handle keeps what small splits need)
+  if (*scratch_cap > (64ull << 20)) {
     CUDA_TRY(g, cudaStreamSynchronize(g->stream));
-    dev_free(g, *scratch);
-    *scratch = nullptr; *scratch_cap = 0;
+    release_scratch();
   }
   return AMPNET_OK;
 }

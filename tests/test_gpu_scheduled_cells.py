@@ -288,3 +288,75 @@ def test_program_offsets_beyond_32_bits_void_the_program(scan_lib, n, each, fits
         want = np.arange(n, dtype=np.uint64) * each
         np.testing.assert_array_equal(counts[0].cpu().numpy().astype(np.uint32), want.astype(np.uint32))
         np.testing.assert_array_equal(hdr[:, 0].cpu().numpy(), np.arange(n))
+
+
+class _Refusing:
+    """torch.empty as the engine's allocator calls it, with requests refused while `refuse(bytes)` says so."""
+
+    def __init__(self, monkeypatch, refuse):
+        import torch
+        self.real, self.refuse, self.refused = torch.empty, refuse, []
+        monkeypatch.setattr(torch, "empty", self)
+
+    def __call__(self, *a, **kw):
+        if kw.get("dtype") is not None and str(kw["dtype"]) == "torch.uint8" and self.refuse(a[0]):
+            self.refused.append(a[0])
+            raise MemoryError
+        return self.real(*a, **kw)
+
+
+@pytest.mark.parametrize("family,size,n,limit,when", [("rnn", (14, 64, 64, 10), 6000, 1 << 20, "load"), ("rnn", (14, 64, 64, 10), 6000, 24 << 20, "load"),
+                                                      ("rnn", (14, 64, 64, 10), 8, 40 << 10, "load"), ("tree", (60, 36, 21, 5), 300, 1 << 20, "epoch"),
+                                                      ("ggnn", (15, 24, 3), 60, 1 << 20, "epoch")])
+def test_without_memory_for_programs_or_arenas_the_other_engines_run(oracle_mod, monkeypatch, family, size, n, limit, when):
+    """Requests of the encoder (its scratch, headers, programs) or of the scheduled engine's arenas are refused: the split is loaded and
+    its epoch runs, with the results of any order of execution."""
+    import paper_1705_09786_b200 as amp
+    g, inst = _case(family, size, n)
+    p = wp.init_params(g)
+    o, e = oracle_mod.Oracle(g), amp.Engine(g)
+    o.load_instances(inst)
+    o.set_params(p)
+    e.set_params(p)
+    closed = [when == "load"]
+    gate = _Refusing(monkeypatch, lambda nbytes: closed[0] and nbytes > limit and (when == "load" or not gate.refused))
+    e.load_instances(inst)
+    held = len(e._blocks)
+    closed[0] = when == "epoch"
+    _, oloss = o.run_epoch(mak=1, muf=1 << 30, lr=1e-5)
+    st, eloss = e.run_epoch(mak=8, muf=1 << 30, lr=1e-5, timeout_s=60)
+    assert gate.refused and st.instances == n
+    np.testing.assert_allclose(eloss, oloss, rtol=1e-5, atol=2e-6)
+    closed[0] = False
+    e.load_instances(inst)                                              # with memory again, the split is encoded
+    assert when != "load" or len(e._blocks) > held
+    np.testing.assert_allclose(e.run_epoch(mak=8, muf=1 << 30, lr=0.0, timeout_s=60)[1], o.run_epoch(mak=1, muf=1 << 30, lr=0.0)[1], rtol=2e-5, atol=4e-6)
+    e.close()
+
+
+def test_static_epoch_whose_scheduled_scratch_is_too_large_runs_on_another_engine():
+    """The fixed scratch holds some runs that are too large for the scheduled engine: they are served, not refused."""
+    import paper_1705_09786_b200 as amp
+    g = ir.rnn()
+    inst = data.list_instances(n=40)
+    e = amp.Engine(g)
+    e.load_instances(inst)
+    p = wp.init_params(g)
+    sizes = []
+    for mak in (256, 512, 768, 904, 920, 940, 960, 980, 1280):        # (between the two limits lie some sixty keys)
+        runs = {}
+        for engine in ("", "direct"):
+            if engine:
+                os.environ["AMPNET_ENGINE"] = engine
+            try:
+                e.set_params(p)
+                st, loss = e.run_epoch(mak=mak, muf=1 << 30, lr=0.0, timeout_s=60, static_scratch=True)
+                runs[engine] = loss
+            except amp.AmpnetError as err:
+                assert err.status == 1
+            finally:
+                os.environ.pop("AMPNET_ENGINE", None)
+        sizes.append((mak, "" in runs, "direct" in runs))
+        assert "" in runs or "direct" not in runs, sizes
+    assert any(ok for _, ok, _ in sizes) and not all(ok for _, ok, _ in sizes), sizes
+    e.close()
