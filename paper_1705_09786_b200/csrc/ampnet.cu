@@ -15,6 +15,7 @@
 
 #include "../../include/ampnet.h"
 #include "engine.cuh"
+#include "kernel_smem.h"
 #include "wave.h"
 #include "wave_sizes.h"
 
@@ -1222,7 +1223,7 @@ ampnet_status_t execute(ampnet_graph* g, int split, int mak, int det, int eval, 
     if (le == cudaErrorCooperativeLaunchTooLarge) return set_err(g, AMPNET_EINVAL, "%d CTAs cannot be co-resident", R.ctx.n_ctas);
     if (le != cudaSuccess) return set_err(g, AMPNET_ECUDA, "launch of the direct-delivery engine failed: %s", cudaGetErrorString(le));
   } else {
-    CUDA_TRY(g, cudaFuncSetAttribute(ampnet_engine, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)R.smem_bytes));
+    CUDA_TRY(g, allow_dynamic_smem((const void*)ampnet_engine, R.smem_bytes));
     int per_sm = 0;
     CUDA_TRY(g, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ampnet_engine, THREADS, R.smem_bytes));
     if (per_sm < 1 || (long long)per_sm * g->n_sms < R.ctx.n_ctas)

@@ -20,6 +20,7 @@
 #include <cuda_runtime.h>
 
 #include "engine_types.h"
+#include "kernel_smem.h"
 #include "tc_tile.cuh"
 
 namespace ampf {
@@ -1915,7 +1916,7 @@ extern "C" cudaError_t ampnet_direct_static_smem(size_t* bytes) {
   return e;
 }
 extern "C" cudaError_t ampnet_direct_launch(const amp::Ctx* ctx, int n_ctas, size_t smem_bytes, cudaStream_t stream, int n_sms) {
-  cudaError_t e = cudaFuncSetAttribute(ampnet_engine_direct, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
+  cudaError_t e = amp::allow_dynamic_smem((const void*)ampnet_engine_direct, smem_bytes);
   if (e != cudaSuccess) return e;
   int per_sm = 0;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ampnet_engine_direct, ampf::FT, smem_bytes);

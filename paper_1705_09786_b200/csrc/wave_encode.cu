@@ -2,6 +2,7 @@
 // writes the instance's program (wave.h).  A payload is a list of row records, a row record a list of terms.
 #include <cuda_runtime.h>
 
+#include "kernel_smem.h"
 #include "wave.h"
 
 namespace wave {
@@ -734,15 +735,9 @@ int encode_warps_per_block() { return EW; }
 
 static cudaError_t run_encode(const EncModel* m, const DevInst& inst, unsigned* scratch, int blocks, int warps, const Program& prog, InstHdr* hdr, unsigned* counts, Term* ov,
                               EncTotals* totals, int emit, cudaStream_t st) {
-  static size_t set[64] = {};
   const size_t smem = (size_t)warps * ((size_t)m->stack_cap * sizeof(Item) + (m->near_scratch ? (size_t)m->scratch_words * 4 : 0));
-  int dev = 0;
-  cudaGetDevice(&dev);
-  if (smem > 40 * 1024 && (dev < 0 || dev >= 64 || set[dev] < smem)) {
-    const cudaError_t e = cudaFuncSetAttribute(encode_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    if (dev >= 0 && dev < 64) set[dev] = smem;
-  }
+  const cudaError_t e = allow_dynamic_smem((const void*)encode_kernel, smem);
+  if (e != cudaSuccess) return e;
   encode_kernel<<<blocks, warps * 32, smem, st>>>(*m, inst, scratch, prog, hdr, counts, ov, totals, emit);
   return cudaGetLastError();
 }

@@ -13,6 +13,7 @@
 // updates of the one before; 2 otherwise: the reload then never waits).
 #include <cuda_bf16.h>
 
+#include "kernel_smem.h"
 #include "tc_tile.cuh"
 #include "wave.h"
 
@@ -1735,14 +1736,8 @@ extern "C" __global__ void __launch_bounds__(NT, 1) ENGINE_KERNEL(const __grid_c
 
 // ---- host hooks ---------------------------------------------------------------------------------------------------------------
 cudaError_t launch(const Run* run, int n_ctas, size_t smem, cudaStream_t st) {
-  static size_t set[64] = {};
-  int dev = 0;
-  cudaGetDevice(&dev);
-  if (dev < 0 || dev >= 64 || set[dev] < smem) {
-    const cudaError_t e = cudaFuncSetAttribute(ENGINE_KERNEL, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    if (dev >= 0 && dev < 64) set[dev] = smem;
-  }
+  const cudaError_t e = allow_dynamic_smem((const void*)ENGINE_KERNEL, smem);
+  if (e != cudaSuccess) return e;
   void* args[] = {const_cast<Run*>(run)};
   return cudaLaunchCooperativeKernel((void*)ENGINE_KERNEL, dim3(n_ctas), dim3(NT), args, smem, st);
 }
