@@ -1139,7 +1139,10 @@ ampnet_status_t wave_execute(ampnet_graph* g, HostDataset& D, const WavePlan& P,
   std::memcpy(g->last_stats.data(), g->host_read + S.stats_at, g->ppts.size() * sizeof(PPTStats));
   g->last_node_msgs.resize(g->hnodes.size() * 2);
   std::memcpy(g->last_node_msgs.data(), g->host_read + S.node_msgs_at, g->last_node_msgs.size() * sizeof(unsigned long long));
-  if (per_instance_loss) std::memcpy(per_instance_loss, g->host_read + S.loss_at, (size_t)D.n * sizeof(float));
+  if (per_instance_loss) {
+    const double* sums = reinterpret_cast<const double*>(g->host_read + S.loss_at);
+    for (long long i = 0; i < D.n; i++) per_instance_loss[i] = (float)sums[i];
+  }
   if (getenv("AMPNET_DEBUG")) {
     const unsigned long long* ph = reinterpret_cast<const unsigned long long*>(g->host_read + S.phases_at);
     for (size_t k = 0; k < P.teams.size(); k++) {
@@ -1574,7 +1577,7 @@ ampnet_status_t ampnet_load_instances(ampnet_graph_t* g, int32_t split, const am
   if (in->labels_f) if ((st = upload_raw(g, D, in->labels_f, (size_t)n, &V.labels_f)) != AMPNET_OK) return st;
   if ((st = flush_uploads(g, D)) != AMPNET_OK) return st;
   infer_domains(g, D);
-  if ((st = ensure_host_read(g, sizeof(Globals) + g->ppts.size() * sizeof(PPTStats) + 16384 + (size_t)n * sizeof(float))) != AMPNET_OK) return st;
+  if ((st = ensure_host_read(g, sizeof(Globals) + g->ppts.size() * sizeof(PPTStats) + 16384 + (size_t)n * sizeof(double))) != AMPNET_OK) return st;
   if ((st = wave_encode(g, D, g->wave, D.wave, &g->enc_scratch, &g->enc_scratch_cap)) != AMPNET_OK) return st;
   CUDA_TRY(g, cudaStreamSynchronize(g->stream));
   D.loaded = true;

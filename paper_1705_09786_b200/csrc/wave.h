@@ -127,7 +127,7 @@ struct Core {                          // what every CTA keeps in shared memory
   float4* arena; unsigned slot4; int copies;     // floats of a key / 4; arenas a key alternates between
   const long long* order; long long n_order;
   const unsigned char* inference_only;
-  float* loss_out;
+  double* loss_out;                    // per instance: sums over its Loss messages, whatever order they come in
   unsigned long long* phases;          // [teams][N_PHASES]
   const float* dense; int dense_dim;
   int n_teams, mak, eval, bf16, lag, pace, n_ctas;      // pace: most instances admitted in one round

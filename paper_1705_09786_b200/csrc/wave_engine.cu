@@ -1406,7 +1406,7 @@ __device__ __noinline__ void head_main(const int team, float* smem, RowD* rows, 
         for (int j = lj; j < outp; j += G) d[j] = j == 0 ? rnd(bf16, 2.f * e) * act_grad(T.act, y[0]) : 0.f;
       }
       if (live && lj == 0) {
-        atomicAdd(S.core.loss_out + (r.inst & 0x7fffffff), loss);
+        atomicAdd(S.core.loss_out + (r.inst & 0x7fffffff), (double)loss);
         if (inf) inf_sum += loss; else loss_sum += loss;
       }
     }

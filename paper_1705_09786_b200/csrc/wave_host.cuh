@@ -522,8 +522,8 @@ static WaveScratch wave_carve(ampnet_graph* g, HostDataset& D, const WaveModel& 
   R.core.phases = C.take<unsigned long long>(MAX_CELLS * N_PHASES);
   S.phases_at = C.used - MAX_CELLS * N_PHASES * sizeof(unsigned long long);
   const size_t nl = (size_t)std::max<long long>(D.n, 1);
-  R.core.loss_out = C.take<float>(nl);
-  S.loss_at = C.used - nl * sizeof(float);
+  R.core.loss_out = C.take<double>(nl);
+  S.loss_at = C.used - nl * sizeof(double);
   S.read_bytes = C.used;
   R.core.progress = C.take<unsigned>(MAX_CELLS * 16);
   g->d_stats.assign(np, nullptr);

@@ -349,3 +349,17 @@ def test_static_epoch_whose_scheduled_scratch_is_too_large_runs_on_another_engin
     assert (e.alloc_calls, e.free_calls) == calls
     np.testing.assert_allclose(eloss, o.run_epoch(mak=1, muf=1 << 30, lr=0.01)[1], rtol=1e-5, atol=2e-6)
     e.close()
+
+
+def test_losses_of_an_evaluation_are_the_same_bits_every_time():
+    """A tree's loss is a sum over its nodes that arrives in any order: it is kept in 64 bits, so what is left of the order (2^-53 of the
+    sum) disappears when it is rounded to a float."""
+    import paper_1705_09786_b200 as amp
+    g, inst = ir.tree(500, 36, 21, 5), data.tree_instances(n=300, vocab=500, min_leaves=30, max_leaves=200)
+    e = amp.Engine(g)
+    e.load_instances(inst)
+    e.set_params(wp.init_params(g))
+    first = e.eval(split=0, mak=64)[2]
+    for mak in (64, 64, 64, 64):
+        np.testing.assert_array_equal(e.eval(split=0, mak=mak)[2], first)
+    e.close()
