@@ -206,7 +206,8 @@ ampnet_status_t ampnet_set_params(ampnet_graph_t*, int32_t node, int32_t which, 
  * the whole model on several GPUs are averaged in place at the end of an epoch (Sec. 5) by a collective library.     */
 ampnet_status_t ampnet_param_device_ptr(ampnet_graph_t*, int32_t node, int32_t which, float** dev, int64_t* n);
 
-/* Statistics of the last run.  staleness_hist: 64 bins (updates between a gradient's forward and backward).
+/* Statistics of the last run.  staleness_hist: 64 bins (updates between a gradient's forward and backward).  The
+ * asynchronous engines for single-row messages and message programs do not count it for embeddings (their rows have no version).
  * fwd_msgs / bwd_msgs (messages consumed by the node) and the route fingerprint are collected in the
  * deterministic schedule only; the asynchronous schedule counts the total of node messages.                   */
 ampnet_status_t ampnet_get_node_stats(ampnet_graph_t*, int32_t node, int64_t* n_updates, int64_t* n_grads_applied,
@@ -216,35 +217,42 @@ ampnet_status_t ampnet_get_update_log(ampnet_graph_t*, int32_t node, int32_t* n_
 /* Key bookkeeping of the last deterministic run: instance, slot, admission round, release round.             */
 ampnet_status_t ampnet_get_key_log(ampnet_graph_t*, int64_t* inst, int32_t* slot, int64_t* admit_round,
                                    int64_t* release_round, int64_t cap, int64_t* n);
-/* Number of keyed cache entries (join counters, recorded origins) still set after the last run; the
- * forward/backward state invariant of Sec. 4 makes this 0.                                                   */
+/* What the last run left unanswered; the forward/backward state invariant of Sec. 4 makes this 0.  Scheduled engine (the usual
+ * one of asynchronous runs): payload rows of the admitted instances' message programs, less the rows the cells worked on, summed
+ * over the cells (that every message of a program is answered was checked when it was made).  Other engines: keyed cache entries
+ * (join counters, recorded origins) still set.                                                                                  */
 ampnet_status_t ampnet_leftover_cache_entries(ampnet_graph_t*, int64_t* n);
-/* Placement chosen for a parameterised node: number of row tiles (CTAs) and micro-batch row capacity.  Asynchronous
- * runs of graphs that the direct-delivery engine takes (single-row messages; Cond, Phi, Isu, Bcast, Concat, Sink and a
- * Loss fed by a Linear node) report the forward row tiles; a Linear node has backward column tiles besides (none for a
- * node that feeds a Loss: each of its tiles holds all rows, does both directions and takes its share of the messages). */
+/* Placement chosen for a parameterised node in the last run: number of CTAs and micro-batch row capacity.  The scheduled engine
+ * reports the CTAs of the node's forward cell (GRU: of its z and r gates) and the rows it stages at a time; gradients and
+ * accumulators have CTAs of their own besides.  The direct-delivery engine reports the forward row tiles, the interpreter engine
+ * the row tiles.                                                                                                                */
 ampnet_status_t ampnet_get_placement(ampnet_graph_t*, int32_t node, int32_t* n_tiles, int32_t* batch_rows);
 
-/* Where the leader tile of a node spent its SM cycles in the last run: [0] waiting for messages, [1] fetching a
+/* Where a node's CTAs spent their SM cycles in the last run.  Scheduled engine: [0..5] first CTA of the forward cell, [8..13] first
+ * CTA of the input-gradient cell (embedding: of the gradient cell), both as {waiting for the round's rows to be listed, waiting for
+ * the cells it reads, gathering rows, product, output and the rest, loss of a loss head}; accumulator: [6] waiting, [7] gathering,
+ * [14] products, [15] the rest and updates.  Interpreter engine, leader tile: [0] waiting for messages, [1] fetching a
  * batch descriptor, [2] loading headers, [3] staging + arithmetic, [4] local updates, [5] barrier among the node's
  * tiles, [6] emission (walking the parameter-free nodes), [7] loop overhead; [8..15] detail of the emission phase
  * ([8] look-ahead scheduling, [9] reduction of partial gradients, [10]/[12] own walks of warps 0/1, [11]/[13] helping
- * other warps, [14] closing barrier).  After a run of the direct-delivery engine the 16 values are diagnostic marks of
+ * other warps, [14] closing barrier).  Direct-delivery engine: the 16 values are diagnostic marks of
  * the node's first forward tile ([0] waiting for and taking messages, [1] keys, routes and staging of the input rows,
  * [2] rest of the arithmetic phase, [3] update / reload of the weights, [4] arrivals and closing barrier, [5] products,
  * [6] activation and stores / Loss and gradients of a loss head, [7] delivery of those gradients) and, for a Linear node with column tiles, [8..14] of its first backward
  * tile in the same order of work (wait, routes and staging, incoming gradient, input gradient and delivery,
  * accumulation, update and publication, arrivals).  cycles16: 16 values.  batches: micro-batches executed.        */
 ampnet_status_t ampnet_get_phase_cycles(ampnet_graph_t*, int32_t node, uint64_t* cycles16, int64_t* batches);
-/* Queue occupancy of a node in the last asynchronous run (the benchmark set's stress configuration asks for it; App. A:
- * every worker owns a queue): the largest number of messages that were waiting in the node's forward and in its
- * backward ring at the moment a micro-batch was taken, as seen by the node's first tile.  The deterministic schedule
- * and graphs that run on the interpreter engine report 0.                                                        */
+/* Most work that was pending for a node at one time in the last asynchronous run (the benchmark set's stress configuration asks for
+ * it; App. A: every worker owns a queue).  Scheduled engine, which has no queues: the largest number of payload rows that one round
+ * had for the node's forward and for its backward cell (the classifier in front of a Loss works in both directions at once: 0
+ * backward; an embedding's two cells each).  Direct-delivery engine: the largest number of messages that were waiting in the node's
+ * forward and in its backward ring at the moment a micro-batch was taken, as seen by the node's first tile.  The deterministic
+ * schedule and the interpreter engine report 0.                                                                                  */
 ampnet_status_t ampnet_get_queue_occupancy(ampnet_graph_t*, int32_t node, int64_t* max_pending_fwd, int64_t* max_pending_bwd);
 /* Micro-batches of a node in the last run by the unit that ran their product (the stress configuration of the benchmark
  * set asks for this split): tensor_core_batches = forward micro-batches whose product Y^T = W X^T ran as tcgen05
- * instructions (bf16 runs on the direct-delivery engine: nodes with out_dim a multiple of 64 and in_dim a multiple of
- * 16; W and the batch as bfloat16 operands in shared memory, fp32 accumulator in tensor memory; the master weights,
+ * instructions (asynchronous bf16 runs and evaluations of graphs whose messages are single rows that go to at most two places: nodes
+ * with out_dim a multiple of 64 and in_dim a multiple of 16, batches of more than four rows; W and the batch as bfloat16 operands in shared memory, fp32 accumulator in tensor memory; the master weights,
  * the input gradient and the accumulation stay fp32), fma_batches = all others (counted like micro_batches of the epoch
  * statistics: by the node's first forward and first backward tile).  Either pointer may be NULL.                 */
 ampnet_status_t ampnet_get_micro_batch_split(ampnet_graph_t*, int32_t node, int64_t* fma_batches, int64_t* tensor_core_batches);

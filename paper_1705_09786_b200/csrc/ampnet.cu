@@ -105,6 +105,7 @@ struct ampnet_graph {
   int ctl_trials = 0, ctl_choice = -1;
   double ctl_rate[2] = {0.0, 0.0};
   std::vector<std::pair<size_t, size_t>> leftover_regions;   // (offset, bytes) inside ctl
+  long long leftover_rows = 0;                               // scheduled engine: program rows of the last run that no cell worked on
   std::vector<std::pair<void*, size_t>> zero_regions;        // parts of the bulk arena that must start a run at zero
   std::vector<PPTStats*> d_stats;
   std::vector<int*> d_update_log;
@@ -1143,8 +1144,21 @@ ampnet_status_t wave_execute(ampnet_graph* g, HostDataset& D, const WavePlan& P,
     const double* sums = reinterpret_cast<const double*>(g->host_read + S.loss_at);
     for (long long i = 0; i < D.n; i++) per_instance_loss[i] = (float)sums[i];
   }
+  const unsigned long long* ph = reinterpret_cast<const unsigned long long*>(g->host_read + S.phases_at);
+  const long long* left = reinterpret_cast<const long long*>(g->host_read + S.rows_left_at);
+  for (size_t k = 0; k < P.teams.size(); k++) {                  // (cycles of the cells' first CTAs, as ampnet_get_phase_cycles lays them out)
+    g->leftover_rows += std::llabs(left[k]);
+    const wave::Team& t = P.teams[k].t;
+    const unsigned long long* c = ph + k * wave::N_PHASES;
+    unsigned long long* to = g->last_stats[t.ppt].phase_cycles;
+    switch (t.kind) {
+      case wave::LIN_F: case wave::HEAD: case wave::GRU_ZR: case wave::LOOKUP_F: std::copy(c, c + wave::N_PHASES, to); break;
+      case wave::LIN_DX: case wave::GRU_DC: case wave::LOOKUP_B: std::copy(c, c + wave::N_PHASES, to + 8); break;
+      case wave::ACC: if (!t.pad) { to[6] = c[0] + c[1]; to[7] = c[2]; to[14] = c[3]; to[15] = c[4] + c[5]; } break;
+      default: break;
+    }
+  }
   if (getenv("AMPNET_DEBUG")) {
-    const unsigned long long* ph = reinterpret_cast<const unsigned long long*>(g->host_read + S.phases_at);
     for (size_t k = 0; k < P.teams.size(); k++) {
       const wave::Team& t = P.teams[k].t;
       static const char* names[] = {"LOOKUP_F", "LOOKUP_B", "LIN_F", "LIN_DX", "ACC", "HEAD", "GRU_ZR", "GRU_C", "GRU_DC", "GRU_DZR"};
@@ -1182,6 +1196,7 @@ ampnet_status_t execute(ampnet_graph* g, int split, int mak, int det, int eval, 
   const bool dbg = getenv("AMPNET_DEBUG") != nullptr;
   CUDA_TRY(g, cudaSetDevice(g->device));
   g->have_run = false;                // planning re-targets the statistics pointers: the previous run's are gone from here on
+  g->leftover_rows = 0;
   WavePlan wp;
   ampnet_status_t st = AMPNET_ENOMEM;
   if (scheduled && wave_takes(g, D, mak, det, eval, cfg, n_order, wp)) st = wave_execute(g, D, wp, mak, eval, cfg, order, n_order, out, per_instance_loss, accuracy, inference_only, inference);
@@ -1714,7 +1729,7 @@ ampnet_status_t ampnet_get_key_log(ampnet_graph_t* g, int64_t* inst, int32_t* sl
 ampnet_status_t ampnet_leftover_cache_entries(ampnet_graph_t* g, int64_t* n) {
   if (!g || !n) return AMPNET_EINVAL;
   if (!g->have_run) return set_err(g, AMPNET_ESTATE, "no run yet");
-  int64_t cnt = 0;
+  int64_t cnt = g->leftover_rows;
   std::vector<unsigned char> h;
   for (auto& r : g->leftover_regions) {
     h.resize(r.second);
@@ -1826,5 +1841,6 @@ extern "C" ampnet_status_t ampnet_run_epoch_static(ampnet_graph_t* g, const ampn
   g->arenas_lent = false;
   g->ctl_mem = own_ctl; g->ctl_cap = own_ctl_cap; g->bulk_mem = own_bulk; g->bulk_cap = own_bulk_cap;
   g->leftover_regions.clear();      // they described the lent memory
+  g->leftover_rows = 0;
   return st;
 }

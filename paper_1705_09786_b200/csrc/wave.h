@@ -129,6 +129,7 @@ struct Core {                          // what every CTA keeps in shared memory
   const unsigned char* inference_only;
   double* loss_out;                    // per instance: sums over its Loss messages, whatever order they come in
   unsigned long long* phases;          // [teams][N_PHASES]
+  long long* rows_left;                // [teams]: rows that the instances admitted have for the cell, less those it worked on
   const float* dense; int dense_dim;
   int n_teams, mak, eval, bf16, lag, pace, n_ctas;      // pace: most instances admitted in one round
   float lr; int opt; float mu, beta1, beta2, eps;

@@ -239,7 +239,7 @@ __device__ __forceinline__ int helper_scan(const int v, int& total) {          /
   return s - v + (warp > 0 ? a : 0) + (warp > 1 ? b : 0) + (warp > 2 ? c : 0);
 }
 
-__device__ __noinline__ void helper_main(const int cta, const int tile, const int shard, unsigned char* smem, const unsigned long long t0) {
+__device__ __noinline__ void helper_main(const int team, const int cta, const int tile, const int shard, unsigned char* smem, const unsigned long long t0) {
   IN_SMEM(smem);
   const int ht = threadIdx.x - CT;
   const Team& T = S.team;
@@ -261,7 +261,7 @@ __device__ __noinline__ void helper_main(const int cta, const int tile, const in
   int max_active = 0;
   bool finishing = true;
   unsigned max_rows = 0;
-  long long inf_instances = 0;
+  long long inf_instances = 0, expected = 0;
   bar_helper();
   auto publish = [&](int count, int flags, int n_upd) {
     if (ht == 0) { Head h; h.round = round; h.count = count; h.flags = flags; h.n_upd = n_upd; h.upd_t = n_updates; h.n_updates = n_updates - ((flags & H_UPDATE) ? 1 : 0); h.total = 0; h.pad = 0; S.hd[buf] = h; }
@@ -289,6 +289,7 @@ __device__ __noinline__ void helper_main(const int cta, const int tile, const in
           L.base4[s] = b == home + (unsigned)S.core.copies * S.core.slot4 ? home : b;
           L.inst[s] = (int)i | (ev && !EVALUATING ? (int)0x80000000 : 0);
           if (cta == 0) { node_msgs += ev ? h.msgs_eval : h.msgs; inf_instances += ev && !EVALUATING; }
+          if (tile == 0 && shard == 0 && !(backward && ev)) expected += (long long)__ldg(tab + L.end[s]) - (long long)__ldg(tab + h.tab);
         }
       }
       next += admitted;
@@ -398,7 +399,7 @@ __device__ __noinline__ void helper_main(const int cta, const int tile, const in
     round++;
     if (ht == 0) S.helper_stop = *(volatile int*)&S.stop;
     bar_helper();                                                 // (the slot tables are used up)
-    if (S.helper_stop) return;
+    if (S.helper_stop) { if (expected) atomicAdd(reinterpret_cast<unsigned long long*>(S.core.rows_left + team), (unsigned long long)expected); return; }
   }
   // ---- the end: the leftover gradients are applied once more --------------------------------------------------------------
   int n_upd = 0;
@@ -409,6 +410,7 @@ __device__ __noinline__ void helper_main(const int cta, const int tile, const in
   chunk_empty(&S.empty[buf], parity, t0);
   publish(0, H_END | (n_upd ? H_UPDATE : 0), n_upd);
   // ---- statistics ----------------------------------------------------------------------------------------------------------
+  if (expected) atomicAdd(reinterpret_cast<unsigned long long*>(S.core.rows_left + team), (unsigned long long)expected);
   PPTStats& st = *S.ppt.stats;
   const bool counts_msgs = leader && kind != GRU_C && kind != GRU_DZR && !(kind == ACC && !S.ppt.source_adj);
   if (counts_msgs && n_msgs) atomicAdd(&st.msgs, n_msgs * (kind == HEAD && !EVALUATING ? 2ull : 1ull));
@@ -1699,7 +1701,7 @@ extern "C" __global__ void __launch_bounds__(NT, 1) ENGINE_KERNEL(const __grid_c
   const int T = S.team.T, tile = idx % T, shard = idx / T;
   RowD* const rows = reinterpret_cast<RowD*>(smem + slots_bytes(C.core.mak));
   float* const work = reinterpret_cast<float*>(rows + 2 * S.team.BM);
-  if (tid >= CT) helper_main(cta, tile, shard, smem, t0);
+  if (tid >= CT) helper_main(team, cta, tile, shard, smem, t0);
   else switch (S.team.kind) {
     case LIN_F:
       if (S.team.bf16_tc) forward_main<F_TENSOR>(team, tile, work, rows, t0);
@@ -1719,6 +1721,7 @@ extern "C" __global__ void __launch_bounds__(NT, 1) ENGINE_KERNEL(const __grid_c
 #endif
   }
   __syncthreads();
+  if (tile == 0 && tid == 0 && S.batch_rows) atomicAdd(reinterpret_cast<unsigned long long*>(C.core.rows_left + team), 0ull - S.batch_rows);
   if (idx == 0 && tid < N_PHASES) C.core.phases[team * N_PHASES + tid] = S.phase[tid];
   // micro-batches, staleness
   PPTStats& st = *S.ppt.stats;

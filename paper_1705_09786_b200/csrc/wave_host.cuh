@@ -502,7 +502,7 @@ static WavePlan wave_place(const ampnet_graph* g, const WaveModel& M, const Wave
 // ---- a run -----------------------------------------------------------------------------------------------------------------------
 // Carves the run's scratch from the handle's arenas (dry: sizes only) and fills the kernel's argument.  What the host reads
 // back and what must start at zero lies together at the front of the control arena.
-struct WaveScratch { size_t zero_bytes, read_bytes, stats_at, loss_at, node_msgs_at, phases_at; };
+struct WaveScratch { size_t zero_bytes, read_bytes, stats_at, loss_at, node_msgs_at, phases_at, rows_left_at; };
 static WaveScratch wave_carve(ampnet_graph* g, HostDataset& D, const WaveModel& M, const WaveData& W, const WavePlan& P, int mak, int eval, const ampnet_run_cfg_t* cfg,
                               long long n_order, bool dry, wave::Run& R) {
   using namespace wave;
@@ -521,6 +521,8 @@ static WaveScratch wave_carve(ampnet_graph* g, HostDataset& D, const WaveModel& 
   S.node_msgs_at = C.used - g->hnodes.size() * 2 * sizeof(unsigned long long);
   R.core.phases = C.take<unsigned long long>(MAX_CELLS * N_PHASES);
   S.phases_at = C.used - MAX_CELLS * N_PHASES * sizeof(unsigned long long);
+  R.core.rows_left = C.take<long long>(MAX_CELLS);
+  S.rows_left_at = C.used - MAX_CELLS * sizeof(long long);
   const size_t nl = (size_t)std::max<long long>(D.n, 1);
   R.core.loss_out = C.take<double>(nl);
   S.loss_at = C.used - nl * sizeof(double);

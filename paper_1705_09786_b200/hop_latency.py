@@ -1,10 +1,11 @@
 """Where the time of one instance goes when a single key is in flight: `python -m paper_1705_09786_b200.hop_latency`.
 
-With max_active_keys = 1 nothing overlaps, so the latency of an instance is the sum of its hops and the kernel's own cycle
-counters (ampnet_get_phase_cycles: the first forward and the first backward tile of every parameterised node) split it
-into the time those tiles worked and the time they waited for the next message.  What is left after the work of all
-nodes is the hand-over between tiles: arrival counters, ticket, entry store, the consumer's poll.  The asynchronous mode
-of the MLP, list and tree workloads (the direct-delivery engine) is measured; sizes are kept small (seconds).
+With max_active_keys = 1 no two instances overlap: in every round the cells that have a row of the instance work on it and the cells
+that read them wait.  The kernel's own cycle counters (ampnet_get_phase_cycles: the first CTA of every cell) say how long each cell
+worked.  A dense row is in one cell at a time, so what is left of its latency is the hand-over from one cell to the next: fence,
+counter and poll, and the block barriers around them (the "output" phase holds a cell's own fence).  The tokens of a list and the
+nodes of a tree work side by side, so there the cells' times add up to more than the latency.  Accumulators are beside the way.
+Asynchronous epochs of the MLP, list and tree workloads are measured; sizes are kept small (seconds).
 """
 import argparse
 
@@ -17,8 +18,7 @@ from . import Engine
 CASES = {"mlp": (lambda: ir.mlp((784, 256, 256, 10)), lambda n: data.mlp_instances(n=n), 2048, 32),
          "rnn": (ir.rnn, lambda n: data.list_instances(n=n), 3000, 50),
          "tree": (ir.tree, lambda n: data.tree_instances(n=n), 600, 100)}
-F_PHASES = ("front", "rest", "update", "arrive", "product", "epilogue/loss", "loss-head dx")       # phase marks 1..7 of a forward tile
-B_PHASES = ("front", "dpre", "dx", "accumulate", "update", "arrive")                                # marks 9..14 of a backward tile
+PHASES = ("gather", "product", "output", "loss")       # marks 2..5 of a forward cell, 10..13 of an input-gradient cell
 
 
 def measure(family, sm_mhz):
@@ -36,13 +36,14 @@ def measure(family, sm_mhz):
     for node in g.ppt_nodes():
         a, _ = e.phase_cycles(node)
         us = a.astype(np.float64) / sm_mhz / inst.n                    # microseconds per instance
-        f_busy, b_busy = us[1:8].sum() + us[15], us[9:15].sum()
+        parts = lambda v: ", ".join(f"{k} {x:.2f}" for k, x in zip(PHASES, v) if x >= 0.005)
+        f_busy, b_busy, acc = us[2:6].sum(), us[10:14].sum(), us[7] + us[14] + us[15]
         busy_total += f_busy + b_busy
-        f = ", ".join(f"{k} {v:.2f}" for k, v in zip(F_PHASES, us[1:8]) if v >= 0.005)
-        b = ", ".join(f"{k} {v:.2f}" for k, v in zip(B_PHASES, us[9:15]) if v >= 0.005)
-        lines.append(f"  {g.names[node]:<12} forward tile works {f_busy:6.2f} us per instance ({f})" +
-                     (f"; backward tile {b_busy:6.2f} us ({b})" if b_busy > 0 else ""))
-    lines.append(f"  tiles at work {busy_total:.1f} us, hand-overs and the controller {per_inst - busy_total:.1f} us per instance")
+        lines.append(f"  {g.names[node]:<12} forward cell works {f_busy:6.2f} us per instance ({parts(us[2:6])})" +
+                     (f"; gradient cell {b_busy:6.2f} us ({parts(us[10:14])})" if b_busy > 0 else "") +
+                     (f"; accumulator {acc:6.2f} us" if acc > 0 else ""))
+    lines.append(f"  these cells together {busy_total:.1f} us per instance" +
+                 (f", hand-overs {per_inst - busy_total:.1f} us" if family == "mlp" else " (messages of one instance work in several at a time)"))
     e.close()
     return lines
 

@@ -363,3 +363,33 @@ def test_losses_of_an_evaluation_are_the_same_bits_every_time():
     for mak in (64, 64, 64, 64):
         np.testing.assert_array_equal(e.eval(split=0, mak=mak)[2], first)
     e.close()
+
+
+@pytest.mark.parametrize("family,size,n", [("mlp", (61, 258, 7), 120), ("tree", (60, 36, 21, 5), 60), ("ggnn", (15, 25, 3), 40)])
+def test_statistics_of_an_asynchronous_run_say_what_happened(family, size, n):
+    """Phase cycles of every node's cells, within the run's own time; no row of a program is left over, unless the run gave up."""
+    import paper_1705_09786_b200 as amp
+    g, inst = _case(family, size, n)
+    e = amp.Engine(g)
+    e.load_instances(inst)
+    p = wp.init_params(g)
+    e.set_params(p)
+    st, _ = e.run_epoch(mak=16, muf=20, lr=1e-4, timeout_s=60)
+    assert e.leftover_cache_entries() == 0
+    for i in g.ppt_nodes():
+        c, batches = e.phase_cycles(i)
+        assert batches > 0 and c[2:6].sum() + c[4] > 0, g.names[i]
+        kind, flags = int(g.nodes[i][0]), int(g.nodes[i][7])
+        into_loss = any(s == i and int(g.nodes[d][0]) in (ir.LOSS_CE, ir.LOSS_MSE) for s, _, d, _ in g._edges)
+        assert (c[8:14].sum() > 0) == (kind != ir.LINEAR or not (flags or into_loss)), g.names[i]
+        assert (c[14] > 0) == (kind != ir.LOOKUP), g.names[i]
+        for cell in (c[0:6], c[8:14], c[[6, 7, 14, 15]]):
+            assert cell.sum() <= 2.2e9 * (st.seconds + 1e-3), g.names[i]            # (no SM clock is above 2.2 GHz)
+    e.set_params(p)
+    with pytest.raises(amp.AmpnetError):
+        e.run_epoch(mak=16, muf=20, lr=1e-4, timeout_s=1e-5)
+    assert e.leftover_cache_entries() > 0
+    e.set_params(p)
+    e.run_epoch_mixed(mak=16, muf=20, lr=1e-4, inference_only=(np.arange(n) % 3 == 0), timeout_s=60)
+    assert e.leftover_cache_entries() == 0
+    e.close()
