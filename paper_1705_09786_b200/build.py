@@ -1,4 +1,5 @@
-"""Build step: compiles csrc/ampnet.cu and csrc/engine_fast.cu into libampnet.so (in-tree) for sm_100a with nvcc."""
+"""Build step: compiles the sources under csrc/ into libampnet.so (in-tree) for sm_100a with nvcc."""
+import glob
 import os
 import subprocess
 
@@ -7,8 +8,8 @@ SRC = os.path.join(_DIR, "csrc", "ampnet.cu")
 SRC_HOST = os.path.join(_DIR, "csrc", "ir_builders.cpp")
 SRC_DIRECT = os.path.join(_DIR, "csrc", "engine_fast.cu")
 SRC_WAVE = [os.path.join(_DIR, "csrc", f) for f in ("wave_engine.cu", "wave_forward.cu", "wave_moments.cu", "wave_encode.cu")]
-DEPS = [SRC, SRC_HOST, SRC_DIRECT, *SRC_WAVE, os.path.join(_DIR, "csrc", "engine.cuh"), os.path.join(_DIR, "csrc", "engine_types.h"),
-        os.path.join(os.path.dirname(_DIR), "include", "ampnet.h")]
+# whatever the sources include: every file beside them, and the public header
+DEPS = sorted(glob.glob(os.path.join(_DIR, "csrc", "*"))) + [os.path.join(os.path.dirname(_DIR), "include", "ampnet.h")]
 LIB = os.path.join(_DIR, "libampnet.so")
 
 

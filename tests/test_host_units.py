@@ -45,3 +45,26 @@ def test_shared_memory_limit_of_a_kernel_is_never_lowered_by_another_thread(tmp_
                            str(tmp_path / "smem.cpp"), "-o", str(tmp_path / "smem")])
     bad, calls = (int(v) for v in subprocess.check_output([str(tmp_path / "smem")], text=True, timeout=60).split())
     assert bad == 0 and 1 <= calls < 200
+
+
+def test_a_newer_file_of_the_sources_or_headers_is_a_reason_to_build(monkeypatch, tmp_path):
+    """Every quoted include of the sources is among the files whose time the build looks at."""
+    import re
+
+    from paper_1705_09786_b200 import build
+    csrc = os.path.dirname(build.SRC)
+    deps = {os.path.realpath(d) for d in build.DEPS}
+    for f in os.listdir(csrc):
+        assert os.path.realpath(os.path.join(csrc, f)) in deps
+        for inc in re.findall(r'#include "([^"]+)"', open(os.path.join(csrc, f)).read()):
+            assert os.path.realpath(os.path.join(csrc, inc)) in deps, (f, inc)
+    lib, dep = tmp_path / "lib.so", tmp_path / "wave_host.cuh"
+    lib.write_text("")
+    dep.write_text("")
+    monkeypatch.setattr(build, "LIB", str(lib))
+    monkeypatch.setattr(build, "DEPS", [str(dep)])
+    os.utime(lib, (1000, 1000))
+    os.utime(dep, (900, 900))
+    assert build.up_to_date()
+    os.utime(dep, (1100, 1100))
+    assert not build.up_to_date()
