@@ -781,8 +781,6 @@ struct RunPlan {
   bool direct = false;                // the run goes to the direct-delivery engine
 };
 
-inline bool eval_uses_classic(int) { return false; }
-
 ampnet_status_t plan_run(ampnet_graph* g, int split, int mak, int det, int eval, const ampnet_run_cfg_t* cfg,
                          long long n_order, bool dry, RunPlan& R) {
   HostDataset& D = g->data[split];
@@ -795,7 +793,7 @@ ampnet_status_t plan_run(ampnet_graph* g, int split, int mak, int det, int eval,
   int emit_ctas = (!det && !(tune & 32)) ? ((tune & 64) ? 1 : 2) : 0;
   const int mbr = cfg ? cfg->max_batch_rows : 0;
   ampnet_status_t st = AMPNET_EOVERFLOW;
-  R.direct = !eval_uses_classic(eval) && mbr == 0 && direct_candidate(g, D, det);
+  R.direct = mbr == 0 && direct_candidate(g, D, det);
   if (R.direct) {
     st = place_direct(g, n_ctas, R.roles);
     if (st == AMPNET_EOVERFLOW) R.direct = false;             // too few CTAs for its tiles: the interpreter engine places its own
@@ -1103,7 +1101,7 @@ bool wave_takes(ampnet_graph* g, HostDataset& D, int mak, int det, int eval, con
   // (the placement of the last run of this kind still holds if nothing it depends on has changed)
   const char* env[3] = {getenv("AMPNET_DIRECT_ROWS"), getenv("AMPNET_DIRECT_COLS"), getenv("AMPNET_TENSOR_CORES")};
   const int n_ctas = cfg && cfg->n_ctas > 0 ? std::min(cfg->n_ctas, g->n_sms) : g->n_sms;
-  wave::WavePlanKey key{D.wave.load_id, n_order, mak, cfg ? cfg->min_update_frequency : 1, eval, n_ctas, {env[0] ? atoi(env[0]) : -1, env[1] ? atoi(env[1]) : -1, env[2] ? atoi(env[2]) : -1}};
+  wave::WavePlanKey key{n_order, mak, cfg ? cfg->min_update_frequency : 1, eval, n_ctas, {env[0] ? atoi(env[0]) : -1, env[1] ? atoi(env[1]) : -1, env[2] ? atoi(env[2]) : -1}};
   auto& slot = D.wave_plan[eval ? 1 : 0];
   if (!(slot.first == key)) { slot.first = key; slot.second = wave_place(g, g->wave, D.wave, mak, key.muf, eval != 0, n_order, D.n, n_ctas); }
   P = slot.second;
@@ -1332,7 +1330,7 @@ ampnet_status_t ampnet_graph_create(const ampnet_ir_desc_t* ir, uint64_t init_se
   if (st == AMPNET_OK) {
     std::vector<int> pn;
     for (auto& P : g->ppts) pn.push_back(P.node);
-    wave_model(g->hnodes, g->sources, g->has_it ? g->it_steps + 1 : 1, g->payload_bf16, g->wave, pn);
+    wave_model(g->hnodes, g->sources, g->has_it ? g->it_steps + 1 : 1, g->wave, pn);
   }
   if (st == AMPNET_OK && (cudaEventCreate(&g->ev0) != cudaSuccess || cudaEventCreate(&g->ev1) != cudaSuccess)) st = AMPNET_ECUDA;
   if (st != AMPNET_OK) {

@@ -54,7 +54,7 @@ enum { H_FIRST = 1, H_LAST = 2, H_UPDATE = 4, H_END = 8, H_COPIES = 16, H_LONG =
 // A loop that may call sum_terms keeps nothing in flight across the call, so loops over rows exist twice.
 template <bool V> struct Flag { static constexpr bool value = V; };
 struct __align__(16) RowD { unsigned out4, a4, b4, meta; Term t[4]; int inst; unsigned base4; unsigned pad[2]; };
-struct Head { int round, count, flags, n_upd, upd_t, n_updates, total, pad; };
+struct Head { int round, count, flags, n_upd, upd_t, n_updates; };
 
 // Geometry of an accumulator's tile (floats and fours; smem offsets in floats; s*: powers of two).  It is read from shared memory in every
 // section of a chunk: kept in registers it drives the gradient sums out of them.
@@ -68,8 +68,7 @@ struct Shared {
   int stop, helper_stop, ok, ok2;
   unsigned long long ver;                      // what the ACC team had published `lag` rounds ago: updates << 32 | publications << 16 | round
   int warp_sum[4], sel;
-  unsigned long long batches, batch_rows, msgs, tc_batches;
-  unsigned max_pending;
+  unsigned long long batches, batch_rows, tc_batches;
   unsigned stale_hist[64]; int max_stale;
   int team_n[MAX_CELLS];
   unsigned long long phase[N_PHASES]; long long mark;
@@ -264,7 +263,7 @@ __device__ __noinline__ void helper_main(const int team, const int cta, const in
   long long inf_instances = 0, expected = 0;
   bar_helper();
   auto publish = [&](int count, int flags, int n_upd) {
-    if (ht == 0) { Head h; h.round = round; h.count = count; h.flags = flags; h.n_upd = n_upd; h.upd_t = n_updates; h.n_updates = n_updates - ((flags & H_UPDATE) ? 1 : 0); h.total = 0; h.pad = 0; S.hd[buf] = h; }
+    if (ht == 0) { Head h; h.round = round; h.count = count; h.flags = flags; h.n_upd = n_upd; h.upd_t = n_updates; h.n_updates = n_updates - ((flags & H_UPDATE) ? 1 : 0); S.hd[buf] = h; }
     mbar_arrive(&S.full[buf]);                                     // (release: the rows written before are visible to whoever sees the phase)
     buf ^= 1;
     if (buf == 0) parity ^= 1;

@@ -14,12 +14,11 @@ static Lay lay(int nseg, int w) { return w % 4 == 0 ? Lay{1, nseg * w} : Lay{nse
 // node is fed by a Linear node of its own, and the padded layouts of joined payloads agree.
 using wave::WaveCell; using wave::WaveMat; using wave::WaveModel; using wave::WaveData; using wave::WaveTeam; using wave::WavePlan;
 
-static bool wave_model(const std::vector<DevNode>& nodes, const std::vector<int>& sources, int it_count, bool bf16, WaveModel& M, const std::vector<int>& ppt_nodes) {
+static bool wave_model(const std::vector<DevNode>& nodes, const std::vector<int>& sources, int it_count, WaveModel& M, const std::vector<int>& ppt_nodes) {
   using namespace wave;
   const int n = (int)nodes.size(), np = (int)ppt_nodes.size();
   M = WaveModel{};
   if (n > ENC_MAX_NODES || np > ENC_MAX_PPTS) return false;
-  (void)bf16;
   std::vector<Lay> L(n, Lay{-1, 0});            // -1: not known yet
   std::vector<char> sums(n, 0);
   for (int pass = 0; pass < 2 * n + 4; pass++)
