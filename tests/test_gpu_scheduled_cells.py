@@ -393,3 +393,71 @@ def test_statistics_of_an_asynchronous_run_say_what_happened(family, size, n):
     e.run_epoch_mixed(mak=16, muf=20, lr=1e-4, inference_only=(np.arange(n) % 3 == 0), timeout_s=60)
     assert e.leftover_cache_entries() == 0
     e.close()
+
+
+ENGINES = [("mlp", (61, 258, 7), 60, dict(env="direct")), ("rnn", (14, 36, 36, 10), 60, dict(env="direct")), ("tree", (60, 36, 20, 5), 40, dict(env="direct")),
+           ("rnn", (14, 36, 36, 10), 60, dict(env="classic")), ("ggnn", (15, 25, 3), 30, dict(env="classic")), ("tree_lstm", (60, 36, 20, 5), 30, dict(env="classic")),
+           ("tree", (60, 36, 20, 5), 40, dict(max_batch_rows=16)), ("ggnn", (15, 25, 3), 30, dict(max_batch_rows=32)), ("mlp", (61, 258, 7), 60, dict(mak=2100)),
+           ("ggnn", (15, 25, 3), 30, dict(n_ctas=14))]
+
+
+@pytest.mark.parametrize("family,size,n,how", ENGINES)
+def test_engines_behind_the_scheduled_one_match_oracle(oracle_mod, monkeypatch, family, size, n, how):
+    """Asynchronous epochs that the scheduled engine does not take: forced to another one, with a cap on a micro-batch's rows, with more keys
+    than it has slots for, with fewer CTAs than it has cells.  No update before the flush, so the order of execution cannot matter."""
+    import paper_1705_09786_b200 as amp
+    how = dict(how)
+    if "env" in how:
+        monkeypatch.setenv("AMPNET_ENGINE", how.pop("env"))
+    g, inst = _case(family, size, n)
+    p = wp.init_params(g)
+    o, e = oracle_mod.Oracle(g), amp.Engine(g)
+    for s in (o, e):
+        s.load_instances(inst)
+        s.set_params(p)
+    _, oloss = o.run_epoch(mak=1, muf=1 << 30, lr=1e-4)
+    _, eloss = e.run_epoch(**dict(dict(mak=16, muf=1 << 30, lr=1e-4, timeout_s=60), **how))
+    np.testing.assert_allclose(eloss, oloss, rtol=1e-5, atol=2e-6)
+    assert e.leftover_cache_entries() == 0
+    ep, op = e.get_params(), o.get_params()
+    for k in op:
+        assert np.abs(ep[k] - op[k]).max() <= 1e-4 * np.abs(op[k]).max(), (g.names[k[0]], k[1])
+    e.close()
+
+
+# lists of one digit have two tokens, trees of two leaves two embeddings, one branch and three classifications: with these thresholds every
+# node's updates fall on the end of an instance
+SEQUENCE_CASES = [("mlp", (61, 37, 3), 90, 1, None), ("mlp", (61, 258, 7), 60, 3, "momentum"), ("rnn", (14, 33, 33, 10), 80, 2, None), ("rnn", (14, 32, 32, 10), 80, 6, "adam"),
+                  ("tree", (60, 36, 21, 5), 60, 6, None), ("tree", (5000, 132, 36, 5), 60, 6, "momentum"), ("tree_lstm", (60, 36, 20, 5), 60, 6, None)]
+
+
+@pytest.mark.parametrize("family,size,n,muf,kind", SEQUENCE_CASES)
+def test_many_updates_with_one_key_in_flight_follow_the_oracle(oracle_mod, family, size, n, muf, kind):
+    """With one key in flight and updates that fall between instances there is one order of execution: two epochs of 10 to 180 updates a
+    node give the oracle's losses, update by update, and its parameters.  Rounding errors of 2^-24 per sum are carried on by every update:
+    ten times the tolerances of a single one."""
+    import paper_1705_09786_b200 as amp
+    if family == "rnn":
+        g, inst = ir.rnn(*size[:4]), data.list_instances(n=n, max_len=1)
+    elif family == "mlp":
+        g, inst = _case(family, size, n)
+    else:
+        g, inst = (ir.tree if family == "tree" else ir.tree_lstm)(*size), data.tree_instances(n=n, vocab=size[0], min_leaves=2, max_leaves=2)
+    p = wp.init_params(g)
+    o, e = oracle_mod.Oracle(g), amp.Engine(g)
+    for s in (o, e):
+        s.load_instances(inst)
+        s.set_params(p)
+        if kind:
+            s.set_optimizer(kind=kind, momentum=0.8, beta1=0.85, beta2=0.99, eps=1e-4)
+    for epoch in range(2):
+        _, oloss = o.run_epoch(mak=1, muf=muf, lr=0.02 if kind != "adam" else 0.002)
+        _, eloss = e.run_epoch(mak=1, muf=muf, lr=0.02 if kind != "adam" else 0.002, timeout_s=60)
+        np.testing.assert_allclose(eloss, oloss, rtol=1e-4, atol=2e-5)
+        for i in g.ppt_nodes():
+            assert e.node_stats(i)["n_updates"] == o.node_stats(i)["n_updates"] > 1
+            np.testing.assert_array_equal(e.update_log(i), o.update_log(i))
+        ep, op = e.get_params(), o.get_params()
+        for k in op:
+            assert np.abs(ep[k] - op[k]).max() <= 1e-3 * np.abs(op[k]).max(), (epoch, g.names[k[0]], k[1])
+    e.close()
