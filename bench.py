@@ -31,7 +31,7 @@ WORKLOADS = {
     "rnn": (ir.rnn, data.list_instances, 20000, 16, 50, 0.05),
     "tree": (ir.tree, data.tree_instances, 8544, 64, 100, 0.05),
     "ggnn": (ir.ggnn, data.graph_instances, 130000, 128, 200, 0.01),
-    # the tree model with the leaf operations of a tree grouped into one matrix message (Sec. 6); runs on the interpreter engine
+    # the tree model with the leaf operations of a tree grouped into one matrix message (Sec. 6)
     "tree_grouped": (lambda: ir.tree(grouped_leaves=True), data.tree_instances, 8544, 64, 100, 0.05),
     # the paper's sentiment model proper: binary Tree-LSTM (leaf and branch cells) on the same trees as "tree"
     "tree_lstm": (ir.tree_lstm, data.tree_instances, 8544, 64, 100, 0.05),
@@ -242,7 +242,8 @@ def micro_batch_split(eng, graph):
     total = max(1, c["micro_batches_fma"] + c["micro_batches_tensor_core"])
     return {"fma": c["micro_batches_fma"] / total, "tensor_core": c["micro_batches_tensor_core"] / total, **c,
             "note": "tensor cores (tcgen05, bf16 operands, fp32 accumulation) run the forward products of nodes with out_dim % 64 == 0 "
-                    "and in_dim % 16 == 0 in bf16 runs (the stress configuration's cells); everything else runs on FP32 FMA"}
+                    "and in_dim % 16 == 0 in bf16 runs of single-row graphs (the stress configuration's cells), batches of more than "
+                    "four rows; everything else runs on FP32 FMA"}
 
 
 def average_replicas(views, averaging, average_fn=None):
@@ -274,7 +275,7 @@ def roofline_object(rf, graph, inst, workload, flops, kernel_s, peak_tf, peaks, 
             "peak_derived_kind": f"148 SMs x 128 FP32 lanes x 2 x {sm_mhz:.0f} MHz ({peak_kind} max SM clock)",
             "concurrency_ceiling_instances_per_s": mak * rate_one_key,
             "concurrency_ceiling_kind": f"max_active_keys x the rate at one key in flight ({rate_one_key:.0f}/s on {n1} instances)",
-            "kernel": "one persistent launch per step (ampnet_engine_direct; ampnet_engine for graphs with row-wise groups)",
+            "kernel": "one persistent launch per step (ampnet_engine_scheduled)",
             "kernel_ms": kernel_s * 1e3, "algorithmic_flop_per_launch": flops, "flop_per_instance": F,
             "payload_bytes_per_instance": B, "resident_weight_roofline_instances_per_s": roof_inst,
             "weight_reload_roofline_instances_per_s": float(peaks.get("hbm_gbs", 6650.0)) * 1e9 / (rf.reload_bytes(graph, inst) / inst.n),
@@ -459,7 +460,7 @@ def run_ours(args):
                                replica_sync=averaging["note"]),
                 "roofline": roofline, "cpu_baseline": cpu,
                 "e2e": {"value": e2e_value, "unit": "instances/s", "h2d_bytes_per_step": input_bytes(inst),
-                        "d2h_bytes_per_step": int(inst.n * 4 + 512), "steps": e2e_steps},
+                        "d2h_bytes_per_step": int(inst.n * 8 + 512), "steps": e2e_steps},
                 "clocks": clocks, "gpu_launches": args.steps,
                 "step_ms": {"all": [round(1e3 * v, 3) for v in step_s], "best": 1e3 * min(step_s), "median": 1e3 * float(np.median(step_s)),
                             "note": "this rank's steps (CUDA events around launch + averaging)"},

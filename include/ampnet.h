@@ -5,9 +5,11 @@
  * messages keyed by instance flow through parameterised nodes (Linear, GRU cell, embedding lookup) and
  * control-flow nodes (Cond, Phi, Isu, Concat, Bcast, Group, Ungroup, Flatmap); every parameterised node
  * accumulates gradients locally and applies an SGD update once min_update_frequency gradients have
- * arrived (Sec. 3); max_active_keys bounds the instances in flight (Sec. 3).  On the device this is one
- * persistent kernel whose CTAs own row tiles of the parameterised nodes (weights and fp32 accumulators in
- * shared memory) and exchange messages through lock-free ring queues in device memory.
+ * arrived (Sec. 3); max_active_keys bounds the instances in flight (Sec. 3).  On the device an asynchronous epoch is one
+ * persistent kernel: the message passing of an instance is played through when it is loaded, CTAs own cells (tiles of a
+ * node's weights, or a share of its rows) with weights and fp32 accumulators in shared memory, and the cells execute the
+ * instances' programs in rounds.  The deterministic schedule, and what has no program, runs on kernels whose CTAs exchange
+ * messages through lock-free ring queues in device memory.
  *
  * Conventions.  Every call returns a status; nothing aborts the process or traps the GPU; every device-side
  * wait is bounded and reports AMPNET_ETIMEOUT.  Input arrays are caller-owned HOST memory and are copied.
@@ -159,7 +161,9 @@ typedef struct {
 } ampnet_instances_t;
 
 /* Copies the instances to the device and encodes their structure into routing tables (parents and child
- * slots of trees; out-edge, in-edge and per-type edge lists and ranks of graphs).  split: 0 train, 1 valid.  */
+ * slots of trees; out-edge, in-edge and per-type edge lists and ranks of graphs) and into message programs for the
+ * asynchronous runs (48 bytes of device memory per payload row and cell; a split without the memory for them, or with an
+ * instance beyond the encoder's bounds, is loaded without).  split: 0 train, 1 valid.                               */
 ampnet_status_t ampnet_load_instances(ampnet_graph_t*, int32_t split, const ampnet_instances_t*);
 
 /* ---- training (Sec. 3) ---------------------------------------------------------------------------------- */
@@ -259,8 +263,9 @@ ampnet_status_t ampnet_get_micro_batch_split(ampnet_graph_t*, int32_t node, int6
 
 /* ---- concurrent inference (Sec. 1: inference can run while the model trains; Sec. 6 reports inference throughput) --------
  * A training epoch in which the instances i with inference_only[i] != 0 (host array, one byte per loaded instance of
- * the training split) are only evaluated: their messages carry the evaluation flag, travel through the same queues and
- * micro-batch formation as the training messages (a micro-batch holds one kind only), cache nothing, produce no
+ * the training split) are only evaluated: they take turns with the training instances for keys and share the
+ * cells' rounds (on the engines with queues: the queues and micro-batch formation, a micro-batch holding one kind only),
+ * cache nothing, produce no
  * gradients and count towards no update; they occupy a key like any instance.  out->mean_loss is the mean over the
  * training instances, *inference (may be NULL) receives count, mean loss and accuracy of the others;
  * per_instance_loss is indexed by instance for both kinds.                                                        */

@@ -487,8 +487,11 @@ static WavePlan wave_place(const ampnet_graph* g, const WaveModel& M, const Wave
   // cell's fixed costs hide, admissions are spread over the steps of an instance.
   double entries = 0;
   for (int c : cells) entries += W.tot.entries[c];
-  // An instance that is a chain (a dense row, a list: about one message at a time) gains nothing from more company than keeps
-  // the rounds' fixed costs shared, and its gradients only get staler: four such instances start per round.
+  // An instance that is a chain (a dense row, a list: about one message at a time) brings one row at a time, and more of them in flight make
+  // gradients staler: four such instances start per round, which keeps some seventy lists of 5.5 digits in flight whatever max_active_keys
+  // above that.  Lists with 256 keys, update after 50, learning rate 0.05, ms an epoch / greatest staleness / mean loss after six epochs:
+  // 2 a round 50.1 / 8 / 0.60, 4 a round 29.1 / 15 / 0.62, 8 a round 21.4 / 29 / 0.66, 16 a round 18.7 / 53 / 0.94, all 18.6 / 54 / 0.84
+  // (16 keys: 88.0 / 4 / 0.61).  With Adam, update after 200, learning rate 2e-5: 51.6, 27.9, 19.3, 16.3, 16.2 ms and no loss for it.
   P.pace = mak;
   double forward_rows = 0;
   for (int c : cells) if (M.cells[c].forward && M.cells[c].kind != LOOKUP_F && M.cells[c].kind != GRU_C) forward_rows += W.tot.entries[c];
