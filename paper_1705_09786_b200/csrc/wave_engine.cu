@@ -1508,57 +1508,50 @@ __device__ __noinline__ void lookup_main(const int team, RowD* rows, const unsig
   });
   if ((end.flags & H_END) && tid == 0) red_relaxed(S.core.progress + team * 16 + (end.round & 15));      // nothing more is read
 }
-// A small table (its sums fit in shared memory): a thread owns columns and adds up its slice of the rows in a copy of the sums of
-// its own, several loads in flight.  Zipf-like ids pile up on a few rows, so the work is dealt by row, not by id.
-__device__ __noinline__ void lookup_grad_small_main(const int team, float* smem, RowD* rows, const unsigned long long t0) {
+// A small table (its sums fit in shared memory): a tile owns some columns of all rows of the table.  The gradients of a chunk are gathered
+// first, all rows at once (a sum over a graph's messages is three dependent trips to L2, and a thread that walked through the rows made
+// them one after the other: 39,000 cycles a round of the graph net); then a thread adds its slice of the rows to a column of a copy
+// of the sums of its own.  Zipf-like ids pile up on a few rows, so the work is dealt by row, not by id.
+__device__ __noinline__ void lookup_grad_small_main(const int team, const int tile, float* smem, RowD* rows, const unsigned long long t0) {
   IN_SMEM(smem); IN_SMEM(rows);
-  const int tid = threadIdx.x, out = S.ppt.out_dim, ids = S.ppt.in_dim, cols = (out + 31) & ~31, slices = S.team.R;
+  const int tid = threadIdx.x, out = S.ppt.out_dim, ids = S.ppt.in_dim, cw = S.team.C, slices = S.team.R, c0 = tile * cw, cn = min(cw, out - c0), n4 = (cn + 3) >> 2, ldv = cw + 4;
   const PptRun& P = S.ppt;
-  const int sl = tid / cols, c = tid - sl * cols;
-  float* const own = smem + (size_t)sl * ids * out + c;
-  const bool on = sl < slices && c < out;
-  int* const flag = reinterpret_cast<int*>(smem + (size_t)slices * ids * out);      // rows with gradients since the last update
-  const FastDiv dout(out);
-  for (int i = tid; i < slices * ids * out + ids; i += CT) smem[i] = 0.f;
+  const int cols = (cw + 31) & ~31, sl = tid / cols, c = tid - sl * cols;
+  float* const V = smem;                                          // gradients of a chunk's rows
+  float* const sums = V + (size_t)S.team.BM * ldv;
+  float* const own = sums + (size_t)sl * ids * cw + c;
+  const bool on = sl < slices && c < cn;
+  int* const flag = reinterpret_cast<int*>(sums + (size_t)slices * ids * cw);      // rows with gradients since the last update
+  const FastDiv dcw(cw);
+  for (int i = tid; i < slices * ids * cw + ids; i += CT) sums[i] = 0.f;
   bar_compute();
   chunk_loop(rows, team, t0, [&](const Head& h, const RowD* R) {
-    if (on) {
-      const float* const arena = reinterpret_cast<const float*>(S.core.arena);
-      if (h.flags & H_COPIES) {
+    gather_terms(h, R, c0 >> 2, n4, V, ldv);
+    cp_wait();
+    bar_compute();
+    phase(2);
+    if (on)
 #pragma unroll 4
-        for (int b = sl; b < h.count; b += slices) own[R[b].b4 * out] += __ldcg(arena + (size_t)R[b].t[0].src4 * 4 + c);
-      } else {
-#pragma unroll 1
-        for (int b = sl; b < h.count; b += 2 * slices) {
-          float g[2] = {0.f, 0.f};
-#pragma unroll
-          for (int q = 0; q < 2; q++) {
-            if (b + q * slices >= h.count) continue;
-            const RowD& r = R[b + q * slices];
-            const int nt = r.meta & E_NT, cc = c >> 2;
-            if (r.meta & E_OVERFLOW) { const float4 v = sum_terms(S.core.prog.ov + r.t[0].src4, r.base4, nt, cc); g[q] = (c & 3) == 0 ? v.x : (c & 3) == 1 ? v.y : (c & 3) == 2 ? v.z : v.w; continue; }
-#pragma unroll
-            for (int k = 0; k < 4; k++) { const Term t = r.t[k]; const unsigned d = (unsigned)cc - t.col4; if (k < nt && d < t.w4) g[q] += __ldcg(arena + (size_t)(t.src4 + d) * 4 + (c & 3)); }
-          }
-#pragma unroll
-          for (int q = 0; q < 2; q++) if (b + q * slices < h.count) own[R[b + q * slices].b4 * out] += rnd(S.core.bf16, g[q]);
-        }
-      }
-    }
+      for (int b = sl; b < h.count; b += slices) own[R[b].b4 * cw] += V[b * ldv + c];
     for (int b = tid; b < h.count; b += CT) flag[R[b].b4] = 1;
+    phase(3);
     if (h.flags & H_UPDATE) {
       wait_readers(h, t0);
       const OptStep os = opt_step(P.om, P.ov, P.opt_t0, h.n_upd, h.upd_t);
       bar_compute();
 #pragma unroll 1
-      for (int i = tid; i < ids * out; i += CT) {
+      for (int i = tid; i < ids * cw; i += CT) {
+        const int id = dcw.div(i), at = i - id * cw;
         float a = 0.f;
-        for (int s = 0; s < slices; s++) { float* q = smem + (size_t)s * ids * out + i; a += *q; *q = 0.f; }
-        if (flag[dout.div(i)]) P.W[i] = opt_one(os, P.W[i], a, i);      // (the other rows keep their weights and moments)
+#pragma unroll 4
+        for (int s = 0; s < slices; s++) { float* q = sums + (size_t)s * ids * cw + i; a += *q; *q = 0.f; }
+        const size_t k = (size_t)id * out + c0 + at;
+        if (at < cn && flag[id]) P.W[k] = opt_one(os, P.W[k], a, k);      // (the other rows keep their weights and moments)
       }
       bar_compute();
       for (int i = tid; i < ids; i += CT) flag[i] = 0;
       bar_compute();
+      phase(5);
     }
   });
 }
@@ -1737,7 +1730,7 @@ extern "C" __global__ void __launch_bounds__(NT, 1) ENGINE_KERNEL(const __grid_c
     case GRU_DC: input_grad_main<B_DC>(team, tile, work, rows, t0); break;
     case GRU_DZR: input_grad_main<B_DZR>(team, tile, work, rows, t0); break;
     case ACC: accumulate_main(team, tile, work, rows, t0); break;
-    case LOOKUP_B: if (S.team.R) lookup_grad_small_main(team, work, rows, t0); else lookup_grad_main(team, tile, work, rows, t0); break;
+    case LOOKUP_B: if (S.team.R) lookup_grad_small_main(team, tile, work, rows, t0); else lookup_grad_main(team, tile, work, rows, t0); break;
 #endif
   }
   __syncthreads();
@@ -1784,7 +1777,7 @@ size_t smem_bytes(const Team& t, const Mat& m, int mak) {
       break;
     case LIN_DX: case GRU_DC: case GRU_DZR: f = (size_t)t.R * ldo + BM * ldo + BM * pad_ld(t.R); break;
     case ACC: f = (size_t)t.R * (t.C + 4) + ACC_RED + BM * (t.R + 4 + t.C + 4) + t.R + (size_t)(CW / (t.WO * t.WI)) * t.R; break;
-    case LOOKUP_B: f = t.R ? (size_t)(t.R + 1) * t.C : CW * (NEAR + PIECES) + LOOKUP_BITS; break;      // (small table: R copies of C sums)
+    case LOOKUP_B: f = t.R ? BM * (t.C + 4) + (size_t)t.G * (t.R * t.C + 1) : CW * (NEAR + PIECES) + LOOKUP_BITS; break;      // (small table of G rows: R copies of the sums of C columns)
     case HEAD: f = (size_t)m.outp * ldi + m.outp + BM * ldi + 2 * BM * pad_ld(m.outp); break;
     default: break;
   }

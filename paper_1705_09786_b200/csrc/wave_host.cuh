@@ -387,12 +387,18 @@ static bool wave_best(const WaveModel& M, int c, int ctas, double rows, double m
       }
       break;
     default: {    // LOOKUP_B: the sums of a small table in shared memory, otherwise rows dealt to tiles by id
-      const int cols = (h.out_dim + 31) & ~31;
-      if (cols <= 512 && (long long)h.in_dim * h.out_dim * 4 <= 48 * 1024) {
-        Team x = t;
-        x.R = 512 / cols; x.C = h.in_dim * h.out_dim;
-        while (x.R > 1 && (long long)x.R * x.C * 4 > 128 * 1024) x.R--;
-        offer(x, 2500 + rows / x.R * 500 + upd * (1500 + (double)x.C * x.R / 40.0));
+      // (small enough: one copy of the sums in 48 KB)
+      if (h.out_dim <= 512 && (long long)h.in_dim * h.out_dim * 4 <= 48 * 1024) {
+        bool sums = false;                                        // of more messages than a row's descriptor holds
+        for (auto& q : g->hnodes) sums |= q.type == NPT_SUMROWS || q.type == FLATMAP || (q.type == BCAST && q.fn_arg > 4);
+        for (int n = 1; n <= std::min(ctas, (h.out_dim + 3) / 4); n++) {
+          Team x = t;
+          x.C = pad4i((h.out_dim + n - 1) / n); x.T = x.n = (h.out_dim + x.C - 1) / x.C; x.G = h.in_dim;
+          if (x.T != n) continue;
+          x.R = 512 / ((x.C + 31) & ~31);
+          while (x.R > 1 && (long long)x.R * x.C * h.in_dim * 4 > 64 * 1024) x.R--;
+          offer(x, 3000 + std::ceil(rows * x.C / 4 / 512) * (sums ? 2500 : 900) + rows / x.R * 40 + upd * (1500 + (double)x.C * h.in_dim * (x.R + 8) / 200.0));
+        }
         break;
       }
       for (int n = 1; n <= std::min(ctas, std::max(1, h.in_dim / 8)) && (n == 1 || (long long)h.in_dim * n < (1ll << 31)); n++) {      // (the kernel divides ids by multiplication)
