@@ -16,6 +16,7 @@
 #include "../../include/ampnet.h"
 #include "engine.cuh"
 #include "kernel_smem.h"
+#include "tc_split.cuh"
 #include "wave.h"
 #include "wave_sizes.h"
 

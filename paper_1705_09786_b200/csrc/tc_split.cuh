@@ -1,0 +1,153 @@
+// Single-precision products on the tensor cores (sm_100a: tcgen05.mma with the accumulators in tensor memory).
+//
+//   Y[b][o] = sum_k X[b][k] W[o][k]          o < M (64 or 128), b < n rows, K a multiple of four
+//
+// Every operand is held as three bfloat16 parts whose sum is the 32-bit value (8 + 8 + 8 significant bits): x = h + m + l.  Six of the nine
+// products are formed, hh + (hm + mh) + (hl + mm + lh); the three left out are below 2^-24 of the whole.  The instruction truncates its
+// sums, so a long chain drifts towards zero (K = 304 in one chain: 2.3e-7 of the result against 1.2e-7 of a chain of 32-bit
+// multiply-adds): the hh products are dealt to several accumulators of at most CHAIN steps each, which meet in 32 bits, rounded to nearest (four
+// chains: 9e-8).  The small ones need one accumulator per order of magnitude.
+//
+// Operand layout (no swizzle): core matrices of 8 rows x 16 bytes, 128 contiguous bytes; along k they lie CORE_K = 144 bytes apart, so that
+// sixteen lanes which store 8 bytes each of one row's neighbouring columns meet all 32 banks; groups of eight rows lie K / 8 x 144 bytes apart.
+// The parts of the rows follow each other, n rows apart, and serve as one wider operand: W_h x [X_m X_l] is one instruction.
+#pragma once
+#include <stdint.h>
+
+namespace tc3 {
+
+constexpr unsigned CORE_K = 144;
+constexpr int CHAIN = 6;               // k steps (of sixteen) that one accumulator adds up at most
+constexpr int COLUMNS = 512;           // tensor memory of an SM
+
+__host__ __device__ __forceinline__ int k_steps(const int K) { return (K + 15) >> 4; }
+__host__ __device__ __forceinline__ int chains(const int K) { return (k_steps(K) + CHAIN - 1) / CHAIN; }
+__host__ __device__ __forceinline__ unsigned group_bytes(const int K) { return (unsigned)k_steps(K) * 2u * CORE_K; }      // of eight rows
+__host__ __device__ __forceinline__ int rows_padded(const int rows, const int M) { return M == 64 ? (rows + 7) & ~7 : (rows + 15) & ~15; }
+// rows of a chunk that the accumulators of all chains have room for
+__host__ __device__ __forceinline__ int max_rows(const int K) { const int r = COLUMNS / (chains(K) + 2); return r >= 128 ? 128 : r & ~15; }
+
+__device__ __forceinline__ unsigned smem_addr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
+
+// ---- operands ------------------------------------------------------------------------------------------------------
+// Two values as their upper, middle and lower parts, packed for two neighbouring columns.  The upper part is cut off, not rounded: it stays
+// finite where the value is, and the rest is exact.
+__device__ __forceinline__ void split(const float x, const float y, unsigned& h, unsigned& m, unsigned& l) {
+  const unsigned xb = __float_as_uint(x), yb = __float_as_uint(y);
+  h = __byte_perm(xb, yb, 0x7632);
+  float rx = x - __uint_as_float(xb & 0xffff0000u), ry = y - __uint_as_float(yb & 0xffff0000u);
+  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(m) : "f"(ry), "f"(rx));
+  rx -= __uint_as_float(m << 16); ry -= __uint_as_float(m & 0xffff0000u);
+  l = __byte_perm(__float_as_uint(rx), __float_as_uint(ry), 0x7632);      // (eight significant bits are left: exact)
+}
+// Columns 4 c4 .. of row r; the parts lie `part` bytes apart.
+__device__ __forceinline__ void store4(unsigned char* base, const unsigned part, const unsigned group, const int r, const int c4, const float4 v) {
+  unsigned char* const p = base + (unsigned)(r >> 3) * group + (unsigned)(c4 >> 1) * CORE_K + (unsigned)(r & 7) * 16u + (unsigned)(c4 & 1) * 8u;
+  uint2 h, m, l;
+  split(v.x, v.y, h.x, m.x, l.x); split(v.z, v.w, h.y, m.y, l.y);
+  *reinterpret_cast<uint2*>(p) = h; *reinterpret_cast<uint2*>(p + part) = m; *reinterpret_cast<uint2*>(p + 2 * part) = l;
+}
+__device__ __forceinline__ bool finite(const float v) { return fabsf(v) <= 3.4028235e38f; }
+__device__ __forceinline__ float value(const unsigned char* base, const unsigned part, const unsigned group, const int r, const int k) {
+  const unsigned char* const p = base + (unsigned)(r >> 3) * group + (unsigned)(k >> 3) * CORE_K + (unsigned)(r & 7) * 16u + (unsigned)(k & 7) * 2u;
+  auto at = [&](const unsigned o) { return __uint_as_float((unsigned)*reinterpret_cast<const unsigned short*>(p + o) << 16); };
+  const float h = at(0);
+  return finite(h) ? h + (at(part) + at(2 * part)) : h;
+}
+__device__ __forceinline__ void fence_operands() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+
+// ---- tensor memory: one warp allocates and frees ---------------------------------------------------------------------
+__device__ __forceinline__ void tmem_alloc(unsigned* slot_in_smem) {
+  asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" :: "r"(smem_addr(slot_in_smem)), "r"((unsigned)COLUMNS) : "memory");
+  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void tmem_free(const unsigned taddr) { asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(taddr), "r"((unsigned)COLUMNS) : "memory"); }
+
+// ---- the product ------------------------------------------------------------------------------------------------------
+__device__ __forceinline__ uint64_t smem_desc(const unsigned saddr, const unsigned group) {      // K-major: leading offset along k, stride offset between row groups
+  return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)(CORE_K >> 4) << 16) | ((uint64_t)((group >> 4) & 0x3FFFu) << 32) | (1ull << 46);
+}
+__host__ __device__ constexpr uint32_t instr_desc(const int m, const int n) { return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24); }
+__device__ __forceinline__ void mma(const unsigned d, const uint64_t a, const uint64_t b, const uint32_t idesc, const bool add) {
+  asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\ntcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" :: "r"(d), "l"(a), "l"(b), "r"(idesc), "r"((unsigned)add) : "memory");
+}
+// One thread issues the whole product and commits it to the mbarrier at `bar`; operands written, fenced (fence_operands) and the CTA
+// synchronised before.  Accumulators from column 0: the chains of hh, then hm + mh, then hl + mm + lh, n columns each.
+__device__ __forceinline__ void issue(const unsigned taddr, const unsigned char* Wb, const unsigned w_part, const unsigned char* Xb, const unsigned x_part, const unsigned group, const int M, const int n, const int K, const unsigned bar) {
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const int steps = k_steps(K), sets = chains(K);
+  uint64_t wh = smem_desc(smem_addr(Wb), group), xh = smem_desc(smem_addr(Xb), group);
+  const uint64_t wp = w_part >> 4, xp = x_part >> 4;
+  const uint32_t one = instr_desc(M, n), two = instr_desc(M, 2 * n);
+  const unsigned low = taddr + (unsigned)(sets * n), lowest = low + (unsigned)n;
+  unsigned d = taddr;
+  for (int s0 = 0; s0 < steps; s0 += CHAIN, d += (unsigned)n) {
+    const int s1 = min(s0 + CHAIN, steps);
+#pragma unroll 2
+    for (int s = s0; s < s1; s++) {
+      mma(d, wh, xh, one, s > s0);
+      mma(low, wh, xh + xp, two, s > 0);
+      mma(low, wh + wp, xh, two, true);
+      mma(lowest, wh + 2 * wp, xh, one, true);
+      wh += 2 * CORE_K >> 4; xh += 2 * CORE_K >> 4;
+    }
+  }
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" :: "r"(bar) : "memory");
+}
+// Eight columns of an accumulator in this warp's lanes (all lanes of the warp take part).
+__device__ __forceinline__ void load8(const unsigned a, unsigned (&u)[8]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];" : "=r"(u[0]), "=r"(u[1]), "=r"(u[2]), "=r"(u[3]), "=r"(u[4]), "=r"(u[5]), "=r"(u[6]), "=r"(u[7]) : "r"(a) : "memory");
+}
+__device__ __forceinline__ void load_wait(unsigned (&u)[8], unsigned (&v)[8]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;" : "+r"(u[0]), "+r"(u[1]), "+r"(u[2]), "+r"(u[3]), "+r"(u[4]), "+r"(u[5]), "+r"(u[6]), "+r"(u[7]),
+               "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]) :: "memory");
+}
+// One result in 32-bit multiply-adds, where the parts' is not finite: an infinity's lower parts are no numbers, and a sum of parts may pass the
+// largest number where the whole does not.
+static __device__ __noinline__ float dot_plain(const unsigned char* Wb, const unsigned w_part, const unsigned char* Xb, const unsigned x_part, const unsigned group, const int K, const int o, const int b) {
+  float v = 0.f;
+#pragma unroll 1
+  for (int k = 0; k < K; k++) v = fmaf(value(Xb, x_part, group, b, k), value(Wb, w_part, group, o, k), v);
+  return v;
+}
+// After the mbarrier has flipped: the sixteen warps add up the accumulators and store Y[b * ldy + o] for b < count, o < outs.  With M = 64
+// row o sits in lane o mod 16 of quadrant o / 16, otherwise in lane o mod 32 of quadrant o / 32; a warp reaches the quadrant of its index mod 4.
+__device__ __forceinline__ void collect(const unsigned taddr, const unsigned char* Wb, const unsigned w_part, const unsigned char* Xb, const unsigned x_part, const unsigned group, const int M, const int n, const int K, const int count, const int outs,
+                                        float* Y, const int ldy) {
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, q = warp & 3, sets = chains(K);
+  const int o = M == 64 ? 16 * q + lane : 32 * q + lane;
+  const bool mine = (M != 64 || lane < 16) && o < outs;
+  const unsigned t = taddr + ((unsigned)(32 * q) << 16);
+#pragma unroll 1
+  for (int c0 = (warp >> 2) * 8; c0 < count; c0 += 32) {
+    float v[8];
+    unsigned a[8], b[8];
+    load8(t + (unsigned)((sets + 1) * n + c0), a); load8(t + (unsigned)(sets * n + c0), b);
+    load_wait(a, b);
+#pragma unroll
+    for (int j = 0; j < 8; j++) v[j] = __uint_as_float(a[j]) + __uint_as_float(b[j]);
+#pragma unroll 1
+    for (int s = 0; s < sets; s += 2) {
+      load8(t + (unsigned)(s * n + c0), a);
+      if (s + 1 < sets) load8(t + (unsigned)((s + 1) * n + c0), b);
+      load_wait(a, b);
+#pragma unroll
+      for (int j = 0; j < 8; j++) v[j] += s + 1 < sets ? __uint_as_float(a[j]) + __uint_as_float(b[j]) : __uint_as_float(a[j]);
+    }
+    if (mine) {
+#pragma unroll
+      for (int j = 0; j < 8; j++) if (c0 + j < count) Y[(c0 + j) * ldy + o] = v[j];
+      float all = 0.f;                                             // (no number where one of the eight is not finite)
+#pragma unroll
+      for (int j = 0; j < 8; j++) all = fmaf(v[j], 0.f, all);
+      if (all != 0.f)
+#pragma unroll 1
+        for (int j = 0; j < 8; j++)
+          if (c0 + j < count && !finite(Y[(c0 + j) * ldy + o])) Y[(c0 + j) * ldy + o] = dot_plain(Wb, w_part, Xb, x_part, group, K, o, c0 + j);
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+}
+
+}  // namespace tc3

@@ -108,6 +108,7 @@ struct Team {                          // the CTAs of one cell
   int C, WO, WI, LO;                   // ACC: tile columns, warps along rows / columns, lanes along rows
   unsigned wait_mask;                  // cells whose previous round this one reads
   int act, bf16_tc, first, pad;        // first: lowest CTA index
+  int split;                           // M of the tensor-core products of 32-bit operands in three parts (64, 128); 0: multiply-adds
   int H4, lstm;                        // GRU / gate nodes: padded hidden width (float4), gate count
   int reader;                          // LOOKUP_B: team that reads the table's rows (-1: none)
   int keep, k4;                        // LIN_F: a summed input is stored for the accumulator; width of the rows' terms (float4)

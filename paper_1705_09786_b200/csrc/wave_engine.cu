@@ -13,7 +13,10 @@
 // updates of the one before; 2 otherwise: the reload then never waits).
 #include <cuda_bf16.h>
 
+#include <algorithm>
+
 #include "kernel_smem.h"
+#include "tc_split.cuh"
 #include "tc_tile.cuh"
 #include "wave.h"
 
@@ -880,11 +883,116 @@ __device__ __noinline__ void tensor_rows_general(const RowD* R, const int count,
   }
 }
 
+// ---- products of a tile on the tensor cores, 32-bit operands in three parts (tc_split.cuh) ---------------------------------
+struct Parts {                         // an operand in shared memory
+  unsigned char* base; unsigned part, group;
+  __device__ __forceinline__ void put(const int r, const int c4, const float4 v) const { tc3::store4(base, part, group, r, c4, v); }
+  __device__ __forceinline__ float4 get(const int r, const int c4) const {
+    return make_float4(tc3::value(base, part, group, r, 4 * c4), tc3::value(base, part, group, r, 4 * c4 + 1), tc3::value(base, part, group, r, 4 * c4 + 2), tc3::value(base, part, group, r, 4 * c4 + 3));
+  }
+};
+__host__ __device__ __forceinline__ size_t parts_bytes(const int rows, const int K) { return (size_t)3 * ((rows + 7) >> 3) * tc3::group_bytes(K); }
+// What gather_terms does, into parts.  Copies: four loads of a thread in flight whatever rows they belong to.
+template <bool CALL>
+__device__ __noinline__ void gather_general_parts(const RowD* rows, const int count, const int nc, const Parts X) {
+  IN_SMEM(rows); IN_SMEM(X.base);
+  const FastDiv dn(nc);
+#pragma unroll 1
+  for (int i = threadIdx.x; i < count * nc; i += CT) {
+    const int b = dn.div(i), c = i - b * nc;
+    const RowD& r = rows[b];
+    X.put(b, c, (r.meta & (E_DENSE | E_RAW)) ? dense4(r.inst, c) : rnd4(S.core.bf16, row_sum<CALL>(r, c)));
+  }
+}
+__device__ __noinline__ void gather_copies_parts(const RowD* rows, const int count, const int nc, const Parts X) {
+  IN_SMEM(rows); IN_SMEM(X.base);
+  const FastDiv dn(nc);
+  const float4* const arena = S.core.arena;
+  constexpr int U = 4;
+  const int n = count * nc;
+#pragma unroll 1
+  for (int i0 = threadIdx.x; i0 < n; i0 += U * CT) {
+    float4 v[U];
+#pragma unroll
+    for (int u = 0; u < U; u++) {
+      const int i = min(i0 + u * CT, n - 1), b = dn.div(i), c = i - b * nc;
+      const uint4 t = *reinterpret_cast<const uint4*>(&rows[b].t[0]);
+      const int cut = (int)(t.w & 0xffffu);
+      v[u] = ldcg4(arena + (c >= cut ? t.z + (c - cut) : t.x + c));
+    }
+#pragma unroll
+    for (int u = 0; u < U; u++) {
+      const int i = i0 + u * CT, b = dn.div(i), c = i - b * nc;
+      if (i < n) X.put(b, c, v[u]);
+    }
+  }
+}
+__device__ __forceinline__ void gather_parts(const Head& h, const RowD* rows, const int nc, const Parts X) {
+  if (h.flags & H_COPIES) gather_copies_parts(rows, h.count, nc, X);
+  else if (h.flags & H_LONG) gather_general_parts<true>(rows, h.count, nc, X);
+  else gather_general_parts<false>(rows, h.count, nc, X);
+}
+// Weights of a tile as parts: what first_rows / load_rows and first_cols / load_cols do.
+__device__ __noinline__ void first_parts(const Mat& m, const bool cols, const int G, const int gw, const int j0, const int jn, const Parts W, float* bs) {
+  IN_SMEM(&m); IN_SMEM(W.base);
+  const int rows = cols ? jn : G * jn, n4 = (cols ? m.outp : m.inp) >> 2;
+#pragma unroll 1
+  for (int i = threadIdx.x; i < rows * n4; i += CT) {
+    const int rr = i / n4, k = i - rr * n4, g = cols ? 0 : rr / jn, at = j0 + rr - g * jn;
+    float v[4];
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+      const int ro = cols ? real_out(m, 4 * k + q) : real_out(m, g * gw + at), ri = cols ? real_in(m, at) : real_in(m, 4 * k + q);
+      v[q] = (ro >= 0 && ri >= 0) ? m.W[(size_t)ro * m.in_real + ri] : 0.f;
+    }
+    W.put(rr, k, make_float4(v[0], v[1], v[2], v[3]));
+  }
+  if (!cols)
+#pragma unroll 1
+    for (int i = threadIdx.x; i < G * jn; i += CT) { const int g = i / jn, ro = real_out(m, g * gw + j0 + i - g * jn); bs[i] = ro >= 0 ? m.b[ro] : 0.f; }
+}
+__device__ __noinline__ void load_parts(const Mat& m, const unsigned pub, const bool cols, const int G, const int gw, const int j0, const int jn, const Parts W, float* bs) {
+  IN_SMEM(&m); IN_SMEM(W.base);
+  const float* const src = (cols ? m.WTp : m.Wp) + (size_t)(pub % PUB) * m.outp * m.inp;
+  const int width = cols ? m.outp : m.inp, n4 = width >> 2, rows = cols ? jn : G * jn, n = rows * n4;
+  const FastDiv dn(n4), dj(jn);
+  constexpr int U = 4;
+#pragma unroll 1
+  for (int i0 = threadIdx.x; i0 < n; i0 += U * CT) {
+    float4 v[U];
+#pragma unroll
+    for (int u = 0; u < U; u++) {
+      const int i = min(i0 + u * CT, n - 1), rr = dn.div(i), k = i - rr * n4, g = G > 1 ? dj.div(rr) : 0;
+      v[u] = ldcg4(reinterpret_cast<const float4*>(src + (size_t)(g * gw + j0 + rr - g * jn) * width) + k);
+    }
+#pragma unroll
+    for (int u = 0; u < U; u++) { const int i = i0 + u * CT, rr = dn.div(i); if (i < n) W.put(rr, i - rr * n4, v[u]); }
+  }
+  if (!cols) {
+    const float* const bp = m.bp + (size_t)(pub % PUB) * m.outp;
+#pragma unroll 1
+    for (int i = threadIdx.x; i < rows; i += CT) { const int g = G > 1 ? dj.div(i) : 0; bs[i] = __ldcg(bp + g * gw + j0 + i - g * jn); }
+  }
+}
+// Y[b][o] from the two operands; every compute thread comes here with its part of X written.
+__device__ __noinline__ void product_parts(const Parts W, const Parts X, const int M, const int n, const int K, const int count, const int outs, float* Y, const int ldy, unsigned& parity, const unsigned long long t0) {
+  IN_SMEM(W.base); IN_SMEM(X.base); IN_SMEM(Y);
+  tc3::fence_operands();
+  bar_compute();
+  phase(2);
+  if (threadIdx.x == 0) tc3::issue(S.tmem, W.base, W.part, X.base, X.part, W.group, M, n, K, smem_u32(&S.tc_mbar));
+  const bool done = mbar_wait(&S.tc_mbar, parity, t0, 26);
+  if (!done) for (unsigned extra = 0; extra < (1u << 16) && !mbar_try(&S.tc_mbar, parity); extra++) {}      // what was issued still writes the accumulators
+  parity ^= 1;
+  if (__all_sync(0xffffffffu, done)) tc3::collect(S.tmem, W.base, W.part, X.base, X.part, W.group, M, n, K, count, outs, Y, ldy);
+  bar_compute();
+}
+
 // ---- forward cell ----------------------------------------------------------------------------------------------------------
 // A tile holds R columns of every gate group (G = 1 for a Linear node, 2 for a GRU's z and r, 3 or 5 for an LSTM's gates) for all
 // inputs; a shard takes its part of the round's rows.  Bound by the latency of gather -> product -> store at the usual 10-60 rows.
 enum { F_PLAIN, F_TENSOR, F_ZR, F_C, F_LSTM };      // (a function per variant: a round runs through its code once, so it has to be short)
-template <int MODE>
+template <int MODE, bool SPLIT = false>
 __device__ __noinline__ void forward_main(const int team, const int tile, float* smem, RowD* rows, const unsigned long long t0) {
   IN_SMEM(smem);  IN_SMEM(rows);
   const Team& T = S.team; const Mat& m = S.mat;
@@ -893,8 +1001,9 @@ __device__ __noinline__ void forward_main(const int team, const int tile, float*
   const int j0 = tile * T.R, jn = min(T.R, gw - j0), nB = G * jn, K = m.inp, ld = pad_ld(K), n4 = K >> 2;
   constexpr bool tcm = MODE == F_TENSOR, lstm = MODE == F_LSTM;
   const int NTC = (T.BM + 15) & ~15, YP = pad_ld(nB);
-  const size_t w_floats = tcm ? (size_t)tc::M * K / 2 : (size_t)G * T.R * ld, x_floats = tcm ? (size_t)NTC * K / 2 : (size_t)T.BM * ld;
-  float *Ws = smem, *bs = Ws + w_floats, *Xs = bs + ((G * T.R + 3) & ~3), *Ys = Xs + x_floats, *Zs = Ys + (size_t)T.BM * YP;      // Zs: a GRU's z and h columns
+  const size_t w_floats = SPLIT ? parts_bytes(G * T.R, K) / 4 : tcm ? (size_t)tc::M * K / 2 : (size_t)G * T.R * ld;
+  const size_t x_floats = SPLIT ? parts_bytes(tc3::rows_padded(T.BM, T.split), K) / 4 : tcm ? (size_t)NTC * K / 2 : (size_t)T.BM * ld;
+  float *Ws = smem, *Xs = Ws + w_floats, *bs = Xs + x_floats, *Ys = bs + ((G * T.R + 3) & ~3), *Zs = Ys + (size_t)T.BM * YP;      // Zs: a GRU's z and h columns
   unsigned char *const Wb = reinterpret_cast<unsigned char*>(Ws), *const Xb = reinterpret_cast<unsigned char*>(Xs);
   unsigned have = 0;
   const FastDiv dj4(max(jn >> 2, 1));
@@ -911,7 +1020,15 @@ __device__ __noinline__ void forward_main(const int team, const int tile, float*
     for (size_t i = tid; i < x_floats; i += CT) Xs[i] = 0.f;
     bar_compute();
     fill_w(m.W, m.b);                                              // version 0, which no publication number stands for: they wrap at 2^16
-  } else first_rows(m, G, gw, j0, jn, Ws, ld, bs);
+  }
+  const unsigned group = tc3::group_bytes(K);
+  const Parts Wq{reinterpret_cast<unsigned char*>(Ws), (unsigned)((nB + 7) >> 3) * group, group};
+  if (SPLIT) {
+#pragma unroll 1
+    for (size_t i = tid; i < w_floats + x_floats; i += CT) Ws[i] = 0.f;      // (columns past the width stay zero)
+    bar_compute();
+    first_parts(m, false, G, gw, j0, jn, Wq, bs);
+  } else if (!tcm) first_rows(m, G, gw, j0, jn, Ws, ld, bs);
   unsigned tc_parity = 0;
   bar_compute();
   chunk_loop(rows, team, t0, [&](const Head& h, const RowD* R) {
@@ -966,7 +1083,10 @@ __device__ __noinline__ void forward_main(const int team, const int tile, float*
       if (tile == 0 && !EVALUATING) for (int b = tid; b < count; b += CT) S.core.arena[R[b].out4 + H4] = make_float4(__int_as_float(version), 0.f, 0.f, 0.f);
       return;
     }
-    gather_terms(h, R, 0, n4, Xs, ld);
+    const int np = SPLIT ? tc3::rows_padded(count, T.split) : 0;
+    const Parts Xq{reinterpret_cast<unsigned char*>(Xs), (unsigned)(np >> 3) * group, group};
+    auto x_at = [&](const int b, const int c4) { if constexpr (SPLIT) return Xq.get(b, c4); else return *reinterpret_cast<const float4*>(Xs + b * ld + 4 * c4); };
+    if (SPLIT) gather_parts(h, R, n4, Xq); else gather_terms(h, R, 0, n4, Xs, ld);
     if (kind == GRU_C)                                          // z and h of this tile's columns
 #pragma unroll 1
       for (int i = tid; i < count * (jn >> 2); i += CT) {
@@ -975,10 +1095,13 @@ __device__ __noinline__ void forward_main(const int team, const int tile, float*
         cp16(Zs + b * 2 * jn + jn + 4 * k, S.core.arena + R[b].out4 + H4 + (j0 >> 2) + k);
       }
     cp_wait();
-    bar_compute();
-    phase(2);
-    gemm(Xs, ld, count, Ws, ld, nB, n4, Ys, YP);
-    bar_compute();
+    if (SPLIT) product_parts(Wq, Xq, T.split, np, K, count, nB, Ys, YP, tc_parity, t0);
+    else {
+      bar_compute();
+      phase(2);
+      gemm(Xs, ld, count, Ws, ld, nB, n4, Ys, YP);
+      bar_compute();
+    }
     phase(3);
     const int ow = m.out_w, w4 = jn >> 2;
     if constexpr (MODE == F_PLAIN) {
@@ -1005,7 +1128,7 @@ __device__ __noinline__ void forward_main(const int team, const int tile, float*
       auto clip = [&](float4 v) { if (past > 0) { v.w = 0.f; if (past > 1) v.z = 0.f; if (past > 2) v.y = 0.f; if (past > 3) v.x = 0.f; } return v; };
       if (kind == GRU_ZR) {
         const float4 z = clip(act_fwd4(3, add4(y4[0], b4[0]))), rr = clip(act_fwd4(3, add4(y4[w4], b4[w4])));
-        const float4 hh = *reinterpret_cast<const float4*>(Xs + b * ld + gw + 4 * c4);
+        const float4 hh = x_at(b, H4 + c4);
         out[2 * H4 + c4] = z; out[3 * H4 + c4] = rr;
         out[4 * H4 + c4] = make_float4(rr.x * hh.x, rr.y * hh.y, rr.z * hh.z, rr.w * hh.w);
         continue;
@@ -1040,7 +1163,7 @@ __device__ __noinline__ void forward_main(const int team, const int tile, float*
 #pragma unroll 1
       for (int i = tid; i < count * share; i += CT) {
         const int b = i / share, k = i - b * share;
-        if (k < kn) S.core.arena[(kind == GRU_ZR ? R[b].out4 : R[b].a4) + k0 + k] = *reinterpret_cast<const float4*>(Xs + b * ld + 4 * (k0 + k));
+        if (k < kn) S.core.arena[(kind == GRU_ZR ? R[b].out4 : R[b].a4) + k0 + k] = x_at(b, k0 + k);
       }
     }
     if (tile == 0 && !EVALUATING && kind != GRU_ZR) {
@@ -1052,7 +1175,9 @@ __device__ __noinline__ void forward_main(const int team, const int tile, float*
     const unsigned pub = pub_of(ver);
     if (pub == have) return;
     have = pub;
-    if (tcm) fill_w(m.Wp + (size_t)(pub % PUB) * m.outp * m.inp, m.bp + (size_t)(pub % PUB) * m.outp); else load_rows(m, pub, G, gw, j0, jn, Ws, ld, bs);
+    if (tcm) fill_w(m.Wp + (size_t)(pub % PUB) * m.outp * m.inp, m.bp + (size_t)(pub % PUB) * m.outp);
+    else if (SPLIT) load_parts(m, pub, false, G, gw, j0, jn, Wq, bs);
+    else load_rows(m, pub, G, gw, j0, jn, Ws, ld, bs);
   });
 }
 
@@ -1060,7 +1185,7 @@ __device__ __noinline__ void forward_main(const int team, const int tile, float*
 // A tile holds R input columns of the matrix for all outputs.  The pre-activation gradients of a row are formed while the row
 // is gathered (every tile stores its share of them for the accumulator) and multiplied with the transposed weights.
 enum { B_PLAIN, B_DC, B_DZR, B_LSTM };
-template <int MODE>
+template <int MODE, bool SPLIT = false>
 __device__ __noinline__ void input_grad_main(const int team, const int tile, float* smem, RowD* rows, const unsigned long long t0) {
   IN_SMEM(smem);  IN_SMEM(rows);
   const Team& T = S.team; const Mat& m = S.mat;
@@ -1068,9 +1193,18 @@ __device__ __noinline__ void input_grad_main(const int team, const int tile, flo
   const int tid = threadIdx.x, H4 = T.H4, bf16 = S.core.bf16;
   const int c0 = tile * T.R, cn = min(T.R, m.inp - c0), K = m.outp, ld = pad_ld(K), n4 = K >> 2;
   const int YP = pad_ld(cn);
-  float *Wt = smem, *Gs = Wt + (size_t)T.R * ld, *Ys = Gs + (size_t)T.BM * ld;
+  const size_t w_floats = SPLIT ? parts_bytes(T.R, K) / 4 : (size_t)T.R * ld, g_floats = SPLIT ? parts_bytes(tc3::rows_padded(T.BM, T.split), K) / 4 : (size_t)T.BM * ld;
+  float *Wt = smem, *Gs = Wt + w_floats, *Ys = Gs + g_floats;
   const FastDiv dc4(max(cn >> 2, 1));
-  first_cols(m, c0, cn, Wt, ld);
+  const unsigned group = tc3::group_bytes(K);
+  const Parts Wq{reinterpret_cast<unsigned char*>(Wt), (unsigned)((cn + 7) >> 3) * group, group};
+  unsigned tc_parity = 0;
+  if (SPLIT) {
+#pragma unroll 1
+    for (size_t i = tid; i < w_floats + g_floats; i += CT) Wt[i] = 0.f;      // (columns past the width stay zero)
+    bar_compute();
+    first_parts(m, true, 1, 0, c0, cn, Wq, nullptr);
+  } else first_cols(m, c0, cn, Wt, ld);
   unsigned have = 0;
   constexpr bool lstm = MODE == B_LSTM;
   const bool branch = lstm && T.lstm == 5;
@@ -1079,7 +1213,9 @@ __device__ __noinline__ void input_grad_main(const int team, const int tile, flo
   const int in4 = m.inp >> 2;
   bar_compute();
   chunk_loop(rows, team, t0, [&](const Head& h, const RowD* R) {
-    const int count = h.count;
+    const int count = h.count, np = SPLIT ? tc3::rows_padded(count, T.split) : 0;
+    const Parts Gq{reinterpret_cast<unsigned char*>(Gs), (unsigned)(np >> 3) * group, group};
+    auto put = [&](const int b, const int c4, const float4 v) { if constexpr (SPLIT) Gq.put(b, c4, v); else *reinterpret_cast<float4*>(Gs + b * ld + 4 * c4) = v; };
     auto gather = [&](auto is_long) {
     constexpr bool LONG = decltype(is_long)::value;
 #pragma unroll 1
@@ -1141,22 +1277,25 @@ __device__ __noinline__ void input_grad_main(const int team, const int tile, flo
         for (int k = 0; k < 5; k++)
           if (branch || k == 0 || k > 2) {
             const float4 v = make_float4(out[k][0], out[k][1], out[k][2], out[k][3]);
-            *reinterpret_cast<float4*>(Gs + b * ld + 4 * (g * H4 + c)) = v;
+            put(b, g * H4 + c, v);
             if (mine) dp[g * H4] = v;
             g++;
           }
         if (branch && mine) { dp[L * H4] = make_float4(out[5][0], out[5][1], out[5][2], out[5][3]); dp[(L + 1) * H4] = make_float4(out[6][0], out[6][1], out[6][2], out[6][3]); }
         continue;
       }
-      *reinterpret_cast<float4*>(Gs + b * ld + 4 * c) = d;
+      put(b, c, d);
     }
     };
     if (kind != GRU_DZR && (h.flags & H_LONG)) gather(Flag<true>()); else gather(Flag<false>());
-    cp_wait();
-    bar_compute();
-    phase(2);
-    gemm(Gs, ld, count, Wt, ld, cn, n4, Ys, YP);
-    bar_compute();
+    if (SPLIT) product_parts(Wq, Gq, T.split, np, K, count, cn, Ys, YP, tc_parity, t0);
+    else {
+      cp_wait();
+      bar_compute();
+      phase(2);
+      gemm(Gs, ld, count, Wt, ld, cn, n4, Ys, YP);
+      bar_compute();
+    }
     const int w4c = cn >> 2;
 #pragma unroll 1
     for (int i = tid; i < count * w4c; i += CT) {
@@ -1178,7 +1317,9 @@ __device__ __noinline__ void input_grad_main(const int team, const int tile, flo
     phase(3);
   }, [&](const unsigned long long ver) {
     const unsigned pub = pub_of(ver);
-    if (pub != have) { have = pub; load_cols(m, pub, c0, cn, Wt, ld); }
+    if (pub == have) return;
+    have = pub;
+    if (SPLIT) load_parts(m, pub, true, 1, 0, c0, cn, Wq, nullptr); else load_cols(m, pub, c0, cn, Wt, ld);
   });
 }
 
@@ -1704,9 +1845,9 @@ extern "C" __global__ void __launch_bounds__(NT, 1) ENGINE_KERNEL(const __grid_c
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
-  const bool tcm = S.team.bf16_tc != 0;
-  if (tcm) {
-    if (tid < 32) tc::tmem_alloc(&S.tmem);
+  const bool tcm = S.team.bf16_tc != 0, split = S.team.split != 0;
+  if (tcm || split) {
+    if (tid < 32) { if (split) tc3::tmem_alloc(&S.tmem); else tc::tmem_alloc(&S.tmem); }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -1718,17 +1859,22 @@ extern "C" __global__ void __launch_bounds__(NT, 1) ENGINE_KERNEL(const __grid_c
   else switch (S.team.kind) {
     case LIN_F:
       if (S.team.bf16_tc) forward_main<F_TENSOR>(team, tile, work, rows, t0);
-      else if (S.team.lstm) forward_main<F_LSTM>(team, tile, work, rows, t0);
+      else if (S.team.lstm) { if (split) forward_main<F_LSTM, true>(team, tile, work, rows, t0); else forward_main<F_LSTM>(team, tile, work, rows, t0); }
+      else if (split) forward_main<F_PLAIN, true>(team, tile, work, rows, t0);
       else forward_main<F_PLAIN>(team, tile, work, rows, t0);
       break;
-    case GRU_ZR: forward_main<F_ZR>(team, tile, work, rows, t0); break;
-    case GRU_C: forward_main<F_C>(team, tile, work, rows, t0); break;
+    case GRU_ZR: if (split) forward_main<F_ZR, true>(team, tile, work, rows, t0); else forward_main<F_ZR>(team, tile, work, rows, t0); break;
+    case GRU_C: if (split) forward_main<F_C, true>(team, tile, work, rows, t0); else forward_main<F_C>(team, tile, work, rows, t0); break;
     case HEAD: head_main(team, work, rows, t0); break;
     case LOOKUP_F: lookup_main(team, rows, t0); break;
 #ifndef WAVE_FORWARD
-    case LIN_DX: if (S.team.lstm) input_grad_main<B_LSTM>(team, tile, work, rows, t0); else input_grad_main<B_PLAIN>(team, tile, work, rows, t0); break;
-    case GRU_DC: input_grad_main<B_DC>(team, tile, work, rows, t0); break;
-    case GRU_DZR: input_grad_main<B_DZR>(team, tile, work, rows, t0); break;
+    case LIN_DX:
+      if (S.team.lstm) { if (split) input_grad_main<B_LSTM, true>(team, tile, work, rows, t0); else input_grad_main<B_LSTM>(team, tile, work, rows, t0); }
+      else if (split) input_grad_main<B_PLAIN, true>(team, tile, work, rows, t0);
+      else input_grad_main<B_PLAIN>(team, tile, work, rows, t0);
+      break;
+    case GRU_DC: if (split) input_grad_main<B_DC, true>(team, tile, work, rows, t0); else input_grad_main<B_DC>(team, tile, work, rows, t0); break;
+    case GRU_DZR: if (split) input_grad_main<B_DZR, true>(team, tile, work, rows, t0); else input_grad_main<B_DZR>(team, tile, work, rows, t0); break;
     case ACC: accumulate_main(team, tile, work, rows, t0); break;
     case LOOKUP_B: if (S.team.R) lookup_grad_small_main(team, tile, work, rows, t0); else lookup_grad_main(team, tile, work, rows, t0); break;
 #endif
@@ -1747,7 +1893,7 @@ extern "C" __global__ void __launch_bounds__(NT, 1) ENGINE_KERNEL(const __grid_c
     if (tid < 64) st.stale_hist[tid] = S.stale_hist[tid];
     if (tid == 0) st.max_staleness = S.max_stale;
   }
-  if (tcm && tid < 32) tc::tmem_free(S.tmem);
+  if (tid < 32) { if (split) tc3::tmem_free(S.tmem); else if (tcm) tc::tmem_free(S.tmem); }
 }
 
 // ---- host hooks ---------------------------------------------------------------------------------------------------------------
@@ -1766,16 +1912,22 @@ cudaError_t launch(const Run* run, int n_ctas, size_t smem, cudaStream_t st) {
   return run->core.eval ? forward::launch(run, n_ctas, smem, st) : run->core.opt ? moments::launch(run, n_ctas, smem, st) : training::launch(run, n_ctas, smem, st);
 }
 using namespace training;
+// Both operands of a tile in parts.  An instruction reads M rows of a part of the weights: past the last one it reads on, in what follows.
+static size_t split_floats(const int w_rows, const int K, const Team& t) {
+  const size_t w = parts_bytes(w_rows, K), x = parts_bytes(tc3::rows_padded(t.BM, t.split), K), reach = 2 * (w / 3) + (size_t)(t.split / 8) * tc3::group_bytes(K);
+  return std::max(w + x, reach) / 4;
+}
 size_t smem_bytes(const Team& t, const Mat& m, int mak) {
   const size_t head = slots_bytes(mak) + 2 * (size_t)t.BM * sizeof(RowD);
   const size_t ldi = pad_ld(m.inp), ldo = pad_ld(m.outp), BM = t.BM;
   size_t f = 0;
   switch (t.kind) {
     case LIN_F: case GRU_ZR: case GRU_C:
-      if (t.bf16_tc) f = (size_t)tc::M * m.inp / 2 + tc::M + ((BM + 15) & ~(size_t)15) * m.inp / 2 + BM * pad_ld(tc::M);
+      if (t.split) f = split_floats(t.G * t.R, m.inp, t) + ((t.G * t.R + 3) & ~3) + BM * pad_ld(t.G * t.R) + (t.kind == GRU_C ? BM * 2 * t.R : 0);
+      else if (t.bf16_tc) f = (size_t)tc::M * m.inp / 2 + tc::M + ((BM + 15) & ~(size_t)15) * m.inp / 2 + BM * pad_ld(tc::M);
       else f = (size_t)t.G * t.R * ldi + ((t.G * t.R + 3) & ~3) + BM * ldi + BM * pad_ld(t.G * t.R) + (t.kind == GRU_C ? BM * 2 * t.R : 0);
       break;
-    case LIN_DX: case GRU_DC: case GRU_DZR: f = (size_t)t.R * ldo + BM * ldo + BM * pad_ld(t.R); break;
+    case LIN_DX: case GRU_DC: case GRU_DZR: f = t.split ? split_floats(t.R, m.outp, t) + BM * pad_ld(t.R) : (size_t)t.R * ldo + BM * ldo + BM * pad_ld(t.R); break;
     case ACC: f = (size_t)t.R * (t.C + 4) + ACC_RED + BM * (t.R + 4 + t.C + 4) + t.R + (size_t)(CW / (t.WO * t.WI)) * t.R; break;
     case LOOKUP_B: f = t.R ? BM * (t.C + 4) + (size_t)t.G * (t.R * t.C + 1) : CW * (NEAR + PIECES) + LOOKUP_BITS; break;      // (small table of G rows: R copies of the sums of C columns)
     case HEAD: f = (size_t)m.outp * ldi + m.outp + BM * ldi + 2 * BM * pad_ld(m.outp); break;

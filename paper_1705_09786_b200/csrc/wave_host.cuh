@@ -296,20 +296,24 @@ static bool wave_best(const WaveModel& M, int c, int ctas, double rows, double m
   if (K.mat >= 0) { const WaveMat& w = M.mats[K.mat]; m.outp = w.outp; m.inp = w.inp; m.out_w = w.out_w; m.nso = w.nso; m.in_w = w.in_w; m.nsi = w.nsi; }
   const double upd = eval ? 0.0 : std::min(1.0, rows / std::max(1.0, msgs_per_update));      // rounds with new weights
   bool found = false;
-  auto offer = [&](Team x, double cycles) {
+  auto offer = [&](Team x, double cycles, const double per_chunk = 900.0, const int split_k = 0) {
     static const int caps[] = {128, 96, 64, 48, 32, 24, 16, 8};
     for (int bm : caps) {
       if (bm > 32 && bm >= 2 * rows / x.Sh + 32) continue;              // (no more staging than a round needs)
       if (x.bf16_tc && bm > 64) continue;
+      if (split_k > 0 && tc3::rows_padded(bm, x.split) > tc3::max_rows(split_k)) continue;
       x.BM = bm;
       if (smem_bytes(x, m, mak) > budget) continue;
       const double chunks = std::max(1.0, rows / x.Sh / bm);
-      cycles += 900.0 * (chunks - 1.0);
+      cycles += per_chunk * (chunks - 1.0);
       if (!found || cycles < best.cycles * 0.995) { best.t = x; best.cycles = cycles; found = true; }
       return;
     }
   };
   const double bpc = 36, fma = 40;
+  // products of 32-bit operands on the tensor cores: four instructions a step of sixteen, whatever the rows, and the accumulators' way back
+  const double split_gather = 0.7, split_weights = 1.5, split_chunk = 2500;
+  auto split_product = [](const int k) { return 900 + 4 * 32.0 * tc3::k_steps(k) + 60.0 * tc3::chains(k); };
   int env_rows = 0, env_cols = 0;
   if (const char* e = getenv("AMPNET_DIRECT_ROWS")) env_rows = std::max(1, atoi(e));
   if (const char* e = getenv("AMPNET_DIRECT_COLS")) env_cols = std::max(4, atoi(e));
@@ -334,7 +338,12 @@ static bool wave_best(const WaveModel& M, int c, int ctas, double rows, double m
         const bool sums = K.kind == GRU_ZR || (t.keep && !eval);
         const double gather = 1300 + rs * m.inp / 4 * (sums ? 3.5 : 1.0), weights = std::min(1.0, upd) * outs * m.inp * 4.0 / bpc;
         const double product = tc ? 1500 + rs * m.inp / 8.0 : 600 + (rs + 4) * outs * m.inp / fma;
-        offer(x, gather + weights + product + 1600 + rs * x.R / 4 * (t.lstm ? 20.0 : K.kind == LIN_F ? 2.0 : 3.0));
+        const double rest = 1600 + rs * x.R / 4 * (t.lstm ? 20.0 : K.kind == LIN_F ? 2.0 : 3.0);
+        offer(x, gather + weights + product + rest);
+        if (!tc && outs <= 128) {
+          x.split = outs <= 64 ? 64 : 128;
+          offer(x, gather + rs * m.inp / 4 * split_gather + weights * split_weights + split_product(m.inp) + rest, split_chunk + split_product(m.inp), m.inp);
+        }
         if (tc || env_rows) break;
       }
       break;
@@ -351,7 +360,12 @@ static bool wave_best(const WaveModel& M, int c, int ctas, double rows, double m
         x.n = x.T * x.Sh;
         const double rs = std::max(1.0, rows / x.Sh);
         const double per4 = t.lstm ? 17.0 * t.H4 : m.outp / 4 * (K.kind == GRU_DC ? 12.0 : 3.4);
-        offer(x, 1500 + rs * per4 + std::min(1.0, upd) * x.R * m.outp * 4.0 / bpc + 600 + (rs + 4) * x.R * m.outp / fma + 1700 + rs * x.R / 4 * 1.5);
+        const double weights = std::min(1.0, upd) * x.R * m.outp * 4.0 / bpc, rest = 1700 + rs * x.R / 4 * 1.5;
+        offer(x, 1500 + rs * per4 + weights + 600 + (rs + 4) * x.R * m.outp / fma + rest);
+        if (x.R <= 128) {
+          x.split = x.R <= 64 ? 64 : 128;
+          offer(x, 1500 + rs * (per4 + m.outp / 4 * split_gather) + weights * split_weights + split_product(m.outp) + rest, split_chunk + split_product(m.outp), m.outp);
+        }
         if (env_cols) break;
       }
       break;
