@@ -312,6 +312,7 @@ static bool wave_best(const WaveModel& M, int c, int ctas, double rows, double m
   };
   const double bpc = 36, fma = 40;
   // products of 32-bit operands on the tensor cores: four instructions a step of sixteen, whatever the rows, and the accumulators' way back
+  const double acc_base = 5000, acc_row = 0.17, acc_chunk = 3500;
   const double split_gather = 0.7, split_weights = 1.5, split_chunk = 2500;
   auto split_product = [](const int k) { return 900 + 4 * 32.0 * tc3::k_steps(k) + 60.0 * tc3::chains(k); };
   int env_rows = 0, env_cols = 0;
@@ -370,6 +371,19 @@ static bool wave_best(const WaveModel& M, int c, int ctas, double rows, double m
       }
       break;
     case ACC:
+      // Tiles on the tensor cores: the operands' way into shared memory is what counts, so a tile is as nearly square as its count allows.
+      // Column Ci of the instruction's at most 128 is the bias gradient's.
+      for (int to = 1; to <= std::min(ctas, m.outp / 4); to++) {
+        const int R = pad4i((m.outp + to - 1) / to);
+        if (R > 128 || (m.outp + R - 1) / R != to) continue;
+        for (int ti = 1; to * ti <= ctas && ti <= m.inp / 4; ti++) {
+          Team x = t;
+          x.R = R; x.C = pad4i((m.inp + ti - 1) / ti);
+          if (x.C > 124 || (m.inp + x.C - 1) / x.C != ti) continue;
+          x.T = x.n = to * ti; x.split = R <= 64 ? 64 : 128;
+          offer(x, acc_base + rows * (8 + acc_row * (x.R + x.C)) + upd * acc_chunk + std::min(1.0, upd) * (double)x.R * x.C / 5, acc_chunk);
+        }
+      }
       for (int LO = 1; LO <= 8; LO *= 2)
         for (int WO = 1; WO <= 16; WO *= 2)
           for (int WI = 1; WO * WI <= 16; WI *= 2) {
