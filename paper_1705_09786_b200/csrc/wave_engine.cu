@@ -75,7 +75,6 @@ struct Shared {
   unsigned stale_hist[64]; int max_stale;
   int team_n[MAX_CELLS];
   unsigned long long phase[N_PHASES]; long long mark;
-  float few[CW][32];                           // sums of a product of few rows
 };
 __shared__ Shared S;
 // Pointers into shared memory that reach a function as arguments would be dereferenced as generic addresses.
@@ -640,8 +639,8 @@ __device__ __forceinline__ void gather_terms(const Head& h, const RowD* rows, co
 
 // ---- products ---------------------------------------------------------------------------------------------------------------
 // Y[b][o] = sum_k A[b][k] B[o][k]: all in shared memory, k contiguous, row strides of A and B 4 (mod 8) floats, K4 groups of four,
-// nB a multiple of four.  512 threads (all of them: gemm_few has a barrier inside).  Three shapes:
-//   gemm_few     up to four rows: a warp per eight columns and slice of k, lanes along k
+// nB a multiple of four.  512 threads, no barrier inside.  Three shapes:
+//   gemm_few     up to four rows: a warp per output column, lanes along k
 //   gemm_warps   up to 1,536 outputs: a warp per 4 x 4 outputs, lanes along k, a reduce-scatter of shuffles (short code)
 //   gemm_tiles   4 x 4 outputs per thread, k in four interleaved lanes that meet in a reduce-scatter of shuffles.  The bound is what
 //                shared memory can hand to registers (a 16-byte load costs four cycles of the SM whatever it hits); packed multiply-adds
@@ -736,54 +735,34 @@ __device__ __noinline__ void gemm_tiles(const float* __restrict__ A, const int l
     else Y[b * ldy + o] = v[0];
   }
 }
-// Up to four rows: a warp takes eight columns (32 sums) and every slice-th group of 32 fours of k, so that a row is read once per column
-// group and not once per column; the sums meet in a reduce-scatter (lane l keeps row l / 8, column l mod 8) and, over the slices, in shared
-// memory.  A warp per column read the rows nB times, and with eight columns half of the warps had nothing to do.
 __device__ __noinline__ void gemm_few(const float* __restrict__ A, const int lda, const int nA, const float* __restrict__ B, const int ldb, const int nB, const int K4, float* __restrict__ Y, const int ldy) {
   IN_SMEM(A); IN_SMEM(B); IN_SMEM(Y);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const float4* const A4 = reinterpret_cast<const float4*>(A);
   const float4* const B4 = reinterpret_cast<const float4*>(B);
-  const int ldb4 = ldb >> 2, groups = (nB + 7) >> 3, slices = groups > CW / 2 ? 1 : min(CW / groups, (K4 + 31) >> 5);
-  const int l1 = min(1, nA - 1) * (lda >> 2), l2 = min(2, nA - 1) * (lda >> 2), l3 = min(3, nA - 1) * (lda >> 2);
-  const int slice = warp / groups, first = warp - slice * groups;
-  if (slice < slices)
+  const int ldb4 = ldb >> 2, l1 = nA > 1 ? lda >> 2 : 0, l2 = nA > 2 ? 2 * (lda >> 2) : 0, l3 = nA > 3 ? 3 * (lda >> 2) : 0;
 #pragma unroll 1
-    for (int g = first; g < groups; g += CW) {
-      float v[32];
-#pragma unroll
-      for (int i = 0; i < 32; i++) v[i] = 0.f;
-#pragma unroll 1
-      for (int k4 = 32 * slice + lane; k4 < K4; k4 += 32 * slices) {
-        const float4 x0 = A4[k4], x1 = A4[l1 + k4], x2 = A4[l2 + k4], x3 = A4[l3 + k4];
-#pragma unroll
-        for (int j = 0; j < 8; j++) {
-          const float4 w = B4[min(8 * g + j, nB - 1) * ldb4 + k4];
-          auto dot = [&](const float4 x, float s) { s = fmaf(x.x, w.x, s); s = fmaf(x.y, w.y, s); s = fmaf(x.z, w.z, s); return fmaf(x.w, w.w, s); };
-          v[j] = dot(x0, v[j]); v[8 + j] = dot(x1, v[8 + j]); v[16 + j] = dot(x2, v[16 + j]); v[24 + j] = dot(x3, v[24 + j]);
-        }
-      }
-#pragma unroll
-      for (int H = 16; H >= 1; H >>= 1) {
-        const bool up = lane & H;
-#pragma unroll
-        for (int i = 0; i < H; i++) {
-          const float give = up ? v[i] : v[i + H], keep = up ? v[i + H] : v[i];
-          v[i] = keep + __shfl_xor_sync(0xffffffffu, give, H);
-        }
-      }
-      if (slices > 1) S.few[warp][lane] = v[0];
-      else if ((lane >> 3) < nA && 8 * g + (lane & 7) < nB) Y[(lane >> 3) * ldy + 8 * g + (lane & 7)] = v[0];
+  for (int o = warp; o < nB; o += CW) {
+    float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
+    auto dot = [](const float4 w, const float4 x, float s) { s = fmaf(x.x, w.x, s); s = fmaf(x.y, w.y, s); s = fmaf(x.z, w.z, s); return fmaf(x.w, w.w, s); };
+#pragma unroll 2
+    for (int k4 = lane; k4 < K4; k4 += 32) {
+      const float4 w = B4[o * ldb4 + k4];
+      a0 = dot(w, A4[k4], a0);
+      if (nA > 1) { a1 = dot(w, A4[l1 + k4], a1); a2 = dot(w, A4[l2 + k4], a2); a3 = dot(w, A4[l3 + k4], a3); }
     }
-  if (slices > 1) {
-    bar_compute();
-    const int b = lane >> 3, o = 8 * warp + (lane & 7);
-    if (warp < groups && b < nA && o < nB) {
-      float s = 0.f;
-#pragma unroll 4
-      for (int q = 0; q < slices; q++) s += S.few[q * groups + warp][lane];
-      Y[b * ldy + o] = s;
-    }
+    // lanes 0-15 keep rows 0, 1, lanes 16-31 rows 2, 3; then one row per group of eight lanes
+    const bool hi = lane & 16, mid = lane & 8;
+    float s0 = hi ? a2 : a0, s1 = hi ? a3 : a1;
+    s0 += __shfl_xor_sync(0xffffffffu, hi ? a0 : a2, 16);
+    s1 += __shfl_xor_sync(0xffffffffu, hi ? a1 : a3, 16);
+    float v = mid ? s1 : s0;
+    v += __shfl_xor_sync(0xffffffffu, mid ? s0 : s1, 8);
+    v += __shfl_xor_sync(0xffffffffu, v, 4);
+    v += __shfl_xor_sync(0xffffffffu, v, 2);
+    v += __shfl_xor_sync(0xffffffffu, v, 1);
+    const int b = (hi ? 2 : 0) + (mid ? 1 : 0);
+    if ((lane & 7) == 0 && b < nA) Y[b * ldy + o] = v;
   }
 }
 __device__ __forceinline__ void gemm(const float* A, const int lda, const int nA, const float* B, const int ldb, const int nB, const int K4, float* Y, const int ldy) {
