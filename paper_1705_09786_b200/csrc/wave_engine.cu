@@ -557,16 +557,16 @@ __device__ __forceinline__ void for_rows(const int count, const int n4, const F&
 // ---- gathers ---------------------------------------------------------------------------------------------------------------
 // A sum of more terms than a row's descriptor holds: eight loads in flight (one after another, each is a trip to L2; the sum over a
 // graph's nodes took 24,000 cycles of a round).
-__device__ __noinline__ float4 sum_terms(const Term* t, const unsigned base4, const int nt, const int c) {
+__device__ __noinline__ float4 sum_terms(const Term* t, const unsigned base4, const int nt, const int c, const int first = 0, const int step = 1) {
   float4 v = zero4();
 #pragma unroll 1
-  for (int q0 = 0; q0 < nt; q0 += 8) {
+  for (int q0 = first; q0 < nt; q0 += 8 * step) {
     float4 w[8];
 #pragma unroll
     for (int q = 0; q < 8; q++) {
       w[q] = zero4();
-      if (q0 + q >= nt) continue;
-      const Term u = t[q0 + q];
+      if (q0 + q * step >= nt) continue;
+      const Term u = t[q0 + q * step];
       const unsigned d = (unsigned)c - u.col4;
       if (d < u.w4) w[q] = ldcg4(S.core.arena + base4 + u.src4 + d);
     }
@@ -609,7 +609,39 @@ __device__ __noinline__ float4 dense4(const int inst, const int c) {
 // Columns [c0, c0 + nc) (in fours) of the rows' terms into X; copies are asynchronous (cp_wait before the barrier), sums take up to
 // four loads at a time.  Chunks of plain copies (one source, or a Concat of two) have a loop of their own: what a round costs is
 // mostly how many instructions it walks through.
-template <bool CALL>
+// Chunks with long sums: as many lanes per four columns (up to eight) as the threads allow, each with every so many-th term.  A read-out over a
+// graph's atoms comes eight rows a round: 210 threads with up to four dependent pairs of trips to L2 took 15,000 cycles.
+template <class Put>
+__device__ __forceinline__ void for_long_rows(const RowD* rows, const int count, const int c0, const int nc, const Put& put) {
+  const FastDiv dn(nc);
+  const int items = count * nc;
+  int sh = 0;
+  while (sh < 3 && (items << (sh + 1)) <= CT) sh++;
+#pragma unroll 1
+  for (int j = threadIdx.x; j < ((items << sh) + 31 & ~31); j += CT) {      // (whole warps)
+    const int i = min(j >> sh, items - 1), q = j & ((1 << sh) - 1), b = dn.div(i), k = i - b * nc;
+    const RowD& r = rows[b];
+    float4 v = zero4();
+    if (r.meta & (E_DENSE | E_RAW)) v = dense4(r.inst, c0 + k);
+    else {
+      if (r.meta & E_OVERFLOW) {
+        v = sum_terms(S.core.prog.ov + r.t[0].src4, r.base4, r.meta & E_NT, c0 + k, q, 1 << sh);
+      } else if (q == 0) v = row_sum<false>(r, c0 + k);
+    }
+    if (sh)
+#pragma unroll 1
+      for (int o = 1; o < 1 << sh; o <<= 1) {
+        float4 w;
+        w.x = __shfl_xor_sync(0xffffffffu, v.x, o); w.y = __shfl_xor_sync(0xffffffffu, v.y, o); w.z = __shfl_xor_sync(0xffffffffu, v.z, o); w.w = __shfl_xor_sync(0xffffffffu, v.w, o);
+        if (!(r.meta & (E_DENSE | E_RAW))) v = add4(v, w);
+      }
+    if (q == 0 && j >> sh < items) put(b, k, (r.meta & (E_DENSE | E_RAW)) ? v : rnd4(S.core.bf16, v));
+  }
+}
+__device__ __noinline__ void gather_long(const RowD* rows, const int count, const int c0, const int nc, float* X, const int ldx) {
+  IN_SMEM(rows); IN_SMEM(X);
+  for_long_rows(rows, count, c0, nc, [&](const int b, const int k, const float4 v) { *reinterpret_cast<float4*>(X + b * ldx + 4 * k) = v; });
+}
 __device__ __noinline__ void gather_general(const RowD* rows, const int count, const int c0, const int nc, float* X, const int ldx) {
   IN_SMEM(rows); IN_SMEM(X);
   const FastDiv dn(nc);
@@ -621,11 +653,11 @@ __device__ __noinline__ void gather_general(const RowD* rows, const int count, c
     if (r.meta & (E_DENSE | E_RAW)) {
       if ((S.core.dense_dim & 3) == 0) { if (4 * c < S.core.dense_dim) cp16(dst, S.core.dense + (long long)(r.inst & 0x7fffffff) * S.core.dense_dim + 4 * c); else *reinterpret_cast<float4*>(dst) = zero4(); }
       else *reinterpret_cast<float4*>(dst) = dense4(r.inst, c);
-    } else *reinterpret_cast<float4*>(dst) = rnd4(S.core.bf16, row_sum<CALL>(r, c));
+    } else *reinterpret_cast<float4*>(dst) = rnd4(S.core.bf16, row_sum<false>(r, c));
   }
 }
 __device__ __forceinline__ void gather_terms(const Head& h, const RowD* rows, const int c0, const int nc, float* X, const int ldx) {
-  if (!(h.flags & H_COPIES)) { if (h.flags & H_LONG) gather_general<true>(rows, h.count, c0, nc, X, ldx); else gather_general<false>(rows, h.count, c0, nc, X, ldx); return; }
+  if (!(h.flags & H_COPIES)) { if (h.flags & H_LONG) gather_long(rows, h.count, c0, nc, X, ldx); else gather_general(rows, h.count, c0, nc, X, ldx); return; }
   const float4* const arena = S.core.arena;
   for_rows(h.count, nc, [&](const int b, const int k0, const int step) {
     const uint4 t = *reinterpret_cast<const uint4*>(&rows[b].t[0]);            // {source, columns} twice
@@ -873,7 +905,10 @@ struct Parts {                         // an operand in shared memory
 __host__ __device__ __forceinline__ int split_columns(const int Ci) { return (Ci + 1 + 15) & ~15; }      // of an accumulator's instruction: the tile's and the ones
 __host__ __device__ __forceinline__ size_t parts_bytes(const int rows, const int K) { return (size_t)3 * ((rows + 7) >> 3) * tc3::group_bytes(K); }
 // What gather_terms does, into parts.  Copies: four loads of a thread in flight whatever rows they belong to.
-template <bool CALL>
+__device__ __noinline__ void gather_long_parts(const RowD* rows, const int count, const int nc, const Parts X) {
+  IN_SMEM(rows); IN_SMEM(X.base);
+  for_long_rows(rows, count, 0, nc, [&](const int b, const int k, const float4 v) { X.put(b, k, v); });
+}
 __device__ __noinline__ void gather_general_parts(const RowD* rows, const int count, const int nc, const Parts X) {
   IN_SMEM(rows); IN_SMEM(X.base);
   const FastDiv dn(nc);
@@ -881,7 +916,7 @@ __device__ __noinline__ void gather_general_parts(const RowD* rows, const int co
   for (int i = threadIdx.x; i < count * nc; i += CT) {
     const int b = dn.div(i), c = i - b * nc;
     const RowD& r = rows[b];
-    X.put(b, c, (r.meta & (E_DENSE | E_RAW)) ? dense4(r.inst, c) : rnd4(S.core.bf16, row_sum<CALL>(r, c)));
+    X.put(b, c, (r.meta & (E_DENSE | E_RAW)) ? dense4(r.inst, c) : rnd4(S.core.bf16, row_sum<false>(r, c)));
   }
 }
 __device__ __noinline__ void gather_copies_parts(const RowD* rows, const int count, const int nc, const Parts X) {
@@ -909,8 +944,8 @@ __device__ __noinline__ void gather_copies_parts(const RowD* rows, const int cou
 }
 __device__ __forceinline__ void gather_parts(const Head& h, const RowD* rows, const int nc, const Parts X) {
   if (h.flags & H_COPIES) gather_copies_parts(rows, h.count, nc, X);
-  else if (h.flags & H_LONG) gather_general_parts<true>(rows, h.count, nc, X);
-  else gather_general_parts<false>(rows, h.count, nc, X);
+  else if (h.flags & H_LONG) gather_long_parts(rows, h.count, nc, X);
+  else gather_general_parts(rows, h.count, nc, X);
 }
 // Weights of a tile as parts: what first_rows / load_rows and first_cols / load_cols do.
 __device__ __noinline__ void first_parts(const Mat& m, const bool cols, const int G, const int gw, const int j0, const int jn, const Parts W, float* bs) {
@@ -1420,7 +1455,7 @@ __device__ __noinline__ void accumulate_main(const int team, const int tile, flo
           const bool second = c >= (int)(t.w & 0xffffu);
           cp16(Xg + b * ldx + 4 * k, S.core.arena + (second ? t.z + c - (t.w & 0xffffu) : t.x + c));
         }
-      } else gather_general<false>(R, count, i4, x4, Xg, ldx);
+      } else gather_general(R, count, i4, x4, Xg, ldx);
       stale.count_in(h.n_updates, count, tile);
     }
     cp_wait();
@@ -1513,58 +1548,42 @@ __device__ __noinline__ void gather_outer(const Head& h, const RowD* R, const in
   IN_SMEM(R); IN_SMEM(Gq.base); IN_SMEM(Xq.base);
   const volatile AccGeo& Z = S.ag;
   const int tid = threadIdx.x, count = h.count, d4 = Z.d4, x4 = Z.x4, o4 = Z.o0 >> 2, i4 = Z.i0 >> 2, act = S.team.act;
-  const FastDiv dd((unsigned)d4, Z.ddM), dx((unsigned)x4, Z.dxM);
   const float4* const arena = S.core.arena;
-  constexpr int U = 4;
+  const int all4 = d4 + x4, n = ((count + 15) & ~15) * all4;      // (both operands in one loop: one trip to L2)
+  const FastDiv da(all4);
   const Staleness stale(R, count, tile);
-  if (S.ppt.source_adj) {
-#pragma unroll 1
-    for (int i = tid; i < count * d4; i += CT) {
-      const int b = dd.div(i), k = i - b * d4, c = o4 + k;
-      const RowD& r = R[b];
-      if (!(r.meta & E_RAW)) { Gq.put(b, k, ldcg4(arena + r.out4 + c)); continue; }
-      const float4 y = ldcg4(arena + r.a4 + c), g = rnd4(S.core.bf16, row_sum<false>(r, c));
-      Gq.put(b, k, make_float4(g.x * act_grad(act, y.x), g.y * act_grad(act, y.y), g.z * act_grad(act, y.z), g.w * act_grad(act, y.w)));
-    }
-  } else {
-    const int n = count * d4;
-#pragma unroll 1
-    for (int i0 = tid; i0 < n; i0 += U * CT) {
-      float4 v[U];
-#pragma unroll
-      for (int u = 0; u < U; u++) { const int i = min(i0 + u * CT, n - 1), b = dd.div(i); v[u] = ldcg4(arena + R[b].out4 + o4 + (i - b * d4)); }
-#pragma unroll
-      for (int u = 0; u < U; u++) { const int i = i0 + u * CT, b = dd.div(i); if (i < n) Gq.put(b, i - b * d4, v[u]); }
-    }
-  }
-  if (h.flags & H_COPIES) {
-    const int n = count * x4;
+  auto put = [&](const int b, const int k, const float4 v) { if (k < d4) Gq.put(b, k, v); else Xq.put(b, k - d4, v); };
+  if ((h.flags & H_COPIES) && !S.ppt.source_adj) {
+    constexpr int U = 4;
 #pragma unroll 1
     for (int i0 = tid; i0 < n; i0 += U * CT) {
       float4 v[U];
 #pragma unroll
       for (int u = 0; u < U; u++) {
-        const int i = min(i0 + u * CT, n - 1), b = dx.div(i), c = i4 + i - b * x4;
+        const int i = i0 + u * CT, b = da.div(i), k = i - b * all4, c = i4 + k - d4;
+        v[u] = zero4();
+        if (b >= count) continue;
         const uint4 t = *reinterpret_cast<const uint4*>(&R[b].t[0]);
         const int cut = (int)(t.w & 0xffffu);
-        v[u] = ldcg4(arena + (c >= cut ? t.z + (c - cut) : t.x + c));
+        v[u] = ldcg4(arena + (k < d4 ? R[b].out4 + o4 + k : c >= cut ? t.z + (c - cut) : t.x + c));
       }
 #pragma unroll
-      for (int u = 0; u < U; u++) { const int i = i0 + u * CT, b = dx.div(i); if (i < n) Xq.put(b, i - b * x4, v[u]); }
+      for (int u = 0; u < U; u++) { const int i = i0 + u * CT, b = da.div(i); if (i < n) put(b, i - b * all4, v[u]); }
     }
   } else {
 #pragma unroll 1
-    for (int i = tid; i < count * x4; i += CT) {
-      const int b = dx.div(i), k = i - b * x4;
+    for (int i = tid; i < n; i += CT) {
+      const int b = da.div(i), k = i - b * all4;
       const RowD& r = R[b];
-      Xq.put(b, k, (r.meta & (E_DENSE | E_RAW)) ? dense4(r.inst, i4 + k) : rnd4(S.core.bf16, row_sum<false>(r, i4 + k)));
+      float4 v = zero4();
+      if (b >= count) {
+      } else if (k >= d4) v = (r.meta & (E_DENSE | E_RAW)) ? dense4(r.inst, i4 + k - d4) : rnd4(S.core.bf16, row_sum<false>(r, i4 + k - d4));
+      else if (r.meta & E_RAW) {
+        const float4 y = ldcg4(arena + r.a4 + o4 + k), g = rnd4(S.core.bf16, row_sum<false>(r, o4 + k));
+        v = make_float4(g.x * act_grad(act, y.x), g.y * act_grad(act, y.y), g.z * act_grad(act, y.z), g.w * act_grad(act, y.w));
+      } else v = ldcg4(arena + r.out4 + o4 + k);
+      put(b, k, v);
     }
-  }
-  const int pad = -count & 15, all4 = d4 + x4;
-#pragma unroll 1
-  for (int i = tid; i < pad * all4; i += CT) {
-    const int b = i / all4, k = i - b * all4;
-    if (k < d4) Gq.put(count + b, k, zero4()); else Xq.put(count + b, k - d4, zero4());
   }
   stale.count_in(h.n_updates, count, tile);
 }
