@@ -314,7 +314,7 @@ static bool wave_best(const WaveModel& M, int c, int ctas, double rows, double m
   // products of 32-bit operands on the tensor cores: four instructions a step of sixteen, whatever the rows, and the accumulators' way back
   const double acc_base = 5000, acc_row = 0.17, acc_chunk = 3500;
   const double split_gather = 0.7, split_weights = 1.5, split_chunk = 2500;
-  auto split_product = [](const int k) { return 900 + 4 * 32.0 * tc3::k_steps(k) + 60.0 * tc3::chains(k); };
+  auto split_product = [](const int k) { return 1600 + 4 * 57.0 * tc3::k_steps(k) + 150.0 * tc3::chains(k); };
   int env_rows = 0, env_cols = 0;
   if (const char* e = getenv("AMPNET_DIRECT_ROWS")) env_rows = std::max(1, atoi(e));
   if (const char* e = getenv("AMPNET_DIRECT_COLS")) env_cols = std::max(4, atoi(e));
@@ -381,7 +381,7 @@ static bool wave_best(const WaveModel& M, int c, int ctas, double rows, double m
           x.R = R; x.C = pad4i((m.inp + ti - 1) / ti);
           if (x.C > 124 || (m.inp + x.C - 1) / x.C != ti) continue;
           x.T = x.n = to * ti; x.split = R <= 64 ? 64 : 128;
-          offer(x, acc_base + rows * (8 + acc_row * (x.R + x.C)) + upd * acc_chunk + std::min(1.0, upd) * (double)x.R * x.C / 5, acc_chunk);
+          offer(x, 2.4 * (acc_base + rows * (8 + acc_row * (x.R + x.C)) + upd * acc_chunk + std::min(1.0, upd) * (double)x.R * x.C / 5), acc_chunk);
         }
       }
       for (int LO = 1; LO <= 8; LO *= 2)
