@@ -1955,10 +1955,10 @@ __device__ __noinline__ void lookup_grad_main(const int team, const int tile, fl
     int listed = 0;
     auto add_listed = [&]() {
 #pragma unroll 1
-      for (int k0 = 0; k0 < listed; k0 += 4) {
-        float4 v[4];
+      for (int k0 = 0; k0 < listed; k0 += 8) {                     // eight pieces' loads in flight (a frequent word has a dozen rows a round)
+        float4 v[8];
 #pragma unroll
-        for (int k = 0; k < 4; k++) {
+        for (int k = 0; k < 8; k++) {
           v[k] = zero4();
           const int x = k0 + k < listed ? work[k0 + k] : -1, c = 32 * (x >> 8) + lane;
           if (x < 0 || c >= o4) continue;
@@ -1966,7 +1966,7 @@ __device__ __noinline__ void lookup_grad_main(const int team, const int tile, fl
           v[k] = h.flags & H_COPIES ? ldcg4(S.core.arena + r.t[0].src4 + c) : rnd4(S.core.bf16, row_sum<false>(r, c));
         }
 #pragma unroll
-        for (int k = 0; k < 4; k++) {
+        for (int k = 0; k < 8; k++) {
           if (k0 + k >= listed) break;
           const int x = work[k0 + k], q = x >> 8, c = 32 * q + lane;
           const unsigned id = R[x & 255].b4;
@@ -1990,8 +1990,9 @@ __device__ __noinline__ void lookup_grad_main(const int team, const int tile, fl
       const bool ours = b0 + lane < h.count && id - of * NTL == tile;
       if (!__any_sync(0xffffffffu, ours)) continue;
 #pragma unroll 1
-      for (int q = 0; q < segs; q++) {
-        const bool mine = ours && ((of * segs + q) & (CW - 1)) == warp;
+      for (int q0 = 0; q0 < segs; q0 += CW) {                      // (of CW neighbouring pieces exactly one is this warp's)
+        const int q = q0 + ((warp - of * segs - q0) & (CW - 1));
+        const bool mine = ours && q < segs;
         const unsigned all = __ballot_sync(0xffffffffu, mine);
         if (listed + __popc(all) > PIECES) add_listed();
         const unsigned before = (1u << lane) - 1u;
@@ -2009,7 +2010,8 @@ __device__ __noinline__ void lookup_grad_main(const int team, const int tile, fl
       }
     }
     add_listed();
-    if (h.flags & H_UPDATE) { wait_readers(h, t0); update(h.n_upd, h.upd_t); }
+    phase(2);
+    if (h.flags & H_UPDATE) { wait_readers(h, t0); phase(3); update(h.n_upd, h.upd_t); phase(5); }
   });
 }
 
