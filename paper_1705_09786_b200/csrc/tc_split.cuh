@@ -71,28 +71,40 @@ __host__ __device__ constexpr uint32_t instr_desc(const int m, const int n) { re
 __device__ __forceinline__ void mma(const unsigned d, const uint64_t a, const uint64_t b, const uint32_t idesc, const bool add) {
   asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\ntcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" :: "r"(d), "l"(a), "l"(b), "r"(idesc), "r"((unsigned)add) : "memory");
 }
-// One thread issues the whole product and commits it to the mbarrier at `bar`; operands written, fenced (fence_operands) and the CTA
-// synchronised before.  Accumulators from column 0: the chains of hh, then hm + mh, then hl + mm + lh, n columns each.
+// The first warp issues the whole product (one thread of it) and commits it to the mbarrier at `bar`; operands written, fenced
+// (fence_operands) and the CTA synchronised before.  Accumulators from column 0: the chains of hh, then hm + mh, then hl + mm + lh, n columns
+// each.  An instruction takes its operands from uniform registers: descriptors that the warp has agreed on before the loop cost 30 cycles
+// an instruction, one thread's own values 57.
+template <class T> __device__ __forceinline__ T uniform(const T v) { return __shfl_sync(0xffffffffu, v, 0); }
+__device__ __forceinline__ bool elected() {
+  unsigned e;
+  asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}" : "=r"(e));
+  return e != 0;
+}
 __device__ __forceinline__ void issue(const unsigned taddr, const unsigned char* Wb, const unsigned w_part, const unsigned char* Xb, const unsigned x_part, const unsigned group, const int M, const int n, const int K, const unsigned bar) {
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const int steps = k_steps(K), sets = chains(K);
-  uint64_t wh = smem_desc(smem_addr(Wb), group), xh = smem_desc(smem_addr(Xb), group);
-  const uint64_t wp = w_part >> 4, xp = x_part >> 4;
-  const uint32_t one = instr_desc(M, n), two = instr_desc(M, 2 * n);
-  const unsigned low = taddr + (unsigned)(sets * n), lowest = low + (unsigned)n;
-  unsigned d = taddr;
-  for (int s0 = 0; s0 < steps; s0 += CHAIN, d += (unsigned)n) {
-    const int s1 = min(s0 + CHAIN, steps);
-#pragma unroll 2
-    for (int s = s0; s < s1; s++) {
-      mma(d, wh, xh, one, s > s0);
-      mma(low, wh, xh + xp, two, s > 0);
-      mma(low, wh + wp, xh, two, true);
-      mma(lowest, wh + 2 * wp, xh, one, true);
-      wh += 2 * CORE_K >> 4; xh += 2 * CORE_K >> 4;
+  const int steps = uniform(k_steps(K)), un = uniform(n);
+  const uint64_t wh = uniform(smem_desc(smem_addr(Wb), group)), xh = uniform(smem_desc(smem_addr(Xb), group)), wp = uniform((uint64_t)(w_part >> 4)), xp = uniform((uint64_t)(x_part >> 4));
+  const uint32_t two = uniform(instr_desc(M, 2 * n)), one = uniform(instr_desc(M, n));
+  const unsigned t = uniform(taddr), low = uniform(taddr + (unsigned)(chains(K) * n));
+  if (elected()) {
+    unsigned d = t;
+    uint64_t w = wh, x = xh;
+    int left = CHAIN;
+    bool add = false;
+#pragma unroll 1
+    for (int s = 0; s < steps; s++) {
+      mma(d, w, x, one, add);
+      mma(low, w, x + xp, two, s > 0);
+      mma(low, w + wp, x, two, true);
+      mma(low + un, w + 2 * wp, x, one, true);
+      w += 2 * CORE_K >> 4; x += 2 * CORE_K >> 4;
+      add = true;
+      if (--left == 0) { left = CHAIN; add = false; d += un; }
     }
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" :: "r"(bar) : "memory");
   }
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" :: "r"(bar) : "memory");
+  __syncwarp();
 }
 // Eight columns of an accumulator in this warp's lanes (all lanes of the warp take part).
 __device__ __forceinline__ void load8(const unsigned a, unsigned (&u)[8]) {
@@ -160,19 +172,26 @@ __device__ __forceinline__ uint64_t outer_desc(const unsigned saddr, const unsig
 __device__ __forceinline__ void issue_outer(const unsigned taddr, const unsigned char* Gb, const unsigned g_part, const unsigned g_group, const unsigned char* Xb, const unsigned x_part, const unsigned x_group, const int M, const int N, const int steps,
                                             const unsigned bar) {
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  uint64_t g = outer_desc(smem_addr(Gb), g_group), x = outer_desc(smem_addr(Xb), x_group);
-  const uint64_t gp = g_part >> 4, xp = x_part >> 4, gs = 2 * g_group >> 4, xs = 2 * x_group >> 4;
-  const uint32_t mn = 3u << 15, one = instr_desc(M, N) | mn, two = instr_desc(M, 2 * N) | mn;
-  const unsigned low = taddr + (unsigned)(2 * N), lowest = low + (unsigned)N;
+  const uint64_t gd = uniform(outer_desc(smem_addr(Gb), g_group)), xd = uniform(outer_desc(smem_addr(Xb), x_group));
+  const uint64_t gp = uniform((uint64_t)(g_part >> 4)), xp = uniform((uint64_t)(x_part >> 4)), gs = uniform((uint64_t)(2 * g_group >> 4)), xs = uniform((uint64_t)(2 * x_group >> 4));
+  const uint32_t mn = 3u << 15, one = uniform(instr_desc(M, N) | mn), two = uniform(instr_desc(M, 2 * N) | mn);
+  const unsigned t = uniform(taddr), un = uniform((unsigned)N);
+  const int n_steps = uniform(steps);
+  if (elected()) {
+    uint64_t g = gd, x = xd;
+    unsigned d = t, other = t + un;
 #pragma unroll 1
-  for (int s = 0; s < steps; s++) {
-    mma(taddr + (s & 1 ? (unsigned)N : 0u), g, x, one, s > 1);
-    mma(low, g, x + xp, two, s > 0);
-    mma(low, g + gp, x, two, true);
-    mma(lowest, g + 2 * gp, x, one, true);
-    g += gs; x += xs;
+    for (int s = 0; s < n_steps; s++) {
+      mma(d, g, x, one, s > 1);
+      mma(t + 2 * un, g, x + xp, two, s > 0);
+      mma(t + 2 * un, g + gp, x, two, true);
+      mma(t + 3 * un, g + 2 * gp, x, one, true);
+      g += gs; x += xs;
+      const unsigned q = d; d = other; other = q;
+    }
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" :: "r"(bar) : "memory");
   }
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" :: "r"(bar) : "memory");
+  __syncwarp();
 }
 static __device__ __noinline__ float outer_plain(const unsigned char* Gb, const unsigned g_part, const unsigned g_group, const unsigned char* Xb, const unsigned x_part, const unsigned x_group, const int count, const int o, const int i) {
   float v = 0.f;
