@@ -50,7 +50,7 @@ constexpr int HT = 128;                       // helper threads
 constexpr int NT = CT + HT;
 constexpr int SLOT_WORDS = 6;
 constexpr int ACC_RED = CW * 8 * 32 * 4;       // floats of an accumulator's merge buffer
-constexpr int PIECES = 256;                   // pieces of a chunk a warp lists
+constexpr int PIECES = 128;                   // pieces of a chunk a warp lists
 constexpr int NEAR = 128;                     // touched pieces of embedding rows a warp lists in shared memory
 
 enum { H_FIRST = 1, H_LAST = 2, H_UPDATE = 4, H_END = 8, H_COPIES = 16, H_LONG = 32 };      // H_COPIES: every row is one or two copies; H_LONG: a row has more terms than its descriptor holds
@@ -1899,12 +1899,13 @@ __device__ __noinline__ void lookup_grad_main(const int team, const int tile, fl
   const PptRun& P = S.ppt;
   const int segs = (o4 + 31) >> 5, ids = (P.in_dim + NTL - 1) / NTL;
   int* const near_list = reinterpret_cast<int*>(smem) + warp * NEAR;
-  int* const work = reinterpret_cast<int*>(smem) + CW * NEAR + warp * PIECES;      // (segment, row) of the chunk
+  uint4* const work = reinterpret_cast<uint4*>(reinterpret_cast<int*>(smem) + CW * NEAR) + warp * PIECES;      // of the chunk: gradient, table row, segment, row
   // a bit per piece: listed already (in device memory behind the lists where a table is too large)
   const size_t words = ((size_t)ids * segs + 31) >> 5;
-  unsigned* const bits = words <= LOOKUP_BITS ? reinterpret_cast<unsigned*>(smem) + CW * (NEAR + PIECES) : P.touched_bits + (size_t)tile * words;
+  unsigned* const bits = words <= LOOKUP_BITS ? reinterpret_cast<unsigned*>(smem) + CW * (NEAR + 4 * PIECES) : P.touched_bits + (size_t)tile * words;
   if (words <= LOOKUP_BITS) for (int i = threadIdx.x; i < (int)words; i += CT) bits[i] = 0u;
   const FastDiv d_tiles(NTL);
+  const unsigned long long seg_M = segs <= 4 ? ((1ull << 33) + segs - 1) / (unsigned)segs : 0ull;      // piece / segs by a multiplication, exact below 2^31 for up to four segments
   bar_compute();
   int* const far_list = P.touched_list + ((size_t)tile * CW + warp) * ((size_t)ids * segs / CW + segs + 1);
   const bool wide = (out & 3) == 0;
@@ -1918,7 +1919,7 @@ __device__ __noinline__ void lookup_grad_main(const int team, const int tile, fl
       int cq[4];
 #pragma unroll
       for (int u = 0; u < 4; u++) {
-        const int k = min(k0 + u, touched - 1), piece = k < NEAR ? near_list[k] : far_list[k], local = piece / segs, c = (piece - local * segs) * 32 + lane;
+        const int k = min(k0 + u, touched - 1), piece = k < NEAR ? near_list[k] : far_list[k], local = seg_M ? (int)(((unsigned long long)(unsigned)piece * seg_M) >> 33) : piece / segs, c = (piece - local * segs) * 32 + lane;
         r0[u] = ((size_t)local * NTL + tile) * out + 4 * c;
         cq[u] = k0 + u < touched ? out - 4 * c : 0;
         if (wide && cq[u] > 0) {
@@ -1960,17 +1961,16 @@ __device__ __noinline__ void lookup_grad_main(const int team, const int tile, fl
 #pragma unroll
         for (int k = 0; k < 8; k++) {
           v[k] = zero4();
-          const int x = k0 + k < listed ? work[k0 + k] : -1, c = 32 * (x >> 8) + lane;
-          if (x < 0 || c >= o4) continue;
-          const RowD& r = R[x & 255];
-          v[k] = h.flags & H_COPIES ? ldcg4(S.core.arena + r.t[0].src4 + c) : rnd4(S.core.bf16, row_sum<false>(r, c));
+          if (k0 + k >= listed) continue;
+          const uint4 x = work[k0 + k];
+          if ((int)x.z * 32 + lane < o4) v[k] = h.flags & H_COPIES ? ldcg4(S.core.arena + x.x + lane) : rnd4(S.core.bf16, row_sum<false>(R[x.w], (int)x.z * 32 + lane));
         }
 #pragma unroll
         for (int k = 0; k < 8; k++) {
           if (k0 + k >= listed) break;
-          const int x = work[k0 + k], q = x >> 8, c = 32 * q + lane;
-          const unsigned id = R[x & 255].b4;
-          float* const a = P.A + (size_t)id * out + 4 * c;
+          const uint4 x = work[k0 + k];
+          const int c = (int)x.z * 32 + lane;
+          float* const a = P.A + (size_t)x.y * out + 4 * c;
           if (c < o4) {
             if (wide) asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" :: "l"(a), "f"(v[k].x), "f"(v[k].y), "f"(v[k].z), "f"(v[k].w) : "memory");
             else {
@@ -1999,7 +1999,7 @@ __device__ __noinline__ void lookup_grad_main(const int team, const int tile, fl
         const int piece = of * segs + q;
         bool fresh = false;
         if (mine) {
-          work[listed + __popc(all & before)] = (q << 8) | (b0 + lane);
+          work[listed + __popc(all & before)] = make_uint4(R[b0 + lane].t[0].src4 + 32u * (unsigned)q, (unsigned)id, (unsigned)q, (unsigned)(b0 + lane));
           fresh = !(atomicOr(bits + (piece >> 5), 1u << (piece & 31)) >> (piece & 31) & 1u);
         }
         const unsigned news = __ballot_sync(0xffffffffu, fresh);
@@ -2129,7 +2129,7 @@ size_t smem_bytes(const Team& t, const Mat& m, int mak) {
         const size_t steps = (BM + 15) / 16, N = split_columns(t.C), g = (size_t)((t.R + 7) / 8) * tc3::CORE_K, x = N / 8 * tc3::CORE_K, reach = (2 * steps - 1) * 3 * g + 2 * g + (size_t)(t.split / 8) * tc3::CORE_K;
         f = (size_t)t.R * pad_ld((int)N) + ((t.R + 3) & ~3) + std::max(steps * 2 * 3 * (g + x), reach) / 4;
       } else f = (size_t)t.R * (t.C + 4) + ACC_RED + BM * (t.R + 4 + t.C + 4) + t.R + (size_t)(CW / (t.WO * t.WI)) * t.R; break;
-    case LOOKUP_B: f = t.R ? BM * (t.C + 4) + (size_t)t.G * (t.R * t.C + 1) : CW * (NEAR + PIECES) + LOOKUP_BITS; break;      // (small table of G rows: R copies of the sums of C columns)
+    case LOOKUP_B: f = t.R ? BM * (t.C + 4) + (size_t)t.G * (t.R * t.C + 1) : CW * (NEAR + 4 * PIECES) + LOOKUP_BITS; break;      // (small table of G rows: R copies of the sums of C columns)
     case HEAD: f = (size_t)m.outp * ldi + m.outp + BM * ldi + 2 * BM * pad_ld(m.outp); break;
     default: break;
   }
