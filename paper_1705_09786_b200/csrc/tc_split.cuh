@@ -74,20 +74,22 @@ __device__ __forceinline__ void mma(const unsigned d, const uint64_t a, const ui
 // The first warp issues the whole product (one thread of it) and commits it to the mbarrier at `bar`; operands written, fenced
 // (fence_operands) and the CTA synchronised before.  Accumulators from column 0: the chains of hh, then hm + mh, then hl + mm + lh, n columns
 // each.  An instruction takes its operands from uniform registers: descriptors that the warp has agreed on before the loop cost 30 cycles
-// an instruction, one thread's own values 57.
-template <class T> __device__ __forceinline__ T uniform(const T v) { return __shfl_sync(0xffffffffu, v, 0); }
+// an instruction, one thread's own values 57 (training kernels; in the evaluation kernel it is the other way round, K = 100: 6,600 cycles
+// against 4,000, so it takes the first thread's own).
+template <bool AGREED = true, class T> __device__ __forceinline__ T uniform(const T v) { if constexpr (AGREED) return __shfl_sync(0xffffffffu, v, 0); else return v; }
 __device__ __forceinline__ bool elected() {
   unsigned e;
   asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}" : "=r"(e));
   return e != 0;
 }
+template <bool AGREED>
 __device__ __forceinline__ void issue(const unsigned taddr, const unsigned char* Wb, const unsigned w_part, const unsigned char* Xb, const unsigned x_part, const unsigned group, const int M, const int n, const int K, const unsigned bar) {
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const int steps = uniform(k_steps(K)), un = uniform(n);
-  const uint64_t wh = uniform(smem_desc(smem_addr(Wb), group)), xh = uniform(smem_desc(smem_addr(Xb), group)), wp = uniform((uint64_t)(w_part >> 4)), xp = uniform((uint64_t)(x_part >> 4));
-  const uint32_t two = uniform(instr_desc(M, 2 * n)), one = uniform(instr_desc(M, n));
-  const unsigned t = uniform(taddr), low = uniform(taddr + (unsigned)(chains(K) * n));
-  if (elected()) {
+  const int steps = uniform<AGREED>(k_steps(K)), un = uniform<AGREED>(n);
+  const uint64_t wh = uniform<AGREED>(smem_desc(smem_addr(Wb), group)), xh = uniform<AGREED>(smem_desc(smem_addr(Xb), group)), wp = uniform<AGREED>((uint64_t)(w_part >> 4)), xp = uniform<AGREED>((uint64_t)(x_part >> 4));
+  const uint32_t two = uniform<AGREED>(instr_desc(M, 2 * n)), one = uniform<AGREED>(instr_desc(M, n));
+  const unsigned t = uniform<AGREED>(taddr), low = uniform<AGREED>(taddr + (unsigned)(chains(K) * n));
+  if (AGREED ? elected() : (threadIdx.x & 31) == 0) {
     unsigned d = t;
     uint64_t w = wh, x = xh;
     int left = CHAIN;

@@ -995,7 +995,7 @@ __device__ __noinline__ void product_parts(const Parts W, const Parts X, const i
   tc3::fence_operands();
   bar_compute();
   phase(2);
-  if (threadIdx.x < 32) tc3::issue(S.tmem, W.base, W.part, X.base, X.part, W.group, M, n, K, smem_u32(&S.tc_mbar));
+  if (threadIdx.x < 32) tc3::issue<!EVALUATING>(S.tmem, W.base, W.part, X.base, X.part, W.group, M, n, K, smem_u32(&S.tc_mbar));
   const bool done = mbar_wait(&S.tc_mbar, parity, t0, 26);
   if (!done) for (unsigned extra = 0; extra < (1u << 16) && !mbar_try(&S.tc_mbar, parity); extra++) {}      // what was issued still writes the accumulators
   parity ^= 1;
@@ -1958,13 +1958,17 @@ __device__ __noinline__ void lookup_grad_main(const int team, const int tile, fl
 #pragma unroll 1
       for (int k0 = 0; k0 < listed; k0 += 8) {                     // eight pieces' loads in flight (a frequent word has a dozen rows a round)
         float4 v[8];
+        if (h.flags & H_COPIES) {                                  // (loads without a branch between them: nothing waits for one before the next)
 #pragma unroll
-        for (int k = 0; k < 8; k++) {
-          v[k] = zero4();
-          if (k0 + k >= listed) continue;
-          const uint4 x = work[k0 + k];
-          if ((int)x.z * 32 + lane < o4) v[k] = h.flags & H_COPIES ? ldcg4(S.core.arena + x.x + lane) : rnd4(S.core.bf16, row_sum<false>(R[x.w], (int)x.z * 32 + lane));
-        }
+          for (int k = 0; k < 8; k++) { const uint4 x = work[min(k0 + k, listed - 1)]; v[k] = ldcg4(S.core.arena + x.x + min(lane, o4 - 1 - 32 * (int)x.z)); }
+        } else
+#pragma unroll 1
+          for (int k = 0; k < 8; k++) {
+            const uint4 x = work[min(k0 + k, listed - 1)];
+            const float4 e = rnd4(S.core.bf16, row_sum<false>(R[x.w], min(32 * (int)x.z + lane, o4 - 1)));
+#pragma unroll
+            for (int u = 0; u < 8; u++) if (u == k) v[u] = e;
+          }
 #pragma unroll
         for (int k = 0; k < 8; k++) {
           if (k0 + k >= listed) break;

@@ -314,7 +314,7 @@ static bool wave_best(const WaveModel& M, int c, int ctas, double rows, double m
   // products of 32-bit operands on the tensor cores: four instructions a step of sixteen, whatever the rows, and the accumulators' way back
   const double acc_base = 5000, acc_row = 0.17, acc_chunk = 3500;
   const double split_gather = 0.7, split_weights = 1.5, split_chunk = 5000;
-  auto split_product = [](const int k) { return 1300 + 4 * 30.0 * tc3::k_steps(k) + 150.0 * tc3::chains(k); };
+  auto split_product = [eval](const int k) { return 1300 + 4 * (eval ? 57.0 : 30.0) * tc3::k_steps(k) + 150.0 * tc3::chains(k); };
   int env_rows = 0, env_cols = 0;
   if (const char* e = getenv("AMPNET_DIRECT_ROWS")) env_rows = std::max(1, atoi(e));
   if (const char* e = getenv("AMPNET_DIRECT_COLS")) env_cols = std::max(4, atoi(e));
