@@ -1893,6 +1893,8 @@ __device__ __noinline__ void lookup_grad_small_main(const int team, const int ti
 // A large table: rows are dealt to the tiles by id; a piece of 128 columns of a row always belongs to the same warp of the tile and a
 // column to the same lane, so that a thread's adds and its own later reads are in order without fences or barriers.  A warp lists the
 // pieces it has touched since the last update (the list's overflow in device memory) and moves exactly those.
+// Frequent words: adds to one address meet in L2 one after the other, some 1,000 cycles each (a word of the wide tree comes sixty times a
+// round), so up to 16 pieces of a warp have their sums in shared memory instead, the first of those that share a slot until the update.
 __device__ __noinline__ void lookup_grad_main(const int team, const int tile, float* smem, RowD* rows, const unsigned long long t0) {
   IN_SMEM(smem); IN_SMEM(rows);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, out = S.ppt.out_dim, o4 = S.ppt.out4, NTL = S.team.T;
@@ -1906,6 +1908,11 @@ __device__ __noinline__ void lookup_grad_main(const int team, const int tile, fl
   if (words <= LOOKUP_BITS) for (int i = threadIdx.x; i < (int)words; i += CT) bits[i] = 0u;
   const FastDiv d_tiles(NTL);
   const unsigned long long seg_M = segs <= 4 ? ((1ull << 33) + segs - 1) / (unsigned)segs : 0ull;      // piece / segs by a multiplication, exact below 2^31 for up to four segments
+  const int SL = S.team.G;                                        // slots of a warp (a power of two, or none)
+  int* const tag = reinterpret_cast<int*>(smem) + CW * (NEAR + 4 * PIECES) + LOOKUP_BITS + warp * SL;
+  float4* const held = reinterpret_cast<float4*>(reinterpret_cast<int*>(smem) + CW * (NEAR + 4 * PIECES) + LOOKUP_BITS + CW * SL) + (size_t)warp * SL * 32 + lane;
+  for (int k = 0; k < SL; k++) { held[k * 32] = zero4(); if (lane == 0) tag[k] = -1; }
+  auto slot_of = [&](const int piece) { return (piece >> 4) & (SL - 1); };      // (the pieces of a warp are alike modulo CW)
   bar_compute();
   int* const far_list = P.touched_list + ((size_t)tile * CW + warp) * ((size_t)ids * segs / CW + segs + 1);
   const bool wide = (out & 3) == 0;
@@ -1916,13 +1923,21 @@ __device__ __noinline__ void lookup_grad_main(const int team, const int tile, fl
     for (int k0 = 0; k0 < touched; k0 += 4) {                    // four pieces' loads in flight
       float a[4][4], w[4][4];
       size_t r0[4];
-      int cq[4];
+      int cq[4], at[4];
 #pragma unroll
       for (int u = 0; u < 4; u++) {
         const int k = min(k0 + u, touched - 1), piece = k < NEAR ? near_list[k] : far_list[k], local = seg_M ? (int)(((unsigned long long)(unsigned)piece * seg_M) >> 33) : piece / segs, c = (piece - local * segs) * 32 + lane;
         r0[u] = ((size_t)local * NTL + tile) * out + 4 * c;
         cq[u] = k0 + u < touched ? out - 4 * c : 0;
-        if (wide && cq[u] > 0) {
+        at[u] = SL && tag[slot_of(piece)] == piece ? slot_of(piece) : -1;
+        if (at[u] >= 0) {
+          const float4 e = held[at[u] * 32];
+          a[u][0] = e.x; a[u][1] = e.y; a[u][2] = e.z; a[u][3] = e.w;
+          if (wide && cq[u] > 0) { const float4 x = *reinterpret_cast<const float4*>(P.W + r0[u]); w[u][0] = x.x; w[u][1] = x.y; w[u][2] = x.z; w[u][3] = x.w; }
+          else
+#pragma unroll
+            for (int q = 0; q < 4; q++) if (q < cq[u]) w[u][q] = P.W[r0[u] + q];
+        } else if (wide && cq[u] > 0) {
           asm volatile("ld.relaxed.gpu.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(a[u][0]), "=f"(a[u][1]), "=f"(a[u][2]), "=f"(a[u][3]) : "l"(P.A + r0[u]) : "memory");
           const float4 x = *reinterpret_cast<const float4*>(P.W + r0[u]);
           w[u][0] = x.x; w[u][1] = x.y; w[u][2] = x.z; w[u][3] = x.w;
@@ -1935,20 +1950,24 @@ __device__ __noinline__ void lookup_grad_main(const int team, const int tile, fl
       for (int u = 0; u < 4; u++) {
         if (wide && cq[u] > 0 && (SGD || os.opt == 0)) {
           *reinterpret_cast<float4*>(P.W + r0[u]) = sgd4(os.step, make_float4(w[u][0], w[u][1], w[u][2], w[u][3]), make_float4(a[u][0], a[u][1], a[u][2], a[u][3]));
-          asm volatile("st.relaxed.gpu.global.v4.f32 [%0], {%1, %1, %1, %1};" :: "l"(P.A + r0[u]), "f"(0.f) : "memory");
+          if (at[u] < 0) asm volatile("st.relaxed.gpu.global.v4.f32 [%0], {%1, %1, %1, %1};" :: "l"(P.A + r0[u]), "f"(0.f) : "memory");
+          else held[at[u] * 32] = zero4();
           continue;
         }
 #pragma unroll
         for (int q = 0; q < 4; q++)
           if (q < cq[u]) {
             P.W[r0[u] + q] = opt_one(os, w[u][q], a[u][q], r0[u] + q);
-            asm volatile("st.relaxed.gpu.global.f32 [%0], %1;" :: "l"(P.A + r0[u] + q), "f"(0.f) : "memory");
+            if (at[u] < 0) asm volatile("st.relaxed.gpu.global.f32 [%0], %1;" :: "l"(P.A + r0[u] + q), "f"(0.f) : "memory");
           }
+        if (at[u] >= 0 && k0 + u < touched) held[at[u] * 32] = zero4();
       }
     }
 #pragma unroll 1
     for (int k = lane; k < touched; k += 32) { const int piece = k < NEAR ? near_list[k] : far_list[k]; atomicAnd(bits + (piece >> 5), ~(1u << (piece & 31))); }
     touched = 0;
+    __syncwarp();
+    if (lane < SL) tag[lane] = -1;
     __syncwarp();
   };
   chunk_loop(rows, team, t0, [&](const Head& h, const RowD* R) {
@@ -1960,12 +1979,12 @@ __device__ __noinline__ void lookup_grad_main(const int team, const int tile, fl
         float4 v[8];
         if (h.flags & H_COPIES) {                                  // (loads without a branch between them: nothing waits for one before the next)
 #pragma unroll
-          for (int k = 0; k < 8; k++) { const uint4 x = work[min(k0 + k, listed - 1)]; v[k] = ldcg4(S.core.arena + x.x + min(lane, o4 - 1 - 32 * (int)x.z)); }
+          for (int k = 0; k < 8; k++) { const uint4 x = work[min(k0 + k, listed - 1)]; v[k] = ldcg4(S.core.arena + x.x + min(lane, o4 - 1 - 32 * (int)(x.z & 0xffffu))); }
         } else
 #pragma unroll 1
           for (int k = 0; k < 8; k++) {
             const uint4 x = work[min(k0 + k, listed - 1)];
-            const float4 e = rnd4(S.core.bf16, row_sum<false>(R[x.w], min(32 * (int)x.z + lane, o4 - 1)));
+            const float4 e = rnd4(S.core.bf16, row_sum<false>(R[x.w], min(32 * (int)(x.z & 0xffffu) + lane, o4 - 1)));
 #pragma unroll
             for (int u = 0; u < 8; u++) if (u == k) v[u] = e;
           }
@@ -1973,7 +1992,12 @@ __device__ __noinline__ void lookup_grad_main(const int team, const int tile, fl
         for (int k = 0; k < 8; k++) {
           if (k0 + k >= listed) break;
           const uint4 x = work[k0 + k];
-          const int c = (int)x.z * 32 + lane;
+          const int c = (int)(x.z & 0xffffu) * 32 + lane;
+          if (x.z >> 16) {
+            float4* const e = held + ((x.z >> 16) - 1) * 32;
+            *e = add4(*e, v[k]);
+            continue;
+          }
           float* const a = P.A + (size_t)x.y * out + 4 * c;
           if (c < o4) {
             if (wide) asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" :: "l"(a), "f"(v[k].x), "f"(v[k].y), "f"(v[k].z), "f"(v[k].w) : "memory");
@@ -2002,12 +2026,15 @@ __device__ __noinline__ void lookup_grad_main(const int team, const int tile, fl
         const unsigned before = (1u << lane) - 1u;
         const int piece = of * segs + q;
         bool fresh = false;
-        if (mine) {
-          work[listed + __popc(all & before)] = make_uint4(R[b0 + lane].t[0].src4 + 32u * (unsigned)q, (unsigned)id, (unsigned)q, (unsigned)(b0 + lane));
-          fresh = !(atomicOr(bits + (piece >> 5), 1u << (piece & 31)) >> (piece & 31) & 1u);
-        }
+        if (mine) fresh = !(atomicOr(bits + (piece >> 5), 1u << (piece & 31)) >> (piece & 31) & 1u);
+        if (fresh && SL) atomicCAS(tag + slot_of(piece), -1, piece);
         const unsigned news = __ballot_sync(0xffffffffu, fresh);
         if (fresh) { const int x = touched + __popc(news & before); if (x < NEAR) near_list[x] = piece; else far_list[x] = piece; }
+        __syncwarp();
+        if (mine) {
+          const unsigned slot = SL && tag[slot_of(piece)] == piece ? (unsigned)slot_of(piece) + 1u : 0u;
+          work[listed + __popc(all & before)] = make_uint4(R[b0 + lane].t[0].src4 + 32u * (unsigned)q, (unsigned)id, (unsigned)q | slot << 16, (unsigned)(b0 + lane));
+        }
         listed += __popc(all);
         touched += __popc(news);
         __syncwarp();
@@ -2133,7 +2160,7 @@ size_t smem_bytes(const Team& t, const Mat& m, int mak) {
         const size_t steps = (BM + 15) / 16, N = split_columns(t.C), g = (size_t)((t.R + 7) / 8) * tc3::CORE_K, x = N / 8 * tc3::CORE_K, reach = (2 * steps - 1) * 3 * g + 2 * g + (size_t)(t.split / 8) * tc3::CORE_K;
         f = (size_t)t.R * pad_ld((int)N) + ((t.R + 3) & ~3) + std::max(steps * 2 * 3 * (g + x), reach) / 4;
       } else f = (size_t)t.R * (t.C + 4) + ACC_RED + BM * (t.R + 4 + t.C + 4) + t.R + (size_t)(CW / (t.WO * t.WI)) * t.R; break;
-    case LOOKUP_B: f = t.R ? BM * (t.C + 4) + (size_t)t.G * (t.R * t.C + 1) : CW * (NEAR + 4 * PIECES) + LOOKUP_BITS; break;      // (small table of G rows: R copies of the sums of C columns)
+    case LOOKUP_B: f = t.R ? BM * (t.C + 4) + (size_t)t.G * (t.R * t.C + 1) : CW * (NEAR + 4 * PIECES) + LOOKUP_BITS + (size_t)CW * t.G * (1 + 128); break;      // (small table of G rows: R copies of the sums of C columns)
     case HEAD: f = (size_t)m.outp * ldi + m.outp + BM * ldi + 2 * BM * pad_ld(m.outp); break;
     default: break;
   }
