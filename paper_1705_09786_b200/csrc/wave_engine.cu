@@ -1895,123 +1895,123 @@ __device__ __noinline__ void lookup_grad_small_main(const int team, const int ti
 // pieces it has touched since the last update (the list's overflow in device memory) and moves exactly those.
 // Frequent words: adds to one address meet in L2 one after the other, some 1,000 cycles each (a word of the wide tree comes sixty times a
 // round), so up to 16 pieces of a warp have their sums in shared memory instead, the first of those that share a slot until the update.
-__device__ __noinline__ void lookup_grad_main(const int team, const int tile, float* smem, RowD* rows, const unsigned long long t0) {
-  IN_SMEM(smem); IN_SMEM(rows);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, out = S.ppt.out_dim, o4 = S.ppt.out4, NTL = S.team.T;
-  const PptRun& P = S.ppt;
-  const int segs = (o4 + 31) >> 5, ids = (P.in_dim + NTL - 1) / NTL;
-  int* const near_list = reinterpret_cast<int*>(smem) + warp * NEAR;
-  uint4* const work = reinterpret_cast<uint4*>(reinterpret_cast<int*>(smem) + CW * NEAR) + warp * PIECES;      // of the chunk: gradient, table row, segment, row
-  // a bit per piece: listed already (in device memory behind the lists where a table is too large)
-  const size_t words = ((size_t)ids * segs + 31) >> 5;
-  unsigned* const bits = words <= LOOKUP_BITS ? reinterpret_cast<unsigned*>(smem) + CW * (NEAR + 4 * PIECES) : P.touched_bits + (size_t)tile * words;
-  if (words <= LOOKUP_BITS) for (int i = threadIdx.x; i < (int)words; i += CT) bits[i] = 0u;
-  const FastDiv d_tiles(NTL);
-  const unsigned long long seg_M = segs <= 4 ? ((1ull << 33) + segs - 1) / (unsigned)segs : 0ull;      // piece / segs by a multiplication, exact below 2^31 for up to four segments
-  const int SL = S.team.G;                                        // slots of a warp (a power of two, or none)
-  int* const tag = reinterpret_cast<int*>(smem) + CW * (NEAR + 4 * PIECES) + LOOKUP_BITS + warp * SL;
-  float4* const held = reinterpret_cast<float4*>(reinterpret_cast<int*>(smem) + CW * (NEAR + 4 * PIECES) + LOOKUP_BITS + CW * SL) + (size_t)warp * SL * 32 + lane;
-  for (int k = 0; k < SL; k++) { held[k * 32] = zero4(); if (lane == 0) tag[k] = -1; }
-  auto slot_of = [&](const int piece) { return (piece >> 4) & (SL - 1); };      // (the pieces of a warp are alike modulo CW)
-  bar_compute();
-  int* const far_list = P.touched_list + ((size_t)tile * CW + warp) * ((size_t)ids * segs / CW + segs + 1);
+// (Functions of their own: with them inside, the loop over the chunks spills 800 bytes and an epoch of the tree takes half as long again.)
+__device__ __noinline__ void add_pieces(const uint4* work, const int listed, const RowD* R, float4* held, const bool copies) {
+  IN_SMEM(work); IN_SMEM(R); IN_SMEM(held);
+  const int lane = threadIdx.x & 31, out = S.ppt.out_dim, o4 = S.ppt.out4;
   const bool wide = (out & 3) == 0;
-  int touched = 0;                                               // (the same in all lanes)
-  auto update = [&](const int n_upd, const int upd_t) {
-    const OptStep os = opt_step(P.om, P.ov, P.opt_t0, n_upd, upd_t);
+  const float4* const arena = S.core.arena;
+  float* const A = S.ppt.A;
+  constexpr int U = 8;                                            // pieces whose loads are in flight
 #pragma unroll 1
-    for (int k0 = 0; k0 < touched; k0 += 4) {                    // four pieces' loads in flight
-      float a[4][4], w[4][4];
-      size_t r0[4];
-      int cq[4], at[4];
+  for (int k0 = 0; k0 < listed; k0 += U) {
+    float4 v[U];
 #pragma unroll
-      for (int u = 0; u < 4; u++) {
-        const int k = min(k0 + u, touched - 1), piece = k < NEAR ? near_list[k] : far_list[k], local = seg_M ? (int)(((unsigned long long)(unsigned)piece * seg_M) >> 33) : piece / segs, c = (piece - local * segs) * 32 + lane;
-        r0[u] = ((size_t)local * NTL + tile) * out + 4 * c;
-        cq[u] = k0 + u < touched ? out - 4 * c : 0;
-        at[u] = SL && tag[slot_of(piece)] == piece ? slot_of(piece) : -1;
-        if (at[u] >= 0) {
-          const float4 e = held[at[u] * 32];
-          a[u][0] = e.x; a[u][1] = e.y; a[u][2] = e.z; a[u][3] = e.w;
-          if (wide && cq[u] > 0) { const float4 x = *reinterpret_cast<const float4*>(P.W + r0[u]); w[u][0] = x.x; w[u][1] = x.y; w[u][2] = x.z; w[u][3] = x.w; }
-          else
+    for (int k = 0; k < U; k++) {
+      const uint4 x = work[min(k0 + k, listed - 1)];
+      const int c = min(32 * (int)(x.z & 0xffffu) + lane, o4 - 1);
+      if (copies) v[k] = ldcg4(arena + x.x + c);
+      else v[k] = rnd4(S.core.bf16, row_sum<false>(R[x.w], c));
+    }
 #pragma unroll
-            for (int q = 0; q < 4; q++) if (q < cq[u]) w[u][q] = P.W[r0[u] + q];
-        } else if (wide && cq[u] > 0) {
-          asm volatile("ld.relaxed.gpu.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(a[u][0]), "=f"(a[u][1]), "=f"(a[u][2]), "=f"(a[u][3]) : "l"(P.A + r0[u]) : "memory");
-          const float4 x = *reinterpret_cast<const float4*>(P.W + r0[u]);
-          w[u][0] = x.x; w[u][1] = x.y; w[u][2] = x.z; w[u][3] = x.w;
-        } else
+    for (int k = 0; k < U; k++) {
+      if (k0 + k >= listed) break;
+      const uint4 x = work[k0 + k];
+      const int c = 32 * (int)(x.z & 0xffffu) + lane, slot = (int)(x.z >> 16);
+      if (slot) { held[slot * 32] = add4(held[slot * 32], v[k]); continue; }
+      if (c >= o4) continue;
+      float* const a = A + (size_t)x.y * out + 4 * c;
+      if (wide) asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" :: "l"(a), "f"(v[k].x), "f"(v[k].y), "f"(v[k].z), "f"(v[k].w) : "memory");
+      else {
+        const float e[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
 #pragma unroll
-          for (int q = 0; q < 4; q++)
-            if (q < cq[u]) { asm volatile("ld.relaxed.gpu.global.f32 %0, [%1];" : "=f"(a[u][q]) : "l"(P.A + r0[u] + q) : "memory"); w[u][q] = P.W[r0[u] + q]; }
+        for (int y = 0; y < 4; y++) if (4 * c + y < out) asm volatile("red.relaxed.gpu.global.add.f32 [%0], %1;" :: "l"(a + y), "f"(e[y]) : "memory");
       }
+    }
+  }
+}
+// A warp's touched pieces move; their sums, bits and slots start over.
+__device__ __noinline__ void update_pieces(const int* near_list, const int* far_list, const int touched, int* tag, float4* held, const int SL, unsigned* bits, const int tile, const int n_upd, const int upd_t) {
+  IN_SMEM(near_list); IN_SMEM(tag); IN_SMEM(held);
+  const int lane = threadIdx.x & 31, out = S.ppt.out_dim, NTL = S.team.T, segs = (S.ppt.out4 + 31) >> 5;
+  float* const W = S.ppt.W; float* const A = S.ppt.A;
+  const bool wide = (out & 3) == 0;
+  const unsigned long long seg_M = segs <= 4 ? ((1ull << 33) + segs - 1) / (unsigned)segs : 0ull;      // piece / segs by a multiplication, exact below 2^31 for up to four segments
+  const OptStep os = opt_step(S.ppt.om, S.ppt.ov, S.ppt.opt_t0, n_upd, upd_t);
+  constexpr int U = 4;                                            // pieces whose loads are in flight
+#pragma unroll 1
+  for (int k0 = 0; k0 < touched; k0 += U) {
+    float4 a[U], w[U];
+    size_t r0[U];
+    int cq[U], at[U];
 #pragma unroll
-      for (int u = 0; u < 4; u++) {
-        if (wide && cq[u] > 0 && (SGD || os.opt == 0)) {
-          *reinterpret_cast<float4*>(P.W + r0[u]) = sgd4(os.step, make_float4(w[u][0], w[u][1], w[u][2], w[u][3]), make_float4(a[u][0], a[u][1], a[u][2], a[u][3]));
-          if (at[u] < 0) asm volatile("st.relaxed.gpu.global.v4.f32 [%0], {%1, %1, %1, %1};" :: "l"(P.A + r0[u]), "f"(0.f) : "memory");
-          else held[at[u] * 32] = zero4();
-          continue;
-        }
+    for (int u = 0; u < U; u++) {
+      const int k = min(k0 + u, touched - 1), piece = k < NEAR ? near_list[k] : far_list[k];
+      const int local = seg_M ? (int)(((unsigned long long)(unsigned)piece * seg_M) >> 33) : piece / segs, c = (piece - local * segs) * 32 + lane;
+      r0[u] = ((size_t)local * NTL + tile) * out + 4 * c;
+      cq[u] = k0 + u < touched ? out - 4 * c : 0;
+      at[u] = SL && tag[(piece >> 4) & (SL - 1)] == piece ? (piece >> 4) & (SL - 1) : -1;
+      a[u] = w[u] = zero4();
+      if (wide && cq[u] > 0) {
+        if (at[u] < 0) asm volatile("ld.relaxed.gpu.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(a[u].x), "=f"(a[u].y), "=f"(a[u].z), "=f"(a[u].w) : "l"(A + r0[u]) : "memory");
+        w[u] = *reinterpret_cast<const float4*>(W + r0[u]);
+      } else if (cq[u] > 0) {
+        float* const x = &a[u].x; float* const y = &w[u].x;
 #pragma unroll
         for (int q = 0; q < 4; q++)
           if (q < cq[u]) {
-            P.W[r0[u] + q] = opt_one(os, w[u][q], a[u][q], r0[u] + q);
-            if (at[u] < 0) asm volatile("st.relaxed.gpu.global.f32 [%0], %1;" :: "l"(P.A + r0[u] + q), "f"(0.f) : "memory");
+            if (at[u] < 0) asm volatile("ld.relaxed.gpu.global.f32 %0, [%1];" : "=f"(x[q]) : "l"(A + r0[u] + q) : "memory");
+            y[q] = W[r0[u] + q];
           }
-        if (at[u] >= 0 && k0 + u < touched) held[at[u] * 32] = zero4();
       }
     }
-#pragma unroll 1
-    for (int k = lane; k < touched; k += 32) { const int piece = k < NEAR ? near_list[k] : far_list[k]; atomicAnd(bits + (piece >> 5), ~(1u << (piece & 31))); }
-    touched = 0;
-    __syncwarp();
-    if (lane < SL) tag[lane] = -1;
-    __syncwarp();
-  };
-  chunk_loop(rows, team, t0, [&](const Head& h, const RowD* R) {
-// the warp's pieces of the chunk are listed first, so that its loads overlap whatever rows they come from
-    int listed = 0;
-    auto add_listed = [&]() {
-#pragma unroll 1
-      for (int k0 = 0; k0 < listed; k0 += 8) {                     // eight pieces' loads in flight (a frequent word has a dozen rows a round)
-        float4 v[8];
-        if (h.flags & H_COPIES) {                                  // (loads without a branch between them: nothing waits for one before the next)
 #pragma unroll
-          for (int k = 0; k < 8; k++) { const uint4 x = work[min(k0 + k, listed - 1)]; v[k] = ldcg4(S.core.arena + x.x + min(lane, o4 - 1 - 32 * (int)(x.z & 0xffffu))); }
-        } else
-#pragma unroll 1
-          for (int k = 0; k < 8; k++) {
-            const uint4 x = work[min(k0 + k, listed - 1)];
-            const float4 e = rnd4(S.core.bf16, row_sum<false>(R[x.w], min(32 * (int)(x.z & 0xffffu) + lane, o4 - 1)));
-#pragma unroll
-            for (int u = 0; u < 8; u++) if (u == k) v[u] = e;
-          }
-#pragma unroll
-        for (int k = 0; k < 8; k++) {
-          if (k0 + k >= listed) break;
-          const uint4 x = work[k0 + k];
-          const int c = (int)(x.z & 0xffffu) * 32 + lane;
-          if (x.z >> 16) {
-            float4* const e = held + ((x.z >> 16) - 1) * 32;
-            *e = add4(*e, v[k]);
-            continue;
-          }
-          float* const a = P.A + (size_t)x.y * out + 4 * c;
-          if (c < o4) {
-            if (wide) asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" :: "l"(a), "f"(v[k].x), "f"(v[k].y), "f"(v[k].z), "f"(v[k].w) : "memory");
-            else {
-              const float e[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
-#pragma unroll
-              for (int y = 0; y < 4; y++) if (4 * c + y < out) asm volatile("red.relaxed.gpu.global.add.f32 [%0], %1;" :: "l"(a + y), "f"(e[y]) : "memory");
-            }
-          }
-        }
+    for (int u = 0; u < U; u++) {
+      if (k0 + u >= touched) break;
+      if (at[u] >= 0) { a[u] = held[(at[u] + 1) * 32]; held[(at[u] + 1) * 32] = zero4(); }
+      if (cq[u] <= 0) continue;
+      if (wide && (SGD || os.opt == 0)) {
+        *reinterpret_cast<float4*>(W + r0[u]) = sgd4(os.step, w[u], a[u]);
+        if (at[u] < 0) asm volatile("st.relaxed.gpu.global.v4.f32 [%0], {%1, %1, %1, %1};" :: "l"(A + r0[u]), "f"(0.f) : "memory");
+        continue;
       }
-      listed = 0;
-      __syncwarp();
-    };
+      const float x[4] = {a[u].x, a[u].y, a[u].z, a[u].w}, y[4] = {w[u].x, w[u].y, w[u].z, w[u].w};
+#pragma unroll
+      for (int q = 0; q < 4; q++)
+        if (q < cq[u]) {
+          W[r0[u] + q] = opt_one(os, y[q], x[q], r0[u] + q);
+          if (at[u] < 0) asm volatile("st.relaxed.gpu.global.f32 [%0], %1;" :: "l"(A + r0[u] + q), "f"(0.f) : "memory");
+        }
+    }
+  }
+#pragma unroll 1
+  for (int k = lane; k < touched; k += 32) { const int piece = k < NEAR ? near_list[k] : far_list[k]; atomicAnd(bits + (piece >> 5), ~(1u << (piece & 31))); }
+  __syncwarp();
+  if (lane < SL) tag[lane] = -1;
+  __syncwarp();
+}
+__device__ __noinline__ void lookup_grad_main(const int team, const int tile, float* smem, RowD* rows, const unsigned long long t0) {
+  IN_SMEM(smem); IN_SMEM(rows);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, NTL = S.team.T, SL = S.team.G;      // SL: slots of a warp (a power of two, or none)
+  const PptRun& P = S.ppt;
+  const int segs = (P.out4 + 31) >> 5, ids = (P.in_dim + NTL - 1) / NTL;
+  int* const near_list = reinterpret_cast<int*>(smem) + warp * NEAR;
+  uint4* const work = reinterpret_cast<uint4*>(reinterpret_cast<int*>(smem) + CW * NEAR) + warp * PIECES;      // of the chunk: gradient, table row, segment and slot + 1, row
+  // a bit per piece: listed already (in device memory behind the lists where a table is too large)
+  const size_t words = ((size_t)ids * segs + 31) >> 5;
+  unsigned* const near_bits = reinterpret_cast<unsigned*>(smem) + CW * (NEAR + 4 * PIECES);
+  unsigned* const bits = words <= LOOKUP_BITS ? near_bits : P.touched_bits + (size_t)tile * words;
+  if (words <= LOOKUP_BITS) for (int i = threadIdx.x; i < (int)words; i += CT) bits[i] = 0u;
+  int* const tag = reinterpret_cast<int*>(near_bits + LOOKUP_BITS) + warp * SL;
+  float4* const held = reinterpret_cast<float4*>(near_bits + LOOKUP_BITS + CW * SL) + (warp * SL - 1) * 32 + lane;      // slot s at 32 (s + 1)
+  for (int k = 0; k < SL; k++) { held[(k + 1) * 32] = zero4(); if (lane == 0) tag[k] = -1; }
+  const FastDiv d_tiles(NTL);
+  bar_compute();
+  int* const far_list = P.touched_list + ((size_t)tile * CW + warp) * ((size_t)ids * segs / CW + segs + 1);
+  int touched = 0;                                               // (the same in all lanes)
+  chunk_loop(rows, team, t0, [&](const Head& h, const RowD* R) {
+    // the warp's pieces of the chunk are listed first, so that its loads overlap whatever rows they come from
+    int listed = 0;
 #pragma unroll 1
     for (int b0 = 0; b0 < h.count; b0 += 32) {
       const int id = (int)R[min(b0 + lane, h.count - 1)].b4, of = d_tiles.div(id);
@@ -2019,30 +2019,34 @@ __device__ __noinline__ void lookup_grad_main(const int team, const int tile, fl
       if (!__any_sync(0xffffffffu, ours)) continue;
 #pragma unroll 1
       for (int q0 = 0; q0 < segs; q0 += CW) {                      // (of CW neighbouring pieces exactly one is this warp's)
-        const int q = q0 + ((warp - of * segs - q0) & (CW - 1));
+        const int q = q0 + ((warp - of * segs - q0) & (CW - 1)), piece = of * segs + q;
         const bool mine = ours && q < segs;
-        const unsigned all = __ballot_sync(0xffffffffu, mine);
-        if (listed + __popc(all) > PIECES) add_listed();
-        const unsigned before = (1u << lane) - 1u;
-        const int piece = of * segs + q;
+        const unsigned all = __ballot_sync(0xffffffffu, mine), before = (1u << lane) - 1u;
+        if (all == 0) continue;
+        if (listed + __popc(all) > PIECES) { add_pieces(work, listed, R, held, h.flags & H_COPIES); listed = 0; __syncwarp(); }
+        const int slot = SL ? (piece >> 4) & (SL - 1) : 0;          // (the pieces of a warp are alike modulo CW)
         bool fresh = false;
         if (mine) fresh = !(atomicOr(bits + (piece >> 5), 1u << (piece & 31)) >> (piece & 31) & 1u);
-        if (fresh && SL) atomicCAS(tag + slot_of(piece), -1, piece);
+        if (fresh && SL) atomicCAS(tag + slot, -1, piece);
         const unsigned news = __ballot_sync(0xffffffffu, fresh);
         if (fresh) { const int x = touched + __popc(news & before); if (x < NEAR) near_list[x] = piece; else far_list[x] = piece; }
         __syncwarp();
-        if (mine) {
-          const unsigned slot = SL && tag[slot_of(piece)] == piece ? (unsigned)slot_of(piece) + 1u : 0u;
-          work[listed + __popc(all & before)] = make_uint4(R[b0 + lane].t[0].src4 + 32u * (unsigned)q, (unsigned)id, (unsigned)q | slot << 16, (unsigned)(b0 + lane));
-        }
+        if (mine) work[listed + __popc(all & before)] = make_uint4(R[b0 + lane].t[0].src4, (unsigned)id, (unsigned)q | (SL && tag[slot] == piece ? (unsigned)slot + 1u : 0u) << 16, (unsigned)(b0 + lane));
         listed += __popc(all);
         touched += __popc(news);
         __syncwarp();
       }
     }
-    add_listed();
+    if (listed) add_pieces(work, listed, R, held, h.flags & H_COPIES);
+    __syncwarp();
     phase(2);
-    if (h.flags & H_UPDATE) { wait_readers(h, t0); phase(3); update(h.n_upd, h.upd_t); phase(5); }
+    if (h.flags & H_UPDATE) {
+      wait_readers(h, t0);
+      phase(3);
+      update_pieces(near_list, far_list, touched, tag, held, SL, bits, tile, h.n_upd, h.upd_t);
+      touched = 0;
+      phase(5);
+    }
   });
 }
 
