@@ -428,6 +428,10 @@ __device__ __noinline__ void helper_main(const int team, const int cta, const in
   }
 }
 
+// A counter has a line of its own: most CTAs poll one at any time, and neighbours in a line (one slice of the L2) made them wait for each
+// other's requests.
+__device__ __forceinline__ unsigned* progress_of(const int team, const int round) { return S.core.progress + (team * 16 + (round & 15)) * PROGRESS_STRIDE; }
+
 // ---- compute warps: waiting, signalling -------------------------------------------------------------------------------------
 // Warp 0: the publishing cell has finished the round `lag` back; the cells this one reads have finished the previous round, everybody the
 // round DRIFT back (arenas, publications and counters are reused after that).  Returns 1 when only the version is there yet (first
@@ -443,7 +447,7 @@ __device__ __noinline__ int wait_round(const int round, const bool rows, const b
     target = round - DRIFT;
     if (rows && (T.wait_mask >> lane & 1)) target = round - 1;
     if (rows && lane == T.acc) { of_version = true; target = max(target, round - S.core.lag); }
-    if (target >= 0) { n = S.team_n[lane] * ((target >> 4) + 1); p = S.core.progress + lane * 16 + (target & 15); }
+    if (target >= 0) { n = S.team_n[lane] * ((target >> 4) + 1); p = progress_of(lane, target); }
   }
   const unsigned long long* vp = nullptr;
   const int vr = round - S.core.lag;
@@ -451,10 +455,11 @@ __device__ __noinline__ int wait_round(const int round, const bool rows, const b
   unsigned long long v = 0;
   bool ok = true, all = false;
   if (first && (round & 7) == 7 && lane == 0 && over(t0, 23)) ok = false;
+  bool counted = p == nullptr, seen = vp == nullptr;             // (what has been seen is not asked for again)
   for (unsigned it = 1;; it++) {
-    bool ready = true;
-    if (p) ready = (int)ld_acq(p) >= n;
-    if (vp) { v = ld_acq64(vp); ready = (v & 0xffff) == ((unsigned)vr & 0xffffu); }
+    if (!counted) counted = (int)ld_acq(p) >= n;
+    if (!seen) { v = ld_acq64(vp); seen = (v & 0xffff) == ((unsigned)vr & 0xffffu); }
+    const bool ready = counted && seen;
     all = __all_sync(0xffffffffu, ready);
     if (all) break;
     if (first && versioned && __all_sync(0xffffffffu, ready || !of_version)) break;
@@ -473,7 +478,7 @@ __device__ __noinline__ int wait_round(const int round, const bool rows, const b
 __device__ __forceinline__ void wait_readers(const Head& h, const unsigned long long t0) {
   const int reader = S.team.reader, target = (h.flags & H_END) ? h.round : h.round + S.core.lag - 1;
   if ((threadIdx.x & 31) == 0) {
-    const unsigned* const p = S.core.progress + reader * 16 + (target & 15);
+    const unsigned* const p = progress_of(reader, target);
     const int n = S.team_n[reader] * ((target >> 4) + 1);
     for (unsigned it = 1; (int)ld_acq(p) < n; it++)
       if ((it & 63u) == 0 && over(t0, 27)) break;
@@ -517,7 +522,7 @@ __device__ __forceinline__ Head chunk_loop(RowD* rows, const int team, const uns
     } else if (last) idle(h);
     if (any || last) bar_compute();                                // results stored, rows used up
     if (tid == 0) {
-      unsigned* const mine = S.core.progress + team * 16 + (h.round & 15);
+      unsigned* const mine = progress_of(team, h.round);
       if (last) { if (any || !(h.flags & H_FIRST) || T_publishes) red_release(mine); else red_relaxed(mine); }      // (nothing to order in a round without rows)
       mbar_arrive(&S.empty[buf]);
     }
@@ -1841,7 +1846,7 @@ __device__ __noinline__ void lookup_main(const int team, RowD* rows, const unsig
       for (int u = 0; u < 4; u++) if (i0 + u * CT < n) S.core.arena[at[u]] = rnd4(S.core.bf16, v[u]);
     }
   });
-  if ((end.flags & H_END) && tid == 0) red_relaxed(S.core.progress + team * 16 + (end.round & 15));      // nothing more is read
+  if ((end.flags & H_END) && tid == 0) red_relaxed(progress_of(team, end.round));      // nothing more is read
 }
 // A small table (its sums fit in shared memory): a tile owns some columns of all rows of the table.  The gradients of a chunk are gathered
 // first, all rows at once (a sum over a graph's messages is three dependent trips to L2, and a thread that walked through the rows made

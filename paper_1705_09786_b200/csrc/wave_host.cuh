@@ -565,7 +565,7 @@ static WaveScratch wave_carve(ampnet_graph* g, HostDataset& D, const WaveModel& 
   R.core.loss_out = C.take<double>(nl);
   S.loss_at = C.used - nl * sizeof(double);
   S.read_bytes = C.used;
-  R.core.progress = C.take<unsigned>(MAX_CELLS * 16);
+  R.core.progress = C.take<unsigned>((size_t)MAX_CELLS * 16 * PROGRESS_STRIDE);
   g->d_stats.assign(np, nullptr);
   g->d_update_log.assign(np, nullptr);
   R.core.n_teams = (int)P.teams.size(); R.n_mats = (int)M.mats.size(); R.n_ppts = (int)np; R.core.n_ctas = P.n_ctas;
