@@ -71,6 +71,7 @@ struct Shared {
   int stop, helper_stop, ok, ok2;
   unsigned long long ver;                      // what the ACC team had published `lag` rounds ago: updates << 32 | publications << 16 | round
   int warp_sum[4], sel;
+  int own_rows[4];
   unsigned long long batches, batch_rows, tc_batches;
   unsigned stale_hist[64]; int max_stale;
   int team_n[MAX_CELLS];
@@ -1900,6 +1901,11 @@ __device__ __noinline__ void lookup_grad_small_main(const int team, const int ti
 // pieces it has touched since the last update (the list's overflow in device memory) and moves exactly those.
 // Frequent words: adds to one address meet in L2 one after the other, some 1,000 cycles each (a word of the wide tree comes sixty times a
 // round), so up to 16 pieces of a warp have their sums in shared memory instead, the first of those that share a slot until the update.
+// Bits and tags in shared memory by its own instructions: on a generic address the compiler spins on a compare-and-swap, and the sixteen
+// warps' bits share words.
+__device__ __forceinline__ unsigned smem_or(unsigned* p, const unsigned v) { unsigned o; asm volatile("atom.shared.or.b32 %0, [%1], %2;" : "=r"(o) : "r"(smem_u32(p)), "r"(v) : "memory"); return o; }
+__device__ __forceinline__ void smem_and(unsigned* p, const unsigned v) { asm volatile("red.shared.and.b32 [%0], %1;" :: "r"(smem_u32(p)), "r"(v) : "memory"); }
+__device__ __forceinline__ void smem_cas(int* p, const int old, const int v) { int o; asm volatile("atom.shared.cas.b32 %0, [%1], %2, %3;" : "=r"(o) : "r"(smem_u32(p)), "r"(old), "r"(v) : "memory"); }
 // (Functions of their own: with them inside, the loop over the chunks spills 800 bytes and an epoch of the tree takes half as long again.)
 __device__ __noinline__ void add_pieces(const uint4* work, const int listed, const RowD* R, float4* held, const bool copies) {
   IN_SMEM(work); IN_SMEM(R); IN_SMEM(held);
@@ -1936,7 +1942,7 @@ __device__ __noinline__ void add_pieces(const uint4* work, const int listed, con
   }
 }
 // A warp's touched pieces move; their sums, bits and slots start over.
-__device__ __noinline__ void update_pieces(const int* near_list, const int* far_list, const int touched, int* tag, float4* held, const int SL, unsigned* bits, const int tile, const int n_upd, const int upd_t) {
+__device__ __noinline__ void update_pieces(const int* near_list, const int* far_list, const int touched, int* tag, float4* held, const int SL, unsigned* bits, const bool near, const int tile, const int n_upd, const int upd_t) {
   IN_SMEM(near_list); IN_SMEM(tag); IN_SMEM(held);
   const int lane = threadIdx.x & 31, out = S.ppt.out_dim, NTL = S.team.T, segs = (S.ppt.out4 + 31) >> 5;
   float* const W = S.ppt.W; float* const A = S.ppt.A;
@@ -1990,7 +1996,7 @@ __device__ __noinline__ void update_pieces(const int* near_list, const int* far_
     }
   }
 #pragma unroll 1
-  for (int k = lane; k < touched; k += 32) { const int piece = k < NEAR ? near_list[k] : far_list[k]; atomicAnd(bits + (piece >> 5), ~(1u << (piece & 31))); }
+  for (int k = lane; k < touched; k += 32) { const int piece = k < NEAR ? near_list[k] : far_list[k]; const unsigned rest = ~(1u << (piece & 31)); if (near) smem_and(bits + (piece >> 5), rest); else atomicAnd(bits + (piece >> 5), rest); }
   __syncwarp();
   if (lane < SL) tag[lane] = -1;
   __syncwarp();
@@ -2006,49 +2012,61 @@ __device__ __noinline__ void lookup_grad_main(const int team, const int tile, fl
   const size_t words = ((size_t)ids * segs + 31) >> 5;
   unsigned* const near_bits = reinterpret_cast<unsigned*>(smem) + CW * (NEAR + 4 * PIECES);
   unsigned* const bits = words <= LOOKUP_BITS ? near_bits : P.touched_bits + (size_t)tile * words;
-  if (words <= LOOKUP_BITS) for (int i = threadIdx.x; i < (int)words; i += CT) bits[i] = 0u;
+  const bool near = words <= LOOKUP_BITS;
+  if (near) for (int i = threadIdx.x; i < (int)words; i += CT) bits[i] = 0u;
   int* const tag = reinterpret_cast<int*>(near_bits + LOOKUP_BITS) + warp * SL;
   float4* const held = reinterpret_cast<float4*>(near_bits + LOOKUP_BITS + CW * SL) + (warp * SL - 1) * 32 + lane;      // slot s at 32 (s + 1)
   for (int k = 0; k < SL; k++) { held[(k + 1) * 32] = zero4(); if (lane == 0) tag[k] = -1; }
+  uint4* const own = reinterpret_cast<uint4*>(near_bits + LOOKUP_BITS + CW * SL * (1 + 128));      // the tile's rows of a chunk: gradient, table row, its number in the tile, row
   const FastDiv d_tiles(NTL);
   bar_compute();
   int* const far_list = P.touched_list + ((size_t)tile * CW + warp) * ((size_t)ids * segs / CW + segs + 1);
   int touched = 0;                                               // (the same in all lanes)
   chunk_loop(rows, team, t0, [&](const Head& h, const RowD* R) {
-    // the warp's pieces of the chunk are listed first, so that its loads overlap whatever rows they come from
+    // the tile's rows of the chunk, in order (every warp looking through all rows took 5,000 cycles of a chunk of 44); then the pieces of each warp
+    // are listed before they are added, so that its loads overlap whatever rows they come from
+    if (threadIdx.x < 128) {
+      const int b = threadIdx.x, id = b < h.count ? (int)R[b].b4 : 0, of = d_tiles.div(id);
+      const bool ours = b < h.count && id - of * NTL == tile;
+      const unsigned all = __ballot_sync(0xffffffffu, ours);
+      if (ours) own[32 * warp + __popc(all & ((1u << lane) - 1u))] = make_uint4(R[b].t[0].src4, (unsigned)id, (unsigned)of, (unsigned)b);
+      if (lane == 0) S.own_rows[warp] = __popc(all);
+    }
+    bar_compute();
     int listed = 0;
 #pragma unroll 1
-    for (int b0 = 0; b0 < h.count; b0 += 32) {
-      const int id = (int)R[min(b0 + lane, h.count - 1)].b4, of = d_tiles.div(id);
-      const bool ours = b0 + lane < h.count && id - of * NTL == tile;
-      if (!__any_sync(0xffffffffu, ours)) continue;
+    for (int g = 0; g < 4; g++) {
+      const int n = S.own_rows[g];
+      if (n == 0) continue;
+      const uint4 r = own[32 * g + min(lane, n - 1)];
 #pragma unroll 1
       for (int q0 = 0; q0 < segs; q0 += CW) {                      // (of CW neighbouring pieces exactly one is this warp's)
-        const int q = q0 + ((warp - of * segs - q0) & (CW - 1)), piece = of * segs + q;
-        const bool mine = ours && q < segs;
+        const int q = q0 + ((warp - (int)r.z * segs - q0) & (CW - 1)), piece = (int)r.z * segs + q;
+        const bool mine = lane < n && q < segs;
         const unsigned all = __ballot_sync(0xffffffffu, mine), before = (1u << lane) - 1u;
         if (all == 0) continue;
         if (listed + __popc(all) > PIECES) { add_pieces(work, listed, R, held, h.flags & H_COPIES); listed = 0; __syncwarp(); }
         const int slot = SL ? (piece >> 4) & (SL - 1) : 0;          // (the pieces of a warp are alike modulo CW)
         bool fresh = false;
-        if (mine) fresh = !(atomicOr(bits + (piece >> 5), 1u << (piece & 31)) >> (piece & 31) & 1u);
-        if (fresh && SL) atomicCAS(tag + slot, -1, piece);
+        if (mine) { unsigned* const w = bits + (piece >> 5); const unsigned bit = 1u << (piece & 31); fresh = !((near ? smem_or(w, bit) : atomicOr(w, bit)) & bit); }
+        if (fresh && SL) smem_cas(tag + slot, -1, piece);
         const unsigned news = __ballot_sync(0xffffffffu, fresh);
         if (fresh) { const int x = touched + __popc(news & before); if (x < NEAR) near_list[x] = piece; else far_list[x] = piece; }
         __syncwarp();
-        if (mine) work[listed + __popc(all & before)] = make_uint4(R[b0 + lane].t[0].src4, (unsigned)id, (unsigned)q | (SL && tag[slot] == piece ? (unsigned)slot + 1u : 0u) << 16, (unsigned)(b0 + lane));
+        if (mine) work[listed + __popc(all & before)] = make_uint4(r.x, r.y, (unsigned)q | (SL && tag[slot] == piece ? (unsigned)slot + 1u : 0u) << 16, r.w);
         listed += __popc(all);
         touched += __popc(news);
         __syncwarp();
       }
     }
+    phase(0);
     if (listed) add_pieces(work, listed, R, held, h.flags & H_COPIES);
     __syncwarp();
     phase(2);
     if (h.flags & H_UPDATE) {
       wait_readers(h, t0);
       phase(3);
-      update_pieces(near_list, far_list, touched, tag, held, SL, bits, tile, h.n_upd, h.upd_t);
+      update_pieces(near_list, far_list, touched, tag, held, SL, bits, near, tile, h.n_upd, h.upd_t);
       touched = 0;
       phase(5);
     }
@@ -2169,7 +2187,7 @@ size_t smem_bytes(const Team& t, const Mat& m, int mak) {
         const size_t steps = (BM + 15) / 16, N = split_columns(t.C), g = (size_t)((t.R + 7) / 8) * tc3::CORE_K, x = N / 8 * tc3::CORE_K, reach = (2 * steps - 1) * 3 * g + 2 * g + (size_t)(t.split / 8) * tc3::CORE_K;
         f = (size_t)t.R * pad_ld((int)N) + ((t.R + 3) & ~3) + std::max(steps * 2 * 3 * (g + x), reach) / 4;
       } else f = (size_t)t.R * (t.C + 4) + ACC_RED + BM * (t.R + 4 + t.C + 4) + t.R + (size_t)(CW / (t.WO * t.WI)) * t.R; break;
-    case LOOKUP_B: f = t.R ? BM * (t.C + 4) + (size_t)t.G * (t.R * t.C + 1) : CW * (NEAR + 4 * PIECES) + LOOKUP_BITS + (size_t)CW * t.G * (1 + 128); break;      // (small table of G rows: R copies of the sums of C columns)
+    case LOOKUP_B: f = t.R ? BM * (t.C + 4) + (size_t)t.G * (t.R * t.C + 1) : CW * (NEAR + 4 * PIECES) + LOOKUP_BITS + (size_t)CW * t.G * (1 + 128) + 4 * 128; break;      // (small table of G rows: R copies of the sums of C columns)
     case HEAD: f = (size_t)m.outp * ldi + m.outp + BM * ldi + 2 * BM * pad_ld(m.outp); break;
     default: break;
   }
