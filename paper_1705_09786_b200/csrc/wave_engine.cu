@@ -50,7 +50,7 @@ constexpr int HT = 128;                       // helper threads
 constexpr int NT = CT + HT;
 constexpr int SLOT_WORDS = 6;
 constexpr int ACC_RED = CW * 8 * 32 * 4;       // floats of an accumulator's merge buffer
-constexpr int PIECES = 128;                   // pieces of a chunk a warp lists
+constexpr int PIECES = 256;                   // pieces of a chunk a warp lists
 constexpr int NEAR = 128;                     // touched pieces of embedding rows a warp lists in shared memory
 
 enum { H_FIRST = 1, H_LAST = 2, H_UPDATE = 4, H_END = 8, H_COPIES = 16, H_LONG = 32 };      // H_COPIES: every row is one or two copies; H_LONG: a row has more terms than its descriptor holds
@@ -71,7 +71,6 @@ struct Shared {
   int stop, helper_stop, ok, ok2;
   unsigned long long ver;                      // what the ACC team had published `lag` rounds ago: updates << 32 | publications << 16 | round
   int warp_sum[4], sel;
-  int own_rows[4];
   unsigned long long batches, batch_rows, tc_batches;
   unsigned stale_hist[64]; int max_stale;
   int team_n[MAX_CELLS];
@@ -1899,177 +1898,123 @@ __device__ __noinline__ void lookup_grad_small_main(const int team, const int ti
 // A large table: rows are dealt to the tiles by id; a piece of 128 columns of a row always belongs to the same warp of the tile and a
 // column to the same lane, so that a thread's adds and its own later reads are in order without fences or barriers.  A warp lists the
 // pieces it has touched since the last update (the list's overflow in device memory) and moves exactly those.
-// Frequent words: adds to one address meet in L2 one after the other, some 1,000 cycles each (a word of the wide tree comes sixty times a
-// round), so up to 16 pieces of a warp have their sums in shared memory instead, the first of those that share a slot until the update.
-// Bits and tags in shared memory by its own instructions: on a generic address the compiler spins on a compare-and-swap, and the sixteen
-// warps' bits share words.
-__device__ __forceinline__ unsigned smem_or(unsigned* p, const unsigned v) { unsigned o; asm volatile("atom.shared.or.b32 %0, [%1], %2;" : "=r"(o) : "r"(smem_u32(p)), "r"(v) : "memory"); return o; }
-__device__ __forceinline__ void smem_and(unsigned* p, const unsigned v) { asm volatile("red.shared.and.b32 [%0], %1;" :: "r"(smem_u32(p)), "r"(v) : "memory"); }
-__device__ __forceinline__ void smem_cas(int* p, const int old, const int v) { int o; asm volatile("atom.shared.cas.b32 %0, [%1], %2, %3;" : "=r"(o) : "r"(smem_u32(p)), "r"(old), "r"(v) : "memory"); }
-// (Functions of their own: with them inside, the loop over the chunks spills 800 bytes and an epoch of the tree takes half as long again.)
-__device__ __noinline__ void add_pieces(const uint4* work, const int listed, const RowD* R, float4* held, const bool copies) {
-  IN_SMEM(work); IN_SMEM(R); IN_SMEM(held);
-  const int lane = threadIdx.x & 31, out = S.ppt.out_dim, o4 = S.ppt.out4;
-  const bool wide = (out & 3) == 0;
-  const float4* const arena = S.core.arena;
-  float* const A = S.ppt.A;
-  constexpr int U = 8;                                            // pieces whose loads are in flight
-#pragma unroll 1
-  for (int k0 = 0; k0 < listed; k0 += U) {
-    float4 v[U];
-#pragma unroll
-    for (int k = 0; k < U; k++) {
-      const uint4 x = work[min(k0 + k, listed - 1)];
-      const int c = min(32 * (int)(x.z & 0xffffu) + lane, o4 - 1);
-      if (copies) v[k] = ldcg4(arena + x.x + c);
-      else v[k] = rnd4(S.core.bf16, row_sum<false>(R[x.w], c));
-    }
-#pragma unroll
-    for (int k = 0; k < U; k++) {
-      if (k0 + k >= listed) break;
-      const uint4 x = work[k0 + k];
-      const int c = 32 * (int)(x.z & 0xffffu) + lane, slot = (int)(x.z >> 16);
-      if (slot) { held[slot * 32] = add4(held[slot * 32], v[k]); continue; }
-      if (c >= o4) continue;
-      float* const a = A + (size_t)x.y * out + 4 * c;
-      if (wide) asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" :: "l"(a), "f"(v[k].x), "f"(v[k].y), "f"(v[k].z), "f"(v[k].w) : "memory");
-      else {
-        const float e[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
-#pragma unroll
-        for (int y = 0; y < 4; y++) if (4 * c + y < out) asm volatile("red.relaxed.gpu.global.add.f32 [%0], %1;" :: "l"(a + y), "f"(e[y]) : "memory");
-      }
-    }
-  }
-}
-// A warp's touched pieces move; their sums, bits and slots start over.
-__device__ __noinline__ void update_pieces(const int* near_list, const int* far_list, const int touched, int* tag, float4* held, const int SL, unsigned* bits, const bool near, const int tile, const int n_upd, const int upd_t) {
-  IN_SMEM(near_list); IN_SMEM(tag); IN_SMEM(held);
-  const int lane = threadIdx.x & 31, out = S.ppt.out_dim, NTL = S.team.T, segs = (S.ppt.out4 + 31) >> 5;
-  float* const W = S.ppt.W; float* const A = S.ppt.A;
-  const bool wide = (out & 3) == 0;
-  const unsigned long long seg_M = segs <= 4 ? ((1ull << 33) + segs - 1) / (unsigned)segs : 0ull;      // piece / segs by a multiplication, exact below 2^31 for up to four segments
-  const OptStep os = opt_step(S.ppt.om, S.ppt.ov, S.ppt.opt_t0, n_upd, upd_t);
-  constexpr int U = 4;                                            // pieces whose loads are in flight
-#pragma unroll 1
-  for (int k0 = 0; k0 < touched; k0 += U) {
-    float4 a[U], w[U];
-    size_t r0[U];
-    int cq[U], at[U];
-#pragma unroll
-    for (int u = 0; u < U; u++) {
-      const int k = min(k0 + u, touched - 1), piece = k < NEAR ? near_list[k] : far_list[k];
-      const int local = seg_M ? (int)(((unsigned long long)(unsigned)piece * seg_M) >> 33) : piece / segs, c = (piece - local * segs) * 32 + lane;
-      r0[u] = ((size_t)local * NTL + tile) * out + 4 * c;
-      cq[u] = k0 + u < touched ? out - 4 * c : 0;
-      at[u] = SL && tag[(piece >> 4) & (SL - 1)] == piece ? (piece >> 4) & (SL - 1) : -1;
-      a[u] = w[u] = zero4();
-      if (wide && cq[u] > 0) {
-        if (at[u] < 0) asm volatile("ld.relaxed.gpu.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(a[u].x), "=f"(a[u].y), "=f"(a[u].z), "=f"(a[u].w) : "l"(A + r0[u]) : "memory");
-        w[u] = *reinterpret_cast<const float4*>(W + r0[u]);
-      } else if (cq[u] > 0) {
-        float* const x = &a[u].x; float* const y = &w[u].x;
-#pragma unroll
-        for (int q = 0; q < 4; q++)
-          if (q < cq[u]) {
-            if (at[u] < 0) asm volatile("ld.relaxed.gpu.global.f32 %0, [%1];" : "=f"(x[q]) : "l"(A + r0[u] + q) : "memory");
-            y[q] = W[r0[u] + q];
-          }
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < U; u++) {
-      if (k0 + u >= touched) break;
-      if (at[u] >= 0) { a[u] = held[(at[u] + 1) * 32]; held[(at[u] + 1) * 32] = zero4(); }
-      if (cq[u] <= 0) continue;
-      if (wide && (SGD || os.opt == 0)) {
-        *reinterpret_cast<float4*>(W + r0[u]) = sgd4(os.step, w[u], a[u]);
-        if (at[u] < 0) asm volatile("st.relaxed.gpu.global.v4.f32 [%0], {%1, %1, %1, %1};" :: "l"(A + r0[u]), "f"(0.f) : "memory");
-        continue;
-      }
-      const float x[4] = {a[u].x, a[u].y, a[u].z, a[u].w}, y[4] = {w[u].x, w[u].y, w[u].z, w[u].w};
-#pragma unroll
-      for (int q = 0; q < 4; q++)
-        if (q < cq[u]) {
-          W[r0[u] + q] = opt_one(os, y[q], x[q], r0[u] + q);
-          if (at[u] < 0) asm volatile("st.relaxed.gpu.global.f32 [%0], %1;" :: "l"(A + r0[u] + q), "f"(0.f) : "memory");
-        }
-    }
-  }
-#pragma unroll 1
-  for (int k = lane; k < touched; k += 32) { const int piece = k < NEAR ? near_list[k] : far_list[k]; const unsigned rest = ~(1u << (piece & 31)); if (near) smem_and(bits + (piece >> 5), rest); else atomicAnd(bits + (piece >> 5), rest); }
-  __syncwarp();
-  if (lane < SL) tag[lane] = -1;
-  __syncwarp();
-}
 __device__ __noinline__ void lookup_grad_main(const int team, const int tile, float* smem, RowD* rows, const unsigned long long t0) {
   IN_SMEM(smem); IN_SMEM(rows);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, NTL = S.team.T, SL = S.team.G;      // SL: slots of a warp (a power of two, or none)
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, out = S.ppt.out_dim, o4 = S.ppt.out4, NTL = S.team.T;
   const PptRun& P = S.ppt;
-  const int segs = (P.out4 + 31) >> 5, ids = (P.in_dim + NTL - 1) / NTL;
+  const int segs = (o4 + 31) >> 5, ids = (P.in_dim + NTL - 1) / NTL;
   int* const near_list = reinterpret_cast<int*>(smem) + warp * NEAR;
-  uint4* const work = reinterpret_cast<uint4*>(reinterpret_cast<int*>(smem) + CW * NEAR) + warp * PIECES;      // of the chunk: gradient, table row, segment and slot + 1, row
+  int* const work = reinterpret_cast<int*>(smem) + CW * NEAR + warp * PIECES;      // (segment, row) of the chunk
   // a bit per piece: listed already (in device memory behind the lists where a table is too large)
   const size_t words = ((size_t)ids * segs + 31) >> 5;
-  unsigned* const near_bits = reinterpret_cast<unsigned*>(smem) + CW * (NEAR + 4 * PIECES);
-  unsigned* const bits = words <= LOOKUP_BITS ? near_bits : P.touched_bits + (size_t)tile * words;
-  const bool near = words <= LOOKUP_BITS;
-  if (near) for (int i = threadIdx.x; i < (int)words; i += CT) bits[i] = 0u;
-  int* const tag = reinterpret_cast<int*>(near_bits + LOOKUP_BITS) + warp * SL;
-  float4* const held = reinterpret_cast<float4*>(near_bits + LOOKUP_BITS + CW * SL) + (warp * SL - 1) * 32 + lane;      // slot s at 32 (s + 1)
-  for (int k = 0; k < SL; k++) { held[(k + 1) * 32] = zero4(); if (lane == 0) tag[k] = -1; }
-  uint4* const own = reinterpret_cast<uint4*>(near_bits + LOOKUP_BITS + CW * SL * (1 + 128));      // the tile's rows of a chunk: gradient, table row, its number in the tile, row
+  unsigned* const bits = words <= LOOKUP_BITS ? reinterpret_cast<unsigned*>(smem) + CW * (NEAR + PIECES) : P.touched_bits + (size_t)tile * words;
+  if (words <= LOOKUP_BITS) for (int i = threadIdx.x; i < (int)words; i += CT) bits[i] = 0u;
   const FastDiv d_tiles(NTL);
   bar_compute();
   int* const far_list = P.touched_list + ((size_t)tile * CW + warp) * ((size_t)ids * segs / CW + segs + 1);
+  const bool wide = (out & 3) == 0;
   int touched = 0;                                               // (the same in all lanes)
-  chunk_loop(rows, team, t0, [&](const Head& h, const RowD* R) {
-    // the tile's rows of the chunk, in order (every warp looking through all rows took 5,000 cycles of a chunk of 44); then the pieces of each warp
-    // are listed before they are added, so that its loads overlap whatever rows they come from
-    if (threadIdx.x < 128) {
-      const int b = threadIdx.x, id = b < h.count ? (int)R[b].b4 : 0, of = d_tiles.div(id);
-      const bool ours = b < h.count && id - of * NTL == tile;
-      const unsigned all = __ballot_sync(0xffffffffu, ours);
-      if (ours) own[32 * warp + __popc(all & ((1u << lane) - 1u))] = make_uint4(R[b].t[0].src4, (unsigned)id, (unsigned)of, (unsigned)b);
-      if (lane == 0) S.own_rows[warp] = __popc(all);
+  auto update = [&](const int n_upd, const int upd_t) {
+    const OptStep os = opt_step(P.om, P.ov, P.opt_t0, n_upd, upd_t);
+#pragma unroll 1
+    for (int k0 = 0; k0 < touched; k0 += 4) {                    // four pieces' loads in flight
+      float a[4][4], w[4][4];
+      size_t r0[4];
+      int cq[4];
+#pragma unroll
+      for (int u = 0; u < 4; u++) {
+        const int k = min(k0 + u, touched - 1), piece = k < NEAR ? near_list[k] : far_list[k], local = piece / segs, c = (piece - local * segs) * 32 + lane;
+        r0[u] = ((size_t)local * NTL + tile) * out + 4 * c;
+        cq[u] = k0 + u < touched ? out - 4 * c : 0;
+        if (wide && cq[u] > 0) {
+          asm volatile("ld.relaxed.gpu.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(a[u][0]), "=f"(a[u][1]), "=f"(a[u][2]), "=f"(a[u][3]) : "l"(P.A + r0[u]) : "memory");
+          const float4 x = *reinterpret_cast<const float4*>(P.W + r0[u]);
+          w[u][0] = x.x; w[u][1] = x.y; w[u][2] = x.z; w[u][3] = x.w;
+        } else
+#pragma unroll
+          for (int q = 0; q < 4; q++)
+            if (q < cq[u]) { asm volatile("ld.relaxed.gpu.global.f32 %0, [%1];" : "=f"(a[u][q]) : "l"(P.A + r0[u] + q) : "memory"); w[u][q] = P.W[r0[u] + q]; }
+      }
+#pragma unroll
+      for (int u = 0; u < 4; u++) {
+        if (wide && cq[u] > 0 && (SGD || os.opt == 0)) {
+          *reinterpret_cast<float4*>(P.W + r0[u]) = sgd4(os.step, make_float4(w[u][0], w[u][1], w[u][2], w[u][3]), make_float4(a[u][0], a[u][1], a[u][2], a[u][3]));
+          asm volatile("st.relaxed.gpu.global.v4.f32 [%0], {%1, %1, %1, %1};" :: "l"(P.A + r0[u]), "f"(0.f) : "memory");
+          continue;
+        }
+#pragma unroll
+        for (int q = 0; q < 4; q++)
+          if (q < cq[u]) {
+            P.W[r0[u] + q] = opt_one(os, w[u][q], a[u][q], r0[u] + q);
+            asm volatile("st.relaxed.gpu.global.f32 [%0], %1;" :: "l"(P.A + r0[u] + q), "f"(0.f) : "memory");
+          }
+      }
     }
-    bar_compute();
+#pragma unroll 1
+    for (int k = lane; k < touched; k += 32) { const int piece = k < NEAR ? near_list[k] : far_list[k]; atomicAnd(bits + (piece >> 5), ~(1u << (piece & 31))); }
+    touched = 0;
+    __syncwarp();
+  };
+  chunk_loop(rows, team, t0, [&](const Head& h, const RowD* R) {
+// the warp's pieces of the chunk are listed first, so that its loads overlap whatever rows they come from
     int listed = 0;
+    auto add_listed = [&]() {
 #pragma unroll 1
-    for (int g = 0; g < 4; g++) {
-      const int n = S.own_rows[g];
-      if (n == 0) continue;
-      const uint4 r = own[32 * g + min(lane, n - 1)];
+      for (int k0 = 0; k0 < listed; k0 += 4) {
+        float4 v[4];
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+          v[k] = zero4();
+          const int x = k0 + k < listed ? work[k0 + k] : -1, c = 32 * (x >> 8) + lane;
+          if (x < 0 || c >= o4) continue;
+          const RowD& r = R[x & 255];
+          v[k] = h.flags & H_COPIES ? ldcg4(S.core.arena + r.t[0].src4 + c) : rnd4(S.core.bf16, row_sum<false>(r, c));
+        }
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+          if (k0 + k >= listed) break;
+          const int x = work[k0 + k], q = x >> 8, c = 32 * q + lane;
+          const unsigned id = R[x & 255].b4;
+          float* const a = P.A + (size_t)id * out + 4 * c;
+          if (c < o4) {
+            if (wide) asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" :: "l"(a), "f"(v[k].x), "f"(v[k].y), "f"(v[k].z), "f"(v[k].w) : "memory");
+            else {
+              const float e[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
+#pragma unroll
+              for (int y = 0; y < 4; y++) if (4 * c + y < out) asm volatile("red.relaxed.gpu.global.add.f32 [%0], %1;" :: "l"(a + y), "f"(e[y]) : "memory");
+            }
+          }
+        }
+      }
+      listed = 0;
+      __syncwarp();
+    };
 #pragma unroll 1
-      for (int q0 = 0; q0 < segs; q0 += CW) {                      // (of CW neighbouring pieces exactly one is this warp's)
-        const int q = q0 + ((warp - (int)r.z * segs - q0) & (CW - 1)), piece = (int)r.z * segs + q;
-        const bool mine = lane < n && q < segs;
-        const unsigned all = __ballot_sync(0xffffffffu, mine), before = (1u << lane) - 1u;
-        if (all == 0) continue;
-        if (listed + __popc(all) > PIECES) { add_pieces(work, listed, R, held, h.flags & H_COPIES); listed = 0; __syncwarp(); }
-        const int slot = SL ? (piece >> 4) & (SL - 1) : 0;          // (the pieces of a warp are alike modulo CW)
+    for (int b0 = 0; b0 < h.count; b0 += 32) {
+      const int id = (int)R[min(b0 + lane, h.count - 1)].b4, of = d_tiles.div(id);
+      const bool ours = b0 + lane < h.count && id - of * NTL == tile;
+      if (!__any_sync(0xffffffffu, ours)) continue;
+#pragma unroll 1
+      for (int q = 0; q < segs; q++) {
+        const bool mine = ours && ((of * segs + q) & (CW - 1)) == warp;
+        const unsigned all = __ballot_sync(0xffffffffu, mine);
+        if (listed + __popc(all) > PIECES) add_listed();
+        const unsigned before = (1u << lane) - 1u;
+        const int piece = of * segs + q;
         bool fresh = false;
-        if (mine) { unsigned* const w = bits + (piece >> 5); const unsigned bit = 1u << (piece & 31); fresh = !((near ? smem_or(w, bit) : atomicOr(w, bit)) & bit); }
-        if (fresh && SL) smem_cas(tag + slot, -1, piece);
+        if (mine) {
+          work[listed + __popc(all & before)] = (q << 8) | (b0 + lane);
+          fresh = !(atomicOr(bits + (piece >> 5), 1u << (piece & 31)) >> (piece & 31) & 1u);
+        }
         const unsigned news = __ballot_sync(0xffffffffu, fresh);
         if (fresh) { const int x = touched + __popc(news & before); if (x < NEAR) near_list[x] = piece; else far_list[x] = piece; }
-        __syncwarp();
-        if (mine) work[listed + __popc(all & before)] = make_uint4(r.x, r.y, (unsigned)q | (SL && tag[slot] == piece ? (unsigned)slot + 1u : 0u) << 16, r.w);
         listed += __popc(all);
         touched += __popc(news);
         __syncwarp();
       }
     }
-    phase(0);
-    if (listed) add_pieces(work, listed, R, held, h.flags & H_COPIES);
-    __syncwarp();
-    phase(2);
-    if (h.flags & H_UPDATE) {
-      wait_readers(h, t0);
-      phase(3);
-      update_pieces(near_list, far_list, touched, tag, held, SL, bits, near, tile, h.n_upd, h.upd_t);
-      touched = 0;
-      phase(5);
-    }
+    add_listed();
+    if (h.flags & H_UPDATE) { wait_readers(h, t0); update(h.n_upd, h.upd_t); }
   });
 }
 
@@ -2187,7 +2132,7 @@ size_t smem_bytes(const Team& t, const Mat& m, int mak) {
         const size_t steps = (BM + 15) / 16, N = split_columns(t.C), g = (size_t)((t.R + 7) / 8) * tc3::CORE_K, x = N / 8 * tc3::CORE_K, reach = (2 * steps - 1) * 3 * g + 2 * g + (size_t)(t.split / 8) * tc3::CORE_K;
         f = (size_t)t.R * pad_ld((int)N) + ((t.R + 3) & ~3) + std::max(steps * 2 * 3 * (g + x), reach) / 4;
       } else f = (size_t)t.R * (t.C + 4) + ACC_RED + BM * (t.R + 4 + t.C + 4) + t.R + (size_t)(CW / (t.WO * t.WI)) * t.R; break;
-    case LOOKUP_B: f = t.R ? BM * (t.C + 4) + (size_t)t.G * (t.R * t.C + 1) : CW * (NEAR + 4 * PIECES) + LOOKUP_BITS + (size_t)CW * t.G * (1 + 128) + 4 * 128; break;      // (small table of G rows: R copies of the sums of C columns)
+    case LOOKUP_B: f = t.R ? BM * (t.C + 4) + (size_t)t.G * (t.R * t.C + 1) : CW * (NEAR + PIECES) + LOOKUP_BITS; break;      // (small table of G rows: R copies of the sums of C columns)
     case HEAD: f = (size_t)m.outp * ldi + m.outp + BM * ldi + 2 * BM * pad_ld(m.outp); break;
     default: break;
   }

@@ -432,8 +432,6 @@ static bool wave_best(const WaveModel& M, int c, int ctas, double rows, double m
       for (int n = 1; n <= std::min(ctas, std::max(1, h.in_dim / 8)) && (n == 1 || (long long)h.in_dim * n < (1ll << 31)); n++) {      // (the kernel divides ids by multiplication)
         Team x = t;
         x.T = x.n = n;
-        x.G = 16;                                                  // pieces a warp has room for in shared memory (8 KB), as many as leave a chunk room
-        for (x.BM = 64; x.G > 0 && smem_bytes(x, m, mak) > budget;) x.G = x.G > 2 ? x.G / 2 : 0;
         const double pieces = std::max((h.out_dim + 127) / 128 / 16.0 / n, 0.02);      // of a row, per warp of a tile (frequent ids keep one warp busy)
         offer(x, 4000 + rows * (40 + pieces * 1300) + upd * (4000 + std::min(msgs_per_update, (double)h.in_dim) * pieces * 1500));
       }
