@@ -2058,7 +2058,7 @@ extern "C" __global__ void __launch_bounds__(NT, 1) ENGINE_KERNEL(const __grid_c
   else switch (S.team.kind) {
     case LIN_F:
       if (S.team.bf16_tc) forward_main<F_TENSOR>(team, tile, work, rows, t0);
-      else if (S.team.lstm) { if (split) forward_main<F_LSTM, true>(team, tile, work, rows, t0); else forward_main<F_LSTM>(team, tile, work, rows, t0); }
+      else if (S.team.lstm) forward_main<F_LSTM>(team, tile, work, rows, t0);
       else if (split) forward_main<F_PLAIN, true>(team, tile, work, rows, t0);
       else forward_main<F_PLAIN>(team, tile, work, rows, t0);
       break;
@@ -2068,7 +2068,7 @@ extern "C" __global__ void __launch_bounds__(NT, 1) ENGINE_KERNEL(const __grid_c
     case LOOKUP_F: lookup_main(team, rows, t0); break;
 #ifndef WAVE_FORWARD
     case LIN_DX:
-      if (S.team.lstm) { if (split) input_grad_main<B_LSTM, true>(team, tile, work, rows, t0); else input_grad_main<B_LSTM>(team, tile, work, rows, t0); }
+      if (S.team.lstm) input_grad_main<B_LSTM>(team, tile, work, rows, t0);
       else if (split) input_grad_main<B_PLAIN, true>(team, tile, work, rows, t0);
       else input_grad_main<B_PLAIN>(team, tile, work, rows, t0);
       break;

@@ -341,7 +341,7 @@ static bool wave_best(const WaveModel& M, int c, int ctas, double rows, double m
         const double product = tc ? 1500 + rs * m.inp / 8.0 : 600 + (rs + 4) * outs * m.inp / fma;
         const double rest = 1600 + rs * x.R / 4 * (t.lstm ? 20.0 : K.kind == LIN_F ? 2.0 : 3.0);
         offer(x, gather + weights + product + rest);
-        if (!tc && outs <= 128) {
+        if (!tc && !t.lstm && outs <= 128) {
           x.split = outs <= 64 ? 64 : 128;
           offer(x, gather + rs * m.inp / 4 * split_gather + weights * split_weights + split_product(m.inp) + rest, split_chunk + split_product(m.inp), m.inp);
         }
@@ -363,7 +363,7 @@ static bool wave_best(const WaveModel& M, int c, int ctas, double rows, double m
         const double per4 = t.lstm ? 17.0 * t.H4 : m.outp / 4 * (K.kind == GRU_DC ? 12.0 : 3.4);
         const double weights = std::min(1.0, upd) * x.R * m.outp * 4.0 / bpc, rest = 1700 + rs * x.R / 4 * 1.5;
         offer(x, 1500 + rs * per4 + weights + 600 + (rs + 4) * x.R * m.outp / fma + rest);
-        if (x.R <= 128) {
+        if (!t.lstm && x.R <= 128) {
           x.split = x.R <= 64 ? 64 : 128;
           offer(x, 1500 + rs * (per4 + m.outp / 4 * split_gather) + weights * split_weights + split_product(m.outp) + rest, split_chunk + split_product(m.outp), m.outp);
         }
