@@ -296,6 +296,7 @@ static bool wave_best(const WaveModel& M, int c, int ctas, double rows, double m
   if (K.mat >= 0) { const WaveMat& w = M.mats[K.mat]; m.outp = w.outp; m.inp = w.inp; m.out_w = w.out_w; m.nso = w.nso; m.in_w = w.in_w; m.nsi = w.nsi; }
   const double upd = eval ? 0.0 : std::min(1.0, rows / std::max(1.0, msgs_per_update));      // rounds with new weights
   bool found = false;
+  auto handicap = [](const Team& x) { return x.split ? 1.25 : 1.0; };
   auto offer = [&](Team x, double cycles, const double per_chunk = 900.0, const int split_k = 0) {
     static const int caps[] = {128, 96, 64, 48, 32, 24, 16, 8};
     for (int bm : caps) {
@@ -306,7 +307,7 @@ static bool wave_best(const WaveModel& M, int c, int ctas, double rows, double m
       if (smem_bytes(x, m, mak) > budget) continue;
       const double chunks = std::max(1.0, rows / x.Sh / bm);
       cycles += per_chunk * (chunks - 1.0);
-      if (!found || cycles < best.cycles * 0.995) { best.t = x; best.cycles = cycles; found = true; }
+      if (!found || cycles * handicap(x) < best.cycles * 0.995 * handicap(best.t)) { best.t = x; best.cycles = cycles; found = true; }
       return;
     }
   };
