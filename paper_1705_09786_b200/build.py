@@ -7,7 +7,7 @@ _DIR = os.path.dirname(os.path.abspath(__file__))
 SRC = os.path.join(_DIR, "csrc", "ampnet.cu")
 SRC_HOST = os.path.join(_DIR, "csrc", "ir_builders.cpp")
 SRC_DIRECT = os.path.join(_DIR, "csrc", "engine_fast.cu")
-SRC_WAVE = [os.path.join(_DIR, "csrc", f) for f in ("wave_engine.cu", "wave_forward.cu", "wave_moments.cu", "wave_encode.cu")]
+SRC_WAVE = [os.path.join(_DIR, "csrc", f) for f in ("wave_engine.cu", "wave_forward.cu", "wave_moments.cu", "wave_split.cu", "wave_forward_split.cu", "wave_encode.cu")]
 # whatever the sources include: every file beside them, and the public header
 DEPS = sorted(glob.glob(os.path.join(_DIR, "csrc", "*"))) + [os.path.join(os.path.dirname(_DIR), "include", "ampnet.h")]
 LIB = os.path.join(_DIR, "libampnet.so")

@@ -1102,7 +1102,7 @@ bool wave_takes(ampnet_graph* g, HostDataset& D, int mak, int det, int eval, con
   // (the placement of the last run of this kind still holds if nothing it depends on has changed)
   const char* env[3] = {getenv("AMPNET_DIRECT_ROWS"), getenv("AMPNET_DIRECT_COLS"), getenv("AMPNET_TENSOR_CORES")};
   const int n_ctas = cfg && cfg->n_ctas > 0 ? std::min(cfg->n_ctas, g->n_sms) : g->n_sms;
-  wave::WavePlanKey key{n_order, mak, cfg ? cfg->min_update_frequency : 1, eval, n_ctas, {env[0] ? atoi(env[0]) : -1, env[1] ? atoi(env[1]) : -1, env[2] ? atoi(env[2]) : -1}};
+  wave::WavePlanKey key{n_order, mak, cfg ? cfg->min_update_frequency : 1, eval, n_ctas, {env[0] ? atoi(env[0]) : -1, env[1] ? atoi(env[1]) : -1, env[2] ? atoi(env[2]) : -1}, g->opt};
   auto& slot = D.wave_plan[eval ? 1 : 0];
   if (!(slot.first == key)) { slot.first = key; slot.second = wave_place(g, g->wave, D.wave, mak, key.muf, eval != 0, n_order, D.n, n_ctas); }
   P = slot.second;
@@ -1161,8 +1161,8 @@ ampnet_status_t wave_execute(ampnet_graph* g, HostDataset& D, const WavePlan& P,
     for (size_t k = 0; k < P.teams.size(); k++) {
       const wave::Team& t = P.teams[k].t;
       static const char* names[] = {"LOOKUP_F", "LOOKUP_B", "LIN_F", "LIN_DX", "ACC", "HEAD", "GRU_ZR", "GRU_C", "GRU_DC", "GRU_DZR"};
-      fprintf(stderr, "[team] %-8s node %2d CTAs %3d T %2d Sh %2d R %3d C %3d BM %3d rows/round %7.1f est %6.0f | wait-rows %6.0f wait %6.0f gather %6.0f product %6.0f rest %6.0f update %6.0f", names[t.kind], g->ppts[t.ppt].node,
-              t.n, t.T, t.Sh, t.R, t.C, t.BM, (double)D.wave.tot.entries[t.cell] / std::max<double>(1, (double)G.rounds), P.teams[k].cycles, (double)ph[k * 6] / G.rounds, (double)ph[k * 6 + 1] / G.rounds,
+      fprintf(stderr, "[team] %-8s node %2d CTAs %3d T %2d Sh %2d R %3d C %3d M %3d BM %3d rows/round %7.1f est %6.0f | wait-rows %6.0f wait %6.0f gather %6.0f product %6.0f rest %6.0f update %6.0f", names[t.kind], g->ppts[t.ppt].node,
+              t.n, t.T, t.Sh, t.R, t.C, t.split, t.BM, (double)D.wave.tot.entries[t.cell] / std::max<double>(1, (double)G.rounds), P.teams[k].cycles, (double)ph[k * 6] / G.rounds, (double)ph[k * 6 + 1] / G.rounds,
               (double)ph[k * 6 + 2] / G.rounds, (double)ph[k * 6 + 3] / G.rounds, (double)ph[k * 6 + 4] / G.rounds, (double)ph[k * 6 + 5] / G.rounds);
       fprintf(stderr, "\n");
     }

@@ -165,9 +165,9 @@ struct WaveData {
 };
 struct WavePlanKey {                   // (of one loaded split: a load starts with none)
   long long n_order = 0;
-  int mak = 0, muf = 0, eval = 0, n_ctas = 0, env[3] = {0, 0, 0};
+  int mak = 0, muf = 0, eval = 0, n_ctas = 0, env[3] = {0, 0, 0}, opt = 0;
   bool operator==(const WavePlanKey& o) const {
-    return n_order == o.n_order && mak == o.mak && muf == o.muf && eval == o.eval && n_ctas == o.n_ctas && env[0] == o.env[0] && env[1] == o.env[1] && env[2] == o.env[2];
+    return n_order == o.n_order && mak == o.mak && muf == o.muf && eval == o.eval && n_ctas == o.n_ctas && env[0] == o.env[0] && env[1] == o.env[1] && env[2] == o.env[2] && opt == o.opt;
   }
 };
 struct WaveTeam { Team t; double cycles = 0; };

@@ -20,10 +20,18 @@
 #include "tc_tile.cuh"
 #include "wave.h"
 
-#ifdef WAVE_FORWARD
+#if defined(WAVE_FORWARD) && defined(WAVE_SPLIT)
+#define ENGINE_KERNEL ampnet_engine_scheduled_forward_tensor
+#define EVALUATING true
+#define ENGINE_NAMESPACE forward_tensor
+#elif defined(WAVE_FORWARD)
 #define ENGINE_KERNEL ampnet_engine_scheduled_forward
 #define EVALUATING true
 #define ENGINE_NAMESPACE forward
+#elif defined(WAVE_SPLIT)
+#define ENGINE_KERNEL ampnet_engine_scheduled_tensor
+#define EVALUATING false
+#define ENGINE_NAMESPACE training_tensor
 #elif defined(WAVE_MOMENTS)
 #define ENGINE_KERNEL ampnet_engine_scheduled_moments
 #define EVALUATING false
@@ -45,6 +53,11 @@ constexpr bool SGD = true;                    // (momentum and Adam: wave_moment
 #define OPT_STEP_INLINE __forceinline__
 #endif
 
+#ifdef WAVE_SPLIT
+constexpr bool WITH_SPLIT = true;
+#else
+constexpr bool WITH_SPLIT = false;
+#endif
 constexpr int CT = 512, CW = CT / 32;         // compute threads
 constexpr int HT = 128;                       // helper threads
 constexpr int NT = CT + HT;
@@ -2044,7 +2057,12 @@ extern "C" __global__ void __launch_bounds__(NT, 1) ENGINE_KERNEL(const __grid_c
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
-  const bool tcm = S.team.bf16_tc != 0, split = S.team.split != 0;
+  const bool tcm = S.team.bf16_tc != 0;
+#ifdef WAVE_SPLIT
+  const bool split = S.team.split != 0;
+#else
+  constexpr bool split = false;                                  // (the kernels without: wave_split.cu)
+#endif
   if (tcm || split) {
     if (tid < 32) { if (split) tc3::tmem_alloc(&S.tmem); else tc::tmem_alloc(&S.tmem); }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -2059,22 +2077,23 @@ extern "C" __global__ void __launch_bounds__(NT, 1) ENGINE_KERNEL(const __grid_c
     case LIN_F:
       if (S.team.bf16_tc) forward_main<F_TENSOR>(team, tile, work, rows, t0);
       else if (S.team.lstm) forward_main<F_LSTM>(team, tile, work, rows, t0);
-      else if (split) forward_main<F_PLAIN, true>(team, tile, work, rows, t0);
+      else if (split) forward_main<F_PLAIN, WITH_SPLIT>(team, tile, work, rows, t0);
       else forward_main<F_PLAIN>(team, tile, work, rows, t0);
       break;
-    case GRU_ZR: if (split) forward_main<F_ZR, true>(team, tile, work, rows, t0); else forward_main<F_ZR>(team, tile, work, rows, t0); break;
-    case GRU_C: if (split) forward_main<F_C, true>(team, tile, work, rows, t0); else forward_main<F_C>(team, tile, work, rows, t0); break;
+    case GRU_ZR: if (split) forward_main<F_ZR, WITH_SPLIT>(team, tile, work, rows, t0); else forward_main<F_ZR>(team, tile, work, rows, t0); break;
+    case GRU_C: if (split) forward_main<F_C, WITH_SPLIT>(team, tile, work, rows, t0); else forward_main<F_C>(team, tile, work, rows, t0); break;
     case HEAD: head_main(team, work, rows, t0); break;
     case LOOKUP_F: lookup_main(team, rows, t0); break;
 #ifndef WAVE_FORWARD
     case LIN_DX:
       if (S.team.lstm) input_grad_main<B_LSTM>(team, tile, work, rows, t0);
-      else if (split) input_grad_main<B_PLAIN, true>(team, tile, work, rows, t0);
+      else if (split) input_grad_main<B_PLAIN, WITH_SPLIT>(team, tile, work, rows, t0);
       else input_grad_main<B_PLAIN>(team, tile, work, rows, t0);
       break;
-    case GRU_DC: if (split) input_grad_main<B_DC, true>(team, tile, work, rows, t0); else input_grad_main<B_DC>(team, tile, work, rows, t0); break;
-    case GRU_DZR: if (split) input_grad_main<B_DZR, true>(team, tile, work, rows, t0); else input_grad_main<B_DZR>(team, tile, work, rows, t0); break;
-    case ACC: if (split) accumulate_split_main(team, tile, work, rows, t0); else accumulate_main(team, tile, work, rows, t0); break;
+    case GRU_DC: if (split) input_grad_main<B_DC, WITH_SPLIT>(team, tile, work, rows, t0); else input_grad_main<B_DC>(team, tile, work, rows, t0); break;
+    case GRU_DZR: if (split) input_grad_main<B_DZR, WITH_SPLIT>(team, tile, work, rows, t0); else input_grad_main<B_DZR>(team, tile, work, rows, t0); break;
+    case ACC: if constexpr (WITH_SPLIT) if (split) { accumulate_split_main(team, tile, work, rows, t0); break; }
+      accumulate_main(team, tile, work, rows, t0); break;
     case LOOKUP_B: if (S.team.R) lookup_grad_small_main(team, tile, work, rows, t0); else lookup_grad_main(team, tile, work, rows, t0); break;
 #endif
   }
@@ -2104,10 +2123,15 @@ cudaError_t launch(const Run* run, int n_ctas, size_t smem, cudaStream_t st) {
 }
 }  // namespace ENGINE_NAMESPACE
 
-#if !defined(WAVE_FORWARD) && !defined(WAVE_MOMENTS)
+#if !defined(WAVE_FORWARD) && !defined(WAVE_MOMENTS) && !defined(WAVE_SPLIT)
 namespace forward { cudaError_t launch(const Run* run, int n_ctas, size_t smem, cudaStream_t st); }      // wave_forward.cu
 namespace moments { cudaError_t launch(const Run* run, int n_ctas, size_t smem, cudaStream_t st); }      // wave_moments.cu
+namespace training_tensor { cudaError_t launch(const Run* run, int n_ctas, size_t smem, cudaStream_t st); }      // wave_split.cu
+namespace forward_tensor { cudaError_t launch(const Run* run, int n_ctas, size_t smem, cudaStream_t st); }      // wave_forward_split.cu
 cudaError_t launch(const Run* run, int n_ctas, size_t smem, cudaStream_t st) {
+  bool split = false;
+  for (int k = 0; k < run->core.n_teams; k++) split |= run->teams[k].split != 0;
+  if (split) return run->core.eval ? forward_tensor::launch(run, n_ctas, smem, st) : training_tensor::launch(run, n_ctas, smem, st);
   return run->core.eval ? forward::launch(run, n_ctas, smem, st) : run->core.opt ? moments::launch(run, n_ctas, smem, st) : training::launch(run, n_ctas, smem, st);
 }
 using namespace training;

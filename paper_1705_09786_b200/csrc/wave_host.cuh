@@ -281,7 +281,7 @@ static ampnet_status_t wave_encode(ampnet_graph* g, HostDataset& D, WaveModel& M
 // nothing gains.  The estimate (in cycles) counts the latency of a gather, its bytes, the multiply-adds at the rate the
 // products reach, the reload of updated weights and, for accumulators, the merge at updates.
 
-static bool wave_best(const WaveModel& M, int c, int ctas, double rows, double msgs_per_update, bool eval, size_t budget, int mak, bool use_tc, const ampnet_graph* g, WaveTeam& best) {
+static bool wave_best(const WaveModel& M, int c, int ctas, double rows, double msgs_per_update, bool eval, size_t budget, int mak, bool use_tc, bool use_split, const ampnet_graph* g, WaveTeam& best) {
   using namespace wave;
   const WaveCell& K = M.cells[c];
   const EncPpt& P = M.enc.ppts[K.ppt];
@@ -296,7 +296,6 @@ static bool wave_best(const WaveModel& M, int c, int ctas, double rows, double m
   if (K.mat >= 0) { const WaveMat& w = M.mats[K.mat]; m.outp = w.outp; m.inp = w.inp; m.out_w = w.out_w; m.nso = w.nso; m.in_w = w.in_w; m.nsi = w.nsi; }
   const double upd = eval ? 0.0 : std::min(1.0, rows / std::max(1.0, msgs_per_update));      // rounds with new weights
   bool found = false;
-  auto handicap = [](const Team& x) { return x.split ? 1.25 : 1.0; };
   auto offer = [&](Team x, double cycles, const double per_chunk = 900.0, const int split_k = 0) {
     static const int caps[] = {128, 96, 64, 48, 32, 24, 16, 8};
     for (int bm : caps) {
@@ -307,7 +306,7 @@ static bool wave_best(const WaveModel& M, int c, int ctas, double rows, double m
       if (smem_bytes(x, m, mak) > budget) continue;
       const double chunks = std::max(1.0, rows / x.Sh / bm);
       cycles += per_chunk * (chunks - 1.0);
-      if (!found || cycles * handicap(x) < best.cycles * 0.995 * handicap(best.t)) { best.t = x; best.cycles = cycles; found = true; }
+      if (!found || cycles < best.cycles * 0.995) { best.t = x; best.cycles = cycles; found = true; }
       return;
     }
   };
@@ -342,7 +341,7 @@ static bool wave_best(const WaveModel& M, int c, int ctas, double rows, double m
         const double product = tc ? 1500 + rs * m.inp / 8.0 : 600 + (rs + 4) * outs * m.inp / fma;
         const double rest = 1600 + rs * x.R / 4 * (t.lstm ? 20.0 : K.kind == LIN_F ? 2.0 : 3.0);
         offer(x, gather + weights + product + rest);
-        if (!tc && !t.lstm && outs <= 128) {
+        if (use_split && !tc && !t.lstm && outs <= 128) {
           x.split = outs <= 64 ? 64 : 128;
           offer(x, gather + rs * m.inp / 4 * split_gather + weights * split_weights + split_product(m.inp) + rest, split_chunk + split_product(m.inp), m.inp);
         }
@@ -364,7 +363,7 @@ static bool wave_best(const WaveModel& M, int c, int ctas, double rows, double m
         const double per4 = t.lstm ? 17.0 * t.H4 : m.outp / 4 * (K.kind == GRU_DC ? 12.0 : 3.4);
         const double weights = std::min(1.0, upd) * x.R * m.outp * 4.0 / bpc, rest = 1700 + rs * x.R / 4 * 1.5;
         offer(x, 1500 + rs * per4 + weights + 600 + (rs + 4) * x.R * m.outp / fma + rest);
-        if (!t.lstm && x.R <= 128) {
+        if (use_split && !t.lstm && x.R <= 128) {
           x.split = x.R <= 64 ? 64 : 128;
           offer(x, 1500 + rs * (per4 + m.outp / 4 * split_gather) + weights * split_weights + split_product(m.outp) + rest, split_chunk + split_product(m.outp), m.outp);
         }
@@ -374,7 +373,7 @@ static bool wave_best(const WaveModel& M, int c, int ctas, double rows, double m
     case ACC:
       // Tiles on the tensor cores: the operands' way into shared memory is what counts, so a tile is as nearly square as its count allows.
       // Column Ci of the instruction's at most 128 is the bias gradient's.
-      for (int to = 1; to <= std::min(ctas, m.outp / 4); to++) {
+      for (int to = 1; use_split && to <= std::min(ctas, m.outp / 4); to++) {
         const int R = pad4i((m.outp + to - 1) / to);
         if (R > 128 || (m.outp + R - 1) / R != to) continue;
         for (int ti = 1; to * ti <= ctas && ti <= m.inp / 4; ti++) {
@@ -442,7 +441,7 @@ static bool wave_best(const WaveModel& M, int c, int ctas, double rows, double m
 }
 
 
-static WavePlan wave_place(const ampnet_graph* g, const WaveModel& M, const WaveData& W, int mak, int muf, bool eval, long long n_order, long long n_loaded, int n_ctas) {
+static WavePlan wave_place_with(const ampnet_graph* g, const WaveModel& M, const WaveData& W, int mak, int muf, bool eval, long long n_order, long long n_loaded, int n_ctas, bool use_split) {
   using namespace wave;
   WavePlan P;
   if (!M.ok || !W.ok || mak > max_keys() || n_loaded < 1) return P;
@@ -462,7 +461,7 @@ static WavePlan wave_place(const ampnet_graph* g, const WaveModel& M, const Wave
   P.teams.resize(nc);
   auto rows_of = [&](int c) { return keys * W.tot.entries[c] / std::max(1.0, steps); };
   auto muf_of = [&](int c) { const int o = g->nodes[M.enc.ppts[M.cells[c].ppt].node].muf_override; return (double)(o > 0 ? o : muf); };
-  auto best = [&](int k, int n, WaveTeam& t) { return wave_best(M, cells[k], n, rows_of(cells[k]), muf_of(cells[k]), eval, budget, mak, use_tc, g, t); };
+  auto best = [&](int k, int n, WaveTeam& t) { return wave_best(M, cells[k], n, rows_of(cells[k]), muf_of(cells[k]), eval, budget, mak, use_tc, use_split, g, t); };
   int used = 0;
   for (int k = 0; k < nc; k++) {
     int n = 1;
@@ -534,6 +533,24 @@ static WavePlan wave_place(const ampnet_graph* g, const WaveModel& M, const Wave
   else if (keys * entries / std::max(1.0, steps) >= 64.0) P.pace = (int)std::max(1.0, std::ceil(keys * (double)n_loaded / std::max(1.0, steps)));
   P.ok = true;
   return P;
+}
+
+// The kernels with products of 32-bit operands on the tensor cores are taken where the cells' estimates fall by a seventh in all: for graph
+// nets, whose cells have some hundred rows a round (ggnn_train 607,000 -> 438,000 estimated, 47.2 -> 44.8 ms; its evaluation 13.3 -> 10.8 ms), not for
+// trees, whose epoch hangs on the embedding's gradients (133,000 -> 121,000 estimated, 31.1 -> 31.9 ms).  Lists and small requests, where the
+// placement itself counts, have no cell of 24 rows a round and are placed once.
+static WavePlan wave_place(const ampnet_graph* g, const WaveModel& M, const WaveData& W, int mak, int muf, bool eval, long long n_order, long long n_loaded, int n_ctas) {
+  using namespace wave;
+  const WavePlan P = wave_place_with(g, M, W, mak, muf, eval, n_order, n_loaded, n_ctas, false);
+  if (!eval && g->opt != 0) return P;                              // (momentum and Adam have no such kernel)
+  if (const char* e = getenv("AMPNET_TENSOR_CORES")) if (atoi(e) == 0) return P;
+  const double steps = std::max(1.0, (double)(eval ? W.tot.steps_eval_sum : W.tot.steps_sum)), keys = (double)std::max<long long>(1, std::min<long long>(mak, n_order));
+  bool rows = false;
+  for (size_t c = 0; c < M.cells.size(); c++) rows |= M.cells[c].mat >= 0 && M.cells[c].kind != HEAD && keys * W.tot.entries[c] / steps >= 24.0;
+  if (!rows) return P;
+  const WavePlan Q = wave_place_with(g, M, W, mak, muf, eval, n_order, n_loaded, n_ctas, true);
+  auto sum = [](const WavePlan& p) { double s = 0; for (auto& t : p.teams) s += t.cycles; return s; };
+  return Q.ok && (!P.ok || sum(Q) < 0.86 * sum(P)) ? Q : P;
 }
 
 // ---- a run -----------------------------------------------------------------------------------------------------------------------

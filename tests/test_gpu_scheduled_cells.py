@@ -461,3 +461,38 @@ def test_many_updates_with_one_key_in_flight_follow_the_oracle(oracle_mod, famil
         for k in op:
             assert np.abs(ep[k] - op[k]).max() <= 1e-3 * np.abs(op[k]).max(), (epoch, g.names[k[0]], k[1])
     e.close()
+
+
+@pytest.mark.parametrize("hidden,n,mak", [(52, 400, 256), (100, 300, 128), (61, 400, 200)])
+def test_tensor_core_products_of_32_bit_operands_match_oracle(oracle_mod, monkeypatch, capfd, hidden, n, mak):
+    """Graph nets whose cells have rows enough for the tensor cores (operands in three bfloat16 parts): widths that end inside a step of
+    sixteen and inside a group of eight, rounds of more rows than a chunk.  The parts' products are as exact as 32-bit multiply-adds,
+    so the tolerances are those of the other epochs."""
+    g, inst = _case("ggnn", (15, hidden, 3), n)
+    monkeypatch.setenv("AMPNET_DEBUG", "1")
+    _epochs_match(oracle_mod, g, inst, mak, 1e-6).close()
+    teams = [line.split() for line in capfd.readouterr().err.splitlines() if line.startswith("[team]")]
+    on_tensor_cores = {t[1] for t in teams if t[t.index("M") + 1] != "0"}
+    assert {"LIN_F", "LIN_DX", "GRU_ZR", "GRU_C", "GRU_DC", "GRU_DZR"} <= on_tensor_cores, on_tensor_cores
+
+
+def test_tensor_core_products_keep_infinities_where_they_belong(oracle_mod, monkeypatch, capfd):
+    """An infinite embedding: its parts are no numbers, but the rows of a tile that hold finite values stay what they are, and an instance has a
+    finite loss exactly where the oracle has one."""
+    import paper_1705_09786_b200 as amp
+    g, inst = _case("ggnn", (15, 52, 3), 400)
+    p = wp.init_params(g)
+    key = next(k for k, v in p.items() if v.shape == (15, 52))
+    p[key][14, 5] = np.inf
+    monkeypatch.setenv("AMPNET_DEBUG", "1")
+    o, e = oracle_mod.Oracle(g), amp.Engine(g)
+    for s in (o, e):
+        s.load_instances(inst, split=1)
+        s.set_params(p)
+    want, got = o.eval(split=1)[2], e.eval(split=1, mak=256)[2]
+    assert any(line.startswith("[team] LIN_F") and line.split()[line.split().index("M") + 1] != "0" for line in capfd.readouterr().err.splitlines())
+    finite = np.isfinite(want)
+    assert 0 < finite.sum() < len(want)
+    np.testing.assert_array_equal(np.isfinite(got), finite)
+    np.testing.assert_allclose(got[finite], want[finite], rtol=3e-5, atol=6e-6)
+    e.close()
