@@ -1454,7 +1454,14 @@ __device__ __noinline__ void accumulate_main(const int team, const int tile, flo
     {
       const int d4 = Z.d4, x4 = Z.x4, ldd = Z.ldd, ldx = Z.ldx, o4 = Z.o0 >> 2, i4 = Z.i0 >> 2;
       float* const Dg = smem + Z.dg; float* const Xg = smem + Z.xg;
-      const Staleness stale(R, count, tile);
+      // staleness: updates of the node since the forward pass (Sec. 3); a warp per 32 rows, loaded before the rows and counted after
+      float version = 0.f;
+      bool message = false, stamped = false;
+      if (tile == 0 && tid < count) {
+        const RowD& r = R[tid];
+        message = r.meta & E_MSG_END; stamped = message && r.a4 != NONE;
+        if (stamped) version = __ldcg(reinterpret_cast<const float*>(S.core.arena + r.a4 + ((r.meta & E_RAW) ? (m.outp >> 2) : 0)));
+      }
       const FastDiv dd((unsigned)d4, Z.ddM);
 #pragma unroll 1
       for (int i = tid; i < count * d4; i += CT) {
@@ -1474,7 +1481,11 @@ __device__ __noinline__ void accumulate_main(const int team, const int tile, flo
           cp16(Xg + b * ldx + 4 * k, S.core.arena + (second ? t.z + c - (t.w & 0xffffu) : t.x + c));
         }
       } else gather_general(R, count, i4, x4, Xg, ldx);
-      stale.count_in(h.n_updates, count, tile);
+      if (tile == 0 && (tid & ~31) < count) {
+        const int stale = message ? (stamped ? max(0, h.n_updates - __float_as_int(version)) : 0) : -1;
+        const unsigned same = __match_any_sync(0xffffffffu, stale);
+        if (stale >= 0 && (same & ((1u << (tid & 31)) - 1u)) == 0) { atomicAdd(&S.stale_hist[min(stale, 63)], __popc(same)); atomicMax(&S.max_stale, stale); }
+      }
     }
     cp_wait();
     bar_compute();
@@ -1549,14 +1560,37 @@ __device__ __noinline__ void accumulate_main(const int team, const int tile, flo
       phase(5);
     }
     if (!(h.flags & H_LAST)) return;
-    if (dirty) {
+    if (dirty) {                                                // publish: for the forward tiles, and transposed for the input-gradient tiles
       pubs++;
       dirty = false;
-      publish_tile(m, pubs, T.G != 0, smem, smem + Z.bm);
+      const int x4 = Z.x4, d4 = Z.d4, ro = Z.ro, o0 = Z.o0, i0 = Z.i0, ldw = Z.ldw;
+      const FastDiv dd((unsigned)d4, Z.ddM), dx((unsigned)x4, Z.dxM);
+      const float* const Wm = smem; const float* const bm = smem + Z.bm;
+      float* const Wp = m.Wp + (size_t)(pubs % PUB) * m.outp * m.inp; float* const WT = m.WTp + (size_t)(pubs % PUB) * m.outp * m.inp;
+#pragma unroll 1
+      for (int i = tid; i < ro * x4; i += CT) { const int o = dx.div(i), c = i - o * x4; *reinterpret_cast<float4*>(Wp + (size_t)(o0 + o) * m.inp + i0 + 4 * c) = *reinterpret_cast<const float4*>(Wm + o * ldw + 4 * c); }
+      if (T.G)
+#pragma unroll 1
+        for (int i = tid; i < d4 * x4; i += CT) {
+          const int c = dd.div(i), o = 4 * (i - c * d4);
+          const float* w = Wm + o * ldw + 4 * c;
+          const float4 a = *reinterpret_cast<const float4*>(w), b = *reinterpret_cast<const float4*>(w + ldw), e = *reinterpret_cast<const float4*>(w + 2 * ldw), f = *reinterpret_cast<const float4*>(w + 3 * ldw);
+          float* t = WT + (size_t)(i0 + 4 * c) * m.outp + o0 + o;
+          *reinterpret_cast<float4*>(t) = make_float4(a.x, b.x, e.x, f.x); *reinterpret_cast<float4*>(t + m.outp) = make_float4(a.y, b.y, e.y, f.y);
+          *reinterpret_cast<float4*>(t + 2 * (size_t)m.outp) = make_float4(a.z, b.z, e.z, f.z); *reinterpret_cast<float4*>(t + 3 * (size_t)m.outp) = make_float4(a.w, b.w, e.w, f.w);
+        }
+      if (i0 == 0) for (int i = tid; i < ro; i += CT) m.bp[(size_t)(pubs % PUB) * m.outp + o0 + i] = bm[i];
     }
     stamp(h);
   }, Nothing(), stamp);                                         // (a round without rows: the version stays)
-  if (end.flags & H_END) write_back(m, smem, smem + Z.bm);
+  if (!(end.flags & H_END)) return;
+  const int ro = Z.ro, ci = Z.ci, o0 = Z.o0, i0 = Z.i0, ldw = Z.ldw;
+#pragma unroll 1
+  for (int i = tid; i < ro * ci; i += CT) {
+    const int o = i / ci, c = i - o * ci, r = real_out(m, o0 + o), k = real_in(m, i0 + c);
+    if (r >= 0 && k >= 0) m.W[(size_t)r * m.in_real + k] = smem[o * ldw + c];
+  }
+  if (i0 == 0) for (int i = tid; i < ro; i += CT) { const int r = real_out(m, o0 + i); if (r >= 0) m.b[r] = smem[Z.bm + i]; }
 }
 
 // The same cell with its sums on the tensor cores: G[b][o]^T X[b][i] over the rows of a chunk, operands in three parts (tc_split.cuh).  After

@@ -463,8 +463,8 @@ def test_many_updates_with_one_key_in_flight_follow_the_oracle(oracle_mod, famil
     e.close()
 
 
-@pytest.mark.parametrize("hidden,n,mak", [(52, 400, 256), (100, 300, 128), (61, 400, 200)])
-def test_tensor_core_products_of_32_bit_operands_match_oracle(oracle_mod, monkeypatch, capfd, hidden, n, mak):
+@pytest.mark.parametrize("hidden,n,mak,training", [(52, 400, 256, False), (61, 400, 200, False), (97, 600, 256, True), (100, 500, 256, True)])
+def test_tensor_core_products_of_32_bit_operands_match_oracle(oracle_mod, monkeypatch, capfd, hidden, n, mak, training):
     """Graph nets whose cells have rows enough for the tensor cores (operands in three bfloat16 parts): widths that end inside a step of
     sixteen and inside a group of eight, rounds of more rows than a chunk.  The parts' products are as exact as 32-bit multiply-adds,
     so the tolerances are those of the other epochs."""
@@ -473,7 +473,7 @@ def test_tensor_core_products_of_32_bit_operands_match_oracle(oracle_mod, monkey
     _epochs_match(oracle_mod, g, inst, mak, 1e-6).close()
     teams = [line.split() for line in capfd.readouterr().err.splitlines() if line.startswith("[team]")]
     on_tensor_cores = {t[1] for t in teams if t[t.index("M") + 1] != "0"}
-    assert {"LIN_F", "LIN_DX", "GRU_ZR", "GRU_C", "GRU_DC", "GRU_DZR"} <= on_tensor_cores, on_tensor_cores
+    assert {"LIN_F", "GRU_ZR", "GRU_C"} <= on_tensor_cores and (not training or {"LIN_DX", "GRU_DC", "GRU_DZR"} <= on_tensor_cores), on_tensor_cores
 
 
 def test_tensor_core_products_keep_infinities_where_they_belong(oracle_mod, monkeypatch, capfd):
@@ -483,7 +483,9 @@ def test_tensor_core_products_keep_infinities_where_they_belong(oracle_mod, monk
     g, inst = _case("ggnn", (15, 52, 3), 400)
     p = wp.init_params(g)
     key = next(k for k, v in p.items() if v.shape == (15, 52))
-    p[key][14, 5] = np.inf
+    holders = [len({i for i in range(inst.n) if token in inst.tokens[inst.offsets[i]:inst.offsets[i + 1]]}) for token in range(15)]
+    token = next(t for t in range(15) if 0.1 < holders[t] / inst.n < 0.9)
+    p[key][token, 5] = np.inf
     monkeypatch.setenv("AMPNET_DEBUG", "1")
     o, e = oracle_mod.Oracle(g), amp.Engine(g)
     for s in (o, e):
