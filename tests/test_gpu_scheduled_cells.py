@@ -477,24 +477,30 @@ def test_tensor_core_products_of_32_bit_operands_match_oracle(oracle_mod, monkey
 
 
 def test_tensor_core_products_keep_infinities_where_they_belong(oracle_mod, monkeypatch, capfd):
-    """An infinite embedding: its parts are no numbers, but the rows of a tile that hold finite values stay what they are, and an instance has a
-    finite loss exactly where the oracle has one."""
+    """An infinite embedding: its parts are no numbers.  Graphs without the token keep their losses; the others' infinities and no-numbers
+    travel through the gates to the read-out, whose ReLU makes a zero of a no-number and keeps an infinity, as in the oracle."""
     import paper_1705_09786_b200 as amp
     g, inst = _case("ggnn", (15, 52, 3), 400)
     p = wp.init_params(g)
     key = next(k for k, v in p.items() if v.shape == (15, 52))
-    holders = [len({i for i in range(inst.n) if token in inst.tokens[inst.offsets[i]:inst.offsets[i + 1]]}) for token in range(15)]
-    token = next(t for t in range(15) if 0.1 < holders[t] / inst.n < 0.9)
-    p[key][token, 5] = np.inf
+    holds = np.array([[token in inst.tokens[inst.offsets[i]:inst.offsets[i + 1]] for i in range(inst.n)] for token in range(15)])
+    token = next(t for t in range(15) if 0.1 < holds[t].mean() < 0.9)
     monkeypatch.setenv("AMPNET_DEBUG", "1")
     o, e = oracle_mod.Oracle(g), amp.Engine(g)
     for s in (o, e):
         s.load_instances(inst, split=1)
-        s.set_params(p)
-    want, got = o.eval(split=1)[2], e.eval(split=1, mak=256)[2]
-    assert any(line.startswith("[team] LIN_F") and line.split()[line.split().index("M") + 1] != "0" for line in capfd.readouterr().err.splitlines())
-    finite = np.isfinite(want)
-    assert 0 < finite.sum() < len(want)
-    np.testing.assert_array_equal(np.isfinite(got), finite)
-    np.testing.assert_allclose(got[finite], want[finite], rtol=3e-5, atol=6e-6)
+    losses = []
+    for value in (p[key][token, 5], np.inf):
+        p[key][token, 5] = value
+        for s in (o, e):
+            s.set_params(p)
+        want, got = o.eval(split=1)[2], e.eval(split=1, mak=256)[2]
+        np.testing.assert_array_equal(np.isfinite(got), np.isfinite(want))
+        finite = np.isfinite(want)
+        np.testing.assert_allclose(got[finite], want[finite], rtol=3e-5, atol=6e-6)
+        losses.append(got)
+    changed = losses[0] != losses[1]
+    assert changed[holds[token]].any() and not changed[~holds[token]].any()
+    teams = [line.split() for line in capfd.readouterr().err.splitlines() if line.startswith("[team]")]
+    assert any(t[1] == "LIN_F" and t[t.index("M") + 1] != "0" for t in teams)
     e.close()
