@@ -99,7 +99,6 @@ struct Mat {
 constexpr int PUB = 8;                 // published versions kept (readers lag by less than DRIFT + lag rounds)
 constexpr int LOOKUP_BITS = 8192;      // words of the bit map of touched rows that a tile of a large table keeps in shared memory
 constexpr int N_PHASES = 6;            // cycle counters of a cell's first CTA
-constexpr int PROGRESS_STRIDE = 32;     // words from one progress counter to the next
 constexpr int DRIFT = 4;               // no CTA runs more than this many rounds ahead of another
 
 struct Team {                          // the CTAs of one cell
@@ -125,7 +124,7 @@ struct PptRun {
 struct Core {                          // what every CTA keeps in shared memory
   Program prog;
   amp::Globals* g;
-  unsigned* progress;                  // [teams][16] counters: CTAs that have finished round r, in slot r mod 16
+  unsigned* progress;                  // [teams][16]: CTAs that have finished round r, in slot r mod 16
   float4* arena; unsigned slot4; int copies;     // floats of a key / 4; arenas a key alternates between
   const long long* order; long long n_order;
   const unsigned char* inference_only;

@@ -441,9 +441,7 @@ __device__ __noinline__ void helper_main(const int team, const int cta, const in
   }
 }
 
-// A counter has a line of its own: most CTAs poll one at any time, and neighbours in a line (one slice of the L2) made them wait for each
-// other's requests.
-__device__ __forceinline__ unsigned* progress_of(const int team, const int round) { return S.core.progress + (team * 16 + (round & 15)) * PROGRESS_STRIDE; }
+__device__ __forceinline__ unsigned* progress_of(const int team, const int round) { return S.core.progress + team * 16 + (round & 15); }
 
 // ---- compute warps: waiting, signalling -------------------------------------------------------------------------------------
 // Warp 0: the publishing cell has finished the round `lag` back; the cells this one reads have finished the previous round, everybody the

@@ -581,7 +581,7 @@ static WaveScratch wave_carve(ampnet_graph* g, HostDataset& D, const WaveModel& 
   R.core.loss_out = C.take<double>(nl);
   S.loss_at = C.used - nl * sizeof(double);
   S.read_bytes = C.used;
-  R.core.progress = C.take<unsigned>((size_t)MAX_CELLS * 16 * PROGRESS_STRIDE);
+  R.core.progress = C.take<unsigned>(MAX_CELLS * 16);
   g->d_stats.assign(np, nullptr);
   g->d_update_log.assign(np, nullptr);
   R.core.n_teams = (int)P.teams.size(); R.n_mats = (int)M.mats.size(); R.n_ppts = (int)np; R.core.n_ctas = P.n_ctas;
@@ -614,7 +614,9 @@ static WaveScratch wave_carve(ampnet_graph* g, HostDataset& D, const WaveModel& 
     if (H.kind == LOOKUP) {
       auto zeroed = [&](size_t n_floats) { float* a = B.take<float>(n_floats); if (!dry) g->zero_regions.push_back({a, n_floats * sizeof(float)}); return a; };
       int T = 1;
-      for (auto& t : P.teams) if (t.t.kind == LOOKUP_B && t.t.ppt == (int)p) T = t.t.T;
+      bool small = false;                                          // (a small table's sums stay in shared memory)
+      for (auto& t : P.teams) if (t.t.kind == LOOKUP_B && t.t.ppt == (int)p) { T = t.t.T; small = t.t.R > 0; }
+      if (small) continue;
       Q.A = zeroed(H.nW);
       const size_t segs = (size_t)(Q.out4 + 31) / 32, ids = (size_t)(H.in + T - 1) / T;      // a list per tile and warp
       const size_t words = (ids * segs + 31) / 32;
