@@ -1034,7 +1034,7 @@ __device__ __noinline__ void forward_main(const int team, const int tile, float*
   const int NTC = (T.BM + 15) & ~15, YP = pad_ld(nB);
   const size_t w_floats = SPLIT ? parts_bytes(G * T.R, K) / 4 : tcm ? (size_t)tc::M * K / 2 : (size_t)G * T.R * ld;
   const size_t x_floats = SPLIT ? parts_bytes(tc3::rows_padded(T.BM, T.split), K) / 4 : tcm ? (size_t)NTC * K / 2 : (size_t)T.BM * ld;
-  float *Ws = smem, *Xs = Ws + w_floats, *bs = Xs + x_floats, *Ys = bs + ((G * T.R + 3) & ~3), *Zs = Ys + (size_t)T.BM * YP;      // Zs: a GRU's z and h columns
+  float *Ws = smem, *bs = Ws + w_floats + (SPLIT ? x_floats : 0), *Xs = SPLIT ? Ws + w_floats : bs + ((G * T.R + 3) & ~3), *Ys = SPLIT ? bs + ((G * T.R + 3) & ~3) : Xs + x_floats, *Zs = Ys + (size_t)T.BM * YP;      // Zs: a GRU's z and h columns
   unsigned char *const Wb = reinterpret_cast<unsigned char*>(Ws), *const Xb = reinterpret_cast<unsigned char*>(Xs);
   unsigned have = 0;
   const FastDiv dj4(max(jn >> 2, 1));
