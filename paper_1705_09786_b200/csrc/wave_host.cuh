@@ -311,8 +311,9 @@ static bool wave_best(const WaveModel& M, int c, int ctas, double rows, double m
     }
   };
   const double bpc = 36, fma = 40;
-  // products of 32-bit operands on the tensor cores: four instructions a step of sixteen, whatever the rows, and the accumulators' way back
-  const double acc_base = 5000, acc_row = 0.17, acc_chunk = 3500;
+  // Products of 32-bit operands on the tensor cores: four instructions a step of sixteen, whatever the rows, and the accumulators' way back; splitting
+  // costs the gather and the weights' reload half as much again.  Estimated and measured cycles: edge cell of 102 rows 20,900 / 25,900 (two chunks in
+  // one round of five), 82 rows 12,800 / 17,400; in evaluation, 49 rows, 10,700 / 11,700.
   const double split_gather = 0.7, split_weights = 1.5, split_chunk = 5000;
   auto split_product = [eval](const int k) { return 1300 + 4 * (eval ? 57.0 : 30.0) * tc3::k_steps(k) + 150.0 * tc3::chains(k); };
   int env_rows = 0, env_cols = 0;
@@ -371,8 +372,9 @@ static bool wave_best(const WaveModel& M, int c, int ctas, double rows, double m
       }
       break;
     case ACC:
-      // Tiles on the tensor cores: the operands' way into shared memory is what counts, so a tile is as nearly square as its count allows.
-      // Column Ci of the instruction's at most 128 is the bias gradient's.
+      // Tiles on the tensor cores: the operands' way into shared memory is what counts, so a tile is as large as its count allows (whole matrices of
+      // 100 x 100, 82 rows a round: estimated 25,800, measured 27,000-28,700 cycles in one CTA, multiply-adds 33,000; tiles of 20 x 20 take 69,000 for
+      // 509 rows, multiply-adds 36,000).  Column Ci of the instruction's at most 128 is the bias gradient's.
       for (int to = 1; use_split && to <= std::min(ctas, m.outp / 4); to++) {
         const int R = pad4i((m.outp + to - 1) / to);
         if (R > 128 || (m.outp + R - 1) / R != to) continue;
@@ -381,7 +383,7 @@ static bool wave_best(const WaveModel& M, int c, int ctas, double rows, double m
           x.R = R; x.C = pad4i((m.inp + ti - 1) / ti);
           if (x.C > 124 || (m.inp + x.C - 1) / x.C != ti) continue;
           x.T = x.n = to * ti; x.split = R <= 64 ? 64 : 128;
-          offer(x, 2.4 * (acc_base + rows * (8 + acc_row * (x.R + x.C)) + upd * acc_chunk + std::min(1.0, upd) * (double)x.R * x.C / 5), acc_chunk);
+          offer(x, 12000 + rows * (19 + 0.41 * (x.R + x.C)) + upd * 8400 + std::min(1.0, upd) * (double)x.R * x.C / 2, 3500.0);
         }
       }
       for (int LO = 1; LO <= 8; LO *= 2)
