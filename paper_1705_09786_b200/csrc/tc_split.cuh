@@ -54,6 +54,14 @@ __device__ __forceinline__ float value(const unsigned char* base, const unsigned
   const float h = at(0);
   return finite(h) ? h + (at(part) + at(2 * part)) : h;
 }
+// Columns 4 c4 .. of row r: the 32-bit values themselves.
+__device__ __forceinline__ float4 load4(const unsigned char* base, const unsigned part, const unsigned group, const int r, const int c4) {
+  const unsigned char* const p = base + (unsigned)(r >> 3) * group + (unsigned)(c4 >> 1) * CORE_K + (unsigned)(r & 7) * 16u + (unsigned)(c4 & 1) * 8u;
+  const uint2 h = *reinterpret_cast<const uint2*>(p), m = *reinterpret_cast<const uint2*>(p + part), l = *reinterpret_cast<const uint2*>(p + 2 * part);
+  auto low = [](const unsigned a, const unsigned b, const unsigned c) { const float x = __uint_as_float(a << 16); return finite(x) ? x + (__uint_as_float(b << 16) + __uint_as_float(c << 16)) : x; };
+  auto high = [](const unsigned a, const unsigned b, const unsigned c) { const float x = __uint_as_float(a & 0xffff0000u); return finite(x) ? x + (__uint_as_float(b & 0xffff0000u) + __uint_as_float(c & 0xffff0000u)) : x; };
+  return make_float4(low(h.x, m.x, l.x), high(h.x, m.x, l.x), low(h.y, m.y, l.y), high(h.y, m.y, l.y));
+}
 __device__ __forceinline__ void fence_operands() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
 // ---- tensor memory: one warp allocates and frees ---------------------------------------------------------------------

@@ -914,9 +914,7 @@ __device__ __noinline__ void tensor_rows_general(const RowD* R, const int count,
 struct Parts {                         // an operand in shared memory
   unsigned char* base; unsigned part, group;
   __device__ __forceinline__ void put(const int r, const int c4, const float4 v) const { tc3::store4(base, part, group, r, c4, v); }
-  __device__ __forceinline__ float4 get(const int r, const int c4) const {
-    return make_float4(tc3::value(base, part, group, r, 4 * c4), tc3::value(base, part, group, r, 4 * c4 + 1), tc3::value(base, part, group, r, 4 * c4 + 2), tc3::value(base, part, group, r, 4 * c4 + 3));
-  }
+  __device__ __forceinline__ float4 get(const int r, const int c4) const { return tc3::load4(base, part, group, r, c4); }
 };
 __host__ __device__ __forceinline__ int split_columns(const int Ci) { return (Ci + 1 + 15) & ~15; }      // of an accumulator's instruction: the tile's and the ones
 __host__ __device__ __forceinline__ size_t parts_bytes(const int rows, const int K) { return (size_t)3 * ((rows + 7) >> 3) * tc3::group_bytes(K); }
