@@ -344,7 +344,10 @@ static bool wave_best(const WaveModel& M, int c, int ctas, double rows, double m
         offer(x, gather + weights + product + rest);
         if (use_split && !tc && !t.lstm && outs <= 128) {
           x.split = outs <= 64 ? 64 : 128;
-          offer(x, gather + rs * m.inp / 4 * split_gather + weights * split_weights + split_product(m.inp) + rest, split_chunk + split_product(m.inp), m.inp);
+          // (a gate's exponentials and its share of the input that is kept, of 66 rows 9,000-10,000 cycles in training; without them the gates get too few
+          // CTAs and the epoch of the graph net is 44.0 ms, with half as much 41.6, with these 39.6)
+          const double gates = eval || K.kind == LIN_F ? 0.0 : rs * x.R / 4 * (K.kind == GRU_ZR ? 24.0 : 16.0);
+          offer(x, gather + rs * m.inp / 4 * split_gather + weights * split_weights + split_product(m.inp) + rest + gates, split_chunk + split_product(m.inp), m.inp);
         }
         if (tc || env_rows) break;
       }
@@ -538,7 +541,7 @@ static WavePlan wave_place_with(const ampnet_graph* g, const WaveModel& M, const
 }
 
 // The kernels with products of 32-bit operands on the tensor cores are taken where the cells' estimates fall by a seventh in all: for graph
-// nets, whose cells have some hundred rows a round (ggnn_train 607,000 -> 438,000 estimated, 47.2 -> 44.8 ms; its evaluation 13.3 -> 10.8 ms), not for
+// nets, whose cells have some hundred rows a round (607,000 -> 450,000 estimated, an epoch 47.2 -> 39.6 ms; evaluation 13.3 -> 10.8 ms), not for
 // trees, whose epoch hangs on the embedding's gradients (133,000 -> 121,000 estimated, 31.1 -> 31.9 ms).  Lists and small requests, where the
 // placement itself counts, have no cell of 24 rows a round and are placed once.
 static WavePlan wave_place(const ampnet_graph* g, const WaveModel& M, const WaveData& W, int mak, int muf, bool eval, long long n_order, long long n_loaded, int n_ctas) {
